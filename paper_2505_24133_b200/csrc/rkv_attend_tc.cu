@@ -121,7 +121,7 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     constexpr bool kFp8 = kSrc != 0;            // the tiles pass through the softmax threads on their way to the tensor cores
     constexpr int kDim = kSrc == 2 ? 64 : kHeadDim;          // head dimension of the caches, the queries and the output
     extern __shared__ uint8_t att_tc_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(att_tc_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *smem = align_smem(att_tc_raw);
     const uint32_t sbase = smem_u32(smem);
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + kOffMisc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + kOffMisc + 4);

@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
     using namespace sm100;
     constexpr int D = kHeadDim;
     extern __shared__ uint8_t prep_tc_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(prep_tc_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *smem = align_smem(prep_tc_raw);
     uint8_t *bop = smem + kPrepTcBufs * kPrepTcTile;
     const uint32_t sbase = smem_u32(smem);
     __shared__ __align__(8) unsigned long long bars[kPrepTcBufs + 1];      // tile landed (per buffer); product done
@@ -492,7 +492,7 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
     using namespace sm100;
     constexpr int D = kHeadDim;
     extern __shared__ uint8_t prep_tc_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(prep_tc_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *smem = align_smem(prep_tc_raw);
     uint8_t *bop = smem + kFusedOffB;
     const uint32_t sbase = smem_u32(smem);
     __shared__ __align__(8) unsigned long long bars[3];      // stored tile landed (per stage); product done

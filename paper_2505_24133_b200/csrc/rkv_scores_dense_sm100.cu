@@ -70,7 +70,7 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 {
     unsigned long long *const item_count = p.counters + kDenseWords, *const ticket = item_count + 1;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *smem = align_smem(smem_raw);
     const uint32_t sbase = smem_u32(smem);
     int4 *items = reinterpret_cast<int4 *>(smem + kOffItems);
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + kOffMisc);

@@ -92,7 +92,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                            int q_rows_pad)
 {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *smem = align_smem(smem_raw);
     const uint32_t sbase = smem_u32(smem);
     const SmemPlan pl = make_plan(q_rows_pad);
     int4 *items = reinterpret_cast<int4 *>(smem + pl.off_items);

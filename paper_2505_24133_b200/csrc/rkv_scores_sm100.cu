@@ -70,7 +70,7 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
                     int row_blocks, int q_rows_pad)
 {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *smem = align_smem(smem_raw);
     const uint32_t sbase = smem_u32(smem);
     float *r_s = reinterpret_cast<float *>(smem + kOffR);
     float *sum_s = reinterpret_cast<float *>(smem + kOffS);

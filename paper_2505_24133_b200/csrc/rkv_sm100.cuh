@@ -13,6 +13,10 @@ constexpr long long kWaitCycles = 4000000000ll;   // default limit of a wait, ab
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// The dynamic shared memory from its first 1024-byte boundary on, by pointer arithmetic: an address that has been through an
+// integer is a generic one to the compiler, and every access through it is resolved at run time.
+__device__ __forceinline__ uint8_t *align_smem(uint8_t *raw) { return raw + ((1024u - (smem_u32(raw) & 1023u)) & 1023u); }
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
@@ -38,17 +42,30 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// The same, the thread asleep for up to about 20 us while the phase is not complete: warps that poll take issue slots from
+// those that work.
+__device__ __forceinline__ bool mbar_try_wait_asleep(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(20000u)
+        : "memory");
+    return ok != 0;
+}
+
 // Bounded wait.  Returns false if the block is aborting (this wait ran out of time, or another one did).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, const ErrSink &sink)
 {
     if (mbar_try_wait(bar, parity)) return true;
     const long long start = clock64();
-    for (uint32_t it = 1;; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((it & 63u) == 0u) {
-            if (*abort_flag) return false;
-            if (clock64() - start > sink.wait_cycles) break;
-        }
+    while (true) {
+        if (mbar_try_wait_asleep(bar, parity)) return true;
+        if (*abort_flag) return false;
+        if (clock64() - start > sink.wait_cycles) break;
     }
     *abort_flag = 1;
     report_timeout(sink);
