@@ -1,0 +1,119 @@
+"""Kernels and dispatch rules at the sizes where they can go wrong: tile remainders, the smallest and largest of a range,
+the points where one variant hands over to another.  Tolerances are those of parity_util and test_gpu_decode."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import rkv_inputs as ri
+from test_gpu_parity import rkv, run_and_check, small_spec  # noqa: F401  (rkv: the fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,beta,T", [("bf16", 1, 0.5), ("bf16", 3, 0.5), ("bf16", 1, 0.9), ("fp8", 2, 0.5)])
+@pytest.mark.parametrize("budget,buffer,lens", [(100, 36, [136, 135, 101]), (256, 137, [393, 265, 264]), (17, 8, [25, 18, 17])])
+def test_row_block_scoring_of_256_dimensions(rkv, dtype, beta, T, budget, buffer, lens):  # noqa: F811
+    """Operand tiles in two 128-column blocks: one row tile and two, n = 128, 127, 385, 257, 256, a cache of one small tile."""
+    spec = small_spec("rb256", batch=3, hkv=2, hq=8, budget=budget, buffer=buffer, head_dim=256, dtype=dtype, span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=401 + budget, seq_lens=torch.tensor(lens))
+    rep, comp = run_and_check(rkv, wl, beta=beta, T=T)
+    assert rep.ok(), rep.errors
+    assert rep.compressed_heads == 2 * sum(L > budget for L in lens)
+    comp.check_status()
+
+
+@pytest.mark.parametrize("head_dim,hq,alpha", [(64, 2, 8), (128, 8, 8), (128, 18, 8), (256, 6, 5)])
+@pytest.mark.parametrize("budget,buffer,lens", [(40, 32, [72, 71, 41]), (110, 90, [200, 137, 136])])
+def test_cuda_core_scoring_tiles(rkv, head_dim, hq, alpha, budget, buffer, lens):  # noqa: F811
+    """64-row blocks and 64- (d = 256: 32-) key steps: n = 64, 63, 33, 192, 129, 128; one and two passes over the query rows
+    (72 rows: more than a block of 64)."""
+    spec = small_spec("simt", batch=3, hkv=2, hq=hq, budget=budget, buffer=buffer, alpha=alpha, head_dim=head_dim, dtype="f32", span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=411 + hq, seq_lens=torch.tensor(lens))
+    for b, L in enumerate(lens):
+        wl.k_cache[b, :, L:] = float("nan")
+    rep, comp = run_and_check(rkv, wl, beta=2)
+    assert rep.ok(), rep.errors
+    comp.check_status()
+
+
+@pytest.mark.parametrize("batch,hkv,hq,cap", [(1, 1, 4, 128), (1, 1, 4, 8192), (2, 1, 8, 2176), (1, 2, 2, 1920), (1, 2, 2, 1921),
+                                              (40, 8, 16, 640)])
+def test_decode_attention_splits(rkv, batch, hkv, hq, cap):  # noqa: F811
+    """One block per head up to the largest cluster (16 blocks), more key tiles than one block holds (15), many heads with a
+    single split; lengths that leave the last blocks of a cluster without a row."""
+    spec = ri.CacheSpec("split", 1, batch, hkv, hq, 128, cap - 64, 64, 8, 0.1, "bf16", 16, 0.3, 0.05, 4, 8.0)
+    lens = [(cap, cap - 1, 1, cap // 2, 129)[b % 5] if b else cap for b in range(batch)]
+    if batch == 1:
+        lens = [max(1, cap - 130)]
+    wl = ri.make_workload(spec, device="cuda", seed=421, seq_lens=torch.tensor(lens))
+    for b, L in enumerate(lens):
+        wl.k_cache[b, :, L:] = float("nan")
+        wl.v_cache[b, :, L:] = float("nan")
+    g = torch.Generator(device="cuda").manual_seed(7)
+    q_new = torch.randn(batch, hq, 128, generator=g, device="cuda").to(torch.bfloat16)
+    comp = rkv.Compressor(batch, hkv, hq, spec.budget, spec.buffer, spec.alpha, 0.1)
+    out = torch.full((batch, hq, 128), 7.0, device="cuda")
+    for _ in range(2):                              # back to back: the second starts while the first is still running
+        assert rkv.rkv_decode_attention(comp.desc, wl.k_cache, wl.v_cache, q_new, wl.seq_lens, out, spec.budget, spec.buffer) == 0
+    torch.cuda.synchronize()
+    comp.check_status()
+    K, V = (torch.nan_to_num(t.float(), nan=0.0).cpu().numpy() for t in (wl.k_cache, wl.v_cache))
+    ref = oracle.oracle_decode_attention(K, V, q_new.float().cpu().numpy(), np.array(lens, dtype=np.int32))
+    got = out.cpu().numpy().astype(np.float64)
+    scale = np.maximum(np.abs(ref).max(axis=-1, keepdims=True), 1e-30)
+    assert (np.abs(got - ref) <= 1e-3 * scale + 1e-7).all(), float((np.abs(got - ref) / scale).max())
+
+
+@pytest.mark.parametrize("hkv,head_dim,dtype", [(1, 64, torch.bfloat16), (32, 128, torch.float32)])
+def test_append_rows_of_one_block(rkv, hkv, head_dim, dtype):  # noqa: F811
+    """A sequence's new rows are moved by one block: 8 vectors and 1024 (several per thread); appends in a row, the last one
+    into a cache that is full by then."""
+    batch, budget, buffer = 3, 24, 8
+    cap = budget + buffer
+    comp = rkv.Compressor(batch, hkv, hkv, budget, buffer, 8, 0.1, dtype=dtype, head_dim=head_dim)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    k = torch.randn(batch, hkv, cap, head_dim, generator=g, device="cuda").to(dtype)
+    v, want_k, want_v = k + 1, k.clone(), k + 1
+    lens = torch.tensor([0, cap - 2, cap], dtype=torch.int32, device="cuda")
+    length = lens.tolist()
+    for step in range(3):
+        kn = torch.randn(batch, hkv, head_dim, generator=g, device="cuda").to(dtype)
+        vn = kn * 2
+        assert rkv.rkv_append(comp.desc, k, v, kn, vn, lens, budget, buffer) == 0
+        for b in range(batch):
+            if length[b] < cap:
+                want_k[b, :, length[b]], want_v[b, :, length[b]] = kn[b], vn[b]
+                length[b] += 1
+    torch.cuda.synchronize()
+    assert lens.tolist() == length == [3, cap, cap]
+    assert torch.equal(k, want_k) and torch.equal(v, want_v)
+    assert int(comp.status.item()) == 1              # the full cache was reported
+
+
+@pytest.mark.parametrize("batch", [7, 17])
+def test_host_buffers_in_pieces(rkv, batch):  # noqa: F811
+    """The host-buffer form cuts larger batches into pieces of whole sequences: uneven pieces (33 and 80 MB of caches), two
+    calls in a row on the same buffers' copies, ragged lengths, per-sequence budgets."""
+    spec = small_spec("pieces", batch=batch, hkv=8, hq=16, budget=1024, buffer=128, span=32)
+    lens = [spec.cap - 9 * (b % 5) for b in range(batch)]
+    lens[2] = 900
+    budgets = torch.tensor([spec.budget - 13 * (b % 3) for b in range(batch)])
+    wl = ri.make_workload(spec, device="cuda", seed=431, seq_lens=torch.tensor(lens))
+    ch = rkv.Compressor(batch, 8, 16, spec.budget, spec.buffer, 8, 0.1, host_staging=True, budgets=budgets)
+    got = []
+    for _ in range(2):
+        hk, hv, hq, hs = (t.cpu().pin_memory() for t in (wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens))
+        hidx = torch.empty(batch, 8, spec.budget, dtype=torch.int32).pin_memory()
+        ch.compress_host(hk, hv, hq, hs, hidx)
+        got.append((hk, hv, hs, hidx))
+    cd = rkv.Compressor(batch, 8, 16, spec.budget, spec.buffer, 8, 0.1, budgets=budgets)
+    idx = cd.compress(wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens)
+    torch.cuda.synchronize()
+    ch.check_status()
+    for hk, hv, hs, hidx in got:
+        assert torch.equal(hidx, idx.cpu()) and torch.equal(hs, wl.seq_lens.cpu())
+        for b in range(batch):
+            n = int(hs[b])
+            assert torch.equal(hk[b, :, :n].view(torch.int16), wl.k_cache[b, :, :n].cpu().view(torch.int16))
+            assert torch.equal(hv[b, :, :n].view(torch.int16), wl.v_cache[b, :, :n].cpu().view(torch.int16))
