@@ -392,11 +392,10 @@ cudaError_t launch_attend(const void *k_cache, const void *v_cache, const void *
     p.block_table = block_table;
     p.d_out = head_dim;
     cudaError_t e;
-    if (attend_uses_tc(G, dtype))
-        e = launch_attend_tc(k_cache, v_cache, q_new, seq_lens, out, partial, batch, hkv, hq, cap, splits, status, wait_cycles,
-                             block_table, pool_pages, dtype == RKV_FP8_E4M3 ? 1 : (head_dim == 64 ? 2 : 0), s);
-    else
-        e = launch_dtype<float>(p, G, s);
+    if (attend_uses_tc(G, dtype))           // (merges its splits itself)
+        return launch_attend_tc(k_cache, v_cache, q_new, seq_lens, out, batch, hkv, hq, cap, splits, status, wait_cycles,
+                                block_table, pool_pages, dtype == RKV_FP8_E4M3 ? 1 : (head_dim == 64 ? 2 : 0), s);
+    e = launch_dtype<float>(p, G, s);
     if (e != cudaSuccess || splits == 1) return e;
     attend_merge_kernel<<<(unsigned)(batch * hkv * G), kHeadDim, 0, s>>>(p, G);
     return cudaGetLastError();

@@ -17,7 +17,9 @@
 // maximum per query over the whole split is taken, so the weights need no running rescale; then the V tiles stream
 // through the same ring while the softmax threads turn score columns into P tiles (double-buffered).  Every weight
 // is split into two bf16 parts (rows g and 8 + g of P: N = 16 has the room), so the products carry fp32-accurate
-// weights; the sum of the weights is taken from the same parts.  Splits are merged by attend_merge_kernel.
+// weights; the sum of the weights is taken from the same parts.  The splits of a head are one thread-block cluster: each
+// leaves its partial result in its shared memory, then every block merges a share of the outputs from all of them (a merge
+// kernel of its own behind this one took 4 us of a decode step's 33 per layer).
 //
 // Warps 0..3: softmax (thread = TMEM lane = key row of a tile, later = output dimension), warp 4: TMA producer,
 // warp 5: MMA issuer and TMEM owner.
@@ -28,7 +30,7 @@
 // row.  Rows beyond the length are written as zeros there.
 //
 // Every mbarrier wait is bounded; on expiry the block records RKV_ERR_TIMEOUT,
-// writes zeros and leaves through the common exit that frees TMEM.  No TMA multicast, no cluster launch.
+// writes zeros and leaves through the common exit that frees TMEM.  No TMA multicast.
 #include "rkv_sm100.cuh"
 
 namespace rkv {
@@ -40,6 +42,7 @@ using namespace sm100;
 constexpr int kTcThreads = 192;
 constexpr int kTcStages = 3;                         // ring of key / value tiles
 constexpr int kTcMaxTiles = 15;                      // key tiles per block
+constexpr int kTcMaxSplits = 16;                     // blocks of a cluster
 constexpr int kTcHalf = kTile * 64 * 2;              // one TMA box: 128 rows x 64 bf16
 constexpr int kTcTileBytes = 2 * kTcHalf;            // 32 KB
 constexpr int kTcSmall = 16 * kHeadDim * 2;          // a [16 x 128] bf16 operand (Q^T or P): two [16 x 64] halves of 2 KB
@@ -75,7 +78,6 @@ static_assert(16 + 16 * kTcMaxTiles <= (int)kTcTmemCols, "TMEM columns");
 struct AttendTcParams {
     const int32_t *seq_lens;
     float *out;                 // [batch][hq][d]
-    float *partial;             // [P][splits][G][d + 2]: unnormalised output, maximum (base-2 domain), sum of weights
     int batch, hkv, hq, cap, splits, tiles_per_split;
     int32_t *status;
     long long wait_cycles;
@@ -97,6 +99,19 @@ __device__ __forceinline__ void tmem_wait16(uint32_t (&r)[16])
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
                    "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
                  :: "memory");
+}
+// a float of block `rank` of the cluster, at the shared-memory address `addr` of this block
+__device__ __forceinline__ float ld_cluster(uint32_t addr, int rank)
+{
+    uint32_t remote;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // barrier among the 128 softmax threads only
 __device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
@@ -132,32 +147,6 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     const int head = blockIdx.x / p.splits, split = blockIdx.x % p.splits;
     const int b = head / p.hkv, h = head % p.hkv;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int L = p.seq_lens[b];
-    if (L < 0 || L > p.cap) {               // reported, and treated as an empty cache
-        report(p.status, RKV_ERR_INVALID_ARG);
-        L = 0;
-    }
-    const int t0 = split * p.tiles_per_split;                       // first key tile of this block
-    const int T = min(min(p.tiles_per_split, kTcMaxTiles), (L + kTile - 1) / kTile - t0);      // its tiles (<= 0: none)
-    constexpr int kStride = kHeadDim + 2;
-    float *part = p.partial + ((size_t)head * p.splits + split) * G * kStride;
-    float *out = p.out + ((size_t)b * p.hq + (size_t)h * G) * kDim;
-
-    if (T <= 0) {       // no cached row falls into this split (uniform for the block: nothing was allocated yet)
-        for (int x = threadIdx.x; x < G * kDim; x += kTcThreads) {
-            const int g = x / kDim, c = x % kDim;
-            if (p.splits == 1) {
-                out[(size_t)g * kDim + c] = 0.f;
-            } else {
-                part[g * kStride + c] = 0.f;
-                if (c == 0) {
-                    part[g * kStride + kHeadDim] = -INFINITY;
-                    part[g * kStride + kHeadDim + 1] = 0.f;
-                }
-            }
-        }
-        return;
-    }
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kTcStages; ++s) {
@@ -192,13 +181,34 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
+    pdl_trigger();
+    pdl_wait();                             // what is above reads nothing that an earlier kernel writes
+
+    int L = p.seq_lens[b];
+    if (L < 0 || L > p.cap) {               // reported, and treated as an empty cache
+        report(p.status, RKV_ERR_INVALID_ARG);
+        L = 0;
+    }
+    const int t0 = split * p.tiles_per_split;                       // first key tile of this block
+    const int T = min(min(p.tiles_per_split, kTcMaxTiles), (L + kTile - 1) / kTile - t0);      // its tiles (<= 0: none)
+    constexpr int kStride = kHeadDim + 2;
+    float *part = reinterpret_cast<float *>(smem + kOffP);          // [G][d + 2]: unnormalised output, maximum (base-2 domain), sum of weights
+    static_assert(G * kStride * 4 <= 2 * kTcSmall, "the partial result takes the room of P");
+    float *out = p.out + ((size_t)b * p.hq + (size_t)h * G) * kDim;
 
     // where key tile t of the head starts, in rows of the 2-D [rows][d] view of the caches
     auto tile_y = [&](int t) -> int {
         return p.block_table ? p.block_table[(size_t)head * (p.cap / kTile) + t] * kTile : head * p.cap + t * kTile;
     };
 
-    if (warp == 4) {
+    if (T <= 0) {       // no cached row falls into this split (uniform for the block)
+        if (p.splits == 1) {
+            for (int x = threadIdx.x; x < G * kDim; x += kTcThreads) out[x] = 0.f;
+        } else if (threadIdx.x < G) {
+            part[threadIdx.x * kStride + kHeadDim] = -INFINITY;
+            part[threadIdx.x * kStride + kHeadDim + 1] = 0.f;
+        }
+    } else if (warp == 4) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
             mbar_expect_tx(bar(kBarQ), kSrc == 2 ? kTcSmall / 2 : kTcSmall);
@@ -401,6 +411,32 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
         }
     }
 
+    // ---- merge the splits: out = sum_s 2^(m_s - m) num_s / sum_s 2^(m_s - m) l_s, block r of the cluster taking its share
+    if (p.splits > 1) {
+        __syncwarp();
+        cluster_sync();
+        const uint32_t base = smem_u32(part);
+        for (int x = split * kTcThreads + threadIdx.x; x < G * kDim; x += p.splits * kTcThreads) {
+            const int g = x / kDim, c = x % kDim;
+            const uint32_t row = base + (uint32_t)(g * kStride) * 4u;
+            float ms[kTcMaxSplits], m = -INFINITY, num = 0.f, den = 0.f;
+#pragma unroll
+            for (int s = 0; s < kTcMaxSplits; ++s) {
+                ms[s] = s < p.splits ? ld_cluster(row + kHeadDim * 4u, s) : -INFINITY;
+                m = fmaxf(m, ms[s]);
+            }
+#pragma unroll
+            for (int s = 0; s < kTcMaxSplits; ++s) {                   // fixed order; a split without rows has m = -inf
+                if (ms[s] == -INFINITY) continue;
+                const float w = exp2f(ms[s] - m);
+                num = fmaf(w, ld_cluster(row + (uint32_t)c * 4u, s), num);
+                den = fmaf(w, ld_cluster(row + (kHeadDim + 1) * 4u, s), den);
+            }
+            out[x] = den > 0.f ? num / den : 0.f;
+        }
+        cluster_sync();                     // nobody leaves while its partial result is still being read
+    }
+
     // ---------------------------------------------------------------------- common exit
     tc_fence_before();
     __syncthreads();
@@ -415,10 +451,12 @@ template <int G, int kSrc>
 cudaError_t launch_tc_one(const AttendTcParams &p, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
                           cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(attend_tc_kernel<G, kSrc>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-    if (e != cudaSuccess) return e;
-    attend_tc_kernel<G, kSrc><<<(unsigned)(p.batch * p.hkv * p.splits), kTcThreads, kTcSmem, s>>>(p, mk, mv, mq);
-    return cudaGetLastError();
+    static std::atomic<unsigned long long> done{0ull};
+    int dev = 0, sms = 0;
+    cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, attend_tc_kernel<G, kSrc>, kTcSmem, true)) != cudaSuccess) return e;
+    return launch_early(attend_tc_kernel<G, kSrc>, (unsigned)(p.batch * p.hkv * p.splits), kTcThreads, kTcSmem, s,
+                        (unsigned)p.splits, p, mk, mv, mq);
 }
 template <int G>
 cudaError_t launch_tc_for(const AttendTcParams &p, int src, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
@@ -430,26 +468,33 @@ cudaError_t launch_tc_for(const AttendTcParams &p, int src, const CUtensorMap &m
 
 }  // namespace
 
-// Splits of a head's key tiles for the tensor-core kernel: enough blocks for two waves of resident blocks (2 per SM),
-// never more than kTcMaxTiles tiles per block, never finer than a tile.
+// Splits of a head's key tiles (blocks of a cluster) for the tensor-core kernel: at most kTcMaxTiles tiles per block, and
+// among those the number with the shortest run: waves of resident blocks (2 per SM) times what a block spends, its tiles and
+// about two tiles' worth of set-up and merge.  (128 heads of 33 tiles: 4 splits, two waves of 9 tiles, where the earlier rule,
+// the fewest splits that give two waves of blocks, took three waves of 7.)
 int attend_tc_splits(int heads, int cap, int sms)
 {
     const int tiles = (cap + kTile - 1) / kTile;
-    int splits = (4 * sms + heads - 1) / heads;
-    const int least = (tiles + kTcMaxTiles - 1) / kTcMaxTiles;
-    splits = splits < least ? least : splits;
-    return splits > tiles ? tiles : splits;
+    int best = 0;
+    long long best_cost = 0;
+    for (int s = (tiles + kTcMaxTiles - 1) / kTcMaxTiles; s <= tiles && s <= kTcMaxSplits; ++s) {
+        const int per = (tiles + s - 1) / s;
+        if (s > 1 && (tiles + per - 1) / per < s) continue;          // the last blocks would have no tile
+        const long long waves = ((long long)heads * s + 2 * sms - 1) / (2 * sms);
+        const long long cost = waves * (per + 2);
+        if (best == 0 || cost < best_cost) best = s, best_cost = cost;
+    }
+    return best;
 }
 
 cudaError_t launch_attend_tc(const void *k_cache, const void *v_cache, const void *q_new, const int32_t *seq_lens, float *out,
-                             float *partial, int batch, int hkv, int hq, int cap, int splits, int32_t *status,
-                             long long wait_cycles, const int32_t *block_table, long long pool_pages, int src, cudaStream_t s)
+                             int batch, int hkv, int hq, int cap, int splits, int32_t *status, long long wait_cycles,
+                             const int32_t *block_table, long long pool_pages, int src, cudaStream_t s)
 {
     const int tiles = (cap + kTile - 1) / kTile;
     AttendTcParams p;
     p.seq_lens = seq_lens;
     p.out = out;
-    p.partial = partial;
     p.batch = batch;
     p.hkv = hkv;
     p.hq = hq;
@@ -465,7 +510,7 @@ cudaError_t launch_attend_tc(const void *k_cache, const void *v_cache, const voi
     // src: 0 = bf16 caches of 128 dimensions, 1 = E4M3 codes of 128 dimensions, 2 = bf16 caches of 64 dimensions
     const bool maps_ok = src != 0 ? (sm100::make_map_row128(&mk, k_cache, rows, src == 1) && sm100::make_map_row128(&mv, v_cache, rows, src == 1))
                                   : (sm100::make_map(&mk, k_cache, rows, kTile) && sm100::make_map(&mv, v_cache, rows, kTile));
-    const bool q_ok = src == 2 ? sm100::make_map_q64(&mq, q_new, (uint64_t)batch * hq) : sm100::make_map(&mq, q_new, (uint64_t)batch * hq, 16);
+    const bool q_ok = src == 2 ? sm100::make_map_rows(&mq, q_new, (uint64_t)batch * hq, 64, 16) : sm100::make_map(&mq, q_new, (uint64_t)batch * hq, 16);
     if (!maps_ok || !q_ok) return cudaErrorInvalidValue;
     switch (hq / hkv) {
         case 1: return launch_tc_for<1>(p, src, mk, mv, mq, s);

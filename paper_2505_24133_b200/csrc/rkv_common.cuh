@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "rkv.h"
 
 namespace rkv {
@@ -209,6 +211,59 @@ __device__ __forceinline__ void widen16(const uint4 &codes, uint4 *lo, uint4 *hi
     *hi = make_uint4(out[4], out[5], out[6], out[7]);
 }
 
+// ---- launches that overlap the end of the kernel before them (programmatic dependent launch) ----------------------------
+// A kernel launched through launch_early() may become resident while its predecessor in the stream is still running: it
+// lets its own successor in (pdl_trigger) and waits for the predecessor's results (pdl_wait) before it touches global
+// memory.  Between the short kernels of a decode step the launch gap, 2-3 us, is most of the time.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... Args>
+cudaError_t launch_early(void (*kernel)(Args...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, unsigned cluster, Args... args)
+{
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// What a launch asks the runtime for, asked once per device (both idempotent, so threads may race).
+constexpr int kDeviceSlots = 64;
+inline cudaError_t device_sms(int *dev, int *sms)
+{
+    static std::atomic<int> known[kDeviceSlots];
+    cudaError_t e = cudaGetDevice(dev);
+    if (e != cudaSuccess) return e;
+    const bool slot = *dev >= 0 && *dev < kDeviceSlots;
+    *sms = slot ? known[*dev].load(std::memory_order_relaxed) : 0;
+    if (*sms > 0) return cudaSuccess;
+    e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev);
+    if (e == cudaSuccess && slot) known[*dev].store(*sms, std::memory_order_relaxed);
+    return e;
+}
+// The kernel's dynamic shared memory limit (and clusters of more than 8 blocks), set once per device.  `done`: the caller's
+// bit per device.
+template <class Kernel>
+inline cudaError_t allow_smem_once(std::atomic<unsigned long long> &done, int dev, Kernel kernel, int bytes, bool wide_cluster = false)
+{
+    const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+    if (bit && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && wide_cluster) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
+
 // launchers (one per stage); each returns cudaGetLastError() of its launch
 cudaError_t launch_prep(const Params &p, cudaStream_t s);
 cudaError_t launch_widen_keys(const Params &stored, __nv_bfloat16 *wide, int wide_d, const void *q_src, void *q_dst,
@@ -226,8 +281,8 @@ cudaError_t launch_attend(const void *k_cache, const void *v_cache, const void *
                           float *partial, int batch, int hkv, int hq, int cap, int splits, int dtype, int32_t *status,
                           long long wait_cycles, const int32_t *block_table, long long pool_pages, int head_dim, cudaStream_t s);
 cudaError_t launch_attend_tc(const void *k_cache, const void *v_cache, const void *q_new, const int32_t *seq_lens, float *out,
-                             float *partial, int batch, int hkv, int hq, int cap, int splits, int32_t *status,
-                             long long wait_cycles, const int32_t *block_table, long long pool_pages, int src, cudaStream_t s);
+                             int batch, int hkv, int hq, int cap, int splits, int32_t *status, long long wait_cycles,
+                             const int32_t *block_table, long long pool_pages, int src, cudaStream_t s);
 int attend_tc_splits(int heads, int cap, int sms);
 int attend_max_group();
 int attend_splits(int heads, int cap, int sms, int G, int dtype);

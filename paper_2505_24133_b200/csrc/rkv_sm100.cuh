@@ -283,19 +283,23 @@ inline uint64_t key_rows_total(const Params &p)
     return p.block_table ? (uint64_t)p.pool_pages * kTile : (uint64_t)p.batch * p.hkv * p.cap;
 }
 
-// 2-D bf16 view [rows][128] of a contiguous tensor, boxes of box_rows x 64 elements, 128-byte swizzle,
-// out-of-range rows read as zero.
-inline bool make_map(CUtensorMap *map, const void *base, uint64_t rows, uint32_t box_rows)
+// 2-D bf16 view [rows][dim] of a contiguous tensor (dim a multiple of 64), boxes of box_rows x 64 elements, 128-byte
+// swizzle, out-of-range rows read as zero.
+inline bool make_map_rows(CUtensorMap *map, const void *base, uint64_t rows, int dim, uint32_t box_rows)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)kHeadDim, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)kHeadDim * 2};
+    const cuuint64_t dims[2] = {(cuuint64_t)dim, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)dim * 2};
     const cuuint32_t box[2] = {64u, box_rows};
     const cuuint32_t estr[2] = {1u, 1u};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+inline bool make_map(CUtensorMap *map, const void *base, uint64_t rows, uint32_t box_rows)
+{
+    return make_map_rows(map, base, rows, kHeadDim, box_rows);
 }
 
 // 2-D view [rows][128 bytes] of a cache whose rows are 128 bytes long -- E4M3 codes of 128 dimensions, or bf16 keys of 64
@@ -310,20 +314,6 @@ inline bool make_map_row128(CUtensorMap *map, const void *base, uint64_t rows, b
     const cuuint32_t estr[2] = {1u, 1u};
     return fn(map, codes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims,
               strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// 2-D bf16 view [rows][64] of query rows of 64 dimensions, boxes of 16 rows, 128-byte swizzle.
-inline bool make_map_q64(CUtensorMap *map, const void *base, uint64_t rows)
-{
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[2] = {64u, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {128u};
-    const cuuint32_t box[2] = {64u, 16u};
-    const cuuint32_t estr[2] = {1u, 1u};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
