@@ -1,10 +1,12 @@
-"""ctypes binding of include/rkv.h: same names, argument marshalling only.
+"""Binding of include/rkv.h: same names, argument marshalling only (ctypes; the calls a decode loop makes per layer through
+csrc/pycall.c).
 
 torch is used for device memory and streams; tensors cross the boundary as raw pointers.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional, Sequence
 
@@ -12,7 +14,9 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_PKG, "librkv_b200.so")
+_CALL_PATH = os.path.join(_PKG, "_rkv_call.so")
 _lib = None
+_fast = None        # the calls made per layer and step, marshalled in C (csrc/pycall.c)
 
 RKV_OK = 0
 RKV_BF16, RKV_F32, RKV_FP8_E4M3 = 0, 1, 2
@@ -80,8 +84,26 @@ def lib():
         L.rkv_launch_count_for.restype, L.rkv_launch_count_for.argtypes = ctypes.c_int, [P, I32, I32, I32, U32]
         L.rkv_status_string.restype, L.rkv_status_string.argtypes = ctypes.c_char_p, [ctypes.c_int]
         L.rkv_last_cuda_error.restype, L.rkv_last_cuda_error.argtypes = ctypes.c_char_p, []
+        _load_fast(L)
         _lib = L
     return _lib
+
+
+def _load_fast(L) -> None:
+    global _fast
+    if not os.path.exists(_CALL_PATH):
+        raise ImportError(f"{_CALL_PATH} is missing: run `python paper_2505_24133_b200/build.py`")
+    spec = importlib.util.spec_from_file_location("_rkv_call", _CALL_PATH)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None:               # (a torch built without CUDA)
+        raw, device = (lambda _: _stream(None)), (lambda: 0)
+    address = [ctypes.cast(f, ctypes.c_void_p).value for f in (L.rkv_push_query, L.rkv_append, L.rkv_decode_attention,
+                                                               L.rkv_compress_stages)]
+    module.bind(*address, torch.cuda.is_initialized, device, raw, lambda: _stream(None))
+    _fast = module
 
 
 def _ptr(t) -> Optional[int]:
@@ -142,9 +164,10 @@ def rkv_compress_ex(desc, k_cache, v_cache, q_window, seq_lens, budget, buffer, 
 
 def rkv_compress_stages(desc, k_cache, v_cache, q_window, seq_lens, budget, buffer, alpha, lam, out_idx,
                         stream=None, stage_mask: int = RKV_STAGE_ALL) -> int:
-    return lib().rkv_compress_stages(ctypes.byref(desc), _ptr(k_cache), _ptr(v_cache), _ptr(q_window),
-                                     _ptr(seq_lens), budget, buffer, alpha, float(lam), _ptr(out_idx),
-                                     _stream(stream), stage_mask)
+    if _fast is None:
+        lib()
+    return _fast.compress_stages(desc, k_cache, v_cache, q_window, seq_lens, budget, buffer, alpha, lam, out_idx, stream,
+                                 stage_mask)
 
 
 def rkv_compress_host(desc, host_k, host_v, host_q, host_seq_lens, budget, buffer, alpha, lam, host_out_idx,
@@ -169,13 +192,16 @@ def rkv_compress_static(desc, k_cache, v_cache, q_window, seq_lens, budget, buff
 
 def rkv_append(desc, k_cache, v_cache, k_new, v_new, seq_lens, budget, buffer, stream=None) -> int:
     """The new token of every sequence enters its cache at row seq_lens[b]; seq_lens[b] += 1 (Section 3.1)."""
-    return lib().rkv_append(ctypes.byref(desc), _ptr(k_cache), _ptr(v_cache), _ptr(k_new), _ptr(v_new), _ptr(seq_lens),
-                            budget, buffer, _stream(stream))
+    if _fast is None:
+        lib()
+    return _fast.append(desc, k_cache, v_cache, k_new, v_new, seq_lens, budget, buffer, stream)
 
 
 def rkv_push_query(desc, q_window, q_new, alpha, slot, stream=None) -> int:
     """q_new becomes row `slot` of every query head's observation window (Algorithm 1's M_alpha as a ring)."""
-    return lib().rkv_push_query(ctypes.byref(desc), _ptr(q_window), _ptr(q_new), alpha, slot, _stream(stream))
+    if _fast is None:
+        lib()
+    return _fast.push_query(desc, q_window, q_new, alpha, slot, stream)
 
 
 def rkv_decode_workspace_bytes(desc, budget: int, buffer: int) -> int:
@@ -185,8 +211,9 @@ def rkv_decode_workspace_bytes(desc, budget: int, buffer: int) -> int:
 def rkv_decode_attention(desc, k_cache, v_cache, q_new, seq_lens, out, budget, buffer, stream=None) -> int:
     """The new token's queries attend over the cached keys and values of their KV heads (Section 3.1, Eq. 1);
     out [batch, n_q_heads, head_dim] float32."""
-    return lib().rkv_decode_attention(ctypes.byref(desc), _ptr(k_cache), _ptr(v_cache), _ptr(q_new), _ptr(seq_lens),
-                                      _ptr(out), budget, buffer, _stream(stream))
+    if _fast is None:
+        lib()
+    return _fast.decode_attention(desc, k_cache, v_cache, q_new, seq_lens, out, budget, buffer, stream)
 
 
 def rkv_selftest_wait_expiry(device_status, report_words, limit_cycles: int, stream=None) -> int:

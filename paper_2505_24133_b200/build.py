@@ -5,11 +5,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "librkv_b200.so")
+CALL = os.path.join(PKG, "_rkv_call.so")            # argument marshalling of the per-layer calls
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-shared",
@@ -29,7 +31,15 @@ def stale() -> bool:
     return any(os.path.getmtime(f) > t for f in deps)
 
 
+def build_call(force: bool = False) -> None:
+    src = os.path.join(CSRC, "pycall.c")
+    if force or not os.path.exists(CALL) or os.path.getmtime(src) > os.path.getmtime(CALL):
+        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-fvisibility=hidden",
+                        "-I", sysconfig.get_paths()["include"], "-o", CALL, src], check=True)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_call(force)
     if force or stale():
         cmd = [NVCC] + FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB] + sources()
         subprocess.run(cmd, check=True)
