@@ -109,8 +109,8 @@ typedef struct rkv_desc {
     int32_t head_dim;    /* d: 64, 128 or 256.  The tensor-core scoring kernels are built for bf16 keys with d = 128;
                             bf16 and 8-bit caches with d = 64 are scored by them on a copy of the keys (and of the
                             observation queries) padded with zeros to 128 in the workspace -- dot products and norms do
-                            not see the padding --; d = 256 and fp32 caches are scored by the CUDA-core kernel
-                            (correct, but far slower) */
+                            not see the padding --; d = 256 by a tensor-core kernel that forms the whole similarity
+                            matrix; fp32 caches by the CUDA-core kernel (fp32 arithmetic, slower) */
     int32_t dtype;       /* rkv_dtype_t of k_cache and v_cache (and of q_window, except for 8-bit caches: bf16) */
     int32_t pool_w;      /* W of Eq. 4; 0 = no pooling.  Range [0, 64].  Default 4 (the paper prints no value) */
     int32_t beta;        /* beta of Section 3.3; 0 = rule off.  Default 1 (the paper prints no value) */
@@ -215,9 +215,11 @@ RKV_API int rkv_compress_stages(const rkv_desc_t *desc, void *k_cache, void *v_c
 /*
  * End-to-end form with HOST buffers (pinned memory recommended): copies host_k_cache, host_v_cache,
  * host_q_window and host_seq_lens to device staging inside desc->workspace, runs the step, and copies back
- * rows [0, budget) of K and V of every head, seq_lens and out_idx -- all asynchronously on `stream`; the
+ * rows [0, budget) of K and V of every head, seq_lens and out_idx -- all asynchronously, in order with `stream`; the
  * results are valid once the stream is synchronised.  desc->workspace must hold rkv_host_workspace_bytes().
- * Shapes and semantics as rkv_compress.
+ * Shapes and semantics as rkv_compress.  Larger batches go through in pieces of whole sequences, the copies of one piece
+ * under the compression of another, on copy streams of the library's own (a bounded pool); a wait that runs out (see
+ * rkv_compress) then leaves the caches of its own piece unmodified.
  */
 RKV_API size_t rkv_host_workspace_bytes(const rkv_desc_t *desc, int32_t budget, int32_t buffer, int32_t alpha);
 RKV_API int rkv_compress_host(const rkv_desc_t *desc, void *host_k_cache, void *host_v_cache, const void *host_q_window,

@@ -17,6 +17,11 @@
 //                    against the resident G*alpha query rows (N operand), so every thread ends up with all
 //                    G*alpha logits of one key and takes the max over the group locally.
 //
+// Head dimension 256 (its only tensor-core route) runs the same kernel with every operand tile as two 128-column blocks of
+// 32 KB: the row blocks' tiles take twice the room, the ring brings a key tile in two stages, and a product is complete
+// after both.  (Measured with 16 layers x 4 sequences x 4 KV heads of 1152 tokens: 231 us for this kernel, where the CUDA-core kernel
+// took 29.7 ms.)
+//
 // Warp roles (320 threads): warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner, warps 2..9 = epilogue
 // (warp w may touch TMEM lanes 32 (w % 4) .. +31; warps 2-5 serve accumulator half 0, warps 6-9 half 1).
 // Every wait on an mbarrier is bounded; on expiry the block records RKV_ERR_TIMEOUT, stops issuing work,
@@ -32,52 +37,59 @@ namespace {
 using namespace sm100;
 
 constexpr int kThreads = 320;
-constexpr int kStages = 3;                       // ring depth of streamed key tiles
 constexpr int kHalfBytes = kTile * 64 * 2;       // one TMA box: 128 rows x 64 bf16 (128-byte swizzled rows)
-constexpr int kTileBytes = 2 * kHalfBytes;       // 32 KB: a 128 x 128 bf16 operand tile
+constexpr int kTileBytes = 2 * kHalfBytes;       // 32 KB: a 128 x 128 bf16 operand block
 constexpr int kRowsPerBlock = 2 * kTile;         // 256 matrix rows per row block
 constexpr uint32_t kTmemCols = 512;
+constexpr int kMaxStages = 3;
 
-// shared memory carve-up (offsets from a 1024-byte aligned base)
-constexpr int kOffB = 0;                                   // kStages streamed key tiles
-constexpr int kOffA = kOffB + kStages * kTileBytes;        // 2 resident tiles (row blocks) / the query tile
-constexpr int kOffR = kOffA + 2 * kTileBytes;              // inverse norms of the head, up to RKV_MAX_CAP floats
-constexpr int kOffS = kOffR + RKV_MAX_CAP * 4;             // sum_j Kbar_j, 128 floats
-constexpr int kOffBar = kOffS + kHeadDim * 4;              // mbarriers
-constexpr int kNumBars = 2 * kStages + 4 + 1;
-constexpr int kOffMisc = kOffBar + kNumBars * 8;           // tmem base, abort flag
-constexpr int kSmemBytes = kOffMisc + 16 + 1024;           // + slack for the manual 1024-byte alignment
-// The query block stages up to 128 x 128 fp32 logits in the second resident tile and the norm vector behind it
-// (neither is used there): 64 KB, contiguous.
-constexpr int kOffStage = kOffA + kTileBytes;
-static_assert(kOffStage + RKV_MAX_GROUP_ROWS * kTile * 4 <= kOffS, "logit staging must fit");
-static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+// Shared memory carve-up (offsets from a 1024-byte aligned base) for head dimension kBlocks * 128.
+template <int kBlocks> struct Smem {
+    static constexpr int kStages = kBlocks == 1 ? 3 : 2;              // ring depth: key tiles, or halves of them
+    static constexpr int kOffB = 0;                                   // kStages streamed operand blocks
+    static constexpr int kOffA = kOffB + kStages * kTileBytes;        // 2 resident tiles (row blocks) / the query tile
+    static constexpr int kOffR = kOffA + 2 * kBlocks * kTileBytes;    // inverse norms of the head, up to RKV_MAX_CAP floats
+    static constexpr int kOffS = kOffR + RKV_MAX_CAP * 4;             // sum_j Kbar_j
+    static constexpr int kOffBar = kOffS + kBlocks * kHeadDim * 4;    // mbarriers
+    static constexpr int kNumBars = 2 * kMaxStages + 4 + 1;
+    static constexpr int kOffMisc = kOffBar + kNumBars * 8;           // tmem base, abort flag
+    static constexpr int kBytes = kOffMisc + 16 + 1024;               // + slack for the manual 1024-byte alignment
+    // The query block stages up to 128 x 128 fp32 logits behind the query tile and over the norm vector (not used there):
+    // 64 KB, contiguous.
+    static constexpr int kOffStage = kOffA + kBlocks * kTileBytes;
+    static_assert(kOffStage + RKV_MAX_GROUP_ROWS * kTile * 4 <= kOffS, "logit staging must fit");
+    static_assert(kBytes <= 227 * 1024, "shared memory budget");
+};
 
 __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
-// mbarrier addresses (8 bytes each, from bar0): full[kStages], empty[kStages], acc_full[2], acc_empty[2], resident
+// mbarrier addresses (8 bytes each, from bar0): full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], resident
 struct Barriers {
     uint32_t bar0;
     __device__ __forceinline__ uint32_t full(int s) const { return bar0 + 8 * s; }
-    __device__ __forceinline__ uint32_t empty(int s) const { return bar0 + 8 * (kStages + s); }
-    __device__ __forceinline__ uint32_t acc_full(int a) const { return bar0 + 8 * (2 * kStages + a); }
-    __device__ __forceinline__ uint32_t acc_empty(int a) const { return bar0 + 8 * (2 * kStages + 2 + a); }
-    __device__ __forceinline__ uint32_t resident() const { return bar0 + 8 * (2 * kStages + 4); }
+    __device__ __forceinline__ uint32_t empty(int s) const { return bar0 + 8 * (kMaxStages + s); }
+    __device__ __forceinline__ uint32_t acc_full(int a) const { return bar0 + 8 * (2 * kMaxStages + a); }
+    __device__ __forceinline__ uint32_t acc_empty(int a) const { return bar0 + 8 * (2 * kMaxStages + 2 + a); }
+    __device__ __forceinline__ uint32_t resident() const { return bar0 + 8 * (2 * kMaxStages + 4); }
 };
 
+template <int kBlocks>
 __global__ void __launch_bounds__(kThreads, 1)
 scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,
                     int row_blocks, int q_rows_pad)
 {
+    using S = Smem<kBlocks>;
+    constexpr int kStages = S::kStages, kOffB = S::kOffB, kOffA = S::kOffA, kOffR = S::kOffR, kOffS = S::kOffS;
+    constexpr int kDim = kBlocks * kHeadDim;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = align_smem(smem_raw);
     const uint32_t sbase = smem_u32(smem);
     float *r_s = reinterpret_cast<float *>(smem + kOffR);
     float *sum_s = reinterpret_cast<float *>(smem + kOffS);
-    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + kOffMisc);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + kOffMisc + 4);
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + S::kOffMisc);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + S::kOffMisc + 4);
 
-    const Barriers bar{sbase + kOffBar};
+    const Barriers bar{sbase + S::kOffBar};
 
     // Once any block has recorded an error (a wait that ran out), the blocks still to run return at once
     // instead of each waiting out its own limit.
@@ -130,26 +142,25 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
         if (lane == 0) {
             if (is_q) {
                 const int q_row = (b * p.hq + h * p.group) * p.alpha;
-                mbar_expect_tx(bar.resident(), (uint32_t)(2 * q_rows_pad * 128));
-                tma_load_2d(sbase + kOffA, &map_q, 0, q_row, bar.resident());
-                tma_load_2d(sbase + kOffA + kHalfBytes, &map_q, 64, q_row, bar.resident());
+                mbar_expect_tx(bar.resident(), (uint32_t)(q_rows_pad * kDim * 2));
+                for (int c = 0; c < 2 * kBlocks; ++c) tma_load_2d(sbase + kOffA + c * kHalfBytes, &map_q, 64 * c, q_row, bar.resident());
             } else {
-                mbar_expect_tx(bar.resident(), (uint32_t)(num_m * kTileBytes));
+                mbar_expect_tx(bar.resident(), (uint32_t)(num_m * kBlocks * kTileBytes));
                 for (int m = 0; m < num_m; ++m) {
                     const int y = (int)tile_row0(p, head, row0 / kTile + m);
-                    tma_load_2d(sbase + kOffA + m * kTileBytes, &map_k, 0, y, bar.resident());
-                    tma_load_2d(sbase + kOffA + m * kTileBytes + kHalfBytes, &map_k, 64, y, bar.resident());
+                    for (int c = 0; c < 2 * kBlocks; ++c)
+                        tma_load_2d(sbase + kOffA + m * kBlocks * kTileBytes + c * kHalfBytes, &map_k, 64 * c, y, bar.resident());
                 }
             }
-            for (int t = 0; t < n_iter; ++t) {
-                const int s = t % kStages;
-                const int jt = n_tiles - 1 - t;                       // last tile first
-                if (!mbar_wait(bar.empty(s), ((t / kStages) & 1) ^ 1, abort_flag, sink)) break;
+            for (int u = 0; u < n_iter * kBlocks; ++u) {              // 128-column blocks of the key tiles, last tile first
+                const int s = u % kStages;
+                const int jt = n_tiles - 1 - u / kBlocks, x0 = (u % kBlocks) * kHeadDim;
+                if (!mbar_wait(bar.empty(s), ((u / kStages) & 1) ^ 1, abort_flag, sink)) break;
                 mbar_expect_tx(bar.full(s), kTileBytes);
                 const uint32_t dst = sbase + kOffB + s * kTileBytes;
                 const int y = (int)tile_row0(p, head, jt);
-                tma_load_2d(dst, &map_k, 0, y, bar.full(s));
-                tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar.full(s));
+                tma_load_2d(dst, &map_k, x0, y, bar.full(s));
+                tma_load_2d(dst + kHalfBytes, &map_k, x0 + 64, y, bar.full(s));
             }
         }
     } else if (warp == 1) {
@@ -157,14 +168,14 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
         if (lane == 0) {
             const uint32_t idesc = is_q ? instr_desc(kTile, q_rows_pad) : instr_desc(kTile, kTile);
             bool ok = mbar_wait(bar.resident(), 0, abort_flag, sink);
-            for (int t = 0; ok && t < n_iter; ++t) {
-                const int s = t % kStages, a = t & 1;
-                if (!mbar_wait(bar.full(s), (t / kStages) & 1, abort_flag, sink)) break;
-                if (!mbar_wait(bar.acc_empty(a), ((t >> 1) & 1) ^ 1, abort_flag, sink)) break;
+            for (int u = 0; ok && u < n_iter * kBlocks; ++u) {
+                const int s = u % kStages, t = u / kBlocks, blk = u % kBlocks, a = t & 1;
+                if (!mbar_wait(bar.full(s), (u / kStages) & 1, abort_flag, sink)) break;
+                if (blk == 0 && !mbar_wait(bar.acc_empty(a), ((t >> 1) & 1) ^ 1, abort_flag, sink)) break;
                 tc_fence_after();
                 const uint32_t stage = sbase + kOffB + s * kTileBytes;
                 for (int m = 0; m < num_m; ++m) {
-                    const uint32_t resident = sbase + kOffA + m * kTileBytes;
+                    const uint32_t resident = sbase + kOffA + (m * kBlocks + blk) * kTileBytes;
                     const uint32_t d_tmem = tmem_base + a * 256 + m * 128;
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
@@ -172,11 +183,11 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
                         const uint32_t koff = (k >> 2) * kHalfBytes + (k & 3) * 32;
                         const uint64_t da = smem_desc((is_q ? stage : resident) + koff);
                         const uint64_t db = smem_desc((is_q ? resident : stage) + koff);
-                        umma(d_tmem, da, db, idesc, k > 0);
+                        umma(d_tmem, da, db, idesc, blk > 0 || k > 0);
                     }
                 }
-                umma_commit(bar.empty(s));       // the stage may be refilled once these MMAs have read it
-                umma_commit(bar.acc_full(a));    // the accumulators are complete
+                umma_commit(bar.empty(s));                               // the stage may be refilled once these MMAs have read it
+                if (blk == kBlocks - 1) umma_commit(bar.acc_full(a));    // the accumulators are complete
             }
         }
         __syncwarp();
@@ -195,7 +206,7 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
             const float *inv_norm = p.inv_norm + (size_t)head * p.cap_pad;
             for (int v = et; v < n_tiles * (kTile / 4); v += 256)
                 reinterpret_cast<float4 *>(r_s)[v] = __ldg(reinterpret_cast<const float4 *>(inv_norm) + v);
-            if (et < kHeadDim) sum_s[et] = p.head_sum[(size_t)head * kHeadDim + et];
+            if (et < kDim) sum_s[et] = p.head_sum[(size_t)head * kDim + et];
             epi_barrier();
 
             const int i = row0 + half * kTile + lrow;
@@ -206,10 +217,10 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
             if (ok && warp_active) {
                 // Kbar_i . s - Kbar_i . Kbar_i from the resident (swizzled) tile: 16-byte chunk c of row r sits at
                 // chunk position c ^ (r & 7) of the row's 128 bytes
-                const uint8_t *tile = smem + kOffA + half * kTileBytes;
+                const uint8_t *tile = smem + kOffA + half * kBlocks * kTileBytes;
                 float dot = 0.f, sq = 0.f;
 #pragma unroll
-                for (int hb = 0; hb < 2; ++hb) {
+                for (int hb = 0; hb < 2 * kBlocks; ++hb) {
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
                         const uint4 raw = *reinterpret_cast<const uint4 *>(tile + hb * kHalfBytes + lrow * 128 +
@@ -277,7 +288,7 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
             if (row_ok) p.sbar[(size_t)head * p.cap_pad + i] = (total - removed * ri) / (float)n;
         } else {
             // Eq. 2-3: thread = key, all G * alpha logits of that key in its accumulator row
-            float *stage_f = reinterpret_cast<float *>(smem + kOffStage);           // [q_rows_pad][128] floats
+            float *stage_f = reinterpret_cast<float *>(smem + S::kOffStage);           // [q_rows_pad][128] floats
             float *logits = p.logits + (size_t)head * p.alpha * p.cap_pad;
             const float scale = p.logit_scale;                                    // 1 / sqrt(d)
             for (int t = 0; t < n_iter; ++t) {
@@ -325,6 +336,16 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
         atomicAdd(p.counters, (unsigned long long)(n_iter * num_m));
 }
 
+template <int kBlocks>
+cudaError_t launch_blocks(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q, unsigned grid,
+                          int row_blocks, int q_rows_pad)
+{
+    const cudaError_t e = cudaFuncSetAttribute(scores_sm100_kernel<kBlocks>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<kBlocks>::kBytes);
+    if (e != cudaSuccess) return e;
+    scores_sm100_kernel<kBlocks><<<grid, kThreads, Smem<kBlocks>::kBytes, s>>>(p, map_k, map_q, row_blocks, q_rows_pad);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 bool scores_sm100_available() { return true; }
@@ -335,15 +356,13 @@ cudaError_t launch_scores_sm100(const Params &p, cudaStream_t s)
     const int q_rows = p.group * p.alpha;
     const int q_rows_pad = (q_rows + 15) / 16 * 16;
     CUtensorMap map_k, map_q;
-    if (!make_map(&map_k, p.k_cache, key_rows_total(p), kTile) ||
-        !make_map(&map_q, p.q_window, (uint64_t)p.batch * p.hq * p.alpha, (uint32_t)q_rows_pad))
+    if (!make_map_rows(&map_k, p.k_cache, key_rows_total(p), p.d, kTile) ||
+        !make_map_rows(&map_q, p.q_window, (uint64_t)p.batch * p.hq * p.alpha, p.d, (uint32_t)q_rows_pad))
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(scores_sm100_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
     const int row_blocks = (p.cap + kRowsPerBlock - 1) / kRowsPerBlock;
     const unsigned grid = (unsigned)(row_blocks + 1) * (unsigned)(p.batch * p.hkv);
-    scores_sm100_kernel<<<grid, kThreads, kSmemBytes, s>>>(p, map_k, map_q, row_blocks, q_rows_pad);
-    return cudaGetLastError();
+    return p.d == kHeadDim ? launch_blocks<1>(p, s, map_k, map_q, grid, row_blocks, q_rows_pad)
+                           : launch_blocks<2>(p, s, map_k, map_q, grid, row_blocks, q_rows_pad);
 }
 
 }  // namespace rkv
