@@ -2,6 +2,8 @@
 // See include/rkv.h for the contract of every entry point.
 #include <cstdio>
 #include <cstring>
+#include <memory>
+#include <mutex>
 
 #include "rkv_common.cuh"
 
@@ -25,9 +27,10 @@ struct Layout {
     int cap, cap_pad, tiles, tri;
 };
 
-// The tensor-core scoring kernels are built for bf16 keys of 128 dimensions.  bf16 and 8-bit caches of 128 dimensions
-// use them directly (8-bit: on a widened copy), those of 64 dimensions on a copy padded with zeros to 128 (dot products
-// and norms do not see the padding); fp32 caches, 256 dimensions, or a request for it go to the CUDA-core kernel.
+// The two-pass tensor-core scoring kernels are built for bf16 keys of 128 dimensions.  bf16 and 8-bit caches of 128
+// dimensions use them directly (8-bit: on a widened copy), those of 64 dimensions on a copy padded with zeros to 128 (dot
+// products and norms do not see the padding).  256 dimensions take the row-block tensor-core kernel, which forms the whole
+// similarity matrix; fp32 caches, or a request for it, the CUDA-core kernel.
 // Bytes of a cache element and of a query element.  8-bit caches (E4M3 codes) are scored on a bf16 copy of their keys
 // in the workspace (every E4M3 value is a bf16 value), with bf16 queries.
 size_t cache_esz(const rkv_desc_t *d) { return d->dtype == RKV_BF16 ? 2 : d->dtype == RKV_F32 ? 4 : 1; }
@@ -35,7 +38,7 @@ size_t query_esz(const rkv_desc_t *d) { return d->dtype == RKV_F32 ? 4 : 2; }
 
 bool use_simt(const rkv_desc_t *d)
 {
-    return d->dtype == RKV_F32 || d->head_dim == 256 || (d->flags & RKV_FLAG_SIMT_SCORES);
+    return d->dtype == RKV_F32 || (d->flags & RKV_FLAG_SIMT_SCORES);
 }
 // The head dimension is padded from 64 to 128 in the scoring copy (keys and observation queries).
 bool pads_dim(const rkv_desc_t *d) { return d->head_dim == 64 && !use_simt(d); }
@@ -55,7 +58,7 @@ int fuse_mode(const rkv_desc_t *d, long long cap)
 }
 
 // 1 when the triangle tensor-core kernels score (bf16 caches, unless a cross-check kernel is asked for).
-int use_tri(const rkv_desc_t *d) { return !(use_simt(d) || (d->flags & RKV_FLAG_ROWBLOCK_SCORES)); }
+int use_tri(const rkv_desc_t *d) { return !(use_simt(d) || d->head_dim == 256 || (d->flags & RKV_FLAG_ROWBLOCK_SCORES)); }
 
 // Returns RKV_OK and fills *lay when the shape arguments are usable.
 int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout *lay)
@@ -282,6 +285,67 @@ int host_layout(const rkv_desc_t *d, int budget, int buffer, int alpha, HostLayo
     return RKV_OK;
 }
 
+// Two copy streams and the events between them and the caller's stream, for the host-buffer form.  A call takes one from the
+// pool while it enqueues and gives it back then; the next taker's copies queue up behind what is still in the streams.
+// Creating the two streams for each call took 250 us.
+constexpr int kMaxPieces = 8;
+struct HostPipe {
+    int dev = -1;
+    cudaStream_t up = nullptr, down = nullptr;
+    cudaEvent_t ev[3 * kMaxPieces + 2] = {};
+    bool open(int device)
+    {
+        dev = device;
+        bool ok = cudaStreamCreateWithFlags(&up, cudaStreamNonBlocking) == cudaSuccess &&
+                  cudaStreamCreateWithFlags(&down, cudaStreamNonBlocking) == cudaSuccess;
+        for (cudaEvent_t &x : ev)
+            if (ok) ok = cudaEventCreateWithFlags(&x, cudaEventDisableTiming) == cudaSuccess;
+        return ok;
+    }
+    ~HostPipe()
+    {
+        for (cudaEvent_t x : ev)
+            if (x) cudaEventDestroy(x);
+        if (up) cudaStreamDestroy(up);
+        if (down) cudaStreamDestroy(down);
+    }
+};
+class PipePool {
+public:
+    std::unique_ptr<HostPipe> take(int dev)
+    {
+        {
+            std::lock_guard<std::mutex> guard(lock_);
+            for (auto &x : free_)
+                if (x && x->dev == dev) return std::move(x);
+        }
+        std::unique_ptr<HostPipe> made(new HostPipe);
+        if (!made->open(dev)) {
+            cudaGetLastError();             // (the call then goes through the caller's stream alone)
+            made.reset();
+        }
+        return made;
+    }
+    void give(std::unique_ptr<HostPipe> x)
+    {
+        std::lock_guard<std::mutex> guard(lock_);
+        for (auto &slot : free_)
+            if (!slot) {
+                slot = std::move(x);
+                return;
+            }
+    }                                       // (no slot left: destroyed when its work is done)
+
+private:
+    std::mutex lock_;
+    std::unique_ptr<HostPipe> free_[16];
+};
+PipePool &pipe_pool()
+{
+    static PipePool *pool = new PipePool;   // never destroyed: the CUDA runtime may be gone before this library's statics
+    return *pool;
+}
+
 }  // namespace
 }  // namespace rkv
 
@@ -357,31 +421,79 @@ int rkv_compress_host(const rkv_desc_t *desc, void *host_k_cache, void *host_v_c
     if (!desc->workspace || desc->workspace_bytes < h.total) return RKV_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(desc->workspace) & 255u) return RKV_ERR_WORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // Pieces of whole sequences: while one is compressed, the next comes in and the one before goes out (the link carries both
+    // directions at once).  A copy costs about 5 us beside its bytes, so a piece has 16 MB or more, and the small arrays cross
+    // once per call.  Events, counters and stream capture are for the call as a whole.
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
+    long long pieces = (long long)(2 * h.kv_bytes / (16u << 20));
+    pieces = pieces < kMaxPieces ? pieces : kMaxPieces;
+    pieces = pieces < 1 ? 1 : (pieces < desc->batch ? pieces : desc->batch);
+    if (capturing != cudaStreamCaptureStatusNone || desc->stage_events || desc->kernel_events || desc->dbg_counters) pieces = 1;
+    int dev = 0;
+    std::unique_ptr<HostPipe> pipe;
+    if (pieces > 1 && cudaGetDevice(&dev) == cudaSuccess) pipe = pipe_pool().take(dev);
+    if (!pipe) pieces = 1;
+    cudaStream_t up = pipe ? pipe->up : s, down = pipe ? pipe->down : s;
+    cudaError_t e = cudaSuccess;
+    const char *where = "host to device copy";
+    const size_t P = (size_t)desc->batch * desc->n_kv_heads, cap = (size_t)budget + buffer;
     char *ws = static_cast<char *>(desc->workspace);
-    cudaError_t e;
-    if ((e = cudaMemcpyAsync(ws + h.k, host_k_cache, h.kv_bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(ws + h.v, host_v_cache, h.kv_bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(ws + h.q, host_q_window, h.q_bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(ws + h.seq, host_seq_lens, h.seq_bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess)
-        return cuda_fail(e, "host to device copy");
-    rkv_desc_t inner = *desc;
-    inner.workspace = ws + h.inner;
-    inner.workspace_bytes = desc->workspace_bytes - h.inner;
-    rc = run(&inner, ws + h.k, ws + h.v, ws + h.q, reinterpret_cast<int32_t *>(ws + h.seq), budget, buffer, alpha,
-             lambda, reinterpret_cast<int32_t *>(ws + h.idx), stream, RKV_STAGE_ALL);
-    if (rc != RKV_OK) return rc;
-    // rows [0, budget) of every head come back; rows beyond are unspecified after a compression and are left
-    // as the host has them
-    const size_t P = (size_t)desc->batch * desc->n_kv_heads;
-    const size_t cap = (size_t)budget + buffer;
-    if ((e = cudaMemcpy2DAsync(host_k_cache, cap * h.row_bytes, ws + h.k, cap * h.row_bytes, budget * h.row_bytes, P,
-                               cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaMemcpy2DAsync(host_v_cache, cap * h.row_bytes, ws + h.v, cap * h.row_bytes, budget * h.row_bytes, P,
-                               cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(host_seq_lens, ws + h.seq, h.seq_bytes, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(host_out_idx, ws + h.idx, h.idx_bytes, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-        return cuda_fail(e, "device to host copy");
-    return RKV_OK;
+    char *hk = static_cast<char *>(host_k_cache), *hv = static_cast<char *>(host_v_cache);
+    auto copy = [&](void *dst, const void *src, size_t bytes, cudaMemcpyKind kind, cudaStream_t st) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, kind, st);
+    };
+    auto link = [&](int ev, cudaStream_t from, cudaStream_t to) {
+        if (e == cudaSuccess && pipe && (e = cudaEventRecord(pipe->ev[ev], from)) == cudaSuccess) e = cudaStreamWaitEvent(to, pipe->ev[ev], 0);
+    };
+    // first sequence of piece i: the first and the last piece are half as large, nothing runs beside them
+    auto edge = [&](int i) -> size_t { return i == 0 ? 0 : i == pieces ? desc->batch : (size_t)desc->batch * (2 * i - 1) / (2 * pieces - 2); };
+    link(0, s, up);                         // the staging buffers may still be in use by earlier work of the stream
+    copy(ws + h.q, host_q_window, h.q_bytes, cudaMemcpyHostToDevice, up);
+    copy(ws + h.seq, host_seq_lens, h.seq_bytes, cudaMemcpyHostToDevice, up);
+    for (int i = 0; i < (int)pieces && e == cudaSuccess && rc == RKV_OK; ++i) {
+        const size_t b0 = edge(i), nb = edge(i + 1) - b0;
+        if (nb == 0) continue;
+        const size_t kv0 = h.kv_bytes / desc->batch * b0, kv = h.kv_bytes / desc->batch * nb;
+        copy(ws + h.k + kv0, hk + kv0, kv, cudaMemcpyHostToDevice, up);
+        link(1 + 3 * i, up, s);             // the scores need the keys alone
+        copy(ws + h.v + kv0, hv + kv0, kv, cudaMemcpyHostToDevice, up);
+        if (e != cudaSuccess) break;
+        rkv_desc_t inner = *desc;
+        inner.batch = (int32_t)nb;
+        inner.workspace = ws + h.inner;     // the pieces are compressed one after the other
+        inner.workspace_bytes = desc->workspace_bytes - h.inner;
+        if (inner.budgets) inner.budgets += b0;
+        for (float **dump : {&inner.dbg_I, &inner.dbg_Sbar, &inner.dbg_R, &inner.dbg_Z})
+            if (*dump) *dump += b0 * desc->n_kv_heads * cap;
+        auto stages = [&](uint32_t mask) {
+            return run(&inner, ws + h.k + kv0, ws + h.v + kv0, ws + h.q + h.q_bytes / desc->batch * b0,
+                       reinterpret_cast<int32_t *>(ws + h.seq) + b0, budget, buffer, alpha, lambda,
+                       reinterpret_cast<int32_t *>(ws + h.idx + h.idx_bytes / desc->batch * b0), stream, mask);
+        };
+        if (pipe) {
+            rc = stages(RKV_STAGE_ALL & ~RKV_STAGE_GATHER);
+            link(2 + 3 * i, up, s);
+            if (rc == RKV_OK) rc = stages(RKV_STAGE_GATHER);
+        } else {
+            rc = stages(RKV_STAGE_ALL);
+        }
+        if (rc != RKV_OK) break;
+        where = "device to host copy";
+        link(3 + 3 * i, s, down);
+        // rows [0, budget) of every head come back; rows beyond are unspecified after a compression and are left
+        // as the host has them
+        const size_t pitch = cap * h.row_bytes, width = budget * h.row_bytes, rows = P / desc->batch * nb;
+        if (e == cudaSuccess) e = cudaMemcpy2DAsync(hk + kv0, pitch, ws + h.k + kv0, pitch, width, rows, cudaMemcpyDeviceToHost, down);
+        if (e == cudaSuccess) e = cudaMemcpy2DAsync(hv + kv0, pitch, ws + h.v + kv0, pitch, width, rows, cudaMemcpyDeviceToHost, down);
+    }
+    if (rc == RKV_OK) {
+        copy(host_seq_lens, ws + h.seq, h.seq_bytes, cudaMemcpyDeviceToHost, down);
+        copy(host_out_idx, ws + h.idx, h.idx_bytes, cudaMemcpyDeviceToHost, down);
+        link(3 * kMaxPieces + 1, down, s);
+    }
+    if (pipe) pipe_pool().give(std::move(pipe));
+    return rc != RKV_OK ? rc : (e == cudaSuccess ? RKV_OK : cuda_fail(e, where));
 }
 
 int rkv_append(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *k_new, const void *v_new, int32_t *seq_lens,
@@ -418,7 +530,7 @@ static int attend_plan(const rkv_desc_t *d, int32_t budget, int32_t buffer, int 
     const int G = d->n_q_heads / d->n_kv_heads;
     if (!attend_supported(G, d->dtype, d->head_dim)) return RKV_ERR_UNSUPPORTED;
     int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    if (device_sms(&dev, &sms) != cudaSuccess)
         sms = 148;       // sizing only (no device here): the B200's count
     *splits = attend_splits(d->batch * d->n_kv_heads, budget + buffer, sms, G, d->dtype);
     *bytes = attend_partial_bytes(d->batch * d->n_kv_heads, *splits, G);
