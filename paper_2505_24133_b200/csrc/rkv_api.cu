@@ -22,8 +22,7 @@ int cuda_fail(cudaError_t e, const char *where)
 }
 
 struct Layout {
-    size_t k_wide, q_wide, best, dense, dense_items, inv_norm, norm_split, thr_split, tile_sum, head_sum, logits, row_stat, imp, sbar, left, strag, strag_count, strag_items, self_dot, head_sum_bf16, meta, counters,
-        tile_done, zero_bytes, total;
+    size_t k_wide, q_wide, best, dense, dense_items, inv_norm, norm_split, thr_split, tile_sum, logits, row_stat, imp, sbar, left, strag, strag_count, strag_items, self_dot, head_sum_bf16, meta, counters, total;
     int cap, cap_pad, tiles, tri;
 };
 
@@ -96,7 +95,6 @@ int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout 
         lay->thr_split = off;   off = align_up(off + P * kTile * 16 * sizeof(__nv_bfloat16), 256);
         const size_t hd = (size_t)scoring_dim(d);
         lay->tile_sum = off;  off = align_up(off + P * lay->tiles * hd * sizeof(float), 256);
-        lay->head_sum = off;  off = align_up(off + P * hd * sizeof(float), 256);
         lay->logits = off;    off = align_up(off + P * alpha * lay->cap_pad * sizeof(float), 256);
         lay->row_stat = off;  off = align_up(off + P * alpha * 2 * sizeof(float), 256);
         lay->imp = off;       off = align_up(off + P * lay->cap_pad * sizeof(float), 256);
@@ -113,10 +111,7 @@ int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout 
         lay->self_dot = off;    off = align_up(off + P * lay->cap_pad * sizeof(float), 256);
         lay->head_sum_bf16 = off; off = align_up(off + P * 16 * hd * sizeof(__nv_bfloat16), 256);
         lay->meta = off;        off = align_up(off + 2 * (size_t)d->batch * sizeof(int32_t), 256);
-        // the region the prep stage zeroes: counters and per-head tile tickets
-        lay->counters = off;    off = align_up(off + 32 * sizeof(unsigned long long), 256);
-        lay->tile_done = off;   off = align_up(off + P * sizeof(uint32_t), 256);
-        lay->zero_bytes = off - lay->counters;
+        lay->counters = off;    off = align_up(off + kCounterWords * sizeof(unsigned long long), 256);
         lay->total = off;
     }
     return RKV_OK;
@@ -175,7 +170,6 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
     p.norm_split = reinterpret_cast<__nv_bfloat16 *>(ws + lay.norm_split);
     p.thr_split = reinterpret_cast<__nv_bfloat16 *>(ws + lay.thr_split);
     p.tile_sum = reinterpret_cast<float *>(ws + lay.tile_sum);
-    p.head_sum = reinterpret_cast<float *>(ws + lay.head_sum);
     p.logits = reinterpret_cast<float *>(ws + lay.logits);
     p.row_stat = reinterpret_cast<float *>(ws + lay.row_stat);
     p.imp = reinterpret_cast<float *>(ws + lay.imp);
@@ -192,8 +186,6 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
     p.head_sum_bf16 = reinterpret_cast<__nv_bfloat16 *>(ws + lay.head_sum_bf16);
     p.meta = reinterpret_cast<int32_t *>(ws + lay.meta);
     p.counters = reinterpret_cast<unsigned long long *>(ws + lay.counters);
-    p.tile_done = reinterpret_cast<uint32_t *>(ws + lay.tile_done);
-    p.zero_bytes = lay.zero_bytes;
     p.tri = lay.tri;
     p.status = d->device_status;
     p.budgets = d->budgets;
@@ -229,7 +221,6 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
         p.fuse_table = stored.block_table;
     }
     if (stages & RKV_STAGE_PREP) {
-        if ((e = cudaMemsetAsync(p.counters, 0, p.zero_bytes, s)) != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
         if (needs_copy(d) &&
             (e = launch_widen_keys(stored, static_cast<__nv_bfloat16 *>(p.k_cache), p.d, pads_dim(d) ? stored.q_window : nullptr,
                                    pads_dim(d) ? ws + lay.q_wide : nullptr, p.fuse_mode == 0, s)) != cudaSuccess)

@@ -56,7 +56,6 @@ struct Params {
                                   // to that tile's rows; the dot product of the two kinds of slice is -T / (r_i r_j)
                                   // to fp32 accuracy.  Both are written by the prep stage (two-pass route only).
     float *tile_sum;     // [P][tiles][128]      sum over the tile's candidate rows of r_i * k_i
-    float *head_sum;     // [P][128]             sum over all candidate rows of r_i * k_i (the tile sums added up)
     float *logits;       // [P][alpha][cap_pad]  Eq. 2-3: group-max of scaled logits
     float *row_stat;     // [P][alpha][2]        Eq. 3 per row: max logit, 1 / sum of exp(logit - max)
     float *imp;          // [P][cap_pad]         Eq. 4: importance I (head_mean: overwritten with Z by select_kernel)
@@ -73,15 +72,15 @@ struct Params {
     int4 *dense_items;   // [P * ceil(tiles/2)]  its work list: {head, pair of row tiles, n, -}
     int dense_ok;        // the symmetric route may be chosen (beta = 1, not switched off)
     float *self_dot;     // [P][cap_pad]         Kbar_i . Kbar_i (1 up to rounding and eps; 0 for a zero key)
-    __nv_bfloat16 *head_sum_bf16;   // [P][16][128] head_sum split into three bf16 rows (hi, mid, lo), 13 zero rows
+    __nv_bfloat16 *head_sum_bf16;   // [P][16][128] the tile sums of a head added up, as three bf16 rows (hi, mid, lo), 13 zero rows
     int32_t *meta;       // [2][batch]           snapshot of seq_lens (kMetaInvalid if out of range), then each
                          //                      sequence's budget (p.budget unless the caller gave per-sequence ones)
     const int32_t *budgets;   // optional [batch]: per-sequence budgets (alpha < budgets[b] <= budget), else null
     const int32_t *block_table;   // optional [P][cap / 128]: paged caches, page (= key tile) ids into the pools, else null
     int pages_per_head;           // cap / 128 (paged caches)
     long long pool_pages;         // pages in the pools (paged caches)
-    // zeroed by the prep stage's memset, in this order, contiguous:
-    unsigned long long *counters;   // [8]       [0] = similarity tiles computed by the tcgen05 kernels, [1] = item
+    // zeroed by the prep kernel:
+    unsigned long long *counters;   // [32]      [0] = similarity tiles computed by the tcgen05 kernels, [1] = item
                                     //           ticket of the first scoring pass, [2] = entries in strag_items,
                                     //           [3] = item ticket of the second pass, [4] = the call's abort word
                                     //           (non-zero once a bounded wait ran out: later kernels of the call
@@ -89,8 +88,6 @@ struct Params {
                                     //           [5] = listed-token x key-tile pairs the second pass has to form,
                                     //           [8 + 2 r], [9 + 2 r] = work items and item ticket of its round r,
                                     //           [16], [17] = the same for the symmetric route
-    uint32_t *tile_done;            // [P]       tiles of the head finished by the prep stage
-    size_t zero_bytes;              // bytes from `counters` to the end of `tile_done`
     int tri;                        // 1: the triangle kernels score (bf16 default); 0: another kernel does
     // optional outputs
     void *const *kernel_events;     // see rkv_desc_t
@@ -114,6 +111,7 @@ __device__ __forceinline__ void report(int32_t *status, int code)
     if (status) atomicCAS(status, 0, code);
 }
 
+constexpr int kCounterWords = 32;
 constexpr int kAbortWord = 4;       // index of the call's abort word in Params::counters
 constexpr int kPairsWord = 5;       // index of the second pass's useful-work count
 constexpr int kDenseWords = 16;     // counters[16], [17]: work items and item ticket of the symmetric route

@@ -26,6 +26,8 @@ __global__ void __launch_bounds__(kGatherThreads) gather_kernel(Params p)
     constexpr int kRows = kChunkRows * kSplit;                                  // rows per chunk: 16 KB in flight per block
     constexpr int kVecPerThread = kRows * kVecPerSlice / kGatherThreads;       // 4 or 8
     constexpr int kRowsPerStep = kGatherThreads / kVecPerSlice;
+    pdl_trigger();
+    pdl_wait();
     const int slice = blockIdx.x % kSplit;
     const int stream = blockIdx.x / kSplit;
     const int head = stream >> 1;
@@ -70,19 +72,17 @@ cudaError_t launch_gather(const Params &p, cudaStream_t s)
     const unsigned streams = 2u * (unsigned)(p.batch * p.hkv);
     int dev = 0, sms = 0;
     cudaError_t e;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = device_sms(&dev, &sms)) != cudaSuccess) return e;
     // Few streams: cut the rows into column slices, as many (4, 2) as still fit the SMs in one wave of resident blocks
     // (8 per SM): a second, partly filled wave would leave SMs idle for much of the kernel.
     const unsigned wave = 8u * (unsigned)sms;
     const int split = streams * 4u <= wave ? 4 : (streams * 2u <= wave ? 2 : (streams < wave ? 4 : 1));
     const int vec_per_row = p.store_row_bytes / 16;      // 16-byte vectors per row: 4 .. 64
-#define RKV_GATHER_CASE(V)                                                                      \
-    case V:                                                                                     \
-        if (split == 4) gather_kernel<V, 4><<<streams * 4u, kGatherThreads, 0, s>>>(p);         \
-        else if (split == 2) gather_kernel<V, 2><<<streams * 2u, kGatherThreads, 0, s>>>(p);    \
-        else gather_kernel<V, 1><<<streams, kGatherThreads, 0, s>>>(p);                         \
-        break;
+#define RKV_GATHER_CASE(V)                                                                                          \
+    case V:                                                                                                         \
+        return split == 4   ? launch_early(gather_kernel<V, 4>, streams * 4u, kGatherThreads, 0, s, 1, p)           \
+               : split == 2 ? launch_early(gather_kernel<V, 2>, streams * 2u, kGatherThreads, 0, s, 1, p)           \
+                            : launch_early(gather_kernel<V, 1>, streams, kGatherThreads, 0, s, 1, p);
     switch (vec_per_row) {
         RKV_GATHER_CASE(4)
         RKV_GATHER_CASE(8)
@@ -92,7 +92,6 @@ cudaError_t launch_gather(const Params &p, cudaStream_t s)
         default: return cudaErrorInvalidValue;
     }
 #undef RKV_GATHER_CASE
-    return cudaGetLastError();
 }
 
 }  // namespace rkv

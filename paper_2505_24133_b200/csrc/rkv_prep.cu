@@ -5,7 +5,8 @@
 // scoring stage obtain sum_j S[j][i] = Kbar_i . (sum_j Kbar_j) - Kbar_i . Kbar_i (Eq. 6 before the
 // retention rule) without accumulating the n x n matrix element by element.
 // Rows i >= n (observation tokens, unused capacity) get r_i = 0 and contribute nothing.
-// The last block to finish a head also leaves sum_i r_i * k_i over the whole head (head_sum).
+// The call's counters start at zero: the first block clears them (a memset in front of this kernel cost a small call 3 us;
+// the first of a block's waits could record that it ran out many microseconds later at the earliest).
 // Kbar_i . Kbar_i is kept per row as well (self_dot).
 //
 // HBM-bound: each block brings its tile of K into shared memory with one bulk copy (cp.async.bulk, bounded wait
@@ -19,6 +20,11 @@ namespace rkv {
 
 namespace {
 
+__device__ __forceinline__ void clear_counters(const Params &p)
+{
+    if (blockIdx.x == 0 && threadIdx.x < kCounterWords) p.counters[threadIdx.x] = 0ull;
+}
+
 constexpr int kPrepThreads = 256;
 constexpr int kPrepWarps = kPrepThreads / 32;
 
@@ -30,6 +36,9 @@ __global__ void __launch_bounds__(kPrepThreads, D <= 128 ? 5 : 2) prep_kernel(Pa
     constexpr int kTileBytesT = kTile * D * (int)sizeof(T);
     __shared__ int abort_flag;
     const ErrSink sink = make_sink(p);
+    pdl_trigger();
+    pdl_wait();
+    clear_counters(p);
     constexpr int kPerVec = Elem<T>::kPerVec;            // elements per 16-byte vector
     constexpr int kVecPerLane = 2;                       // 16-byte vectors of a row held by one lane
     constexpr int kLanesPerRow = D / (kPerVec * kVecPerLane);     // 8 (bf16) or 16 (fp32)
@@ -196,34 +205,6 @@ __global__ void __launch_bounds__(kPrepThreads, D <= 128 ? 5 : 2) prep_kernel(Pa
         for (int w = 0; w < kPrepWarps; ++w) s += part[w][threadIdx.x];
         p.tile_sum[((size_t)head * p.tiles + tile) * D + threadIdx.x] = s;
     }
-
-    // The block that finishes a head's last tile adds the tile sums up, always in tile order, so the result does
-    // not depend on which block that is.  (tile_done is zeroed by the memset that precedes this kernel.)
-    __shared__ bool last_block;
-    __syncthreads();                       // the block's tile sums are written ...
-    if (threadIdx.x == 0) {
-        __threadfence();                   // ... and made visible device-wide before the ticket is drawn
-        last_block = (atomicAdd(&p.tile_done[head], 1u) == (unsigned)p.tiles - 1u);
-    }
-    __syncthreads();
-    if (last_block && threadIdx.x < D) {
-        __threadfence();
-        const float *ts = p.tile_sum + (size_t)head * p.tiles * D + threadIdx.x;
-        float s = 0.f;
-        for (int t = 0; t < p.tiles; ++t) s += __ldcg(ts + (size_t)t * D);
-        p.head_sum[(size_t)head * D + threadIdx.x] = s;
-        // the same vector as three bf16 rows whose sum is s to fp32 accuracy (rows 3..15 of the 16-row block are
-        // zero): appended to the query rows, it lets the tensor cores form Kbar_i . s along with the logits
-        __nv_bfloat16 *hs = p.head_sum_bf16 + (size_t)head * 16 * D + threadIdx.x;
-        float rest = s;
-#pragma unroll
-        for (int part_i = 0; part_i < 3; ++part_i) {
-            const __nv_bfloat16 h16 = __float2bfloat16_rn(rest);
-            hs[part_i * D] = h16;
-            rest -= __bfloat162float(h16);
-        }
-        for (int z = 3; z < 16; ++z) hs[z * D] = __float2bfloat16_rn(0.f);
-    }
 }
 
 // ---- the same stage for bf16 caches with d = 128 (the tensor-core route): sum_i r_i k_i on the tensor cores ------------
@@ -310,7 +291,6 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
         for (int q = 0; q < kPrepTcBufs; ++q) mbar_init(bar_tile0 + 8u * q, 1);
         mbar_init(bar_mma, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        for (int q = 0; q < kPrepTcBufs - 1; ++q) issue_copy(q);
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -324,6 +304,11 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
     tc_fence_after();
     const uint32_t tmem = tmem_holder;
     uint32_t mma_parity = 0;
+    pdl_trigger();
+    pdl_wait();                             // the set-up above touches no global memory
+    clear_counters(p);
+    if (t == 0)
+        for (int q = 0; q < kPrepTcBufs - 1; ++q) issue_copy(q);
 
     int k = 0;
     for (int idx = (int)blockIdx.x; idx < total; idx += (int)gridDim.x, ++k) {
@@ -524,7 +509,6 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
         mbar_init(bar_raw0 + 8u, 1);
         mbar_init(bar_mma, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        issue_copy(0);
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -537,6 +521,10 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
     tc_fence_after();
     const uint32_t tmem = tmem_holder;
     uint32_t mma_parity = 0;
+    pdl_trigger();
+    pdl_wait();
+    clear_counters(p);
+    if (t == 0) issue_copy(0);
 
     int k = 0;
     for (int idx = (int)blockIdx.x; idx < total; idx += (int)gridDim.x, ++k) {
@@ -699,11 +687,12 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
 __global__ void __launch_bounds__(kHeadDim) head_sum_kernel(Params p)
 {
     constexpr int D = kHeadDim;
+    pdl_trigger();
+    pdl_wait();
     const int head = blockIdx.x, t = threadIdx.x;
     const float *ts = p.tile_sum + (size_t)head * p.tiles * D + t;
     float s = 0.f;
     for (int q = 0; q < p.tiles; ++q) s += ts[(size_t)q * D];
-    p.head_sum[(size_t)head * D + t] = s;
     __nv_bfloat16 *hs = p.head_sum_bf16 + (size_t)head * 16 * D + t;
     float rest = s;
 #pragma unroll
@@ -718,19 +707,33 @@ __global__ void __launch_bounds__(kHeadDim) head_sum_kernel(Params p)
 }  // namespace
 
 template <typename T, int D>
-static cudaError_t launch_prep_for(const Params &p, cudaStream_t s)
+static cudaError_t launch_prep_for(const Params &p, int dev, cudaStream_t s)
 {
+    static std::atomic<unsigned long long> done{0ull};
     const unsigned grid = (unsigned)p.tiles * (unsigned)(p.batch * p.hkv);
     const int smem = kTile * D * (int)sizeof(T) + 16;
-    cudaError_t e = cudaFuncSetAttribute(prep_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = allow_smem_once(done, dev, prep_kernel<T, D>, smem);
     if (e != cudaSuccess) return e;
-    prep_kernel<T, D><<<grid, kPrepThreads, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_early(prep_kernel<T, D>, grid, kPrepThreads, smem, s, 1, p);
+}
+
+template <bool kCodes>
+static cudaError_t launch_fused_for(const Params &p, const CUtensorMap &map_src, const CUtensorMap &map_wide, unsigned grid, int total, int dev,
+                                    cudaStream_t s)
+{
+    static std::atomic<unsigned long long> done{0ull};
+    const cudaError_t e = allow_smem_once(done, dev, prep_fused_kernel<kCodes>, kFusedSmem);
+    if (e != cudaSuccess) return e;
+    return launch_early(prep_fused_kernel<kCodes>, grid, kPrepTcThreads, kFusedSmem, s, 1, p, map_src, map_wide, p.fuse_table, total);
 }
 
 cudaError_t launch_prep(const Params &p, cudaStream_t s)
 {
     const bool bf16 = p.dtype == RKV_BF16;
+    int dev = 0, sms = 0;
+    cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess) return e;
+    const int total = p.tiles * p.batch * p.hkv;
     if (p.fuse_mode != 0) {                 // the tensor-core form that also writes the scoring copy
         const uint64_t wide_rows = (uint64_t)p.batch * p.hkv * p.cap + kTile;
         const uint64_t src_rows = p.fuse_table ? (uint64_t)p.pool_pages * kTile : (uint64_t)p.batch * p.hkv * p.cap;
@@ -738,41 +741,25 @@ cudaError_t launch_prep(const Params &p, cudaStream_t s)
         if (!sm100::make_map_row128(&map_src, p.fuse_src, src_rows, p.fuse_mode == 1) ||
             !sm100::make_map(&map_wide, p.k_cache, wide_rows, kTile))
             return cudaErrorInvalidValue;
-        int dev = 0, sms = 0;
-        cudaError_t e;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        const int total = p.tiles * p.batch * p.hkv;
         const unsigned grid = (unsigned)std::min(total, kFusedBlocks * sms);
-        if (p.fuse_mode == 1) {
-            if ((e = cudaFuncSetAttribute(prep_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmem)) != cudaSuccess) return e;
-            prep_fused_kernel<true><<<grid, kPrepTcThreads, kFusedSmem, s>>>(p, map_src, map_wide, p.fuse_table, total);
-        } else {
-            if ((e = cudaFuncSetAttribute(prep_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmem)) != cudaSuccess) return e;
-            prep_fused_kernel<false><<<grid, kPrepTcThreads, kFusedSmem, s>>>(p, map_src, map_wide, p.fuse_table, total);
-        }
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        head_sum_kernel<<<(unsigned)(p.batch * p.hkv), kHeadDim, 0, s>>>(p);
-        return cudaGetLastError();
+        e = p.fuse_mode == 1 ? launch_fused_for<true>(p, map_src, map_wide, grid, total, dev, s)
+                             : launch_fused_for<false>(p, map_src, map_wide, grid, total, dev, s);
+        if (e != cudaSuccess) return e;
+        return launch_early(head_sum_kernel, (unsigned)(p.batch * p.hkv), kHeadDim, 0, s, 1, p);
     }
     if (bf16 && p.d == kHeadDim) {          // the tensor-core form
+        static std::atomic<unsigned long long> done{0ull};
         CUtensorMap map_k;
         if (!sm100::make_map(&map_k, p.k_cache, sm100::key_rows_total(p), kTile)) return cudaErrorInvalidValue;
-        cudaError_t e = cudaFuncSetAttribute(prep_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepTcSmem);
+        if ((e = allow_smem_once(done, dev, prep_tc_kernel, kPrepTcSmem)) != cudaSuccess) return e;
+        e = launch_early(prep_tc_kernel, (unsigned)std::min(total, kPrepTcBlocks * sms), kPrepTcThreads, kPrepTcSmem, s, 1, p, map_k, total);
         if (e != cudaSuccess) return e;
-        int dev = 0, sms = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        const int total = p.tiles * p.batch * p.hkv;
-        prep_tc_kernel<<<(unsigned)std::min(total, kPrepTcBlocks * sms), kPrepTcThreads, kPrepTcSmem, s>>>(p, map_k, total);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        head_sum_kernel<<<(unsigned)(p.batch * p.hkv), kHeadDim, 0, s>>>(p);
-        return cudaGetLastError();
+        return launch_early(head_sum_kernel, (unsigned)(p.batch * p.hkv), kHeadDim, 0, s, 1, p);
     }
     switch (p.d) {
-        case 64: return bf16 ? launch_prep_for<__nv_bfloat16, 64>(p, s) : launch_prep_for<float, 64>(p, s);
-        case 128: return bf16 ? launch_prep_for<__nv_bfloat16, 128>(p, s) : launch_prep_for<float, 128>(p, s);
-        case 256: return bf16 ? launch_prep_for<__nv_bfloat16, 256>(p, s) : launch_prep_for<float, 256>(p, s);
+        case 64: return bf16 ? launch_prep_for<__nv_bfloat16, 64>(p, dev, s) : launch_prep_for<float, 64>(p, dev, s);
+        case 128: return bf16 ? launch_prep_for<__nv_bfloat16, 128>(p, dev, s) : launch_prep_for<float, 128>(p, dev, s);
+        case 256: return bf16 ? launch_prep_for<__nv_bfloat16, 256>(p, dev, s) : launch_prep_for<float, 256>(p, dev, s);
         default: return cudaErrorInvalidValue;
     }
 }

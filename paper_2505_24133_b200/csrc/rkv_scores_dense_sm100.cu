@@ -80,6 +80,8 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
     auto bar = [bar0](int idx) -> uint32_t { return bar0 + 8u * (uint32_t)idx; };
 
     const ErrSink sink = make_sink(p);
+    pdl_trigger();
+    pdl_wait();
     if (threadIdx.x == 0) *bail = (call_aborted(p) || *item_count == 0ull) ? 1 : 0;     // nothing listed for this route
     __syncthreads();
     if (*bail) return;
@@ -389,6 +391,8 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
 {
     // work unit = (head, chunk of 256 tokens), handed out with the grid as stride.  When no head took the route (the
     // common case: no work item of the symmetric scan was ever listed) the blocks return at once.
+    pdl_trigger();
+    pdl_wait();
     const int chunks = (p.cap + kFinishThreads - 1) / kFinishThreads;
     const long long units = (long long)p.batch * p.hkv * chunks;
     if (call_aborted(p) || p.counters[kDenseWords] == 0ull) return;
@@ -423,20 +427,20 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
 
 cudaError_t launch_scores_dense_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns, int sms)
 {
-    cudaError_t e = cudaFuncSetAttribute(scores_dense_sm100_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesD);
-    if (e != cudaSuccess) return e;
+    static std::atomic<unsigned long long> done{0ull};
+    int dev = 0;
+    cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_dense_sm100_kernel, kSmemBytesD)) != cudaSuccess) return e;
     const unsigned long long max_items = (unsigned long long)(p.batch * p.hkv) * (unsigned long long)((p.tiles + 1) / 2);
     const unsigned grid = (unsigned)(max_items < (unsigned long long)sms ? max_items : (unsigned long long)sms);
-    scores_dense_sm100_kernel<<<grid, kThreadsD, kSmemBytesD, s>>>(p, map_k, map_ns);
-    return cudaGetLastError();
+    return launch_early(scores_dense_sm100_kernel, grid, kThreadsD, kSmemBytesD, s, 1, p, map_k, map_ns);
 }
 
 cudaError_t launch_dense_finish(const Params &p, cudaStream_t s, int sms)
 {
     const unsigned long long units = (unsigned long long)(p.batch * p.hkv) * (unsigned long long)((p.cap + kFinishThreads - 1) / kFinishThreads);
     const unsigned long long wave = 8ull * (unsigned long long)sms;             // resident blocks of this size
-    dense_finish_kernel<<<(unsigned)(units < wave ? units : wave), kFinishThreads, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch_early(dense_finish_kernel, (unsigned)(units < wave ? units : wave), kFinishThreads, 0, s, 1, p);
 }
 
 }  // namespace rkv

@@ -105,6 +105,8 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
 
     // Once a bounded wait of this call has run out, the blocks still to start return at once.
     const ErrSink sink = make_sink(p);
+    pdl_trigger();
+    pdl_wait();
     if (threadIdx.x == 0) *bail = call_aborted(p) ? 1 : 0;
     __syncthreads();
     if (*bail) return;
@@ -509,19 +511,19 @@ cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUt
 {
     const SmemPlan pl = make_plan(q_rows_pad);
     if (pl.stages < 2) return cudaErrorInvalidConfiguration;
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(scores_stream_sm100_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.total)) !=
-        cudaSuccess)
-        return e;
+    // (how much shared memory a call needs depends on its query group: the most that any may need is allowed once)
+    static std::atomic<unsigned long long> done{0ull};
+    int dev = 0;
+    cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel, kSmemLimit)) != cudaSuccess) return e;
     const int heads = p.batch * p.hkv;
     // a head is cut into parts when there are too few heads to give every SM several items
     int splits = (4 * sms + heads - 1) / heads;
     splits = splits < 1 ? 1 : (splits > p.tiles ? p.tiles : splits);
     const unsigned long long total_items = (unsigned long long)splits * (unsigned long long)heads;
     const unsigned grid = (unsigned)(total_items < (unsigned long long)sms ? total_items : (unsigned long long)sms);
-    scores_stream_sm100_kernel<<<grid, kThreadsP1, pl.total, s>>>(p, map_k, map_q, map_hs, map_ns, map_ts, splits, total_items,
-                                                                  q_rows_pad);
-    return cudaGetLastError();
+    return launch_early(scores_stream_sm100_kernel, grid, kThreadsP1, (size_t)pl.total, s, 1, p, map_k, map_q, map_hs, map_ns, map_ts, splits,
+                        total_items, q_rows_pad);
 }
 
 }  // namespace rkv

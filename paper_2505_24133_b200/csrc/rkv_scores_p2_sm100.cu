@@ -104,6 +104,8 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
     // invalid length does not stop the others: it just has no candidates).  Pass 2 has nothing to do when the list
     // is empty.
     const ErrSink sink = make_sink(p);
+    pdl_trigger();
+    pdl_wait();
     if (threadIdx.x == 0) {
         int b = call_aborted(p) ? 1 : 0;
         if (*item_count == 0ull) b = 1;
@@ -555,6 +557,8 @@ __global__ void __launch_bounds__(kCompactThreads) strag_compact_kernel(Params p
 {
     __shared__ int warp_tot[kCompactThreads / 32];
     __shared__ int running;
+    pdl_trigger();
+    pdl_wait();
     const int head = blockIdx.x;
     const int n = seq_candidates(p, head / p.hkv);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -651,12 +655,10 @@ cudaError_t launch_scores_tri_sm100(const Params &p, cudaStream_t s)
         !make_map_k16(&map_ts, p.thr_split, (uint64_t)p.batch * p.hkv * kTile))
         return cudaErrorInvalidValue;
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(scores_pass2_sm100_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes)) !=
-        cudaSuccess)
-        return e;
+    static std::atomic<unsigned long long> done{0ull};
     int dev = 0, sms = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = device_sms(&dev, &sms)) != cudaSuccess || (e = allow_smem_once(done, dev, scores_pass2_sm100_kernel, kSmemBytes)) != cudaSuccess)
+        return e;
     const int heads = p.batch * p.hkv;
     if ((e = launch_scores_pass1_sm100(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad, sms)) != cudaSuccess) return e;
     if ((e = mark_kernel(p, 0, s)) != cudaSuccess) return e;
@@ -672,11 +674,9 @@ cudaError_t launch_scores_tri_sm100(const Params &p, cudaStream_t s)
     int below = 0;
     for (int r = 0; r < rounds; ++r) {
         const int width = r == rounds - 1 ? (1 << 20) : kRoundTiles[r];
-        strag_compact_kernel<<<(unsigned)heads, kCompactThreads, 0, s>>>(p, r, below, width);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_early(strag_compact_kernel, (unsigned)heads, kCompactThreads, 0, s, 1, p, r, below, width)) != cudaSuccess) return e;
         if (r == 0 && (e = mark_kernel(p, 1, s)) != cudaSuccess) return e;
-        scores_pass2_sm100_kernel<<<grid2, kThreads, kSmemBytes, s>>>(p, map_k, map_ns, r);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_early(scores_pass2_sm100_kernel, grid2, kThreads, kSmemBytes, s, 1, p, map_k, map_ns, r)) != cudaSuccess) return e;
         // the heads the first listing sent to the symmetric route (none on inputs where similar keys are common:
         // the kernel then returns at once)
         if (r == 0 && dense_possible && (e = launch_scores_dense_sm100(p, s, map_k, map_ns, sms)) != cudaSuccess) return e;

@@ -92,6 +92,8 @@ __global__ void __launch_bounds__(kSimtThreads, D <= 128 ? 3 : 2) scores_simt_ke
     extern __shared__ __align__(16) float smem[];
     float *tileA = smem, *tileB = smem + kRowsA * S::kPad;
     __shared__ float rB[kCols];
+    pdl_trigger();
+    pdl_wait();
 
     const int blocks_per_head = row_blocks + key_blocks;
     const int head = blockIdx.x / blocks_per_head;
@@ -206,10 +208,11 @@ cudaError_t launch_simt_for(const Params &p, cudaStream_t s)
     using S = SimtShape<D>;
     const int row_blocks = (p.cap + kRowsA - 1) / kRowsA, key_blocks = (p.cap + S::kCols - 1) / S::kCols;
     const unsigned grid = (unsigned)(row_blocks + key_blocks) * (unsigned)(p.batch * p.hkv);
-    cudaError_t e = cudaFuncSetAttribute(scores_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes);
-    if (e != cudaSuccess) return e;
-    scores_simt_kernel<T, D><<<grid, kSimtThreads, S::kBytes, s>>>(p, row_blocks, key_blocks);
-    return cudaGetLastError();
+    static std::atomic<unsigned long long> done{0ull};
+    int dev = 0, sms = 0;
+    cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_simt_kernel<T, D>, S::kBytes)) != cudaSuccess) return e;
+    return launch_early(scores_simt_kernel<T, D>, grid, kSimtThreads, S::kBytes, s, 1, p, row_blocks, key_blocks);
 }
 
 }  // namespace

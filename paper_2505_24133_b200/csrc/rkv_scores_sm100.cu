@@ -95,6 +95,8 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
     // instead of each waiting out its own limit.
     __shared__ int bail;
     const ErrSink sink = make_sink(p);
+    pdl_trigger();
+    pdl_wait();
     if (threadIdx.x == 0) bail = call_aborted(p) ? 1 : 0;      // a wait of this call has run out: nothing more is started
     __syncthreads();
     if (bail) return;
@@ -206,7 +208,12 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
             const float *inv_norm = p.inv_norm + (size_t)head * p.cap_pad;
             for (int v = et; v < n_tiles * (kTile / 4); v += 256)
                 reinterpret_cast<float4 *>(r_s)[v] = __ldg(reinterpret_cast<const float4 *>(inv_norm) + v);
-            if (et < kDim) sum_s[et] = p.head_sum[(size_t)head * kDim + et];
+            if (et < kDim) {                 // the tile sums added up in tile order
+                const float *ts = p.tile_sum + (size_t)head * p.tiles * kDim + et;
+                float sum = 0.f;
+                for (int q = 0; q < p.tiles; ++q) sum += ts[(size_t)q * kDim];
+                sum_s[et] = sum;
+            }
             epi_barrier();
 
             const int i = row0 + half * kTile + lrow;
@@ -340,10 +347,11 @@ template <int kBlocks>
 cudaError_t launch_blocks(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q, unsigned grid,
                           int row_blocks, int q_rows_pad)
 {
-    const cudaError_t e = cudaFuncSetAttribute(scores_sm100_kernel<kBlocks>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<kBlocks>::kBytes);
-    if (e != cudaSuccess) return e;
-    scores_sm100_kernel<kBlocks><<<grid, kThreads, Smem<kBlocks>::kBytes, s>>>(p, map_k, map_q, row_blocks, q_rows_pad);
-    return cudaGetLastError();
+    static std::atomic<unsigned long long> done{0ull};
+    int dev = 0, sms = 0;
+    cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_sm100_kernel<kBlocks>, Smem<kBlocks>::kBytes)) != cudaSuccess) return e;
+    return launch_early(scores_sm100_kernel<kBlocks>, grid, kThreads, Smem<kBlocks>::kBytes, s, 1, p, map_k, map_q, row_blocks, q_rows_pad);
 }
 
 }  // namespace

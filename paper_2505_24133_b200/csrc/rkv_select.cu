@@ -69,6 +69,8 @@ constexpr int kImpTokens = 1024;     // tokens per importance block
 __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(Params p)
 {
     __shared__ float scratch[kStatThreads / 32];
+    pdl_trigger();
+    pdl_wait();
     const int head = blockIdx.x / p.alpha, j = blockIdx.x % p.alpha;
     const int n = seq_candidates(p, head / p.hkv);
     if (n == 0) return;
@@ -101,6 +103,8 @@ __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(Params p)
 // Eq. 4 for kImpTokens tokens of one head.
 __global__ void __launch_bounds__(kImpThreads) importance_kernel(Params p)
 {
+    pdl_trigger();
+    pdl_wait();
     const int chunks = (p.cap + kImpTokens - 1) / kImpTokens;
     const int head = blockIdx.x / chunks, i0 = (blockIdx.x % chunks) * kImpTokens;
     const int n = seq_candidates(p, head / p.hkv);
@@ -250,6 +254,8 @@ constexpr int kImp8Tokens = kImp8Threads * 8;
 
 __global__ void __launch_bounds__(kImp8Threads) importance_w4_kernel(Params p)
 {
+    pdl_trigger();
+    pdl_wait();
     const int chunks = (p.cap + kImp8Tokens - 1) / kImp8Tokens;
     const int head = blockIdx.x / chunks;
     const int i0 = (blockIdx.x % chunks) * kImp8Tokens + threadIdx.x * 8;     // first token of this thread
@@ -308,6 +314,8 @@ __global__ void __launch_bounds__(kFused ? kSelThreadsFused : kSelThreadsSplit, 
                                                    // kFused: then [cap_pad] importance and [alpha][cap_pad] logits
     __shared__ float stat_s[2 * RKV_MAX_GROUP_ROWS];
     __shared__ float scratch[kSelWarps];
+    pdl_trigger();
+    pdl_wait();
 
     const int head = blockIdx.x;
     const int b = head / p.hkv;
@@ -426,6 +434,8 @@ __global__ void __launch_bounds__(kSelThreadsSplit, 4) select_mean_kernel(Params
 {
     constexpr int kSelThreads = kSelThreadsSplit;
     extern __shared__ float row[];
+    pdl_trigger();
+    pdl_wait();
     const int b = blockIdx.x, tid = threadIdx.x;
     const int L = p.meta[b];
     if (call_aborted(p)) return;    // select_kernel has written -1 everywhere
@@ -448,43 +458,35 @@ bool select_is_fused(int cap_pad, int alpha) { return (size_t)(alpha + 2) * cap_
 
 static cudaError_t launch_select_mean(const Params &p, cudaStream_t s)
 {
-    const size_t smem = (size_t)p.cap_pad * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(select_mean_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    select_mean_kernel<<<(unsigned)p.batch, kSelThreadsSplit, smem, s>>>(p);
-    return cudaGetLastError();
+    // (up to 32 KB of shared memory: RKV_MAX_CAP words)
+    return launch_early(select_mean_kernel, (unsigned)p.batch, kSelThreadsSplit, (size_t)p.cap_pad * sizeof(float), s, 1, p);
 }
 
 cudaError_t launch_select(const Params &p, cudaStream_t s)
 {
     const unsigned heads = (unsigned)(p.batch * p.hkv);
-    cudaError_t e;
+    int dev = 0, sms = 0;
+    cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess) return e;
     if (select_is_fused(p.cap_pad, p.alpha)) {
         // small caches: one kernel does row statistics, importance and selection
+        static std::atomic<unsigned long long> done{0ull};
         if ((e = mark_kernel(p, 2, s)) != cudaSuccess || (e = mark_kernel(p, 3, s)) != cudaSuccess) return e;
-        const size_t smem = (size_t)(p.alpha + 2) * p.cap_pad * sizeof(float);
-        if ((e = cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
-            return e;
-        select_kernel<true><<<heads, kSelThreadsFused, smem, s>>>(p);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = allow_smem_once(done, dev, select_kernel<true>, (int)kFusedSmemLimit)) != cudaSuccess) return e;
+        e = launch_early(select_kernel<true>, heads, kSelThreadsFused, (size_t)(p.alpha + 2) * p.cap_pad * sizeof(float), s, 1, p);
+        if (e != cudaSuccess) return e;
         return p.head_mean ? launch_select_mean(p, s) : cudaSuccess;
     }
-    row_stats_kernel<<<heads * (unsigned)p.alpha, kStatThreads, 0, s>>>(p);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_early(row_stats_kernel, heads * (unsigned)p.alpha, kStatThreads, 0, s, 1, p)) != cudaSuccess) return e;
     if ((e = mark_kernel(p, 2, s)) != cudaSuccess) return e;
     if (p.pool_w == 4 && !p.mean_then_pool)
-        importance_w4_kernel<<<heads * (unsigned)((p.cap + kImp8Tokens - 1) / kImp8Tokens), kImp8Threads, 0, s>>>(p);
+        e = launch_early(importance_w4_kernel, heads * (unsigned)((p.cap + kImp8Tokens - 1) / kImp8Tokens), kImp8Threads, 0, s, 1, p);
     else
-        importance_kernel<<<heads * (unsigned)((p.cap + kImpTokens - 1) / kImpTokens), kImpThreads, 0, s>>>(p);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_early(importance_kernel, heads * (unsigned)((p.cap + kImpTokens - 1) / kImpTokens), kImpThreads, 0, s, 1, p);
+    if (e != cudaSuccess) return e;
     if ((e = mark_kernel(p, 3, s)) != cudaSuccess) return e;
-    const size_t smem = (size_t)p.cap_pad * sizeof(float);
-    if ((e = cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-        cudaSuccess)
-        return e;
-    select_kernel<false><<<heads, kSelThreadsSplit, smem, s>>>(p);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_early(select_kernel<false>, heads, kSelThreadsSplit, (size_t)p.cap_pad * sizeof(float), s, 1, p);
+    if (e != cudaSuccess) return e;
     return p.head_mean ? launch_select_mean(p, s) : cudaSuccess;
 }
 

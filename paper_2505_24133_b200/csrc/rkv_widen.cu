@@ -25,6 +25,8 @@ __global__ void __launch_bounds__(kWidenThreads)
 widen_keys_kernel(Params p, int key_blocks, __nv_bfloat16 *wide, int src_vecs, int dst_vecs, int codes, const uint4 *q_src, uint4 *q_dst,
                   int q_rows)
 {
+    pdl_trigger();
+    pdl_wait();
     if ((int)blockIdx.x >= key_blocks) {
         // queries: rows of src_q_vecs = dst_vecs / 2 vectors (bf16, 64 dimensions) -> rows of dst_vecs, zero-padded
         const int q_vecs = dst_vecs / 2;
@@ -75,9 +77,8 @@ cudaError_t launch_widen_keys(const Params &stored, __nv_bfloat16 *wide, int wid
     const unsigned key_blocks = keys ? (unsigned)stored.tiles * (unsigned)(stored.batch * stored.hkv) : 0u;
     const unsigned grid = key_blocks + (unsigned)((q_rows + kTile - 1) / kTile);
     if (grid == 0u) return cudaSuccess;
-    widen_keys_kernel<<<grid, kWidenThreads, 0, s>>>(stored, (int)key_blocks, wide, stored.store_row_bytes / 16, wide_d * 2 / 16, codes,
-                                                     static_cast<const uint4 *>(q_src), static_cast<uint4 *>(q_dst), q_rows);
-    return cudaGetLastError();
+    return launch_early(widen_keys_kernel, grid, kWidenThreads, 0, s, 1, stored, (int)key_blocks, wide, stored.store_row_bytes / 16,
+                        wide_d * 2 / 16, codes, static_cast<const uint4 *>(q_src), static_cast<uint4 *>(q_dst), q_rows);
 }
 
 }  // namespace rkv
