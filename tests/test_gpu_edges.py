@@ -117,3 +117,45 @@ def test_host_buffers_in_pieces(rkv, batch):  # noqa: F811
             n = int(hs[b])
             assert torch.equal(hk[b, :, :n].view(torch.int16), wl.k_cache[b, :, :n].cpu().view(torch.int16))
             assert torch.equal(hv[b, :, :n].view(torch.int16), wl.v_cache[b, :, :n].cpu().view(torch.int16))
+
+
+@pytest.mark.parametrize("head_dim,dtype", [(64, "fp8"), (64, "bf16"), (128, "bf16"), (256, "bf16"), (256, "f32")])
+@pytest.mark.parametrize("pattern", ["runs", "last_k", "sparse", "identity"])
+def test_compaction_by_bulk_copies(rkv, head_dim, dtype, pattern):  # noqa: F811
+    """More streams than SMs: the gather stage alone on hand-made ascending lists, every row width; runs that cross chunks,
+    single rows, a long shift, a list in place already, a budget that is not a whole number of chunks; ragged lengths."""
+    batch, hkv, budget, buffer, alpha = 19, 4, 333, 83, 8
+    spec = small_spec("bulk", batch=batch, hkv=hkv, hq=hkv, budget=budget, buffer=buffer, head_dim=head_dim, dtype=dtype)
+    cap = spec.cap
+    lens = torch.tensor([budget - 5 if b % 7 == 3 else cap - b % 5 for b in range(batch)])
+    wl = ri.make_workload(spec, device="cuda", seed=441, seq_lens=lens)
+    comp = rkv.Compressor(batch, hkv, hkv, budget, buffer, alpha, 0.1, dtype=spec.torch_dtype, head_dim=head_dim)
+    comp.compress(wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens, stages=rkv.RKV_STAGE_PREP)       # records lengths
+    g = torch.Generator().manual_seed(5)
+    idx = torch.empty(batch, hkv, budget, dtype=torch.int32)
+    for b in range(batch):
+        L = int(lens[b])
+        for h in range(hkv):
+            if pattern == "identity" or L <= budget:
+                row = torch.arange(budget)
+            elif pattern == "last_k":
+                row = torch.arange(L - budget, L)
+            elif pattern == "sparse":
+                row = torch.randperm(L, generator=g)[:budget].sort().values
+            else:                                    # what is dropped comes in spans
+                keep = torch.ones(L, dtype=torch.bool)
+                drop = L - budget
+                start = int(torch.randint(0, L - drop, (1,), generator=g))
+                keep[start:start + drop] = False
+                row = keep.nonzero().flatten()
+            idx[b, h] = row.int()
+    comp.out_idx.copy_(idx)
+    u8 = lambda t: t.view(torch.uint8)  # noqa: E731
+    k0, v0 = u8(wl.k_cache).clone(), u8(wl.v_cache).clone()
+    comp.compress(wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens, stages=rkv.RKV_STAGE_GATHER)
+    torch.cuda.synchronize()
+    comp.check_status()
+    take = idx.long().cuda()[..., None].expand(-1, -1, -1, k0.shape[-1])
+    assert torch.equal(u8(wl.k_cache)[:, :, :budget], k0.gather(2, take))
+    assert torch.equal(u8(wl.v_cache)[:, :, :budget], v0.gather(2, take))
+    assert wl.seq_lens.tolist() == [min(int(x), budget) for x in lens]
