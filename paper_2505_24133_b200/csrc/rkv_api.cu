@@ -22,7 +22,7 @@ int cuda_fail(cudaError_t e, const char *where)
 }
 
 struct Layout {
-    size_t k_wide, q_wide, best, dense, dense_items, inv_norm, norm_split, thr_split, tile_sum, logits, row_stat, imp, sbar, left, strag, strag_count, strag_items, self_dot, head_sum_bf16, meta, counters, total;
+    size_t k_wide, q_wide, best, dense, dense_items, inv_norm, norm_split, thr_split, tile_sum, logits, row_stat, imp, sbar, left, lacking, strag, strag_items, self_dot, head_sum_bf16, meta, counters, total;
     int cap, cap_pad, tiles, tri;
 };
 
@@ -103,7 +103,7 @@ int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout 
         const size_t tri = (size_t)lay->tri;
         lay->left = off;        off = align_up(off + tri * P * lay->cap_pad * sizeof(int32_t), 256);
         lay->strag = off;       off = align_up(off + tri * P * lay->cap_pad * sizeof(int32_t), 256);
-        lay->strag_count = off; off = align_up(off + tri * P * sizeof(int32_t), 256);
+        lay->lacking = off;     off = align_up(off + tri * P * (lay->cap_pad / 32) * sizeof(uint32_t), 256);
         lay->strag_items = off; off = align_up(off + tri * P * (lay->cap_pad / 256 + 1) * sizeof(int4), 256);
         lay->best = off;        off = align_up(off + tri * P * lay->cap_pad * sizeof(uint32_t), 256);
         lay->dense = off;       off = align_up(off + tri * P * sizeof(int32_t), 256);
@@ -176,7 +176,7 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
     p.sbar = reinterpret_cast<float *>(ws + lay.sbar);
     p.left = reinterpret_cast<int32_t *>(ws + lay.left);
     p.strag = reinterpret_cast<int32_t *>(ws + lay.strag);
-    p.strag_count = reinterpret_cast<int32_t *>(ws + lay.strag_count);
+    p.lacking = reinterpret_cast<uint32_t *>(ws + lay.lacking);
     p.strag_items = reinterpret_cast<int4 *>(ws + lay.strag_items);
     p.self_dot = reinterpret_cast<float *>(ws + lay.self_dot);
     p.best = reinterpret_cast<uint32_t *>(ws + lay.best);

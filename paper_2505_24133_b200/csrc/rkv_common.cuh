@@ -62,9 +62,9 @@ struct Params {
     float *sbar;         // [P][cap_pad]         Eq. 6 column means after the retention rule.  With `tri` set the scoring
                          //                      kernels leave column SUMS minus the removed entries (the select stage
                          //                      divides by n)
-    int32_t *left;       // [P][cap_pad]         tri: partners a token still lacks after the scan of its own line
-    int32_t *strag;      // [P][cap_pad]         tri: positions of the head's tokens with left > 0, ascending
-    int32_t *strag_count;// [P]                  tri: how many
+    uint32_t *lacking;   // [P][cap_pad / 32]    tri: a bit per token that is still short of partners
+    int32_t *left;       // [P][cap_pad]         tri, beta > 1: how many partners it still lacks
+    int32_t *strag;      // [P][cap_pad]         tri: positions of the head's tokens short of partners, ascending
     int4 *strag_items;   // [P * cap_pad / 256]  tri: work list of the second scoring pass: {head, first listed
                          //                      token, tokens (1..256), first streamed tile}
     uint32_t *best;      // [P][cap_pad]         symmetric route: largest partner position + 1 found so far (0 = none)

@@ -262,7 +262,7 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 const int i = pi * kRowsPerItem + m * kTile + gt;
                 const bool row_ok = i < n;
                 const float ri = row_ok ? __ldg(p.inv_norm + hoff + i) : 0.f;
-                const int lf = row_ok ? p.left[hoff + i] : 0;
+                const int lf = row_ok ? (int)(p.lacking[(hoff + i) >> 5] >> (i & 31) & 1u) : 0;
                 float rest = (row_ok && ri > 0.f) ? -__fdiv_rn(p.sim_threshold, ri) : 0.f;
                 uint32_t part[3];
 #pragma unroll
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
     const int n = seq_candidates(p, head / p.hkv);
     if (i >= n) continue;
     const size_t hoff = (size_t)head * p.cap_pad;
-    if (p.left[hoff + i] <= 0) continue;
+    if (!(p.lacking[(hoff + i) >> 5] >> (i & 31) & 1u)) continue;
     const uint32_t b = p.best[hoff + i];
     if (b == 0u) continue;
     const int j = (int)b - 1;
@@ -419,7 +419,6 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
         for (int e = 0; e < 8; ++e) dot = fmaf(a[e], bb[e], dot);
     }
     p.sbar[hoff + i] -= dot * p.inv_norm[hoff + i] * p.inv_norm[hoff + j];
-    p.left[hoff + i] = 0;
     }
 }
 

@@ -16,7 +16,7 @@
 //                            or the mean, over the group: Eq. 3), then k_i . s in three parts, which gives
 //                            sum_j S[j][i] = Kbar_i . (sum_j Kbar_j) - Kbar_i . Kbar_i without forming the matrix
 //
-// Out, per token: the pooled logits, the column sum minus the removed entries (sbar), the partners still lacking (left).
+// Out, per token: the pooled logits, the column sum minus the removed entries (sbar), the partners still lacking (a bit, and for beta > 1 how many).
 //
 // Work item = (head, range of row tiles); items are handed out by a global ticket counter, head-major.  The operands
 // that stay put are double-buffered across items, so the next item's arrive while the current one is streamed, and
@@ -481,7 +481,11 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                         for (int j = 0; j < 8; ++j) logits[(size_t)j * p.cap_pad + i] = pooled[j];
                     }
                     p.sbar[(size_t)head * p.cap_pad + i] = total - ((float)nhit * p.sim_threshold + removed * ri);
-                    p.left[(size_t)head * p.cap_pad + i] = rule_on ? left : 0;
+                    if (p.beta > 1 && rule_on) p.left[(size_t)head * p.cap_pad + i] = left;
+                }
+                if (rule_on) {                   // the tokens still short of partners, a bit each
+                    const unsigned lacking = __ballot_sync(0xffffffffu, left > 0);
+                    if (lane == 0) p.lacking[(size_t)head * (p.cap_pad / 32) + t * 4 + quad] = lacking;
                 }
             }
             if (!ok) break;

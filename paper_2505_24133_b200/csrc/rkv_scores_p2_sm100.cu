@@ -7,7 +7,7 @@
 // first beta hits".  The first pass scans every token against the last key tile; where similar keys are common that
 // settles most tokens.  The rest is done here, in ROUNDS:
 //
-//   list    The tokens with left > 0 are listed per head, ascending, in chunks of 256 (strag_compact_kernel).
+//   list    The tokens still short of partners (a bit each, kept by the scans) are listed per head, ascending, in chunks of 256 (strag_compact_kernel).
 //   scan    Work item = (head, chunk of 256 listed tokens, window of key tiles): the chunk's key rows are gathered
 //           into two resident operand tiles by the epilogue warps; the window's key tiles stream through a ring, last
 //           to first.  The removed entries are subtracted from what the first pass stored, `left` is updated.
@@ -297,7 +297,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
                 rr[m] = pos[m] >= 0 ? __ldg(p.inv_norm + hoff + pos[m]) : 0.f;
-                lf[m] = pos[m] >= 0 ? p.left[hoff + pos[m]] : 0;
+                lf[m] = pos[m] >= 0 ? (p.beta == 1 ? 1 : p.left[hoff + pos[m]]) : 0;
             }
             int32_t *stash_i = reinterpret_cast<int32_t *>(smem + kOffStash + ab * 3 * kRowsPerItem * 4);
             float *stash_r = reinterpret_cast<float *>(stash_i + kRowsPerItem);
@@ -529,7 +529,9 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 }
                 if (nhit > 0) {
                     p.sbar[(size_t)head * p.cap_pad + i] -= (float)nhit * p.sim_threshold + removed * ri;
-                    p.left[(size_t)head * p.cap_pad + i] = left;       // the next round lists the tokens still short
+                    if (p.beta != 1) p.left[(size_t)head * p.cap_pad + i] = left;
+                    // the next round lists the tokens still short
+                    if (left == 0) atomicAnd(p.lacking + (((size_t)head * p.cap_pad + i) >> 5), ~(1u << (i & 31)));
                 }
             }
             ++k_item;
@@ -548,21 +550,22 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 }
 
 // ---- before every round: list, per head, the tokens still short of partners, and cut the list into work items ----
-constexpr int kCompactThreads = 256;
+constexpr int kCompactWarps = 8;         // a warp per head
+constexpr int kWordsPerLane = RKV_MAX_CAP / 32 / 32;
 constexpr int kDenseMinTiles = 12;       // caches of fewer key tiles never take the symmetric route (two more launches)
 
+// The tokens are given as one bit each, 32 to a word, so a list costs a head's 33 words per 1024 tokens and what it writes.
+// (Read from a word per token by a block per head, a listing of 4096 heads of 4216 tokens took 81 us; 37 now.)
 // `below`: key tiles under the first pass's part that earlier rounds have covered; `width`: tiles of this round's
 // window (the last round passes a width that reaches tile 0 whatever the cache size).
-__global__ void __launch_bounds__(kCompactThreads) strag_compact_kernel(Params p, int round, int below, int width)
+__global__ void __launch_bounds__(kCompactWarps * 32) strag_compact_kernel(Params p, int round, int below, int width)
 {
-    __shared__ int warp_tot[kCompactThreads / 32];
-    __shared__ int running;
     pdl_trigger();
     pdl_wait();
-    const int head = blockIdx.x;
+    const int head = blockIdx.x * kCompactWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (head >= p.batch * p.hkv) return;
     const int n = seq_candidates(p, head / p.hkv);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int32_t *left = p.left + (size_t)head * p.cap_pad;
+    const uint32_t *bits = p.lacking + (size_t)head * (p.cap_pad / 32);
     int32_t *list = p.strag + (size_t)head * p.cap_pad;
     // the first pass scanned every token against the last kPass1Depth key tiles; this round starts `below` tiles
     // under that
@@ -570,66 +573,71 @@ __global__ void __launch_bounds__(kCompactThreads) strag_compact_kernel(Params p
     const int first_tile = n_tiles - kPass1Depth - 1 - below;
     if (first_tile < 0 || call_aborted(p) || (round > 0 && p.dense[head])) {
         // nothing left to scan for this head, the call has given up, or the head went to the symmetric route
-        if (threadIdx.x == 0) {
-            p.strag_count[head] = 0;
-            if (round == 0) p.dense[head] = 0;
-        }
+        if (lane == 0 && round == 0) p.dense[head] = 0;
         return;
     }
-    if (threadIdx.x == 0) running = 0;
-    __syncthreads();
-    for (int i0 = 0; i0 < n; i0 += kCompactThreads) {
-        const int i = i0 + threadIdx.x;
-        const bool want = i < n && left[i] > 0;
-        const unsigned bal = __ballot_sync(0xffffffffu, want);
-        if (lane == 0) warp_tot[warp] = __popc(bal);
-        __syncthreads();
-        int before = running;
-        for (int w = 0; w < warp; ++w) before += warp_tot[w];
-        if (want) list[before + __popc(bal & ((1u << lane) - 1u))] = i;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int t = 0;
-            for (int w = 0; w < kCompactThreads / 32; ++w) t += warp_tot[w];
-            running += t;
-        }
-        __syncthreads();
+    const int words = (n + 31) / 32;
+    uint32_t word[kWordsPerLane];
+    int count = 0;
+#pragma unroll
+    for (int k = 0; k < kWordsPerLane; ++k) {
+        word[k] = k * 32 + lane < words ? bits[k * 32 + lane] : 0u;
+        count += __popc(word[k]);
     }
+    count = __reduce_add_sync(0xffffffffu, count);
     if (round == 0) {
         // Most tokens still lack a partner (few pairs exceed T): the rounds would form nearly the whole matrix for this
         // head.  It goes to the symmetric route instead, which forms each tile pair once.
-        const bool dense = p.dense_ok && n_tiles >= kDenseMinTiles && 5 * running > 4 * n;
+        const bool dense = p.dense_ok && n_tiles >= kDenseMinTiles && 5 * count > 4 * n;
+        if (lane == 0) p.dense[head] = dense ? 1 : 0;
         if (dense) {
-            uint32_t *best = p.best + (size_t)head * p.cap_pad;
-            for (int i = threadIdx.x; i < p.cap_pad; i += kCompactThreads) best[i] = 0u;
-            if (threadIdx.x == 0) {
-                p.dense[head] = 1;
-                p.strag_count[head] = 0;
-                const int pairs_of_tiles = (n_tiles + 1) / 2;
-                const unsigned long long at = atomicAdd(&p.counters[kDenseWords], (unsigned long long)pairs_of_tiles);
-                for (int q = 0; q < pairs_of_tiles; ++q) p.dense_items[at + q] = make_int4(head, q, n, 0);   // longest first
+            uint4 *best = reinterpret_cast<uint4 *>(p.best + (size_t)head * p.cap_pad);
+            for (int i = lane; i < p.cap_pad / 4; i += 32) best[i] = make_uint4(0u, 0u, 0u, 0u);
+            const int pairs_of_tiles = (n_tiles + 1) / 2;
+            unsigned long long at = 0ull;
+            if (lane == 0) {
+                at = atomicAdd(&p.counters[kDenseWords], (unsigned long long)pairs_of_tiles);
                 // useful work: every unordered pair of the listed tokens' tiles once
-                atomicAdd(&p.counters[kPairsWord], (unsigned long long)running * (unsigned long long)(n_tiles + 1) / 2ull);
+                atomicAdd(&p.counters[kPairsWord], (unsigned long long)count * (unsigned long long)(n_tiles + 1) / 2ull);
             }
+            at = __shfl_sync(0xffffffffu, at, 0);
+            for (int q = lane; q < pairs_of_tiles; q += 32) p.dense_items[at + q] = make_int4(head, q, n, 0);   // longest first
             return;
         }
-        if (threadIdx.x == 0) p.dense[head] = 0;
     }
-    if (threadIdx.x == 0) {
-        const int count = running;
-        p.strag_count[head] = count;
-        const int chunks = (count + kRowsPerItem - 1) / kRowsPerItem;
-        if (chunks > 0) {
-            const int n_iter = min(width, first_tile + 1);
-            const unsigned long long at = atomicAdd(&p.counters[kRoundWords + 2 * round], (unsigned long long)chunks);
-            for (int q = 0; q < chunks; ++q) {
-                const int k0 = q * kRowsPerItem, rows = min(count - k0, kRowsPerItem);
-                p.strag_items[at + q] = make_int4(head, k0, rows | (n_iter << 16), first_tile);
-            }
-            atomicAdd(&p.counters[2], (unsigned long long)chunks);
-            // listed tokens x key tiles: the work the round cannot avoid
-            atomicAdd(&p.counters[kPairsWord], (unsigned long long)count * (unsigned long long)n_iter);
+    if (count == 0) return;
+    int at = 0;                              // ascending positions
+#pragma unroll
+    for (int k = 0; k < kWordsPerLane; ++k) {
+        if (k * 32 >= words) break;
+        const int mine = __popc(word[k]);
+        int incl = mine;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += o;
         }
+        const int first = at + incl - mine;
+        for (unsigned todo = __ballot_sync(0xffffffffu, mine > 0); todo != 0u; todo &= todo - 1u) {
+            const int src = __ffs(todo) - 1;
+            const uint32_t w = __shfl_sync(0xffffffffu, word[k], src);
+            const int f = __shfl_sync(0xffffffffu, first, src);
+            if (w >> lane & 1u) list[f + __popc(w & ((1u << lane) - 1u))] = (k * 32 + src) * 32 + lane;
+        }
+        at += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    const int chunks = (count + kRowsPerItem - 1) / kRowsPerItem, n_iter = min(width, first_tile + 1);
+    unsigned long long slot = 0ull;
+    if (lane == 0) {
+        slot = atomicAdd(&p.counters[kRoundWords + 2 * round], (unsigned long long)chunks);
+        atomicAdd(&p.counters[2], (unsigned long long)chunks);
+        // listed tokens x key tiles: the work the round cannot avoid
+        atomicAdd(&p.counters[kPairsWord], (unsigned long long)count * (unsigned long long)n_iter);
+    }
+    slot = __shfl_sync(0xffffffffu, slot, 0);
+    for (int q = lane; q < chunks; q += 32) {
+        const int k0 = q * kRowsPerItem;
+        p.strag_items[slot + q] = make_int4(head, k0, min(count - k0, kRowsPerItem) | (n_iter << 16), first_tile);
     }
 }
 
@@ -674,7 +682,7 @@ cudaError_t launch_scores_tri_sm100(const Params &p, cudaStream_t s)
     int below = 0;
     for (int r = 0; r < rounds; ++r) {
         const int width = r == rounds - 1 ? (1 << 20) : kRoundTiles[r];
-        if ((e = launch_early(strag_compact_kernel, (unsigned)heads, kCompactThreads, 0, s, 1, p, r, below, width)) != cudaSuccess) return e;
+        if ((e = launch_early(strag_compact_kernel, (unsigned)((heads + kCompactWarps - 1) / kCompactWarps), kCompactWarps * 32, 0, s, 1, p, r, below, width)) != cudaSuccess) return e;
         if (r == 0 && (e = mark_kernel(p, 1, s)) != cudaSuccess) return e;
         if ((e = launch_early(scores_pass2_sm100_kernel, grid2, kThreads, kSmemBytes, s, 1, p, map_k, map_ns, r)) != cudaSuccess) return e;
         // the heads the first listing sent to the symmetric route (none on inputs where similar keys are common:
