@@ -22,7 +22,7 @@ int cuda_fail(cudaError_t e, const char *where)
 }
 
 struct Layout {
-    size_t k_wide, q_wide, best, dense, dense_items, inv_norm, norm_split, thr_split, tile_sum, logits, row_stat, imp, sbar, left, lacking, strag, strag_items, self_dot, head_sum_bf16, meta, counters, total;
+    size_t k_wide, q_wide, best, dense, dense_items, inv_norm, norm_split, thr_split, tile_sum, logits, row_stat, keys, sbar, left, lacking, strag, strag_items, self_dot, head_sum_bf16, meta, counters, total;
     int cap, cap_pad, tiles, tri;
 };
 
@@ -96,8 +96,8 @@ int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout 
         const size_t hd = (size_t)scoring_dim(d);
         lay->tile_sum = off;  off = align_up(off + P * lay->tiles * hd * sizeof(float), 256);
         lay->logits = off;    off = align_up(off + P * alpha * lay->cap_pad * sizeof(float), 256);
-        lay->row_stat = off;  off = align_up(off + P * alpha * 2 * sizeof(float), 256);
-        lay->imp = off;       off = align_up(off + P * lay->cap_pad * sizeof(float), 256);
+        lay->row_stat = off;  off = align_up(off + P * (alpha + 1) * 2 * sizeof(float), 256);
+        lay->keys = off;      off = align_up(off + P * lay->cap_pad * sizeof(float), 256);
         lay->sbar = off;      off = align_up(off + P * lay->cap_pad * sizeof(float), 256);
         lay->tri = use_tri(d);
         const size_t tri = (size_t)lay->tri;
@@ -172,7 +172,7 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
     p.tile_sum = reinterpret_cast<float *>(ws + lay.tile_sum);
     p.logits = reinterpret_cast<float *>(ws + lay.logits);
     p.row_stat = reinterpret_cast<float *>(ws + lay.row_stat);
-    p.imp = reinterpret_cast<float *>(ws + lay.imp);
+    p.keys = reinterpret_cast<uint32_t *>(ws + lay.keys);
     p.sbar = reinterpret_cast<float *>(ws + lay.sbar);
     p.left = reinterpret_cast<int32_t *>(ws + lay.left);
     p.strag = reinterpret_cast<int32_t *>(ws + lay.strag);

@@ -43,7 +43,7 @@ struct Params {
     // hyper-parameters
     int pool_w, beta;
     int head_mean;                  // Algorithm 1's aggregated selection: one kept set per sequence from the
-                                    // head-averaged Z (select_kernel then leaves Z in `imp` and a second kernel selects)
+                                    // head-averaged Z (Z is then left in `keys` and a second kernel selects)
     int gqa_mean_pool;              // Eq. 3 with the mean over the group's query heads instead of the max
     int mean_then_pool;             // importance in Algorithm 1's order (mean over query rows, then pooling)
     float sim_threshold, eps, lambda;
@@ -57,8 +57,8 @@ struct Params {
                                   // to fp32 accuracy.  Both are written by the prep stage (two-pass route only).
     float *tile_sum;     // [P][tiles][128]      sum over the tile's candidate rows of r_i * k_i
     float *logits;       // [P][alpha][cap_pad]  Eq. 2-3: group-max of scaled logits
-    float *row_stat;     // [P][alpha][2]        Eq. 3 per row: max logit, 1 / sum of exp(logit - max)
-    float *imp;          // [P][cap_pad]         Eq. 4: importance I (head_mean: overwritten with Z by select_kernel)
+    float *row_stat;     // [P][alpha + 1][2]    per row of logits (Eq. 3), and of the column means (Eq. 6): maximum, 1 / sum of exp(value - max)
+    uint32_t *keys;      // [P][cap_pad]         Eq. 7: Z as an order-preserving integer (head_mean: Z itself)
     float *sbar;         // [P][cap_pad]         Eq. 6 column means after the retention rule.  With `tri` set the scoring
                          //                      kernels leave column SUMS minus the removed entries (the select stage
                          //                      divides by n)
