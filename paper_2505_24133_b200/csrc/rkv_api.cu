@@ -91,8 +91,8 @@ int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout 
         lay->q_wide = off;
         if (pads_dim(d)) off = align_up(off + (size_t)d->batch * d->n_q_heads * alpha * kHeadDim * sizeof(__nv_bfloat16), 256);
         lay->inv_norm = off;  off = align_up(off + P * lay->cap_pad * sizeof(float), 256);
-        lay->norm_split = off;  off = align_up(off + P * lay->cap_pad * 16 * sizeof(__nv_bfloat16), 256);
-        lay->thr_split = off;   off = align_up(off + P * kTile * 16 * sizeof(__nv_bfloat16), 256);
+        lay->norm_split = off;  off = align_up(off + P * lay->cap_pad * 8 * sizeof(__nv_bfloat16), 256);
+        lay->thr_split = off;   off = align_up(off + P * kTile * 8 * sizeof(__nv_bfloat16), 256);
         const size_t hd = (size_t)scoring_dim(d);
         lay->tile_sum = off;  off = align_up(off + P * lay->tiles * hd * sizeof(float), 256);
         lay->logits = off;    off = align_up(off + P * alpha * lay->cap_pad * sizeof(float), 256);

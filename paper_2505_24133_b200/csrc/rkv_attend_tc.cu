@@ -182,7 +182,7 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
     pdl_trigger();
-    pdl_wait();                             // what is above reads nothing that an earlier kernel writes
+    pdl_wait();                             // what is above uses nothing that an earlier kernel writes
 
     int L = p.seq_lens[b];
     if (L < 0 || L > p.cap) {               // reported, and treated as an empty cache

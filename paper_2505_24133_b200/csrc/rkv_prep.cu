@@ -159,9 +159,8 @@ __global__ void __launch_bounds__(kPrepThreads, D <= 128 ? 5 : 2) prep_kernel(Pa
                 part[c] = (uint32_t)__bfloat16_as_ushort(h16);
                 rest -= __bfloat162float(h16);
             }
-            uint4 *dst = reinterpret_cast<uint4 *>(p.norm_split + ((size_t)head * p.cap_pad + row) * 16);
+            uint4 *dst = reinterpret_cast<uint4 *>(p.norm_split + ((size_t)head * p.cap_pad + row) * sm100::kSliceElems);
             dst[0] = make_uint4(part[0] | (part[1] << 16), part[2] | (part[0] << 16), part[1] | (part[0] << 16), 0u);
-            dst[1] = make_uint4(0u, 0u, 0u, 0u);
             if (tile == (n + kTile - 1) / kTile - 1) {       // the head's last key tile: the first pass's resident operand
                 rest = r_mine > 0.f ? -__fdiv_rn(p.sim_threshold, r_mine) : 0.f;
 #pragma unroll
@@ -170,9 +169,8 @@ __global__ void __launch_bounds__(kPrepThreads, D <= 128 ? 5 : 2) prep_kernel(Pa
                     part[c] = (uint32_t)__bfloat16_as_ushort(h16);
                     rest -= __bfloat162float(h16);
                 }
-                uint4 *thr = reinterpret_cast<uint4 *>(p.thr_split + ((size_t)head * kTile + lr) * 16);
+                uint4 *thr = reinterpret_cast<uint4 *>(p.thr_split + ((size_t)head * kTile + lr) * sm100::kSliceElems);
                 thr[0] = make_uint4(part[0] | (part[0] << 16), part[0] | (part[1] << 16), part[1] | (part[2] << 16), 0u);
-                thr[1] = make_uint4(0u, 0u, 0u, 0u);
             }
         }
     }
@@ -409,9 +407,8 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
                     part[c] = (uint32_t)__bfloat16_as_ushort(h16);
                     rest -= __bfloat162float(h16);
                 }
-                uint4 *dst = reinterpret_cast<uint4 *>(p.norm_split + ((size_t)head * p.cap_pad + row) * 16);
+                uint4 *dst = reinterpret_cast<uint4 *>(p.norm_split + ((size_t)head * p.cap_pad + row) * sm100::kSliceElems);
                 dst[0] = make_uint4(part[0] | (part[1] << 16), part[2] | (part[0] << 16), part[1] | (part[0] << 16), 0u);
-                dst[1] = make_uint4(0u, 0u, 0u, 0u);
                 if (tile == (n + kTile - 1) / kTile - 1) {
                     rest = r > 0.f ? -__fdiv_rn(p.sim_threshold, r) : 0.f;
 #pragma unroll
@@ -420,9 +417,8 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
                         part[c] = (uint32_t)__bfloat16_as_ushort(h16);
                         rest -= __bfloat162float(h16);
                     }
-                    uint4 *thr = reinterpret_cast<uint4 *>(p.thr_split + ((size_t)head * kTile + rt) * 16);
+                    uint4 *thr = reinterpret_cast<uint4 *>(p.thr_split + ((size_t)head * kTile + rt) * sm100::kSliceElems);
                     thr[0] = make_uint4(part[0] | (part[0] << 16), part[0] | (part[1] << 16), part[1] | (part[2] << 16), 0u);
-                    thr[1] = make_uint4(0u, 0u, 0u, 0u);
                 }
             }
         }
@@ -634,9 +630,8 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
                     part[c] = (uint32_t)__bfloat16_as_ushort(h16);
                     rest -= __bfloat162float(h16);
                 }
-                uint4 *dst = reinterpret_cast<uint4 *>(p.norm_split + ((size_t)head * p.cap_pad + row) * 16);
+                uint4 *dst = reinterpret_cast<uint4 *>(p.norm_split + ((size_t)head * p.cap_pad + row) * sm100::kSliceElems);
                 dst[0] = make_uint4(part[0] | (part[1] << 16), part[2] | (part[0] << 16), part[1] | (part[0] << 16), 0u);
-                dst[1] = make_uint4(0u, 0u, 0u, 0u);
                 if (tile == (n + kTile - 1) / kTile - 1) {
                     rest = r > 0.f ? -__fdiv_rn(p.sim_threshold, r) : 0.f;
 #pragma unroll
@@ -645,9 +640,8 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
                         part[c] = (uint32_t)__bfloat16_as_ushort(h16);
                         rest -= __bfloat162float(h16);
                     }
-                    uint4 *thr = reinterpret_cast<uint4 *>(p.thr_split + ((size_t)head * kTile + rt) * 16);
+                    uint4 *thr = reinterpret_cast<uint4 *>(p.thr_split + ((size_t)head * kTile + rt) * sm100::kSliceElems);
                     thr[0] = make_uint4(part[0] | (part[0] << 16), part[0] | (part[1] << 16), part[1] | (part[2] << 16), 0u);
-                    thr[1] = make_uint4(0u, 0u, 0u, 0u);
                 }
             }
         }

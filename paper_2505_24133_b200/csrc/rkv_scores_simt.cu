@@ -4,7 +4,7 @@
 // for bf16 caches.  It forms Eq. 5's matrix in registers and accumulates Eq. 6's sums directly (no closed form), so the
 // kernels reach the same numbers along different routes.
 //
-// Block x of a head, x < row blocks: rows [64 x, 64 x + 64) of the similarity matrix: for each row i the column sum over j
+// Block x of a head, x < row blocks: 64 (small problems: 16) rows of the similarity matrix: for each row i the column sum over j
 // of S[j][i] (S is symmetric before the retention rule, which for token i touches line i only), minus the entries of the
 // up-to-beta largest j with S[j][i] > T.
 // The blocks after those: Eq. 2-3 pooled logits of the head's query group against 64 (d = 256: 32) candidate keys each.
@@ -13,7 +13,9 @@
 // multiply-adds (one thread per row with the whole head dimension, the earlier form, issued two loads per multiply-add:
 // 256 heads of 1144 tokens took 30 ms, a single head of 88 tokens 70 us).  Rows are D + 4 floats apart: the 16 column rows
 // that a half-warp reads lie in distinct banks, its own rows are broadcasts.  Packed multiply-adds over pairs of
-// dimensions.  Small caches get one block per 64 rows or keys, so that a single head occupies several SMs.
+// dimensions.  Where blocks of 64 rows would leave SMs without one, blocks of 16 rows (a 2 x 4 piece per thread): the time is
+// then one block's, and a quarter of the rows is a quarter of its multiply-adds (a single head of 88 tokens: 19 us with 64
+// rows per block, 9 with 16).
 #include "rkv_common.cuh"
 
 namespace rkv {
@@ -21,15 +23,16 @@ namespace rkv {
 namespace {
 
 constexpr int kSimtThreads = 128;
-constexpr int kRowsA = 64;          // rows of a block
-constexpr int kRowsT = 8;           // ... of which a thread holds: rg, rg + 8, ... (rg = thread / 16)
-
-template <int D> struct SimtShape {
+// kRowsT: rows that a thread holds of a block's 8 kRowsT: rg, rg + 8, ... (rg = thread / 16)
+template <int D, int kRowsT> struct SimtShape {
+    static constexpr int kRowsA = 8 * kRowsT;
     static constexpr int kPad = D + 4;
     static constexpr int kCols = D <= 128 ? 64 : 32;       // streamed keys per step
     static constexpr int kColsT = kCols / 16;              // ... of which a thread holds: cg, cg + 16, ... (cg = thread % 16)
-    static constexpr int kBytes = (kRowsA + kCols) * kPad * 4;
-    static_assert(RKV_MAX_GROUP_ROWS * (kCols + 1) * 4 <= kBytes, "the logits of a key block are staged in the tiles' room");
+    static constexpr int kChunks = (RKV_MAX_GROUP_ROWS + kRowsA - 1) / kRowsA;       // of the query rows
+    static constexpr int kTiles = (kRowsA + kCols) * kPad * 4;
+    static constexpr int kStage = RKV_MAX_GROUP_ROWS * (kCols + 1) * 4;              // the logits of a key block, in the tiles' room
+    static constexpr int kBytes = kTiles > kStage ? kTiles : kStage;
 };
 
 // kRows rows of D elements, starting at `src` (row first_row of its head), into shared memory as fp32; rows >= valid_rows
@@ -48,15 +51,15 @@ __device__ __forceinline__ void load_rows(const T *src, int first_row, int valid
         Elem<T>::unpack(raw, f);
 #pragma unroll
         for (int e = 0; e < kPerVec; e += 4)
-            *reinterpret_cast<float4 *>(dst + r * SimtShape<D>::kPad + c + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
+            *reinterpret_cast<float4 *>(dst + r * (D + 4) + c + e) = make_float4(f[e], f[e + 1], f[e + 2], f[e + 3]);
     }
 }
 
 // dot[i][c] = row (rg + 8 i) of A . row (cg + 16 c) of B
-template <int D>
-__device__ __forceinline__ void tile_product(const float *A, const float *B, float (&dot)[kRowsT][SimtShape<D>::kColsT])
+template <int D, int kRowsT>
+__device__ __forceinline__ void tile_product(const float *A, const float *B, float (&dot)[kRowsT][SimtShape<D, kRowsT>::kColsT])
 {
-    constexpr int kPad = SimtShape<D>::kPad, kC = SimtShape<D>::kColsT;
+    constexpr int kPad = SimtShape<D, kRowsT>::kPad, kC = SimtShape<D, kRowsT>::kColsT;
     const float *a = A + (threadIdx.x >> 4) * kPad, *b = B + (threadIdx.x & 15) * kPad;
     float2 acc[kRowsT][kC];
 #pragma unroll
@@ -84,11 +87,11 @@ __device__ __forceinline__ void tile_product(const float *A, const float *B, flo
         for (int c = 0; c < kC; ++c) dot[i][c] = acc[i][c].x + acc[i][c].y;
 }
 
-template <typename T, int D>
+template <typename T, int D, int kRowsT>
 __global__ void __launch_bounds__(kSimtThreads, D <= 128 ? 3 : 2) scores_simt_kernel(Params p, int row_blocks, int key_blocks)
 {
-    using S = SimtShape<D>;
-    constexpr int kC = S::kColsT, kCols = S::kCols;
+    using S = SimtShape<D, kRowsT>;
+    constexpr int kC = S::kColsT, kCols = S::kCols, kRowsA = S::kRowsA;
     extern __shared__ __align__(16) float smem[];
     float *tileA = smem, *tileB = smem + kRowsA * S::kPad;
     __shared__ float rB[kCols];
@@ -108,7 +111,7 @@ __global__ void __launch_bounds__(kSimtThreads, D <= 128 ? 3 : 2) scores_simt_ke
     const int t = threadIdx.x, rg = t >> 4, cg = t & 15;
 
     if (x < row_blocks) {
-        // ---------------- Eq. 5-6 + retention rule for rows [64 x, 64 x + 64)
+        // ---------------- Eq. 5-6 + retention rule for rows [kRowsA x, kRowsA x + kRowsA)
         const int i0 = x * kRowsA;
         if (i0 >= n) return;
         load_rows<T, D, kRowsA>(key_rows(i0), i0, n, tileA);
@@ -127,7 +130,7 @@ __global__ void __launch_bounds__(kSimtThreads, D <= 128 ? 3 : 2) scores_simt_ke
             if (t < kCols) rB[t] = j0 + t < n ? inv_norm[j0 + t] : 0.f;
             __syncthreads();
             float s[kRowsT][kC];
-            tile_product<D>(tileA, tileB, s);
+            tile_product<D, kRowsT>(tileA, tileB, s);
             float rj[kC];
 #pragma unroll
             for (int c = 0; c < kC; ++c) rj[c] = rB[cg + 16 * c];
@@ -166,24 +169,24 @@ __global__ void __launch_bounds__(kSimtThreads, D <= 128 ? 3 : 2) scores_simt_ke
         const int rows = p.group * p.alpha;
         const T *Q = static_cast<const T *>(p.q_window) + ((size_t)b * p.hq + (size_t)h * p.group) * p.alpha * D;
         load_rows<T, D, kCols>(key_rows(j0), j0, n, tileB);
-        float lg[2][kRowsT][kC];                         // query rows g * alpha + j, at most 112
+        float lg[S::kChunks][kRowsT][kC];                // query rows g * alpha + j, at most 112
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            if (half * kRowsA >= rows) break;
+        for (int chunk = 0; chunk < S::kChunks; ++chunk) {
+            if (chunk * kRowsA >= rows) break;
             __syncthreads();
-            load_rows<T, D, kRowsA>(Q + (size_t)half * kRowsA * D, half * kRowsA, rows, tileA);
+            load_rows<T, D, kRowsA>(Q + (size_t)chunk * kRowsA * D, chunk * kRowsA, rows, tileA);
             __syncthreads();
-            tile_product<D>(tileA, tileB, lg[half]);
+            tile_product<D, kRowsT>(tileA, tileB, lg[chunk]);
         }
         __syncthreads();                                 // the tiles are no longer read
 #pragma unroll
-        for (int half = 0; half < 2; ++half)
+        for (int chunk = 0; chunk < S::kChunks; ++chunk)
 #pragma unroll
             for (int i = 0; i < kRowsT; ++i) {
-                const int row = half * kRowsA + rg + 8 * i;
+                const int row = chunk * kRowsA + rg + 8 * i;
                 if (row < rows)
 #pragma unroll
-                    for (int c = 0; c < kC; ++c) smem[row * (kCols + 1) + cg + 16 * c] = lg[half][i][c];
+                    for (int c = 0; c < kC; ++c) smem[row * (kCols + 1) + cg + 16 * c] = lg[chunk][i][c];
             }
         __syncthreads();
         const float scale = p.logit_scale;
@@ -202,17 +205,26 @@ __global__ void __launch_bounds__(kSimtThreads, D <= 128 ? 3 : 2) scores_simt_ke
     }
 }
 
+template <typename T, int D, int kRowsT>
+cudaError_t launch_simt_rows(const Params &p, int dev, cudaStream_t s)
+{
+    using S = SimtShape<D, kRowsT>;
+    static std::atomic<unsigned long long> done{0ull};
+    const int row_blocks = (p.cap + S::kRowsA - 1) / S::kRowsA, key_blocks = (p.cap + S::kCols - 1) / S::kCols;
+    const unsigned grid = (unsigned)(row_blocks + key_blocks) * (unsigned)(p.batch * p.hkv);
+    const cudaError_t e = allow_smem_once(done, dev, scores_simt_kernel<T, D, kRowsT>, S::kBytes);
+    if (e != cudaSuccess) return e;
+    return launch_early(scores_simt_kernel<T, D, kRowsT>, grid, kSimtThreads, S::kBytes, s, 1, p, row_blocks, key_blocks);
+}
+
 template <typename T, int D>
 cudaError_t launch_simt_for(const Params &p, cudaStream_t s)
 {
-    using S = SimtShape<D>;
-    const int row_blocks = (p.cap + kRowsA - 1) / kRowsA, key_blocks = (p.cap + S::kCols - 1) / S::kCols;
-    const unsigned grid = (unsigned)(row_blocks + key_blocks) * (unsigned)(p.batch * p.hkv);
-    static std::atomic<unsigned long long> done{0ull};
     int dev = 0, sms = 0;
-    cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_simt_kernel<T, D>, S::kBytes)) != cudaSuccess) return e;
-    return launch_early(scores_simt_kernel<T, D>, grid, kSimtThreads, S::kBytes, s, 1, p, row_blocks, key_blocks);
+    const cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess) return e;
+    const long long blocks = (long long)((p.cap + 63) / 64) * p.batch * p.hkv;       // of 64 rows
+    return blocks < sms ? launch_simt_rows<T, D, 2>(p, dev, s) : launch_simt_rows<T, D, 8>(p, dev, s);
 }
 
 }  // namespace
