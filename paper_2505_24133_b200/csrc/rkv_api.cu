@@ -26,10 +26,10 @@ struct Layout {
     int cap, cap_pad, tiles, tri;
 };
 
-// The two-pass tensor-core scoring kernels are built for bf16 keys of 128 dimensions.  bf16 and 8-bit caches of 128
-// dimensions use them directly (8-bit: on a widened copy), those of 64 dimensions on a copy padded with zeros to 128 (dot
-// products and norms do not see the padding).  256 dimensions take the row-block tensor-core kernel, which forms the whole
-// similarity matrix; fp32 caches, or a request for it, the CUDA-core kernel.
+// The two-pass tensor-core scoring kernels are built for bf16 keys of 64 and 128 dimensions; 8-bit caches use them on a
+// widened copy.  The row-block tensor-core kernel, which forms the whole similarity matrix, takes 256 dimensions, and
+// the others where it is asked for (64 on a copy padded with zeros to 128: dot products and norms do not see the padding);
+// fp32 caches, or a request for it, the CUDA-core kernel.
 // Bytes of a cache element and of a query element.  8-bit caches (E4M3 codes) are scored on a bf16 copy of their keys
 // in the workspace (every E4M3 value is a bf16 value), with bf16 queries.
 size_t cache_esz(const rkv_desc_t *d) { return d->dtype == RKV_BF16 ? 2 : d->dtype == RKV_F32 ? 4 : 1; }
@@ -39,25 +39,22 @@ bool use_simt(const rkv_desc_t *d)
 {
     return d->dtype == RKV_F32 || (d->flags & RKV_FLAG_SIMT_SCORES);
 }
+// 1 when the two-pass tensor-core kernels score (unless a cross-check kernel is asked for).
+int use_tri(const rkv_desc_t *d) { return !(use_simt(d) || d->head_dim == 256 || (d->flags & RKV_FLAG_ROWBLOCK_SCORES)); }
 // The head dimension is padded from 64 to 128 in the scoring copy (keys and observation queries).
-bool pads_dim(const rkv_desc_t *d) { return d->head_dim == 64 && !use_simt(d); }
+bool pads_dim(const rkv_desc_t *d) { return d->head_dim == 64 && !use_simt(d) && !use_tri(d); }
 // The scoring stages read a copy of the keys in the workspace instead of the cache itself.
 bool needs_copy(const rkv_desc_t *d) { return d->dtype == RKV_FP8_E4M3 || pads_dim(d); }
 // Head dimension the scoring stages see.
 int scoring_dim(const rkv_desc_t *d) { return pads_dim(d) ? kHeadDim : d->head_dim; }
-// The prep kernel writes the copy of the keys itself (instead of a widening pass in front of it): stored rows of 128
-// bytes that become 128 bf16, in caches whose capacity is a whole number of 128-row tiles.  1: E4M3 codes, 2: bf16 of
-// 64 dimensions.
-int fuse_mode(const rkv_desc_t *d, long long cap)
-{
-    if (!needs_copy(d) || scoring_dim(d) != kHeadDim || cap % kTile != 0) return 0;
-    if (d->dtype == RKV_FP8_E4M3 && d->head_dim == kHeadDim) return 1;
-    if (d->dtype == RKV_BF16 && d->head_dim == 64) return 2;
-    return 0;
-}
-
-// 1 when the triangle tensor-core kernels score (bf16 caches, unless a cross-check kernel is asked for).
-int use_tri(const rkv_desc_t *d) { return !(use_simt(d) || d->head_dim == 256 || (d->flags & RKV_FLAG_ROWBLOCK_SCORES)); }
+// bf16 caches of 64 dimensions on the two-pass route: a kernel ahead of prep records the lengths.
+bool lengths_ahead(const rkv_desc_t *d) { return d->head_dim == 64 && use_tri(d) && !needs_copy(d); }
+// Tensor-core scoring of 64 dimensions, by either route.  Its workspace has room for the padded copy, used or not: callers
+// have relied on the size.
+bool tensor64(const rkv_desc_t *d) { return d->head_dim == 64 && !use_simt(d); }
+// The prep kernel writes the copy of the keys itself (instead of a widening pass in front of it): rows of 128 E4M3 codes in
+// caches whose capacity is a whole number of 128-row tiles.
+bool fused_codes(const rkv_desc_t *d, long long cap) { return d->dtype == RKV_FP8_E4M3 && d->head_dim == kHeadDim && cap % kTile == 0; }
 
 // Returns RKV_OK and fills *lay when the shape arguments are usable.
 int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout *lay)
@@ -86,14 +83,14 @@ int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout 
         size_t off = 0;
         // the scoring copy (8-bit caches, padded head dimension): the keys as bf16, head after head, plus one tile of zero
         // rows behind the last head; with a padded head dimension the observation queries as well
+        const size_t hd = (size_t)(tensor64(d) ? kHeadDim : d->head_dim);
         lay->k_wide = off;
-        if (needs_copy(d)) off = align_up(off + (P * lay->cap + kTile) * (size_t)scoring_dim(d) * sizeof(__nv_bfloat16), 256);
+        if (needs_copy(d) || tensor64(d)) off = align_up(off + (P * lay->cap + kTile) * hd * sizeof(__nv_bfloat16), 256);
         lay->q_wide = off;
-        if (pads_dim(d)) off = align_up(off + (size_t)d->batch * d->n_q_heads * alpha * kHeadDim * sizeof(__nv_bfloat16), 256);
+        if (tensor64(d)) off = align_up(off + (size_t)d->batch * d->n_q_heads * alpha * kHeadDim * sizeof(__nv_bfloat16), 256);
         lay->inv_norm = off;  off = align_up(off + P * lay->cap_pad * sizeof(float), 256);
         lay->norm_split = off;  off = align_up(off + P * lay->cap_pad * 8 * sizeof(__nv_bfloat16), 256);
         lay->thr_split = off;   off = align_up(off + P * kTile * 8 * sizeof(__nv_bfloat16), 256);
-        const size_t hd = (size_t)scoring_dim(d);
         lay->tile_sum = off;  off = align_up(off + P * lay->tiles * hd * sizeof(float), 256);
         lay->logits = off;    off = align_up(off + P * alpha * lay->cap_pad * sizeof(float), 256);
         lay->row_stat = off;  off = align_up(off + P * (alpha + 1) * 2 * sizeof(float), 256);
@@ -216,14 +213,15 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
         p.dtype = RKV_BF16;
         p.d = scoring_dim(d);
         if (pads_dim(d)) p.q_window = ws + lay.q_wide;
-        p.fuse_mode = fuse_mode(d, lay.cap);
+        p.fused_codes = fused_codes(d, lay.cap) ? 1 : 0;
         p.fuse_src = stored.k_cache;
         p.fuse_table = stored.block_table;
     }
+    p.lengths_done = lengths_ahead(d) ? 1 : 0;
     if (stages & RKV_STAGE_PREP) {
         if (needs_copy(d) &&
             (e = launch_widen_keys(stored, static_cast<__nv_bfloat16 *>(p.k_cache), p.d, pads_dim(d) ? stored.q_window : nullptr,
-                                   pads_dim(d) ? ws + lay.q_wide : nullptr, p.fuse_mode == 0, s)) != cudaSuccess)
+                                   pads_dim(d) ? ws + lay.q_wide : nullptr, !p.fused_codes, s)) != cudaSuccess)
             return cuda_fail(e, "widen launch");
         if ((e = launch_prep(p, s)) != cudaSuccess) return cuda_fail(e, "prep launch");
     }
@@ -561,9 +559,12 @@ int rkv_launch_count(const rkv_desc_t *desc, uint32_t stage_mask)
     int c = 0;
     for (uint32_t bit = 1; bit <= RKV_STAGE_GATHER; bit <<= 1) c += (stage_mask & bit) ? 1 : 0;
     if (stage_mask & RKV_STAGE_SELECT) c += 2;      // row statistics and importance run ahead of the selection kernel
-    // bf16 keys of 128 dimensions: the tile sums are added up per head by a kernel of its own behind the prep kernel
-    if (desc && (stage_mask & RKV_STAGE_PREP) && desc->dtype != RKV_F32 && (desc->head_dim == 0 || scoring_dim(desc) == kHeadDim)) c += 1;
-    if (desc && (stage_mask & RKV_STAGE_PREP) && needs_copy(desc)) c += 1;       // the kernel that writes the scoring copy
+    // bf16 keys of 64 and 128 dimensions: the tile sums are added up per head by a kernel of its own behind the prep kernel
+    if (desc && (stage_mask & RKV_STAGE_PREP) && desc->dtype != RKV_F32 &&
+        (desc->head_dim == 0 || scoring_dim(desc) == kHeadDim || tensor64(desc)))
+        c += 1;
+    // the kernel that writes the scoring copy, or the one that records the lengths
+    if (desc && (stage_mask & RKV_STAGE_PREP) && (needs_copy(desc) || lengths_ahead(desc))) c += 1;
     if (desc && (stage_mask & RKV_STAGE_SELECT) && (desc->flags & RKV_FLAG_HEAD_MEAN)) c += 1;   // per-sequence selection
     // the two-pass scoring path is the first pass plus up to two rounds of (listing, second pass) while the
     // retention rule is on
@@ -580,7 +581,7 @@ int rkv_launch_count_for(const rkv_desc_t *desc, int32_t budget, int32_t buffer,
     if (check_shapes(desc, budget, buffer, alpha, &lay) != RKV_OK) return 0;
     int c = rkv_launch_count(desc, stage_mask);
     // the prep kernel writes the copy of the keys itself and nothing else needs a pass of its own
-    if ((stage_mask & RKV_STAGE_PREP) && fuse_mode(desc, lay.cap) != 0 && !pads_dim(desc)) c -= 1;
+    if ((stage_mask & RKV_STAGE_PREP) && fused_codes(desc, lay.cap)) c -= 1;
     if ((stage_mask & RKV_STAGE_SELECT) && select_is_fused(lay.cap_pad, alpha)) c -= 2;
     if ((stage_mask & RKV_STAGE_SCORES) && use_tri(desc) && desc->beta > 0 && desc->sim_threshold < 1.0f)
     {

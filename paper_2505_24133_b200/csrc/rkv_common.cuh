@@ -35,9 +35,8 @@ struct Params {
     int dtype;                      // of the keys the scoring stages read (bf16 for 8-bit caches: their widened copy)
     int store_row_bytes;            // bytes of a row of the caches as stored (what the gather moves)
     float logit_scale;              // Eq. 2's 1 / sqrt(d) with the caches' own head dimension (d above may be a padded one)
-    // prep writes the scoring copy itself (k_cache above) from the stored keys: 0 = no, 1 = rows of 128 E4M3 codes,
-    // 2 = rows of 64 bf16
-    int fuse_mode;
+    int lengths_done;               // 1: a kernel of its own records the lengths and clears the counters ahead of prep
+    int fused_codes;                // 1: prep writes the scoring copy itself (k_cache above) from stored rows of 128 E4M3 codes
     const void *fuse_src;           // the stored keys
     const int32_t *fuse_table;      // their block table (paged caches), else null
     // hyper-parameters

@@ -205,56 +205,77 @@ __global__ void __launch_bounds__(kPrepThreads, D <= 128 ? 5 : 2) prep_kernel(Pa
     }
 }
 
-// ---- the same stage for bf16 caches with d = 128 (the tensor-core route): sum_i r_i k_i on the tensor cores ------------
+// ---- the same stage for bf16 caches with d = 64 or 128 (the tensor-core route): sum_i r_i k_i on the tensor cores -------
 //
 // The norms stay on the CUDA cores, one thread per row (the row read from shared memory once, packed fp32).  The
 // weighted column sums sum_i r_i k_i[c] -- what made the kernel above instruction-bound -- are ONE small tensor-core
 // product per tile: the key tile as TMA leaves it (rows of 128 d-elements, 128-byte swizzle) is used TRANSPOSED as the A
 // operand (MN-major: M = d, K = the 128 rows), the B operand holds r_i in three bf16 parts (N = 16, rows 0..2), so
 // D[c][0..2] sum to sum_i r_i k_i[c] to fp32 accuracy.  Eight K = 16 steps, accumulator = 16 TMEM columns.
+//
+// 64 dimensions: a unit of work is two tiles of a head, one behind the other in the same 32 KB.  They are the two halves of
+// M, their r_i are rows 0..2 and 3..5 of the B operand, and each half of the lanes reads its own three columns.  (One tile
+// per unit would leave half the bytes in flight for the same chain of waits.  8192 heads of 2168 tokens: 1276 us while the
+// keys were written out once more, padded to 128 dimensions, for kernels that knew no other size; 537 now.)
 constexpr int kPrepTcThreads = 128;                         // one thread per row of the tile
-constexpr int kPrepTcTile = kTile * kHeadDim * 2;          // 32 KB
+constexpr int kPrepTcTile = kTile * kHeadDim * 2;          // a unit: 32 KB, one tile of 128 dimensions or two of 64
 constexpr int kPrepTcB = 8 * 16 * 32;                      // 8 K-steps x [16 n][16 k] bf16, 32-byte rows (32-byte swizzle)
 constexpr int kPrepTcBufs = 2;                             // tile buffers of a block: one in use, the others being filled
 constexpr int kPrepTcBlocks = 3;                           // blocks per SM
 constexpr int kPrepTcSmem = kPrepTcBufs * kPrepTcTile + kPrepTcB + 1024; // + slack for the 1024-byte alignment
 constexpr uint32_t kPrepTcTmemCols = 32;
 
-// One key tile of the work list: which head-problem, which tile, how many candidate rows it holds.
-struct PrepTile {
-    int head, tile, b, n, rows_here;
+// One unit of the work list: which head-problem, which tiles, how many candidate rows from its first tile on.
+struct PrepUnit {
+    int head, tile, n, rows_here;
 };
 
-__device__ __forceinline__ PrepTile prep_tile_at(const Params &p, int idx, bool write_meta)
+// kSub: tiles of a unit.  With write_meta the length is recorded, and reported where it is invalid.
+template <int kSub>
+__device__ __forceinline__ PrepUnit prep_unit_at(const Params &p, int idx, bool write_meta)
 {
-    PrepTile w;
-    w.tile = idx % p.tiles;
-    w.head = idx / p.tiles;               // head-problem index b * hkv + h
-    w.b = w.head / p.hkv;
-    int L = p.seq_lens[w.b];
-    int budget_b = p.budgets ? p.budgets[w.b] : p.budget;             // Section 4.2's per-sequence (ratio) budgets
+    PrepUnit w;
+    const int units = (p.tiles + kSub - 1) / kSub;
+    w.tile = idx % units * kSub;
+    w.head = idx / units;                 // head-problem index b * hkv + h
+    const int b = w.head / p.hkv;
+    int L = p.seq_lens[b];
+    int budget_b = p.budgets ? p.budgets[b] : p.budget;             // Section 4.2's per-sequence (ratio) budgets
     if (L < 0 || L > p.cap || budget_b <= p.alpha || budget_b > p.budget) {
         if (write_meta) report(p.status, RKV_ERR_INVALID_ARG);
         L = kMetaInvalid;
         budget_b = p.budget;
     }
     if (write_meta && w.tile == 0 && w.head % p.hkv == 0) {
-        p.meta[w.b] = L;
-        p.meta[p.batch + w.b] = budget_b;
+        p.meta[b] = L;
+        p.meta[p.batch + b] = budget_b;
     }
     w.n = candidates_from_meta(L, budget_b, p.alpha);
-    w.rows_here = min(max(w.n - w.tile * kTile, 0), kTile);
+    w.rows_here = min(max(w.n - w.tile * kTile, 0), kSub * kTile);
     return w;
+}
+
+// bf16 caches of 64 dimensions: the lengths are recorded and the counters cleared ahead of the prep kernel.
+constexpr int kLengthThreads = 256;
+__global__ void __launch_bounds__(kLengthThreads) lengths_kernel(Params p)
+{
+    pdl_trigger();
+    pdl_wait();
+    clear_counters(p);
+    const int b = blockIdx.x * kLengthThreads + threadIdx.x;
+    if (b < p.batch) prep_unit_at<1>(p, b * p.hkv * p.tiles, true);
 }
 
 // Persistent: kPrepTcBlocks blocks per SM, block x takes tiles x, x + gridDim.x, ... of the list (head-major) and
 // keeps the copies of its next kPrepTcBufs - 1 tiles in flight while it works on the present one: what bounds this
 // kernel is how many bytes an SM has under way, not what it does with them.  Barriers, the TMEM columns and the tensor
 // map are set up once per block.
+template <int D>
 __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(Params p, const __grid_constant__ CUtensorMap map_k, int total)
 {
     using namespace sm100;
-    constexpr int D = kHeadDim;
+    constexpr int kSub = kHeadDim / D;                       // tiles of a unit
+    constexpr int kChunks = D / 8;                           // 16-byte vectors of a row
     extern __shared__ uint8_t prep_tc_raw[];
     uint8_t *smem = align_smem(prep_tc_raw);
     uint8_t *bop = smem + kPrepTcBufs * kPrepTcTile;
@@ -266,22 +287,24 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
     const int t = threadIdx.x, warp = t >> 5;
     const uint32_t bar_tile0 = smem_u32(&bars[0]), bar_mma = smem_u32(&bars[kPrepTcBufs]);
 
-    // thread 0: the tile of the block's k-th list entry into buffer k % kPrepTcBufs; an entry without candidates
+    // thread 0: the tiles of the block's k-th list entry into buffer k % kPrepTcBufs; an entry without candidates
     // completes the buffer's barrier phase without a copy, so phases and entries stay in step
     auto issue_copy = [&](int k) {
         const long long idx = (long long)blockIdx.x + (long long)k * gridDim.x;
         if (idx >= total) return;
-        const PrepTile w = prep_tile_at(p, (int)idx, false);
+        const PrepUnit w = prep_unit_at<kSub>(p, (int)idx, false);
         const int buf = k % kPrepTcBufs;
-        const uint32_t bar = bar_tile0 + 8u * buf;
+        const uint32_t bar = bar_tile0 + 8u * buf, dst = sbase + buf * kPrepTcTile;
         if (w.rows_here <= 0) {
             mbar_arrive(bar);
             return;
         }
+        const bool both = kSub == 1 || w.rows_here > kTile;
         const int y = (int)tile_row0(p, w.head, w.tile);
-        mbar_expect_tx(bar, kPrepTcTile);
-        tma_load_2d(sbase + buf * kPrepTcTile, &map_k, 0, y, bar);
-        tma_load_2d(sbase + buf * kPrepTcTile + kPrepTcTile / 2, &map_k, 64, y, bar);
+        mbar_expect_tx(bar, both ? kPrepTcTile : kPrepTcTile / 2);
+        tma_load_2d(dst, &map_k, 0, y, bar);
+        if (kSub == 1) tma_load_2d(dst + kPrepTcTile / 2, &map_k, 64, y, bar);
+        else if (both) tma_load_2d(dst + kPrepTcTile / 2, &map_k, 0, (int)tile_row0(p, w.head, w.tile + 1), bar);
     };
 
     if (t == 0) {
@@ -295,7 +318,7 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
                      ::"r"(smem_u32(&tmem_holder)), "r"(kPrepTcTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // rows 3..15 of the B operand stay zero; rows 0..2 are rewritten in full for every tile
+    // rows 3 kSub..15 of the B operand stay zero; the others are rewritten in full for every unit
     for (int x = t; x < kPrepTcB / 16; x += kPrepTcThreads) reinterpret_cast<uint4 *>(bop)[x] = make_uint4(0u, 0u, 0u, 0u);
     tc_fence_before();
     __syncthreads();
@@ -304,14 +327,14 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
     uint32_t mma_parity = 0;
     pdl_trigger();
     pdl_wait();                             // the set-up above touches no global memory
-    clear_counters(p);
+    if (!p.lengths_done) clear_counters(p);
     if (t == 0)
         for (int q = 0; q < kPrepTcBufs - 1; ++q) issue_copy(q);
 
     int k = 0;
     for (int idx = (int)blockIdx.x; idx < total; idx += (int)gridDim.x, ++k) {
-        const PrepTile w = prep_tile_at(p, idx, t == 0);
-        const int head = w.head, tile = w.tile, n = w.n, rows_here = w.rows_here;
+        const PrepUnit w = prep_unit_at<kSub>(p, idx, t == 0 && !p.lengths_done);
+        const int head = w.head, n = w.n, rows_here = w.rows_here;
         const int buf = k % kPrepTcBufs;
         uint8_t *tile_smem = smem + buf * kPrepTcTile;
         // the buffer entry k - 1 used is free (its product was waited for, by every thread, before the last barrier)
@@ -324,16 +347,20 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
         // (they may hold anything, and 0 x NaN would spoil the product).  Two threads per row were measured slower:
         // the time of a tile is a chain of latencies (barrier, shared-memory loads, product, TMEM load), not of issue slots.
         const int rt = t;
-        const int row = tile * kTile + rt;
-        float r = 0.f, sq = 0.f;
-        if (ok && rows_here > 0) {
-            if (rt < rows_here) {
+        float r[kSub], sq[kSub];
+#pragma unroll
+        for (int u = 0; u < kSub; ++u) {
+            r[u] = sq[u] = 0.f;
+            if (!ok || rows_here <= 0) continue;
+            // chunk c of the row: the first box, or with 128 dimensions the second as well
+            uint8_t *row_smem = tile_smem + u * (kPrepTcTile / 2) + rt * 128;
+            if (u * kTile + rt < rows_here) {
                 float2 sq2[4];                       // four independent chains of packed multiply-adds
 #pragma unroll
                 for (int e = 0; e < 4; ++e) sq2[e] = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const uint4 vec = *reinterpret_cast<const uint4 *>(tile_smem + (c >> 3) * (kPrepTcTile / 2) + rt * 128 + (((c & 7) ^ (rt & 7)) << 4));
+                for (int c = 0; c < kChunks; ++c) {
+                    const uint4 vec = *reinterpret_cast<const uint4 *>(row_smem + (c >> 3) * (kPrepTcTile / 2) + (((c & 7) ^ (rt & 7)) << 4));
                     float f[8];
                     Elem<__nv_bfloat16>::unpack(vec, f);
 #pragma unroll
@@ -342,31 +369,29 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
                         sq2[e] = __ffma2_rn(f2, f2, sq2[e]);
                     }
                 }
-                sq = ((sq2[0].x + sq2[0].y) + (sq2[1].x + sq2[1].y)) + ((sq2[2].x + sq2[2].y) + (sq2[3].x + sq2[3].y));
+                sq[u] = ((sq2[0].x + sq2[0].y) + (sq2[1].x + sq2[1].y)) + ((sq2[2].x + sq2[2].y) + (sq2[3].x + sq2[3].y));
+                const float nrm = sq[u] > 0.f ? sq[u] * rsqrtf(sq[u]) : 0.f;
+                r[u] = __fdividef(1.0f, nrm + p.eps);
             } else {
 #pragma unroll
-                for (int c = 0; c < 16; ++c)
-                    *reinterpret_cast<uint4 *>(tile_smem + (c >> 3) * (kPrepTcTile / 2) + rt * 128 + ((c & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
-            }
-            if (rt < rows_here) {
-                const float nrm = sq > 0.f ? sq * rsqrtf(sq) : 0.f;
-                r = __fdividef(1.0f, nrm + p.eps);
+                for (int c = 0; c < kChunks; ++c)
+                    *reinterpret_cast<uint4 *>(row_smem + (c >> 3) * (kPrepTcTile / 2) + ((c & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
             }
         }
         if (ok) {
-            // r in three bf16 parts: row t of the B operand's K dimension, rows 0..2 of its N dimension
-            float rest = r;
-            uint32_t rp[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const __nv_bfloat16 h16 = __float2bfloat16_rn(rest);
-                rp[c] = (uint32_t)__bfloat16_as_ushort(h16);
-                rest -= __bfloat162float(h16);
-            }
+            // r in three bf16 parts: row t of the B operand's K dimension, rows 3 u..3 u + 2 of its N dimension
             const int s = rt >> 4, kk = rt & 15;
 #pragma unroll
-            for (int nn = 0; nn < 3; ++nn)
-                *reinterpret_cast<unsigned short *>(bop + s * 512 + nn * 32 + ((kk >> 3) << 4) + (kk & 7) * 2) = (unsigned short)rp[nn];
+            for (int u = 0; u < kSub; ++u) {
+                float rest = r[u];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const __nv_bfloat16 h16 = __float2bfloat16_rn(rest);
+                    const int nn = 3 * u + c;        // (32-byte rows, 32-byte swizzle: rows 4..7 have their 16-byte halves swapped)
+                    *reinterpret_cast<__nv_bfloat16 *>(bop + s * 512 + nn * 32 + (((kk >> 3) ^ (nn >> 2)) << 4) + (kk & 7) * 2) = h16;
+                    rest -= __bfloat162float(h16);
+                }
+            }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // generic writes -> tensor-core reads
         __syncthreads();
@@ -394,12 +419,16 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
 
         // ---- what a row leaves behind, written while the product runs
         if (ok) {
-            p.inv_norm[(size_t)head * p.cap_pad + row] = r;
-            p.self_dot[(size_t)head * p.cap_pad + row] = (r * r) * sq;     // Kbar_i . Kbar_i
-            if (p.tri) {
+#pragma unroll
+            for (int u = 0; u < kSub; ++u) {
+                const int tile = w.tile + u, row = tile * kTile + rt;
+                if (kSub > 1 && tile >= p.tiles) break;
+                p.inv_norm[(size_t)head * p.cap_pad + row] = r[u];
+                p.self_dot[(size_t)head * p.cap_pad + row] = (r[u] * r[u]) * sq[u];     // Kbar_i . Kbar_i
+                if (!p.tri) continue;
                 // the threshold slices of the scoring kernels (see prep_kernel above): 1 / r as (n1, n2, n3, n1, n2, n1, 0 ...),
                 // and for the head's last key tile -T / r as (-t1, -t1, -t1, -t2, -t2, -t3, 0 ...)
-                float rest = r > 0.f ? __fdiv_rn(1.0f, r) : 0.f;
+                float rest = r[u] > 0.f ? __fdiv_rn(1.0f, r[u]) : 0.f;
                 uint32_t part[3];
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
@@ -410,7 +439,7 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
                 uint4 *dst = reinterpret_cast<uint4 *>(p.norm_split + ((size_t)head * p.cap_pad + row) * sm100::kSliceElems);
                 dst[0] = make_uint4(part[0] | (part[1] << 16), part[2] | (part[0] << 16), part[1] | (part[0] << 16), 0u);
                 if (tile == (n + kTile - 1) / kTile - 1) {
-                    rest = r > 0.f ? -__fdiv_rn(p.sim_threshold, r) : 0.f;
+                    rest = r[u] > 0.f ? -__fdiv_rn(p.sim_threshold, r[u]) : 0.f;
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
                         const __nv_bfloat16 h16 = __float2bfloat16_rn(rest);
@@ -431,14 +460,15 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
             if (done) {
                 tc_fence_after();
                 uint32_t acc[8];
-                tmem_ld8(tmem + ((uint32_t)(warp * 32) << 16), acc);      // lane = column c of the keys
+                tmem_ld8(tmem + ((uint32_t)(warp * 32) << 16), acc);      // lane = column c of the keys (of tile c / D of the unit)
                 tmem_wait8(acc);
-                tsum = (__uint_as_float(acc[0]) + __uint_as_float(acc[1])) + __uint_as_float(acc[2]);
+                tsum = kSub > 1 && t >= D ? (__uint_as_float(acc[3]) + __uint_as_float(acc[4])) + __uint_as_float(acc[5])
+                                          : (__uint_as_float(acc[0]) + __uint_as_float(acc[1])) + __uint_as_float(acc[2]);
             }
         }
         tc_fence_before();
         done = __syncthreads_and(done);
-        p.tile_sum[((size_t)head * p.tiles + tile) * D + t] = done ? tsum : 0.f;
+        if (kSub == 1 || w.tile + t / D < p.tiles) p.tile_sum[((size_t)head * p.tiles + w.tile) * D + t] = done ? tsum : 0.f;
         if (!done) break;
     }
 
@@ -451,10 +481,10 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
     }
 }
 
-// ---- the same kernel for caches that are scored on a copy: 8-bit codes (d = 128) and bf16 keys of 64 dimensions --------
+// ---- the same kernel for caches that are scored on a copy: 8-bit codes of 128 dimensions --------------------------------
 //
-// Both store a key in 128 bytes.  The tile arrives as stored (16 KB, a ring of two stages); the thread that owns a row
-// widens / pads it into the bf16 operand tile, taking the norm on the way; the tensor cores form the key sums from that
+// The tile arrives as stored (16 KB, a ring of two stages); the thread that owns a row
+// widens it into the bf16 operand tile, taking the norm on the way; the tensor cores form the key sums from that
 // tile as above, and the same tile is written out, by TMA, as the head's part of the scoring copy, which the later
 // stages read.  The stored keys are read once and the copy is not read back here: a separate widening pass in front
 // of prep_tc_kernel cost the prep stage a second sweep over keys twice the stored size.  Only for caches whose
@@ -465,7 +495,6 @@ constexpr int kFusedOffB = kFusedOffRaw + 2 * kFusedRaw;
 constexpr int kFusedSmem = kFusedOffB + kPrepTcB + 1024;
 constexpr int kFusedBlocks = 2;
 
-template <bool kCodes>
 __global__ void __launch_bounds__(kPrepTcThreads, kFusedBlocks)
 prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const __grid_constant__ CUtensorMap map_wide,
                   const int32_t *src_table, int total)
@@ -488,7 +517,7 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
     auto issue_copy = [&](int k) {
         const long long idx = (long long)blockIdx.x + (long long)k * gridDim.x;
         if (idx >= total) return;
-        const PrepTile w = prep_tile_at(p, (int)idx, false);
+        const PrepUnit w = prep_unit_at<1>(p, (int)idx, false);
         const uint32_t bar = bar_raw0 + 8u * (k & 1);
         if (w.rows_here <= 0) {
             mbar_arrive(bar);
@@ -524,7 +553,7 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
 
     int k = 0;
     for (int idx = (int)blockIdx.x; idx < total; idx += (int)gridDim.x, ++k) {
-        const PrepTile w = prep_tile_at(p, idx, t == 0);
+        const PrepUnit w = prep_unit_at<1>(p, idx, t == 0);
         const int head = w.head, tile = w.tile, n = w.n, rows_here = w.rows_here;
         const int buf = k & 1;
         uint8_t *tile_smem = smem + buf * kPrepTcTile;
@@ -555,12 +584,9 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
 #pragma unroll
                 for (int e = 0; e < 4; ++e) sq2[e] = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    if (kCodes) widen16(in[c], &out[2 * c], &out[2 * c + 1]);     // 16 codes -> bf16 chunks 2 c, 2 c + 1
-                    else out[c] = in[c];                                           // 64 dimensions: chunks 0..7, the rest zeros
-                }
+                for (int c = 0; c < 8; ++c) widen16(in[c], &out[2 * c], &out[2 * c + 1]);     // 16 codes -> bf16 chunks 2 c, 2 c + 1
 #pragma unroll
-                for (int c = 0; c < (kCodes ? 16 : 8); ++c) {
+                for (int c = 0; c < 16; ++c) {
                     float f[8];
                     Elem<__nv_bfloat16>::unpack(out[c], f);
 #pragma unroll
@@ -678,9 +704,9 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
 // The tile sums of a head added up in tile order (a launch of its own behind prep_tc_kernel: no tickets, no fences in
 // the streaming kernel), also as three bf16 rows whose sum is s to fp32 accuracy (rows 3..15 of the 16-row block are
 // zero): appended to the query rows, they let the tensor cores form Kbar_i . s along with the logits.
-__global__ void __launch_bounds__(kHeadDim) head_sum_kernel(Params p)
+template <int D>
+__global__ void __launch_bounds__(D) head_sum_kernel(Params p)
 {
-    constexpr int D = kHeadDim;
     pdl_trigger();
     pdl_wait();
     const int head = blockIdx.x, t = threadIdx.x;
@@ -711,14 +737,22 @@ static cudaError_t launch_prep_for(const Params &p, int dev, cudaStream_t s)
     return launch_early(prep_kernel<T, D>, grid, kPrepThreads, smem, s, 1, p);
 }
 
-template <bool kCodes>
-static cudaError_t launch_fused_for(const Params &p, const CUtensorMap &map_src, const CUtensorMap &map_wide, unsigned grid, int total, int dev,
-                                    cudaStream_t s)
+template <int D>
+static cudaError_t launch_prep_tc_for(const Params &p, int dev, int sms, cudaStream_t s)
 {
     static std::atomic<unsigned long long> done{0ull};
-    const cudaError_t e = allow_smem_once(done, dev, prep_fused_kernel<kCodes>, kFusedSmem);
+    CUtensorMap map_k;
+    if (!sm100::make_map_rows(&map_k, p.k_cache, sm100::key_rows_total(p), D, kTile)) return cudaErrorInvalidValue;
+    cudaError_t e = allow_smem_once(done, dev, prep_tc_kernel<D>, kPrepTcSmem);
     if (e != cudaSuccess) return e;
-    return launch_early(prep_fused_kernel<kCodes>, grid, kPrepTcThreads, kFusedSmem, s, 1, p, map_src, map_wide, p.fuse_table, total);
+    if (p.lengths_done &&
+        (e = launch_early(lengths_kernel, (unsigned)((p.batch + kLengthThreads - 1) / kLengthThreads), kLengthThreads, 0, s, 1, p)) != cudaSuccess)
+        return e;
+    const int total = (p.tiles + kHeadDim / D - 1) / (kHeadDim / D) * p.batch * p.hkv;
+    if ((e = launch_early(prep_tc_kernel<D>, (unsigned)std::min(total, kPrepTcBlocks * sms), kPrepTcThreads, kPrepTcSmem, s, 1, p, map_k, total)) !=
+        cudaSuccess)
+        return e;
+    return launch_early(head_sum_kernel<D>, (unsigned)(p.batch * p.hkv), D, 0, s, 1, p);
 }
 
 cudaError_t launch_prep(const Params &p, cudaStream_t s)
@@ -727,32 +761,25 @@ cudaError_t launch_prep(const Params &p, cudaStream_t s)
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess) return e;
-    const int total = p.tiles * p.batch * p.hkv;
-    if (p.fuse_mode != 0) {                 // the tensor-core form that also writes the scoring copy
+    if (p.fused_codes) {                    // the tensor-core form that also writes the scoring copy
+        static std::atomic<unsigned long long> done{0ull};
+        const int total = p.tiles * p.batch * p.hkv;
         const uint64_t wide_rows = (uint64_t)p.batch * p.hkv * p.cap + kTile;
         const uint64_t src_rows = p.fuse_table ? (uint64_t)p.pool_pages * kTile : (uint64_t)p.batch * p.hkv * p.cap;
         CUtensorMap map_src, map_wide;
-        if (!sm100::make_map_row128(&map_src, p.fuse_src, src_rows, p.fuse_mode == 1) ||
-            !sm100::make_map(&map_wide, p.k_cache, wide_rows, kTile))
+        if (!sm100::make_map_row128(&map_src, p.fuse_src, src_rows, true) || !sm100::make_map(&map_wide, p.k_cache, wide_rows, kTile))
             return cudaErrorInvalidValue;
-        const unsigned grid = (unsigned)std::min(total, kFusedBlocks * sms);
-        e = p.fuse_mode == 1 ? launch_fused_for<true>(p, map_src, map_wide, grid, total, dev, s)
-                             : launch_fused_for<false>(p, map_src, map_wide, grid, total, dev, s);
+        if ((e = allow_smem_once(done, dev, prep_fused_kernel, kFusedSmem)) != cudaSuccess) return e;
+        e = launch_early(prep_fused_kernel, (unsigned)std::min(total, kFusedBlocks * sms), kPrepTcThreads, kFusedSmem, s, 1, p, map_src, map_wide,
+                         p.fuse_table, total);
         if (e != cudaSuccess) return e;
-        return launch_early(head_sum_kernel, (unsigned)(p.batch * p.hkv), kHeadDim, 0, s, 1, p);
+        return launch_early(head_sum_kernel<kHeadDim>, (unsigned)(p.batch * p.hkv), kHeadDim, 0, s, 1, p);
     }
-    if (bf16 && p.d == kHeadDim) {          // the tensor-core form
-        static std::atomic<unsigned long long> done{0ull};
-        CUtensorMap map_k;
-        if (!sm100::make_map(&map_k, p.k_cache, sm100::key_rows_total(p), kTile)) return cudaErrorInvalidValue;
-        if ((e = allow_smem_once(done, dev, prep_tc_kernel, kPrepTcSmem)) != cudaSuccess) return e;
-        e = launch_early(prep_tc_kernel, (unsigned)std::min(total, kPrepTcBlocks * sms), kPrepTcThreads, kPrepTcSmem, s, 1, p, map_k, total);
-        if (e != cudaSuccess) return e;
-        return launch_early(head_sum_kernel, (unsigned)(p.batch * p.hkv), kHeadDim, 0, s, 1, p);
-    }
+    if (bf16 && p.d == 128) return launch_prep_tc_for<128>(p, dev, sms, s);          // the tensor-core form
+    if (bf16 && p.d == 64 && p.tri) return launch_prep_tc_for<64>(p, dev, sms, s);
     switch (p.d) {
         case 64: return bf16 ? launch_prep_for<__nv_bfloat16, 64>(p, dev, s) : launch_prep_for<float, 64>(p, dev, s);
-        case 128: return bf16 ? launch_prep_for<__nv_bfloat16, 128>(p, dev, s) : launch_prep_for<float, 128>(p, dev, s);
+        case 128: return launch_prep_for<float, 128>(p, dev, s);
         case 256: return bf16 ? launch_prep_for<__nv_bfloat16, 256>(p, dev, s) : launch_prep_for<float, 256>(p, dev, s);
         default: return cudaErrorInvalidValue;
     }

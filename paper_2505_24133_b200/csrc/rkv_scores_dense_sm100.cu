@@ -33,50 +33,53 @@ using namespace sm100;
 constexpr int kThreadsD = 512;
 constexpr int kPrepWarp0 = 11;                   // first of the 4 warps that prepare slices and stash
 constexpr int kTicketWarpD = 15;
-constexpr int kStagesD = 2;                      // ring depth of streamed tiles
 constexpr int kItemSlotsD = 4;
 constexpr int kHalfBytes = kTile * 64 * 2;
-constexpr int kTileBytes = 2 * kHalfBytes;
 constexpr int kRowsPerItem = 2 * kTile;
 constexpr uint32_t kTmemColsD = 512;
 constexpr int kSliceBytes = kTile * 32;
 
-constexpr int kOffA = 0;                                   // 2 buffers x 2 resident tiles
-constexpr int kOffB = kOffA + 2 * 2 * kTileBytes;          // kStagesD streamed tiles
-constexpr int kOffAugA = kOffB + kStagesD * kTileBytes;    // 2 buffers x 2 slices (rows: -T / r_i)
-constexpr int kOffAugB = kOffAugA + 2 * 2 * kSliceBytes;   // kStagesD slices (keys: 1 / r_j)
-constexpr int kOffStash = kOffAugB + kStagesD * kSliceBytes;            // 2 buffers x kRowsPerItem x left
-constexpr int kOffBar = kOffStash + 2 * kRowsPerItem * 4;
-enum {
-    kBarQFull = 0,
-    kBarQEmpty = kBarQFull + kItemSlotsD,   // producer, 2 MMA threads, 8 epilogue warps, 4 preparing warps
-    kBarAFull = kBarQEmpty + kItemSlotsD,   // [2] resident tiles landed (producer + bytes) and slices / stash written (4 warps)
-    kBarAEmpty = kBarAFull + 2,             // [2] ... no longer read (2 MMA threads, 8 epilogue warps)
-    kBarBFull = kBarAEmpty + 2,
-    kBarBEmpty = kBarBFull + kStagesD,
-    kBarAccFull = kBarBEmpty + kStagesD,    // [2 buffers][2 row tiles]
-    kBarAccEmpty = kBarAccFull + 4,
-    kNumBarsD = kBarAccEmpty + 4
+template <int D>
+struct LayD {                                    // see the second pass's Lay
+    static constexpr int kTileBytes = kTile * D * 2;
+    static constexpr int kStagesD = D == 64 ? 4 : 2;                  // ring depth of streamed tiles
+    static constexpr int kOffA = 0;                                   // 2 buffers x 2 resident tiles
+    static constexpr int kOffB = kOffA + 2 * 2 * kTileBytes;          // kStagesD streamed tiles
+    static constexpr int kOffAugA = kOffB + kStagesD * kTileBytes;    // 2 buffers x 2 slices (rows: -T / r_i)
+    static constexpr int kOffAugB = kOffAugA + 2 * 2 * kSliceBytes;   // kStagesD slices (keys: 1 / r_j)
+    static constexpr int kOffStash = kOffAugB + kStagesD * kSliceBytes;            // 2 buffers x kRowsPerItem x left
+    static constexpr int kOffBar = kOffStash + 2 * kRowsPerItem * 4;
+    static constexpr int kBarQFull = 0;
+    static constexpr int kBarQEmpty = kBarQFull + kItemSlotsD;   // producer, 2 MMA threads, 8 epilogue warps, 4 preparing warps
+    static constexpr int kBarAFull = kBarQEmpty + kItemSlotsD;   // [2] resident tiles landed (producer + bytes) and slices / stash written (4 warps)
+    static constexpr int kBarAEmpty = kBarAFull + 2;             // [2] ... no longer read (2 MMA threads, 8 epilogue warps)
+    static constexpr int kBarBFull = kBarAEmpty + 2;
+    static constexpr int kBarBEmpty = kBarBFull + kStagesD;
+    static constexpr int kBarAccFull = kBarBEmpty + kStagesD;    // [2 buffers][2 row tiles]
+    static constexpr int kBarAccEmpty = kBarAccFull + 4;
+    static constexpr int kNumBarsD = kBarAccEmpty + 4;
+    static constexpr int kOffItems = kOffBar + kNumBarsD * 8;
+    static constexpr int kOffMisc = kOffItems + kItemSlotsD * 16;
+    static constexpr int kSmemBytesD = kOffMisc + 16 + 1024;
+    static_assert(kOffItems % 16 == 0, "item descriptors are read as int4");
+    static_assert(kSmemBytesD <= 227 * 1024, "shared memory budget");
 };
-constexpr int kOffItems = kOffBar + kNumBarsD * 8;
-constexpr int kOffMisc = kOffItems + kItemSlotsD * 16;
-constexpr int kSmemBytesD = kOffMisc + 16 + 1024;
-static_assert(kOffItems % 16 == 0, "item descriptors are read as int4");
-static_assert(kSmemBytesD <= 227 * 1024, "shared memory budget");
 
 // Item descriptor (int4): {head, pair of row tiles p, n, -}.  x < 0: no more items.
+template <int D>
 __global__ void __launch_bounds__(kThreadsD, 1)
 scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_ns)
 {
+    using L = LayD<D>;
     unsigned long long *const item_count = p.counters + kDenseWords, *const ticket = item_count + 1;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = align_smem(smem_raw);
     const uint32_t sbase = smem_u32(smem);
-    int4 *items = reinterpret_cast<int4 *>(smem + kOffItems);
-    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + kOffMisc);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + kOffMisc + 4);
-    volatile int *bail = reinterpret_cast<volatile int *>(smem + kOffMisc + 8);
-    const uint32_t bar0 = sbase + kOffBar;
+    int4 *items = reinterpret_cast<int4 *>(smem + L::kOffItems);
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + L::kOffMisc);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L::kOffMisc + 4);
+    volatile int *bail = reinterpret_cast<volatile int *>(smem + L::kOffMisc + 8);
+    const uint32_t bar0 = sbase + L::kOffBar;
     auto bar = [bar0](int idx) -> uint32_t { return bar0 + 8u * (uint32_t)idx; };
 
     const ErrSink sink = make_sink(p);
@@ -91,20 +94,20 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kItemSlotsD; ++s) {
-            mbar_init(bar(kBarQFull + s), 1);
-            mbar_init(bar(kBarQEmpty + s), 15);
+            mbar_init(bar(L::kBarQFull + s), 1);
+            mbar_init(bar(L::kBarQEmpty + s), 15);
         }
         for (int s = 0; s < 2; ++s) {
-            mbar_init(bar(kBarAFull + s), 5);
-            mbar_init(bar(kBarAEmpty + s), 10);
+            mbar_init(bar(L::kBarAFull + s), 5);
+            mbar_init(bar(L::kBarAEmpty + s), 10);
         }
-        for (int s = 0; s < kStagesD; ++s) {
-            mbar_init(bar(kBarBFull + s), 1);
-            mbar_init(bar(kBarBEmpty + s), 2);
+        for (int s = 0; s < L::kStagesD; ++s) {
+            mbar_init(bar(L::kBarBFull + s), 1);
+            mbar_init(bar(L::kBarBEmpty + s), 2);
         }
         for (int s = 0; s < 4; ++s) {
-            mbar_init(bar(kBarAccFull + s), 1);
-            mbar_init(bar(kBarAccEmpty + s), 4);
+            mbar_init(bar(L::kBarAccFull + s), 1);
+            mbar_init(bar(L::kBarAccEmpty + s), 4);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -129,16 +132,16 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 if (cur >= total_items) break;
                 const int4 desc = p.dense_items[cur];
                 const uint32_t qs = k_item % kItemSlotsD;
-                if (!mbar_wait(bar(kBarQEmpty + qs), ((k_item / kItemSlotsD) & 1) ^ 1, abort_flag, sink)) break;
+                if (!mbar_wait(bar(L::kBarQEmpty + qs), ((k_item / kItemSlotsD) & 1) ^ 1, abort_flag, sink)) break;
                 items[qs] = desc;
-                mbar_arrive(bar(kBarQFull + qs));
+                mbar_arrive(bar(L::kBarQFull + qs));
                 ++k_item;
             }
             if (!*abort_flag) {             // terminator (skipped when the block is aborting)
                 const uint32_t qs = k_item % kItemSlotsD;
-                if (mbar_wait(bar(kBarQEmpty + qs), ((k_item / kItemSlotsD) & 1) ^ 1, abort_flag, sink)) {
+                if (mbar_wait(bar(L::kBarQEmpty + qs), ((k_item / kItemSlotsD) & 1) ^ 1, abort_flag, sink)) {
                     items[qs] = make_int4(-1, 0, 0, 0);
-                    mbar_arrive(bar(kBarQFull + qs));
+                    mbar_arrive(bar(L::kBarQFull + qs));
                 }
             }
         }
@@ -150,34 +153,34 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             bool ok = true;
             while (ok) {
                 const uint32_t qs = k_item % kItemSlotsD;
-                if (!mbar_wait(bar(kBarQFull + qs), (k_item / kItemSlotsD) & 1, abort_flag, sink)) break;
+                if (!mbar_wait(bar(L::kBarQFull + qs), (k_item / kItemSlotsD) & 1, abort_flag, sink)) break;
                 const int4 d = items[qs];
-                mbar_arrive(bar(kBarQEmpty + qs));
+                mbar_arrive(bar(L::kBarQEmpty + qs));
                 if (d.x < 0) break;
                 const int head = d.x, pi = d.y, n = d.z;
                 const int n_tiles = (n + kTile - 1) / kTile;
                 const int num_m = (n - pi * kRowsPerItem > kTile) ? 2 : 1;
                 const uint32_t ab = k_item & 1;
-                if (!mbar_wait(bar(kBarAEmpty + ab), ((k_item >> 1) & 1) ^ 1, abort_flag, sink)) break;
-                mbar_expect_tx(bar(kBarAFull + ab), (uint32_t)(num_m * kTileBytes));
+                if (!mbar_wait(bar(L::kBarAEmpty + ab), ((k_item >> 1) & 1) ^ 1, abort_flag, sink)) break;
+                mbar_expect_tx(bar(L::kBarAFull + ab), (uint32_t)(num_m * L::kTileBytes));
                 for (int m = 0; m < num_m; ++m) {
-                    const uint32_t dst = sbase + kOffA + (ab * 2 + m) * kTileBytes;
+                    const uint32_t dst = sbase + L::kOffA + (ab * 2 + m) * L::kTileBytes;
                     const int y = (int)tile_row0(p, head, 2 * pi + m);
-                    tma_load_2d(dst, &map_k, 0, y, bar(kBarAFull + ab));
-                    tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar(kBarAFull + ab));
+                    tma_load_2d(dst, &map_k, 0, y, bar(L::kBarAFull + ab));
+                    if (D == 128) tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar(L::kBarAFull + ab));
                 }
                 for (int jt = n_tiles - 1; jt >= 2 * pi; --jt) {
-                    const uint32_t s = bcount % kStagesD;
-                    if (!mbar_wait(bar(kBarBEmpty + s), ((bcount / kStagesD) & 1) ^ 1, abort_flag, sink)) {
+                    const uint32_t s = bcount % L::kStagesD;
+                    if (!mbar_wait(bar(L::kBarBEmpty + s), ((bcount / L::kStagesD) & 1) ^ 1, abort_flag, sink)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t dst = sbase + kOffB + s * kTileBytes;
+                    const uint32_t dst = sbase + L::kOffB + s * L::kTileBytes;
                     const int y = (int)tile_row0(p, head, jt);
-                    mbar_expect_tx(bar(kBarBFull + s), kTileBytes + kSliceBytes);
-                    tma_load_2d(dst, &map_k, 0, y, bar(kBarBFull + s));
-                    tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar(kBarBFull + s));
-                    tma_load_2d(sbase + kOffAugB + s * kSliceBytes, &map_ns, 0, head * p.cap_pad + jt * kTile, bar(kBarBFull + s));
+                    mbar_expect_tx(bar(L::kBarBFull + s), L::kTileBytes + kSliceBytes);
+                    tma_load_2d(dst, &map_k, 0, y, bar(L::kBarBFull + s));
+                    if (D == 128) tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar(L::kBarBFull + s));
+                    tma_load_2d(sbase + L::kOffAugB + s * kSliceBytes, &map_ns, 0, head * p.cap_pad + jt * kTile, bar(L::kBarBFull + s));
                     ++bcount;
                 }
                 ++k_item;
@@ -193,47 +196,48 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             bool ok = true;
             while (ok) {
                 const uint32_t qs = k_item % kItemSlotsD;
-                if (!mbar_wait(bar(kBarQFull + qs), (k_item / kItemSlotsD) & 1, abort_flag, sink)) break;
+                if (!mbar_wait(bar(L::kBarQFull + qs), (k_item / kItemSlotsD) & 1, abort_flag, sink)) break;
                 const int4 d = items[qs];
-                mbar_arrive(bar(kBarQEmpty + qs));
+                mbar_arrive(bar(L::kBarQEmpty + qs));
                 if (d.x < 0) break;
                 const int pi = d.y, n = d.z;
                 const int n_tiles = (n + kTile - 1) / kTile;
                 const bool mine = m == 0 || (n - pi * kRowsPerItem > kTile);
                 const uint32_t ab = k_item & 1;
-                if (!mbar_wait(bar(kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink)) break;
+                if (!mbar_wait(bar(L::kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t resident = sbase + kOffA + (ab * 2 + m) * kTileBytes;
-                const uint32_t res_slice = sbase + kOffAugA + (ab * 2 + m) * kSliceBytes;
+                const uint32_t resident = sbase + L::kOffA + (ab * 2 + m) * L::kTileBytes;
+                const uint32_t res_slice = sbase + L::kOffAugA + (ab * 2 + m) * kSliceBytes;
                 for (int jt = n_tiles - 1; jt >= 2 * pi; --jt) {
-                    const uint32_t s = bcount % kStagesD;
-                    if (!mbar_wait(bar(kBarBFull + s), (bcount / kStagesD) & 1, abort_flag, sink)) {
+                    const uint32_t s = bcount % L::kStagesD;
+                    if (!mbar_wait(bar(L::kBarBFull + s), (bcount / L::kStagesD) & 1, abort_flag, sink)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t stage = sbase + kOffB + s * kTileBytes;
+                    const uint32_t stage = sbase + L::kOffB + s * L::kTileBytes;
                     if (mine && jt >= 2 * pi + m) {           // row tile 2 p + 1 leaves key tile 2 p to the column direction
                         const uint32_t a = cnt & 1;
-                        if (!mbar_wait(bar(kBarAccEmpty + a * 2 + m), ((cnt >> 1) & 1) ^ 1, abort_flag, sink)) {
+                        if (!mbar_wait(bar(L::kBarAccEmpty + a * 2 + m), ((cnt >> 1) & 1) ^ 1, abort_flag, sink)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
                         const uint32_t d_tmem = tmem_base + a * 256 + m * 128;
-                        umma_tile_k128(d_tmem, resident, stage, idesc_k);
-                        umma_k16_sw32(d_tmem, res_slice, sbase + kOffAugB + s * kSliceBytes, idesc_k);
-                        umma_commit(bar(kBarAccFull + a * 2 + m));
+                        if (D == 128) umma_tile_k128(d_tmem, resident, stage, idesc_k);
+                        else umma_tile_k64(d_tmem, resident, stage, idesc_k);
+                        umma_k16_sw32(d_tmem, res_slice, sbase + L::kOffAugB + s * kSliceBytes, idesc_k);
+                        umma_commit(bar(L::kBarAccFull + a * 2 + m));
                         ++cnt;
                         ++tiles_done;
-                        umma_commit(bar(kBarBEmpty + s));
+                        umma_commit(bar(L::kBarBEmpty + s));
                     } else {
-                        mbar_arrive(bar(kBarBEmpty + s));
+                        mbar_arrive(bar(L::kBarBEmpty + s));
                     }
                     ++bcount;
                 }
                 if (!ok) break;
-                if (mine) umma_commit(bar(kBarAEmpty + ab));
-                else mbar_arrive(bar(kBarAEmpty + ab));
+                if (mine) umma_commit(bar(L::kBarAEmpty + ab));
+                else mbar_arrive(bar(L::kBarAEmpty + ab));
                 ++k_item;
             }
         }
@@ -247,16 +251,16 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
         uint32_t k_item = 0;
         while (true) {
             const uint32_t qs = k_item % kItemSlotsD;
-            if (!mbar_wait(bar(kBarQFull + qs), (k_item / kItemSlotsD) & 1, abort_flag, sink)) break;
+            if (!mbar_wait(bar(L::kBarQFull + qs), (k_item / kItemSlotsD) & 1, abort_flag, sink)) break;
             const int4 d = items[qs];
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kBarQEmpty + qs));
+            if (lane == 0) mbar_arrive(bar(L::kBarQEmpty + qs));
             if (d.x < 0) break;
             const int head = d.x, pi = d.y, n = d.z;
             const uint32_t ab = k_item & 1;
-            if (!mbar_wait(bar(kBarAEmpty + ab), ((k_item >> 1) & 1) ^ 1, abort_flag, sink)) break;
+            if (!mbar_wait(bar(L::kBarAEmpty + ab), ((k_item >> 1) & 1) ^ 1, abort_flag, sink)) break;
             const size_t hoff = (size_t)head * p.cap_pad;
-            int32_t *stash_left = reinterpret_cast<int32_t *>(smem + kOffStash + ab * kRowsPerItem * 4);
+            int32_t *stash_left = reinterpret_cast<int32_t *>(smem + L::kOffStash + ab * kRowsPerItem * 4);
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
                 const int i = pi * kRowsPerItem + m * kTile + gt;
@@ -271,7 +275,7 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                     part[c] = (uint32_t)__bfloat16_as_ushort(h16);
                     rest -= __bfloat162float(h16);
                 }
-                uint8_t *slice = smem + kOffAugA + (ab * 2 + m) * kSliceBytes + gt * 32;
+                uint8_t *slice = smem + L::kOffAugA + (ab * 2 + m) * kSliceBytes + gt * 32;
                 const int sw = (gt >> 2) & 1;
                 *reinterpret_cast<uint4 *>(slice + (sw << 4)) =
                     make_uint4(part[0] | (part[0] << 16), part[0] | (part[1] << 16), part[1] | (part[2] << 16), 0u);
@@ -280,7 +284,7 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor-core reads
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kBarAFull + ab));
+            if (lane == 0) mbar_arrive(bar(L::kBarAFull + ab));
             ++k_item;
         }
     } else {
@@ -295,10 +299,10 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 
         while (true) {
             const uint32_t qs = k_item % kItemSlotsD;
-            if (!mbar_wait(bar(kBarQFull + qs), (k_item / kItemSlotsD) & 1, abort_flag, sink)) break;
+            if (!mbar_wait(bar(L::kBarQFull + qs), (k_item / kItemSlotsD) & 1, abort_flag, sink)) break;
             const int4 d = items[qs];
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kBarQEmpty + qs));
+            if (lane == 0) mbar_arrive(bar(L::kBarQEmpty + qs));
             if (d.x < 0) break;
             const int head = d.x, pi = d.y, n = d.z;
             const int n_tiles = (n + kTile - 1) / kTile;
@@ -307,9 +311,9 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             const int own_tile = 2 * pi + m;
             const int i = own_tile * kTile + lrow;
             const bool row_ok = active && i < n;
-            bool ok = mbar_wait(bar(kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink);
+            bool ok = mbar_wait(bar(L::kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink);
             bool want = false;                   // the token still lacks its partner
-            if (row_ok && ok) want = reinterpret_cast<const int32_t *>(smem + kOffStash + ab * kRowsPerItem * 4)[m * kTile + lrow] > 0;
+            if (row_ok && ok) want = reinterpret_cast<const int32_t *>(smem + L::kOffStash + ab * kRowsPerItem * 4)[m * kTile + lrow] > 0;
             uint32_t *best = p.best + (size_t)head * p.cap_pad;
             int hit_j = -1;                      // row direction: the largest position above the threshold found by this scan
 
@@ -317,7 +321,7 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 for (int jt = n_tiles - 1; jt >= own_tile; --jt) {     // (row tile 2 p + 1 has no product with key tile 2 p)
                     const int jbase = jt * kTile;
                     const uint32_t a = cnt & 1;
-                    if (ok) ok = mbar_wait(bar(kBarAccFull + a * 2 + m), (cnt >> 1) & 1, abort_flag, sink);
+                    if (ok) ok = mbar_wait(bar(L::kBarAccFull + a * 2 + m), (cnt >> 1) & 1, abort_flag, sink);
                     ++cnt;
                     if (!ok) continue;
                     tc_fence_after();
@@ -361,12 +365,12 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kBarAccEmpty + a * 2 + m));
+                    if (lane == 0) mbar_arrive(bar(L::kBarAccEmpty + a * 2 + m));
                 }
             }
             if (ok && row_ok && hit_j >= 0) atomicMax(best + i, (uint32_t)(hit_j + 1));
             __syncwarp();
-            if (lane == 0 && ok) mbar_arrive(bar(kBarAEmpty + ab));
+            if (lane == 0 && ok) mbar_arrive(bar(L::kBarAEmpty + ab));
             if (!ok) break;
             ++k_item;
         }
@@ -407,11 +411,11 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
     const uint32_t b = p.best[hoff + i];
     if (b == 0u) continue;
     const int j = (int)b - 1;
-    const uint4 *ki = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, i) * kHeadDim);
-    const uint4 *kj = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, j) * kHeadDim);
+    const uint4 *ki = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, i) * p.d);
+    const uint4 *kj = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, j) * p.d);
     float dot = 0.f;
 #pragma unroll 4
-    for (int c = 0; c < kHeadDim / 8; ++c) {
+    for (int c = 0; c < p.d / 8; ++c) {
         float a[8], bb[8];
         Elem<__nv_bfloat16>::unpack(__ldg(ki + c), a);
         Elem<__nv_bfloat16>::unpack(__ldg(kj + c), bb);
@@ -424,19 +428,28 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
 
 }  // namespace
 
-cudaError_t launch_scores_dense_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns, int sms)
+template <int D>
+static cudaError_t launch_dense_for(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns)
 {
     static std::atomic<unsigned long long> done{0ull};
-    int dev = 0;
+    int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_dense_sm100_kernel, kSmemBytesD)) != cudaSuccess) return e;
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_dense_sm100_kernel<D>, LayD<D>::kSmemBytesD)) != cudaSuccess) return e;
     const unsigned long long max_items = (unsigned long long)(p.batch * p.hkv) * (unsigned long long)((p.tiles + 1) / 2);
     const unsigned grid = (unsigned)(max_items < (unsigned long long)sms ? max_items : (unsigned long long)sms);
-    return launch_early(scores_dense_sm100_kernel, grid, kThreadsD, kSmemBytesD, s, 1, p, map_k, map_ns);
+    return launch_early(scores_dense_sm100_kernel<D>, grid, kThreadsD, LayD<D>::kSmemBytesD, s, 1, p, map_k, map_ns);
 }
 
-cudaError_t launch_dense_finish(const Params &p, cudaStream_t s, int sms)
+cudaError_t launch_scores_dense_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns)
 {
+    return p.d == 64 ? launch_dense_for<64>(p, s, map_k, map_ns) : launch_dense_for<128>(p, s, map_k, map_ns);
+}
+
+cudaError_t launch_dense_finish(const Params &p, cudaStream_t s)
+{
+    int dev = 0, sms = 0;
+    const cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess) return e;
     const unsigned long long units = (unsigned long long)(p.batch * p.hkv) * (unsigned long long)((p.cap + kFinishThreads - 1) / kFinishThreads);
     const unsigned long long wave = 8ull * (unsigned long long)sms;             // resident blocks of this size
     return launch_early(dense_finish_kernel, (unsigned)(units < wave ? units : wave), kFinishThreads, 0, s, 1, p);

@@ -36,9 +36,8 @@ using namespace sm100;
 
 constexpr int kThreadsP1 = 320;
 constexpr int kHalfBytes = kTile * 64 * 2;       // one TMA box: 128 rows x 64 bf16 (128-byte swizzled rows)
-constexpr int kTileBytes = 2 * kHalfBytes;       // 32 KB: a 128 x 128 bf16 operand tile
 constexpr int kSliceBytes = kTile * 32;          // the extra K = 16 slice of an operand: 128 rows x 32 bytes (32-byte swizzle)
-constexpr int kMaxStagesA = 6;
+constexpr int kMaxStagesA = 8;
 constexpr uint32_t kTmemColsP1 = 512;            // 2 buffers x (128 key columns + up to 128 query columns)
 constexpr int kSmemLimit = 227 * 1024;
 
@@ -55,20 +54,22 @@ enum {
 // Shared-memory carve-up, offsets from a 1024-byte aligned base.
 struct SmemPlan {
     int stages;          // ring depth
-    int q_bytes;         // bytes of the query block: (q_rows_pad + 16) rows x 256 B
+    int q_bytes;         // bytes of the query block: (q_rows_pad + 16) rows
     int off_aug;         // stages x slice of a streamed tile
-    int off_slot;        // 2 x [B block: rows [0, 128) the last key tile, then the query block; as two 64-column halves |
-                         //      slice of the last key tile]
-    int slot_bytes;      // (128 + q_rows_pad + 16) rows x 256 B; a half is slot_bytes / 2
+    int off_slot;        // 2 x [B block: rows [0, 128) the last key tile, then the query block; as 64-column boxes, one
+                         //      behind the other | slice of the last key tile]
+    int slot_bytes;      // (128 + q_rows_pad + 16) rows; with 128 dimensions a 64-column half is slot_bytes / 2
     int slot_stride;     // slot_bytes + kSliceBytes
     int off_rj;          // 2 x 128 floats: r_j of the last key tile
     int off_bar, off_items, off_misc, total;
 };
 
+template <int D>
 __host__ __device__ inline SmemPlan make_plan(int q_rows_pad)
 {
+    constexpr int kTileBytes = kTile * D * 2;
     SmemPlan pl;
-    pl.q_bytes = (q_rows_pad + 16) * 256;
+    pl.q_bytes = (q_rows_pad + 16) * D * 2;
     pl.slot_bytes = kTileBytes + pl.q_bytes;
     pl.slot_stride = pl.slot_bytes + kSliceBytes;
     const int fixed = 2 * pl.slot_stride + 2 * kTile * 4 + kNumBarsP1 * 8 + 2 * 16 + 16 + 1024;   // + alignment slack
@@ -85,6 +86,7 @@ __host__ __device__ inline SmemPlan make_plan(int q_rows_pad)
 }
 
 // Item descriptor (int4): {head, first row tile, one past the last row tile, n}.  x < 0: no more items.
+template <int D>
 __global__ void __launch_bounds__(kThreadsP1, 1)
 scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,
                            const __grid_constant__ CUtensorMap map_hs, const __grid_constant__ CUtensorMap map_ns,
@@ -94,7 +96,8 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = align_smem(smem_raw);
     const uint32_t sbase = smem_u32(smem);
-    const SmemPlan pl = make_plan(q_rows_pad);
+    constexpr int kTileBytes = kTile * D * 2;        // an operand tile: one 64-column box or two
+    const SmemPlan pl = make_plan<D>(q_rows_pad);
     int4 *items = reinterpret_cast<int4 *>(smem + pl.off_items);
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + pl.off_misc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + pl.off_misc + 4);
@@ -170,16 +173,17 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                     const int q_row = (b * p.hq + h * p.group) * p.alpha;
                     const uint32_t half = (uint32_t)pl.slot_bytes / 2, qdst = slot_addr + kTile * 128;
                     // behind the key tile's rows: the query rows, then 16 rows holding sum_j Kbar_j split into bf16
-                    // parts; both 64-column halves
-                    tma_load_2d(qdst, &map_q, 0, q_row, full);
-                    tma_load_2d(qdst + half, &map_q, 64, q_row, full);
-                    tma_load_2d(qdst + q_rows_pad * 128, &map_hs, 0, head * 16, full);
-                    tma_load_2d(qdst + half + q_rows_pad * 128, &map_hs, 64, head * 16, full);
+                    // parts; every 64-column box
+#pragma unroll
+                    for (int x = 0; x < D / 64; ++x) {
+                        tma_load_2d(qdst + x * half, &map_q, x * 64, q_row, full);
+                        tma_load_2d(qdst + x * half + q_rows_pad * 128, &map_hs, x * 64, head * 16, full);
+                    }
                 }
                 if (rule_on) {
                     const int y = (int)tile_row0(p, head, n_tiles - 1);
                     tma_load_2d(slot_addr, &map_k, 0, y, full);
-                    tma_load_2d(slot_addr + (uint32_t)pl.slot_bytes / 2, &map_k, 64, y, full);
+                    if (D == 128) tma_load_2d(slot_addr + (uint32_t)pl.slot_bytes / 2, &map_k, 64, y, full);
                     // the tile's extra slice: -T / r_j of its keys in three bf16 parts
                     tma_load_2d(slot_addr + (uint32_t)pl.slot_bytes, &map_ts, 0, head * kTile, full);
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -198,7 +202,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                     const int y = (int)tile_row0(p, head, t);
                     mbar_expect_tx(bar(kBarAFull + s), kTileBytes + (rule_on ? kSliceBytes : 0));
                     tma_load_2d(dst, &map_k, 0, y, bar(kBarAFull + s));
-                    tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar(kBarAFull + s));
+                    if (D == 128) tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar(kBarAFull + s));
                     if (rule_on)    // the tile's extra slice: 1 / r_i of its keys in three bf16 parts
                         tma_load_2d(sbase + pl.off_aug + s * kSliceBytes, &map_ns, 0, head * p.cap_pad + t * kTile,
                                     bar(kBarAFull + s));
@@ -246,12 +250,14 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                     const uint32_t tile = sbase + s * kTileBytes;
                     const uint32_t d_tmem = tmem_base + a * 256;
                     if (rule_on) {
-                        umma_tile_k128_halves(d_tmem, tile, kHalfBytes, b_block, b_half, idesc_kq);
+                        if (D == 128) umma_tile_k128_halves(d_tmem, tile, kHalfBytes, b_block, b_half, idesc_kq);
+                        else umma_tile_k64(d_tmem, tile, b_block, idesc_kq);
                         // ... - T / (r_i r_j) onto the key columns: the accumulator's sign is the threshold test
                         umma_k16_sw32(d_tmem, sbase + pl.off_aug + s * kSliceBytes, b_block + (uint32_t)pl.slot_bytes, idesc_k);
                         ++tiles_done;
                     } else {
-                        umma_tile_k128_halves(d_tmem + 128, tile, kHalfBytes, b_block + kTile * 128, b_half, idesc_q);
+                        if (D == 128) umma_tile_k128_halves(d_tmem + 128, tile, kHalfBytes, b_block + kTile * 128, b_half, idesc_q);
+                        else umma_tile_k64(d_tmem + 128, tile, b_block + kTile * 128, idesc_q);
                     }
                     umma_commit(bar(kBarAccFull + a));
                     umma_commit(bar(kBarAEmpty + s));              // the stage may be refilled once these products have read it
@@ -509,25 +515,32 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
 
 }  // namespace
 
-cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q,
-                                      const CUtensorMap &map_hs, const CUtensorMap &map_ns, const CUtensorMap &map_ts,
-                                      int q_rows_pad, int sms)
+template <int D>
+static cudaError_t launch_pass1_for(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q, const CUtensorMap &map_hs,
+                                    const CUtensorMap &map_ns, const CUtensorMap &map_ts, int q_rows_pad)
 {
-    const SmemPlan pl = make_plan(q_rows_pad);
+    const SmemPlan pl = make_plan<D>(q_rows_pad);
     if (pl.stages < 2) return cudaErrorInvalidConfiguration;
     // (how much shared memory a call needs depends on its query group: the most that any may need is allowed once)
     static std::atomic<unsigned long long> done{0ull};
-    int dev = 0;
+    int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel, kSmemLimit)) != cudaSuccess) return e;
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D>, kSmemLimit)) != cudaSuccess) return e;
     const int heads = p.batch * p.hkv;
     // a head is cut into parts when there are too few heads to give every SM several items
     int splits = (4 * sms + heads - 1) / heads;
     splits = splits < 1 ? 1 : (splits > p.tiles ? p.tiles : splits);
     const unsigned long long total_items = (unsigned long long)splits * (unsigned long long)heads;
     const unsigned grid = (unsigned)(total_items < (unsigned long long)sms ? total_items : (unsigned long long)sms);
-    return launch_early(scores_stream_sm100_kernel, grid, kThreadsP1, (size_t)pl.total, s, 1, p, map_k, map_q, map_hs, map_ns, map_ts, splits,
+    return launch_early(scores_stream_sm100_kernel<D>, grid, kThreadsP1, (size_t)pl.total, s, 1, p, map_k, map_q, map_hs, map_ns, map_ts, splits,
                         total_items, q_rows_pad);
+}
+
+cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q,
+                                      const CUtensorMap &map_hs, const CUtensorMap &map_ns, const CUtensorMap &map_ts, int q_rows_pad)
+{
+    return p.d == 64 ? launch_pass1_for<64>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
+                     : launch_pass1_for<128>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
 }
 
 }  // namespace rkv

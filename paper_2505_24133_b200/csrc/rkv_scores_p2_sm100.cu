@@ -42,42 +42,43 @@ using namespace sm100;
 constexpr int kThreads = 512;                    // 16 warps: producer, 2 MMA issuers (warps 1 and 10), 8 epilogue, 4 gather, tickets
 constexpr int kGatherWarp0 = 11;                 // first of the 4 gather warps
 constexpr int kTicketWarp = 15;                  // draws the items and publishes their descriptors, up to three items ahead
-constexpr int kStagesB = 2;                      // ring depth of streamed tiles
 constexpr int kItemSlots = 4;                    // ring depth of item descriptors
 constexpr int kHalfBytes = kTile * 64 * 2;       // one TMA box: 128 rows x 64 bf16 (128-byte swizzled rows)
-constexpr int kTileBytes = 2 * kHalfBytes;       // 32 KB: a 128 x 128 bf16 operand tile
 constexpr int kRowsPerItem = 2 * kTile;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kPass1Depth = 1;                   // key tiles every token is scanned against in the first pass
 constexpr int kRoundWords = 8;                   // Params::counters[kRoundWords + 2 r], [.. + 1]: items and ticket of round r
 
-// shared memory carve-up (offsets from a 1024-byte aligned base)
-constexpr int kOffA = 0;                                   // 2 buffers x 2 resident tiles (the gathered rows of an item)
-constexpr int kOffB = kOffA + 2 * 2 * kTileBytes;          // kStagesB streamed tiles
+// The operand tiles of D-dimensional keys and where everything lies in shared memory (offsets from a 1024-byte aligned base).
 // The extra K = 16 slices of the operands: 128 rows x 32 bytes each (32-byte swizzle), one per resident tile and one
 // per stage of the ring.
 constexpr int kSliceBytes = kTile * 32;
-constexpr int kOffAugA = kOffB + kStagesB * kTileBytes;    // 2 buffers x 2 slices
-constexpr int kOffAugB = kOffAugA + 2 * 2 * kSliceBytes;   // kStagesB slices
-// what the epilogue needs to know about an item's tokens, left by the gather warps: position, r_i, partners lacking
-constexpr int kOffStash = kOffAugB + kStagesB * kSliceBytes;            // 2 buffers x 3 arrays x kRowsPerItem words
-constexpr int kOffBar = kOffStash + 2 * 3 * kRowsPerItem * 4;           // mbarriers
-enum {
-    kBarQFull = 0,                          // [kItemSlots] item descriptor written
-    kBarQEmpty = kBarQFull + kItemSlots,    // [kItemSlots] read by the producer, the 2 MMA threads, the 8 epilogue and the 4 gather warps
-    kBarAFull = kBarQEmpty + kItemSlots,    // [2] resident tiles, slices and stash of the item in place (4 gather warps)
-    kBarAEmpty = kBarAFull + 2,             // [2] ... no longer read (2 MMA threads, 8 epilogue warps)
-    kBarBFull = kBarAEmpty + 2,             // [kStagesB]
-    kBarBEmpty = kBarBFull + kStagesB,      // [kStagesB]
-    kBarAccFull = kBarBEmpty + kStagesB,    // [2 buffers][2 row tiles]
-    kBarAccEmpty = kBarAccFull + 4,         // [2][2], 4 warps each
-    kNumBars = kBarAccEmpty + 4
+template <int D>
+struct Lay {
+    static constexpr int kTileBytes = kTile * D * 2;                  // one 64-column box (16 KB) or two
+    static constexpr int kStagesB = D == 64 ? 4 : 2;                  // ring depth of streamed tiles
+    static constexpr int kOffA = 0;                                   // 2 buffers x 2 resident tiles (the gathered rows of an item)
+    static constexpr int kOffB = kOffA + 2 * 2 * kTileBytes;          // kStagesB streamed tiles
+    static constexpr int kOffAugA = kOffB + kStagesB * kTileBytes;    // 2 buffers x 2 slices
+    static constexpr int kOffAugB = kOffAugA + 2 * 2 * kSliceBytes;   // kStagesB slices
+    // what the epilogue needs to know about an item's tokens, left by the gather warps: position, r_i, partners lacking
+    static constexpr int kOffStash = kOffAugB + kStagesB * kSliceBytes;            // 2 buffers x 3 arrays x kRowsPerItem words
+    static constexpr int kOffBar = kOffStash + 2 * 3 * kRowsPerItem * 4;           // mbarriers
+    static constexpr int kBarQFull = 0;                          // [kItemSlots] item descriptor written
+    static constexpr int kBarQEmpty = kBarQFull + kItemSlots;    // [kItemSlots] read by the producer, the 2 MMA threads, the 8 epilogue and the 4 gather warps
+    static constexpr int kBarAFull = kBarQEmpty + kItemSlots;    // [2] resident tiles, slices and stash of the item in place (4 gather warps)
+    static constexpr int kBarAEmpty = kBarAFull + 2;             // [2] ... no longer read (2 MMA threads, 8 epilogue warps)
+    static constexpr int kBarBFull = kBarAEmpty + 2;             // [kStagesB]
+    static constexpr int kBarBEmpty = kBarBFull + kStagesB;      // [kStagesB]
+    static constexpr int kBarAccFull = kBarBEmpty + kStagesB;    // [2 buffers][2 row tiles]
+    static constexpr int kBarAccEmpty = kBarAccFull + 4;         // [2][2], 4 warps each
+    static constexpr int kNumBars = kBarAccEmpty + 4;
+    static constexpr int kOffItems = kOffBar + kNumBars * 8;          // kItemSlots x int4
+    static constexpr int kOffMisc = kOffItems + kItemSlots * 16;      // tmem base, abort flag, bail flag
+    static constexpr int kSmemBytes = kOffMisc + 16 + 1024;           // + slack for the manual 1024-byte alignment
+    static_assert(kOffItems % 16 == 0, "item descriptors are read as int4");
+    static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 };
-constexpr int kOffItems = kOffBar + kNumBars * 8;          // kItemSlots x int4
-constexpr int kOffMisc = kOffItems + kItemSlots * 16;      // tmem base, abort flag, bail flag
-constexpr int kSmemBytes = kOffMisc + 16 + 1024;           // + slack for the manual 1024-byte alignment
-static_assert(kOffItems % 16 == 0, "item descriptors are read as int4");
-static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 
 struct Bars {
     uint32_t bar0;
@@ -86,19 +87,21 @@ struct Bars {
 
 // Item descriptor (int4): {head, first listed token k0, tokens in the item (1..256) | key tiles of the window << 16,
 // first (highest) streamed tile}.  x < 0: no more items.  `round` selects the round's counters.
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_ns,
                           int round)
 {
+    using L = Lay<D>;
     unsigned long long *const item_count = p.counters + kRoundWords + 2 * round, *const ticket = item_count + 1;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = align_smem(smem_raw);
     const uint32_t sbase = smem_u32(smem);
-    int4 *items = reinterpret_cast<int4 *>(smem + kOffItems);
-    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + kOffMisc);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + kOffMisc + 4);
-    volatile int *bail = reinterpret_cast<volatile int *>(smem + kOffMisc + 8);
-    const Bars bar{sbase + kOffBar};
+    int4 *items = reinterpret_cast<int4 *>(smem + L::kOffItems);
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + L::kOffMisc);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L::kOffMisc + 4);
+    volatile int *bail = reinterpret_cast<volatile int *>(smem + L::kOffMisc + 8);
+    const Bars bar{sbase + L::kOffBar};
 
     // Once a bounded wait of this call has run out, the blocks still to start return at once (a sequence with an
     // invalid length does not stop the others: it just has no candidates).  Pass 2 has nothing to do when the list
@@ -119,21 +122,21 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kItemSlots; ++s) {
-            mbar_init(bar.at(kBarQFull + s), 1);
-            mbar_init(bar.at(kBarQEmpty + s), 15);
+            mbar_init(bar.at(L::kBarQFull + s), 1);
+            mbar_init(bar.at(L::kBarQEmpty + s), 15);
         }
         for (int s = 0; s < 2; ++s) {
             // the 4 gather warps fill the resident tiles; the MMA threads and the epilogue warps read them and the stash
-            mbar_init(bar.at(kBarAFull + s), 4);
-            mbar_init(bar.at(kBarAEmpty + s), 10);
+            mbar_init(bar.at(L::kBarAFull + s), 4);
+            mbar_init(bar.at(L::kBarAEmpty + s), 10);
         }
-        for (int s = 0; s < kStagesB; ++s) {
-            mbar_init(bar.at(kBarBFull + s), 1);
-            mbar_init(bar.at(kBarBEmpty + s), 2);              // both MMA issuers
+        for (int s = 0; s < L::kStagesB; ++s) {
+            mbar_init(bar.at(L::kBarBFull + s), 1);
+            mbar_init(bar.at(L::kBarBEmpty + s), 2);              // both MMA issuers
         }
         for (int s = 0; s < 4; ++s) {
-            mbar_init(bar.at(kBarAccFull + s), 1);
-            mbar_init(bar.at(kBarAccEmpty + s), 4);
+            mbar_init(bar.at(L::kBarAccFull + s), 1);
+            mbar_init(bar.at(L::kBarAccEmpty + s), 4);
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -156,28 +159,28 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             bool ok = true;
             while (ok) {
                 const uint32_t qs = k_item % kItemSlots;
-                if (!mbar_wait(bar.at(kBarQFull + qs), (k_item / kItemSlots) & 1, abort_flag, sink)) break;
+                if (!mbar_wait(bar.at(L::kBarQFull + qs), (k_item / kItemSlots) & 1, abort_flag, sink)) break;
                 const int4 desc = items[qs];            // {head, first listed token, tokens | window, first streamed tile}
-                mbar_arrive(bar.at(kBarQEmpty + qs));
+                mbar_arrive(bar.at(L::kBarQEmpty + qs));
                 if (desc.x < 0) break;
                 const int head = desc.x;
                 const int first_tile = desc.w;             // streamed tiles: first_tile .. first_tile - n_iter + 1
                 const int n_iter = desc.z >> 16;
                 for (int it = 0; it < n_iter; ++it) {
-                    const uint32_t s = bcount % kStagesB;
-                    if (!mbar_wait(bar.at(kBarBEmpty + s), ((bcount / kStagesB) & 1) ^ 1, abort_flag, sink)) {
+                    const uint32_t s = bcount % L::kStagesB;
+                    if (!mbar_wait(bar.at(L::kBarBEmpty + s), ((bcount / L::kStagesB) & 1) ^ 1, abort_flag, sink)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t dst = sbase + kOffB + s * kTileBytes;
+                    const uint32_t dst = sbase + L::kOffB + s * L::kTileBytes;
                     const int jt = first_tile - it;
                     const int y = (int)tile_row0(p, head, jt);
-                    mbar_expect_tx(bar.at(kBarBFull + s), kTileBytes + kSliceBytes);
-                    tma_load_2d(dst, &map_k, 0, y, bar.at(kBarBFull + s));
-                    tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar.at(kBarBFull + s));
+                    mbar_expect_tx(bar.at(L::kBarBFull + s), L::kTileBytes + kSliceBytes);
+                    tma_load_2d(dst, &map_k, 0, y, bar.at(L::kBarBFull + s));
+                    if (D == 128) tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar.at(L::kBarBFull + s));
                     // the tile's extra slice: the norms of its keys in three bf16 parts
-                    tma_load_2d(sbase + kOffAugB + s * kSliceBytes, &map_ns, 0, head * p.cap_pad + jt * kTile,
-                                bar.at(kBarBFull + s));
+                    tma_load_2d(sbase + L::kOffAugB + s * kSliceBytes, &map_ns, 0, head * p.cap_pad + jt * kTile,
+                                bar.at(L::kBarBFull + s));
                     ++bcount;
                 }
                 ++k_item;
@@ -195,17 +198,17 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 if (cur >= total_items) break;
                 const int4 desc = p.strag_items[cur];
                 const uint32_t qs = k_item % kItemSlots;
-                if (!mbar_wait(bar.at(kBarQEmpty + qs), ((k_item / kItemSlots) & 1) ^ 1, abort_flag, sink)) break;
+                if (!mbar_wait(bar.at(L::kBarQEmpty + qs), ((k_item / kItemSlots) & 1) ^ 1, abort_flag, sink)) break;
                 items[qs] = desc;
-                mbar_arrive(bar.at(kBarQFull + qs));
+                mbar_arrive(bar.at(L::kBarQFull + qs));
                 ++k_item;
             }
             // terminator: tells the other roles that no item follows (skipped when the block is aborting)
             if (!*abort_flag) {
                 const uint32_t qs = k_item % kItemSlots;
-                if (mbar_wait(bar.at(kBarQEmpty + qs), ((k_item / kItemSlots) & 1) ^ 1, abort_flag, sink)) {
+                if (mbar_wait(bar.at(L::kBarQEmpty + qs), ((k_item / kItemSlots) & 1) ^ 1, abort_flag, sink)) {
                     items[qs] = make_int4(-1, 0, 0, 0);
-                    mbar_arrive(bar.at(kBarQFull + qs));
+                    mbar_arrive(bar.at(L::kBarQFull + qs));
                 }
             }
         }
@@ -224,48 +227,49 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             bool ok = true;
             while (ok) {
                 const uint32_t qs = k_item % kItemSlots;
-                if (!mbar_wait(bar.at(kBarQFull + qs), (k_item / kItemSlots) & 1, abort_flag, sink)) break;
+                if (!mbar_wait(bar.at(L::kBarQFull + qs), (k_item / kItemSlots) & 1, abort_flag, sink)) break;
                 const int4 d = items[qs];
-                mbar_arrive(bar.at(kBarQEmpty + qs));
+                mbar_arrive(bar.at(L::kBarQEmpty + qs));
                 if (d.x < 0) break;
                 const int num_m = (d.z & 0xffff) > kTile ? 2 : 1;
                 const int n_iter = d.z >> 16;
                 const bool mine = m < num_m;
                 const uint32_t ab = k_item & 1;                  // resident buffer of this item
-                if (!mbar_wait(bar.at(kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink)) break;     // the gathered rows are in place
+                if (!mbar_wait(bar.at(L::kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink)) break;     // the gathered rows are in place
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t resident = sbase + kOffA + (ab * 2 + m) * kTileBytes;
-                const uint32_t res_slice = sbase + kOffAugA + (ab * 2 + m) * kSliceBytes;
+                const uint32_t resident = sbase + L::kOffA + (ab * 2 + m) * L::kTileBytes;
+                const uint32_t res_slice = sbase + L::kOffAugA + (ab * 2 + m) * kSliceBytes;
                 for (int it = 0; it < n_iter; ++it) {
-                    const uint32_t s = bcount % kStagesB;
-                    if (!mbar_wait(bar.at(kBarBFull + s), (bcount / kStagesB) & 1, abort_flag, sink)) {
+                    const uint32_t s = bcount % L::kStagesB;
+                    if (!mbar_wait(bar.at(L::kBarBFull + s), (bcount / L::kStagesB) & 1, abort_flag, sink)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t stage = sbase + kOffB + s * kTileBytes;
+                    const uint32_t stage = sbase + L::kOffB + s * L::kTileBytes;
                     if (mine) {
                         const uint32_t a = cnt & 1;
-                        if (!mbar_wait(bar.at(kBarAccEmpty + a * 2 + m), ((cnt >> 1) & 1) ^ 1, abort_flag, sink)) {
+                        if (!mbar_wait(bar.at(L::kBarAccEmpty + a * 2 + m), ((cnt >> 1) & 1) ^ 1, abort_flag, sink)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
                         const uint32_t d_tmem = tmem_base + a * 256 + m * 128;
-                        umma_tile_k128(d_tmem, resident, stage, idesc_k);
+                        if (D == 128) umma_tile_k128(d_tmem, resident, stage, idesc_k);
+                        else umma_tile_k64(d_tmem, resident, stage, idesc_k);
                         // ... - (T / r_i) (||k_j|| + eps): the accumulator's sign is the threshold test
-                        umma_k16_sw32(d_tmem, res_slice, sbase + kOffAugB + s * kSliceBytes, idesc_k);
-                        umma_commit(bar.at(kBarAccFull + a * 2 + m));
+                        umma_k16_sw32(d_tmem, res_slice, sbase + L::kOffAugB + s * kSliceBytes, idesc_k);
+                        umma_commit(bar.at(L::kBarAccFull + a * 2 + m));
                         ++cnt;
                         ++tiles_done;
-                        umma_commit(bar.at(kBarBEmpty + s));      // the stage may be refilled once these products have read it
+                        umma_commit(bar.at(L::kBarBEmpty + s));      // the stage may be refilled once these products have read it
                     } else {
-                        mbar_arrive(bar.at(kBarBEmpty + s));
+                        mbar_arrive(bar.at(L::kBarBEmpty + s));
                     }
                     ++bcount;
                 }
                 if (!ok) break;
-                if (mine) umma_commit(bar.at(kBarAEmpty + ab));   // so may the resident tiles
-                else mbar_arrive(bar.at(kBarAEmpty + ab));
+                if (mine) umma_commit(bar.at(L::kBarAEmpty + ab));   // so may the resident tiles
+                else mbar_arrive(bar.at(L::kBarAEmpty + ab));
                 ++k_item;
             }
         }
@@ -279,14 +283,14 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
         uint32_t k_item = 0;
         while (true) {
             const uint32_t qs = k_item % kItemSlots;
-            if (!mbar_wait(bar.at(kBarQFull + qs), (k_item / kItemSlots) & 1, abort_flag, sink)) break;
+            if (!mbar_wait(bar.at(L::kBarQFull + qs), (k_item / kItemSlots) & 1, abort_flag, sink)) break;
             const int4 d = items[qs];
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar.at(kBarQEmpty + qs));
+            if (lane == 0) mbar_arrive(bar.at(L::kBarQEmpty + qs));
             if (d.x < 0) break;
             const int head = d.x, k0 = d.y, rows = d.z & 0xffff;
             const uint32_t ab = k_item & 1;
-            if (!mbar_wait(bar.at(kBarAEmpty + ab), ((k_item >> 1) & 1) ^ 1, abort_flag, sink)) break;
+            if (!mbar_wait(bar.at(L::kBarAEmpty + ab), ((k_item >> 1) & 1) ^ 1, abort_flag, sink)) break;
             const int num_m = rows > kTile ? 2 : 1;
             const size_t hoff = (size_t)head * p.cap_pad;
             int pos[2];
@@ -299,21 +303,21 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 rr[m] = pos[m] >= 0 ? __ldg(p.inv_norm + hoff + pos[m]) : 0.f;
                 lf[m] = pos[m] >= 0 ? (p.beta == 1 ? 1 : p.left[hoff + pos[m]]) : 0;
             }
-            int32_t *stash_i = reinterpret_cast<int32_t *>(smem + kOffStash + ab * 3 * kRowsPerItem * 4);
+            int32_t *stash_i = reinterpret_cast<int32_t *>(smem + L::kOffStash + ab * 3 * kRowsPerItem * 4);
             float *stash_r = reinterpret_cast<float *>(stash_i + kRowsPerItem);
             int32_t *stash_left = stash_i + 2 * kRowsPerItem;
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
                 if (m >= num_m) break;
                 const bool row_ok = pos[m] >= 0;
-                uint8_t *tile = smem + kOffA + (ab * 2 + m) * kTileBytes;
+                uint8_t *tile = smem + L::kOffA + (ab * 2 + m) * L::kTileBytes;
                 const uint4 *src = reinterpret_cast<const uint4 *>(
-                    static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, row_ok ? pos[m] : 0) * kHeadDim);
-                uint4 v[16];
+                    static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, row_ok ? pos[m] : 0) * D);
+                uint4 v[D / 8];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) v[c] = row_ok ? __ldg(src + c) : make_uint4(0u, 0u, 0u, 0u);
+                for (int c = 0; c < D / 8; ++c) v[c] = row_ok ? __ldg(src + c) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-                for (int hb = 0; hb < 2; ++hb) {
+                for (int hb = 0; hb < D / 64; ++hb) {
 #pragma unroll
                     for (int c = 0; c < 8; ++c)
                         *reinterpret_cast<uint4 *>(tile + hb * kHalfBytes + gt * 128 + ((c ^ (gt & 7)) << 4)) = v[hb * 8 + c];
@@ -328,7 +332,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                     part[c] = (uint32_t)__bfloat16_as_ushort(h16);
                     rest -= __bfloat162float(h16);
                 }
-                uint8_t *slice = smem + kOffAugA + (ab * 2 + m) * kSliceBytes + gt * 32;
+                uint8_t *slice = smem + L::kOffAugA + (ab * 2 + m) * kSliceBytes + gt * 32;
                 const int sw = (gt >> 2) & 1;
                 *reinterpret_cast<uint4 *>(slice + (sw << 4)) =
                     make_uint4(part[0] | (part[0] << 16), part[0] | (part[1] << 16), part[1] | (part[2] << 16), 0u);
@@ -339,7 +343,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor-core reads
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar.at(kBarAFull + ab));
+            if (lane == 0) mbar_arrive(bar.at(L::kBarAFull + ab));
             ++k_item;
         }
     } else {
@@ -353,10 +357,10 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 
         while (true) {
             const uint32_t qs = k_item % kItemSlots;
-            if (!mbar_wait(bar.at(kBarQFull + qs), (k_item / kItemSlots) & 1, abort_flag, sink)) break;
+            if (!mbar_wait(bar.at(L::kBarQFull + qs), (k_item / kItemSlots) & 1, abort_flag, sink)) break;
             const int4 d = items[qs];
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar.at(kBarQEmpty + qs));
+            if (lane == 0) mbar_arrive(bar.at(L::kBarQEmpty + qs));
             if (d.x < 0) break;
             const int head = d.x;
             const float *inv_norm = p.inv_norm + (size_t)head * p.cap_pad;
@@ -367,11 +371,11 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             const int rows = d.z & 0xffff, first_tile = d.w, last_tile = d.w - (d.z >> 16) + 1;
             const bool active = (m == 0) || (rows > kTile);
             const bool row_ok = active && (m * kTile + lrow) < rows;
-            bool item_ok = mbar_wait(bar.at(kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink);
+            bool item_ok = mbar_wait(bar.at(L::kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink);
             int i = 0, left = 0;
             float ri = 0.f;
             if (row_ok && item_ok) {
-                const int32_t *stash_i = reinterpret_cast<const int32_t *>(smem + kOffStash + ab * 3 * kRowsPerItem * 4);
+                const int32_t *stash_i = reinterpret_cast<const int32_t *>(smem + L::kOffStash + ab * 3 * kRowsPerItem * 4);
                 i = stash_i[m * kTile + lrow];
                 ri = reinterpret_cast<const float *>(stash_i + kRowsPerItem)[m * kTile + lrow];
                 left = stash_i[2 * kRowsPerItem + m * kTile + lrow];
@@ -390,7 +394,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                     // for the chunks that hold partners)
                     const float4 *rj4 = reinterpret_cast<const float4 *>(inv_norm + jbase);
                     const uint32_t a = cnt & 1;
-                    if (ok) ok = mbar_wait(bar.at(kBarAccFull + a * 2 + m), (cnt >> 1) & 1, abort_flag, sink);
+                    if (ok) ok = mbar_wait(bar.at(L::kBarAccFull + a * 2 + m), (cnt >> 1) & 1, abort_flag, sink);
                     ++cnt;
                     if (!ok) continue;
                     tc_fence_after();
@@ -513,13 +517,13 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar.at(kBarAccEmpty + a * 2 + m));
+                    if (lane == 0) mbar_arrive(bar.at(L::kBarAccEmpty + a * 2 + m));
                 }
                 item_ok = ok;
             }
             // the item's resident buffer and stash are no longer read by this warp
             __syncwarp();
-            if (lane == 0 && item_ok) mbar_arrive(bar.at(kBarAEmpty + ab));
+            if (lane == 0 && item_ok) mbar_arrive(bar.at(L::kBarAEmpty + ab));
             if (!item_ok) break;              // (the epilogue warps meet at no barrier of their own: each may leave alone)
             if (row_ok) {
                 // S = T + h r_i r_j for every partner found here
@@ -651,24 +655,25 @@ int scores_pass2_rounds(int tiles)
     return below <= 8 ? 1 : 2;
 }
 
-cudaError_t launch_scores_tri_sm100(const Params &p, cudaStream_t s)
+template <int D>
+static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
 {
     const int q_rows = p.group * p.alpha;
     const int q_rows_pad = (q_rows + 15) / 16 * 16;
     CUtensorMap map_k, map_q, map_hs, map_ns, map_ts;
-    if (!make_map(&map_k, p.k_cache, key_rows_total(p), kTile) ||
-        !make_map(&map_q, p.q_window, (uint64_t)p.batch * p.hq * p.alpha, (uint32_t)q_rows_pad) ||
-        !make_map(&map_hs, p.head_sum_bf16, (uint64_t)p.batch * p.hkv * 16, 16u) ||
+    if (!make_map_rows(&map_k, p.k_cache, key_rows_total(p), D, kTile) ||
+        !make_map_rows(&map_q, p.q_window, (uint64_t)p.batch * p.hq * p.alpha, D, (uint32_t)q_rows_pad) ||
+        !make_map_rows(&map_hs, p.head_sum_bf16, (uint64_t)p.batch * p.hkv * 16, D, 16u) ||
         !make_map_k16(&map_ns, p.norm_split, (uint64_t)p.batch * p.hkv * p.cap_pad) ||
         !make_map_k16(&map_ts, p.thr_split, (uint64_t)p.batch * p.hkv * kTile))
         return cudaErrorInvalidValue;
     cudaError_t e;
     static std::atomic<unsigned long long> done{0ull};
     int dev = 0, sms = 0;
-    if ((e = device_sms(&dev, &sms)) != cudaSuccess || (e = allow_smem_once(done, dev, scores_pass2_sm100_kernel, kSmemBytes)) != cudaSuccess)
+    if ((e = device_sms(&dev, &sms)) != cudaSuccess || (e = allow_smem_once(done, dev, scores_pass2_sm100_kernel<D>, Lay<D>::kSmemBytes)) != cudaSuccess)
         return e;
     const int heads = p.batch * p.hkv;
-    if ((e = launch_scores_pass1_sm100(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad, sms)) != cudaSuccess) return e;
+    if ((e = launch_scores_pass1_sm100(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)) != cudaSuccess) return e;
     if ((e = mark_kernel(p, 0, s)) != cudaSuccess) return e;
     const bool rule_on = p.beta > 0 && p.sim_threshold < 1.0f;
     if (!rule_on || p.tiles < 2) return mark_kernel(p, 1, s);       // nobody can lack partners / the first pass has seen everything
@@ -684,13 +689,15 @@ cudaError_t launch_scores_tri_sm100(const Params &p, cudaStream_t s)
         const int width = r == rounds - 1 ? (1 << 20) : kRoundTiles[r];
         if ((e = launch_early(strag_compact_kernel, (unsigned)((heads + kCompactWarps - 1) / kCompactWarps), kCompactWarps * 32, 0, s, 1, p, r, below, width)) != cudaSuccess) return e;
         if (r == 0 && (e = mark_kernel(p, 1, s)) != cudaSuccess) return e;
-        if ((e = launch_early(scores_pass2_sm100_kernel, grid2, kThreads, kSmemBytes, s, 1, p, map_k, map_ns, r)) != cudaSuccess) return e;
+        if ((e = launch_early(scores_pass2_sm100_kernel<D>, grid2, kThreads, Lay<D>::kSmemBytes, s, 1, p, map_k, map_ns, r)) != cudaSuccess) return e;
         // the heads the first listing sent to the symmetric route (none on inputs where similar keys are common:
         // the kernel then returns at once)
-        if (r == 0 && dense_possible && (e = launch_scores_dense_sm100(p, s, map_k, map_ns, sms)) != cudaSuccess) return e;
+        if (r == 0 && dense_possible && (e = launch_scores_dense_sm100(p, s, map_k, map_ns)) != cudaSuccess) return e;
         below += width;
     }
-    return dense_possible ? launch_dense_finish(p, s, sms) : cudaSuccess;
+    return dense_possible ? launch_dense_finish(p, s) : cudaSuccess;
 }
+
+cudaError_t launch_scores_tri_sm100(const Params &p, cudaStream_t s) { return p.d == 64 ? launch_tri_for<64>(p, s) : launch_tri_for<128>(p, s); }
 
 }  // namespace rkv

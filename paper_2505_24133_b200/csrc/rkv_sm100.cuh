@@ -175,6 +175,12 @@ __device__ __forceinline__ void umma_tile_k128_halves(uint32_t d_tmem, uint32_t 
         ::"r"(d_tmem), "r"(a0), "r"(b0), "r"(hi), "r"(idesc), "r"(a1), "r"(b1)
         : "memory");
 }
+// The product of 64-dimensional keys: the four K = 16 steps of one 64-column box of each operand.
+__device__ __forceinline__ void umma_tile_k64(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc)
+{
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) umma(d_tmem, smem_desc(a_addr + 32 * ks), smem_desc(b_addr + 32 * ks), idesc, ks > 0 ? 1u : 0u);
+}
 // One more K = 16 step onto the accumulator at d_tmem: both operands are 128 rows x 16 bf16 (32-byte rows, 32-byte
 // swizzle, 8-row groups 256 bytes apart, 256-byte aligned).
 __device__ __forceinline__ void umma_k16_sw32(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc)
@@ -361,10 +367,10 @@ inline bool make_map_k16(CUtensorMap *map, const void *base, uint64_t rows)
 // first scoring pass of the two-pass tensor-core route (its own file); the maps are built by the caller
 cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q,
                                       const CUtensorMap &map_hs, const CUtensorMap &map_ns, const CUtensorMap &map_ts,
-                                      int q_rows_pad, int sms);
+                                      int q_rows_pad);
 
 // symmetric route of the second pass (its own file)
-cudaError_t launch_scores_dense_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns, int sms);
-cudaError_t launch_dense_finish(const Params &p, cudaStream_t s, int sms);
+cudaError_t launch_scores_dense_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns);
+cudaError_t launch_dense_finish(const Params &p, cudaStream_t s);
 
 }  // namespace rkv

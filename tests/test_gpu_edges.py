@@ -23,6 +23,22 @@ def test_row_block_scoring_of_256_dimensions(rkv, dtype, beta, T, budget, buffer
     comp.check_status()
 
 
+@pytest.mark.parametrize("dtype,beta,T", [("bf16", 1, 0.5), ("bf16", 3, 0.5), ("bf16", 1, 0.95), ("fp8", 1, 0.5)])
+@pytest.mark.parametrize("budget,buffer,lens", [(100, 36, [136, 135, 101]), (256, 137, [393, 265, 264]), (17, 8, [25, 18, 17]),
+                                                (1500, 164, [1664, 1545, 1544])])
+def test_two_pass_scoring_of_64_dimensions(rkv, dtype, beta, T, budget, buffer, lens):  # noqa: F811
+    """Units of two key tiles: even and odd numbers of tiles, a second tile without a candidate, with one, full; the rounds and
+    (T = 0.95: hardly any pair) the symmetric route."""
+    spec = small_spec("d64", batch=3, hkv=2, hq=8, budget=budget, buffer=buffer, head_dim=64, dtype=dtype, span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=405 + budget, seq_lens=torch.tensor(lens))
+    for b, L in enumerate(lens):
+        wl.k_cache.view(torch.int16 if dtype == "bf16" else torch.uint8)[b, :, L:] = 0x7FC0 if dtype == "bf16" else 0x7F      # NaN
+    rep, comp = run_and_check(rkv, wl, beta=beta, T=T)
+    assert rep.ok(), rep.errors
+    assert rep.compressed_heads == 2 * sum(L > budget for L in lens)
+    comp.check_status()
+
+
 @pytest.mark.parametrize("head_dim,hq,alpha", [(64, 2, 8), (128, 8, 8), (128, 18, 8), (256, 6, 5)])
 @pytest.mark.parametrize("budget,buffer,lens", [(40, 32, [72, 71, 41]), (110, 90, [200, 137, 136])])
 def test_cuda_core_scoring_tiles(rkv, head_dim, hq, alpha, budget, buffer, lens):  # noqa: F811
