@@ -21,6 +21,11 @@
 // epilogue): the screening is a maximum and a sign test with nothing to load per column.  The n x n matrix never
 // leaves TMEM, and no atomics or global flags are involved in the scores.
 //
+// An item of 128 tokens or fewer needs one row tile: with beta = 1 its window's key tiles are then dealt out to both halves of the
+// pipeline in turn (issuer, accumulators, epilogue warps), which merge their findings at the item's end -- the larger position
+// counts.  With one half idle such a tile took 1400 cycles, all of it waits for the other side (8192 heads of 2168 tokens
+// of 64 dimensions, 40 listed per head: the pass 745 us, 516 now).
+//
 // Items are handed out by a global ticket counter, longest first within a head, so neighbouring blocks work on
 // the same head while its keys are in L2.
 // Warp roles (512 threads): warp 15 = tickets (publishes item descriptors up to three items ahead), warps 11..14 =
@@ -72,7 +77,8 @@ struct Lay {
     static constexpr int kBarBEmpty = kBarBFull + kStagesB;      // [kStagesB]
     static constexpr int kBarAccFull = kBarBEmpty + kStagesB;    // [2 buffers][2 row tiles]
     static constexpr int kBarAccEmpty = kBarAccFull + 4;         // [2][2], 4 warps each
-    static constexpr int kNumBars = kBarAccEmpty + 4;
+    static constexpr int kBarMerge = kBarAccEmpty + 4;           // [2] findings of the second half in the stash (its 4 epilogue warps)
+    static constexpr int kNumBars = kBarMerge + 2;
     static constexpr int kOffItems = kOffBar + kNumBars * 8;          // kItemSlots x int4
     static constexpr int kOffMisc = kOffItems + kItemSlots * 16;      // tmem base, abort flag, bail flag
     static constexpr int kSmemBytes = kOffMisc + 16 + 1024;           // + slack for the manual 1024-byte alignment
@@ -87,7 +93,9 @@ struct Bars {
 
 // Item descriptor (int4): {head, first listed token k0, tokens in the item (1..256) | key tiles of the window << 16,
 // first (highest) streamed tile}.  x < 0: no more items.  `round` selects the round's counters.
-template <int D>
+// kOne: beta = 1 (each form without the other's code: the roles share the instruction cache.  1433 -> 1401 us
+// for 4096 heads of 4216 tokens, 591 -> 516 for the 64 dimensions above).
+template <int D, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1)
 scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_ns,
                           int round)
@@ -129,6 +137,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             // the 4 gather warps fill the resident tiles; the MMA threads and the epilogue warps read them and the stash
             mbar_init(bar.at(L::kBarAFull + s), 4);
             mbar_init(bar.at(L::kBarAEmpty + s), 10);
+            mbar_init(bar.at(L::kBarMerge + s), 4);
         }
         for (int s = 0; s < L::kStagesB; ++s) {
             mbar_init(bar.at(L::kBarBFull + s), 1);
@@ -233,12 +242,13 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 if (d.x < 0) break;
                 const int num_m = (d.z & 0xffff) > kTile ? 2 : 1;
                 const int n_iter = d.z >> 16;
-                const bool mine = m < num_m;
+                const bool split = kOne && num_m == 1;    // one row tile, its key tiles dealt out to both issuers
+                const bool mine = m < num_m || split;
                 const uint32_t ab = k_item & 1;                  // resident buffer of this item
                 if (!mbar_wait(bar.at(L::kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink)) break;     // the gathered rows are in place
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t resident = sbase + L::kOffA + (ab * 2 + m) * L::kTileBytes;
-                const uint32_t res_slice = sbase + L::kOffAugA + (ab * 2 + m) * kSliceBytes;
+                const uint32_t resident = sbase + L::kOffA + (ab * 2 + (split ? 0 : m)) * L::kTileBytes;
+                const uint32_t res_slice = sbase + L::kOffAugA + (ab * 2 + (split ? 0 : m)) * kSliceBytes;
                 for (int it = 0; it < n_iter; ++it) {
                     const uint32_t s = bcount % L::kStagesB;
                     if (!mbar_wait(bar.at(L::kBarBFull + s), (bcount / L::kStagesB) & 1, abort_flag, sink)) {
@@ -246,7 +256,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                         break;
                     }
                     const uint32_t stage = sbase + L::kOffB + s * L::kTileBytes;
-                    if (mine) {
+                    if (mine && (!split || (it & 1) == m)) {
                         const uint32_t a = cnt & 1;
                         if (!mbar_wait(bar.at(L::kBarAccEmpty + a * 2 + m), ((cnt >> 1) & 1) ^ 1, abort_flag, sink)) {
                             ok = false;
@@ -301,7 +311,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
                 rr[m] = pos[m] >= 0 ? __ldg(p.inv_norm + hoff + pos[m]) : 0.f;
-                lf[m] = pos[m] >= 0 ? (p.beta == 1 ? 1 : p.left[hoff + pos[m]]) : 0;
+                lf[m] = pos[m] >= 0 ? (kOne ? 1 : p.left[hoff + pos[m]]) : 0;
             }
             int32_t *stash_i = reinterpret_cast<int32_t *>(smem + L::kOffStash + ab * 3 * kRowsPerItem * 4);
             float *stash_r = reinterpret_cast<float *>(stash_i + kRowsPerItem);
@@ -349,11 +359,11 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
     } else {
         // ------------------------------------------------------------------ epilogue warps
         const int ew = warp - 2;                 // 0..7
-        const int m = ew >> 2;                   // row tile of the item this warp serves
+        const int m = ew >> 2;                   // row tile of the item this warp serves, or half of the key tiles of an item of one
         const int quad = warp & 3;               // TMEM lane quadrant this warp may access
         const int lrow = quad * 32 + lane;       // row within the 128-row tile
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
-        uint32_t k_item = 0, cnt = 0;
+        uint32_t k_item = 0, cnt = 0, merge_parity = 0;      // merge_parity: bit b: phase of the merging barrier of buffer b
 
         while (true) {
             const uint32_t qs = k_item % kItemSlots;
@@ -369,16 +379,19 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             // ---- per item: which token this thread owns (left in the stash by the gather warps), where the scan
             // starts and ends
             const int rows = d.z & 0xffff, first_tile = d.w, last_tile = d.w - (d.z >> 16) + 1;
-            const bool active = (m == 0) || (rows > kTile);
-            const bool row_ok = active && (m * kTile + lrow) < rows;
+            const bool split = kOne && rows <= kTile;
+            const bool active = (m == 0) || (rows > kTile) || split;
+            const int r_item = split ? lrow : m * kTile + lrow;               // row of the item
+            const bool row_ok = active && r_item < rows;
             bool item_ok = mbar_wait(bar.at(L::kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink);
+            int32_t *stash_i = reinterpret_cast<int32_t *>(smem + L::kOffStash + ab * 3 * kRowsPerItem * 4);
+            float *stash_r = reinterpret_cast<float *>(stash_i + kRowsPerItem);
             int i = 0, left = 0;
             float ri = 0.f;
             if (row_ok && item_ok) {
-                const int32_t *stash_i = reinterpret_cast<const int32_t *>(smem + L::kOffStash + ab * 3 * kRowsPerItem * 4);
-                i = stash_i[m * kTile + lrow];
-                ri = reinterpret_cast<const float *>(stash_i + kRowsPerItem)[m * kTile + lrow];
-                left = stash_i[2 * kRowsPerItem + m * kTile + lrow];
+                i = stash_i[r_item];
+                ri = stash_r[r_item];
+                left = stash_i[2 * kRowsPerItem + r_item];
             }
 
             float removed = 0.f;
@@ -388,11 +401,15 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             if (active) {
                 // ---- key tiles of the window, last to first
                 bool ok = item_ok;
-                for (int jt = first_tile; jt >= last_tile; --jt) {
+                for (int jt = first_tile - (split ? m : 0); jt >= last_tile; jt -= split ? 2 : 1) {
                     const int jbase = jt * kTile;
-                    // (with beta > 1 the partners' values need the r_j of whole chunks: read through the L1 cache, and only
-                    // for the chunks that hold partners)
-                    const float4 *rj4 = reinterpret_cast<const float4 *>(inv_norm + jbase);
+                    // with beta > 1 the partners' values need the tile's r_j: lane l has those of columns l, 32 + l, ..., under way
+                    // while the product is
+                    float rj[4] = {0.f, 0.f, 0.f, 0.f};
+                    if (!kOne) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) rj[q] = __ldg(inv_norm + jbase + q * 32 + lane);
+                    }
                     const uint32_t a = cnt & 1;
                     if (ok) ok = mbar_wait(bar.at(L::kBarAccFull + a * 2 + m), (cnt >> 1) & 1, abort_flag, sink);
                     ++cnt;
@@ -448,7 +465,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                             }
                         }
                     };
-                    if (p.beta == 1) {
+                    if (kOne) {
                         if (__any_sync(0xffffffffu, want)) {
                             uint32_t ga[32], gb[32];
                             tmem_ld32(base + 96, ga);
@@ -465,54 +482,23 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                             chunk(gb, 0);
                         }
                     } else if (__any_sync(0xffffffffu, want)) {
-                        // Several partners per token.  This loop is kept rolled on purpose: the warps of three roles
-                        // share the instruction cache, and one copy of this body is what fits (unrolled like the
-                        // path above it ran a third slower).
+                        // Several partners per token, S = T + h r_i r_j each.  Most 16-column pieces hold none: the others are
+                        // loaded again and looked at by one copy of this code (the warps of three roles share the
+                        // instruction cache).  4096 heads of 1068 tokens with beta = 4: the pass took 1022 us with every
+                        // chunk of 32 gone through and its r_j loaded where it held a partner, 888 now.
 #pragma unroll 1
-                        for (int ch = 3; ch >= 0; --ch) {
-                            uint32_t g[32];
-                            tmem_ld32(base + ch * 32, g);
-                            float v[32];
-                            uint32_t hits = 0u;
-                            tmem_wait32(g);
-#pragma unroll
-                            for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(g[c]);
-                            float m0 = 0.f, m1 = 0.f;
-#pragma unroll
-                            for (int c = 0; c < 32; c += 4) {
-                                m0 = max3(m0, v[c], v[c + 1]);
-                                m1 = max3(m1, v[c + 2], v[c + 3]);
-                            }
-                            const float cut = want ? 0.f : __int_as_float(0x7f800000);
-                            if (!__any_sync(0xffffffffu, fmaxf(m0, m1) > cut)) continue;
-#pragma unroll
-                            for (int c = 0; c < 32; ++c) hits |= (v[c] > cut) ? (1u << c) : 0u;
-                            const unsigned own = (unsigned)(i - (jbase + ch * 32));           // zero diagonal (Eq. 5)
-                            if (own < 32u) hits &= ~(1u << own);
-                            // the exact mask, cut down to the highest positions if they are more than the token still
-                            // lacks, then the sum of their h r_j (S = T + h r_i r_j per partner)
-                            int taken = __popc(hits);
-                            for (; taken > left; --taken) hits &= hits - 1u;                   // drop the lowest positions
+                        for (unsigned todo = screen128(base, want); todo != 0u;) {
+                            const int piece = 31 - __clz((int)todo), c0 = piece * 16;
+                            todo &= ~(1u << piece);
+                            uint32_t g[16];
+                            tmem_get16(base + c0, g);
+                            uint32_t mask = left > 0 ? 0xffffu : 0u;
+                            const unsigned own = (unsigned)(i - (jbase + c0));                // zero diagonal (Eq. 5)
+                            if (own < 16u) mask &= ~(1u << own);
+                            const float r_lane = piece >= 6 ? rj[3] : piece >= 4 ? rj[2] : piece >= 2 ? rj[1] : rj[0];
+                            const int taken = take_many(g, mask, left, r_lane, (piece & 1) * 16, removed);
                             nhit += taken;
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) {
-                                const float4 R = __ldg(rj4 + ch * 8 + q);
-                                v[4 * q] *= R.x;
-                                v[4 * q + 1] *= R.y;
-                                v[4 * q + 2] *= R.z;
-                                v[4 * q + 3] *= R.w;
-                            }
-                            float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-                            for (int c = 0; c < 32; c += 4) {
-                                s0 += (hits >> c & 1u) ? v[c] : 0.f;
-                                s1 += (hits >> (c + 1) & 1u) ? v[c + 1] : 0.f;
-                                s2 += (hits >> (c + 2) & 1u) ? v[c + 2] : 0.f;
-                                s3 += (hits >> (c + 3) & 1u) ? v[c + 3] : 0.f;
-                            }
-                            removed += (s0 + s1) + (s2 + s3);
                             left -= taken;
-                            if (left == 0) want = false;
                         }
                     }
                     tc_fence_before();
@@ -521,19 +507,36 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 }
                 item_ok = ok;
             }
+            if (split && item_ok) {
+                // the second half leaves its findings where the stash of a second row tile would be
+                if (m == 1) {
+                    stash_i[kTile + lrow] = hit_j;
+                    stash_r[kTile + lrow] = hit_h;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar.at(L::kBarMerge + ab));
+                } else {
+                    item_ok = mbar_wait(bar.at(L::kBarMerge + ab), merge_parity >> ab & 1u, abort_flag, sink);
+                    merge_parity ^= 1u << ab;
+                    if (item_ok && stash_i[kTile + lrow] > hit_j) {
+                        hit_j = stash_i[kTile + lrow];
+                        hit_h = stash_r[kTile + lrow];
+                    }
+                }
+            }
             // the item's resident buffer and stash are no longer read by this warp
             __syncwarp();
             if (lane == 0 && item_ok) mbar_arrive(bar.at(L::kBarAEmpty + ab));
             if (!item_ok) break;              // (the epilogue warps meet at no barrier of their own: each may leave alone)
-            if (row_ok) {
+            if (row_ok && !(split && m == 1)) {
                 // S = T + h r_i r_j for every partner found here
-                if (p.beta == 1 && hit_j >= 0) {
+                if (kOne && hit_j >= 0) {
+                    left = 0;
                     removed = hit_h * __ldg(inv_norm + hit_j);
                     nhit = 1;
                 }
                 if (nhit > 0) {
                     p.sbar[(size_t)head * p.cap_pad + i] -= (float)nhit * p.sim_threshold + removed * ri;
-                    if (p.beta != 1) p.left[(size_t)head * p.cap_pad + i] = left;
+                    if (!kOne) p.left[(size_t)head * p.cap_pad + i] = left;
                     // the next round lists the tokens still short
                     if (left == 0) atomicAnd(p.lacking + (((size_t)head * p.cap_pad + i) >> 5), ~(1u << (i & 31)));
                 }
@@ -655,7 +658,7 @@ int scores_pass2_rounds(int tiles)
     return below <= 8 ? 1 : 2;
 }
 
-template <int D>
+template <int D, bool kOne>
 static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
 {
     const int q_rows = p.group * p.alpha;
@@ -670,7 +673,7 @@ static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
     cudaError_t e;
     static std::atomic<unsigned long long> done{0ull};
     int dev = 0, sms = 0;
-    if ((e = device_sms(&dev, &sms)) != cudaSuccess || (e = allow_smem_once(done, dev, scores_pass2_sm100_kernel<D>, Lay<D>::kSmemBytes)) != cudaSuccess)
+    if ((e = device_sms(&dev, &sms)) != cudaSuccess || (e = allow_smem_once(done, dev, scores_pass2_sm100_kernel<D, kOne>, Lay<D>::kSmemBytes)) != cudaSuccess)
         return e;
     const int heads = p.batch * p.hkv;
     if ((e = launch_scores_pass1_sm100(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)) != cudaSuccess) return e;
@@ -689,7 +692,7 @@ static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
         const int width = r == rounds - 1 ? (1 << 20) : kRoundTiles[r];
         if ((e = launch_early(strag_compact_kernel, (unsigned)((heads + kCompactWarps - 1) / kCompactWarps), kCompactWarps * 32, 0, s, 1, p, r, below, width)) != cudaSuccess) return e;
         if (r == 0 && (e = mark_kernel(p, 1, s)) != cudaSuccess) return e;
-        if ((e = launch_early(scores_pass2_sm100_kernel<D>, grid2, kThreads, Lay<D>::kSmemBytes, s, 1, p, map_k, map_ns, r)) != cudaSuccess) return e;
+        if ((e = launch_early(scores_pass2_sm100_kernel<D, kOne>, grid2, kThreads, Lay<D>::kSmemBytes, s, 1, p, map_k, map_ns, r)) != cudaSuccess) return e;
         // the heads the first listing sent to the symmetric route (none on inputs where similar keys are common:
         // the kernel then returns at once)
         if (r == 0 && dense_possible && (e = launch_scores_dense_sm100(p, s, map_k, map_ns)) != cudaSuccess) return e;
@@ -698,6 +701,10 @@ static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
     return dense_possible ? launch_dense_finish(p, s) : cudaSuccess;
 }
 
-cudaError_t launch_scores_tri_sm100(const Params &p, cudaStream_t s) { return p.d == 64 ? launch_tri_for<64>(p, s) : launch_tri_for<128>(p, s); }
+cudaError_t launch_scores_tri_sm100(const Params &p, cudaStream_t s)
+{
+    if (p.d == 64) return p.beta == 1 ? launch_tri_for<64, true>(p, s) : launch_tri_for<64, false>(p, s);
+    return p.beta == 1 ? launch_tri_for<128, true>(p, s) : launch_tri_for<128, false>(p, s);
+}
 
 }  // namespace rkv
