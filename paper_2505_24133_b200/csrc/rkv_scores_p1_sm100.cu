@@ -86,7 +86,9 @@ __host__ __device__ inline SmemPlan make_plan(int q_rows_pad)
 }
 
 // Item descriptor (int4): {head, first row tile, one past the last row tile, n}.  x < 0: no more items.
-template <int D>
+// kPlain: alpha = 8, beta = 1, the maximum over the group, the retention rule on -- the defaults -- without the code of the other
+// forms: the roles share the instruction cache.
+template <int D, bool kPlain>
 __global__ void __launch_bounds__(kThreadsP1, 1)
 scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,
                            const __grid_constant__ CUtensorMap map_hs, const __grid_constant__ CUtensorMap map_ns,
@@ -115,7 +117,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
     if (*bail) return;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool rule_on = p.beta > 0 && p.sim_threshold < 1.0f;
+    const bool rule_on = kPlain || (p.beta > 0 && p.sim_threshold < 1.0f);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
@@ -326,9 +328,9 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 uint32_t sp[8];
                 tmem_ld8(qbase + q_rows_pad, sp);
                 float pooled[8];
-                if (p.alpha == 8) {
+                if (kPlain || p.alpha == 8) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) pooled[j] = p.gqa_mean_pool ? 0.f : -kInf;
+                    for (int j = 0; j < 8; ++j) pooled[j] = !kPlain && p.gqa_mean_pool ? 0.f : -kInf;
                     for (int g0 = 0; g0 < G; g0 += 4) {       // four query heads per round trip to TMEM
                         uint32_t t0[8], t1[8], t2[8], t3[8];
                         tmem_ld8(qbase + g0 * 8, t0);
@@ -339,7 +341,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                         tmem_wait8(t1);
                         tmem_wait8(t2);
                         tmem_wait8(t3);
-                        if (p.gqa_mean_pool) {        // the variant: sum over the group (scaled to the mean below)
+                        if (!kPlain && p.gqa_mean_pool) {        // the variant: sum over the group (scaled to the mean below)
                             const bool h1 = g0 + 1 < G, h2 = g0 + 2 < G, h3 = g0 + 3 < G;
 #pragma unroll
                             for (int j = 0; j < 8; ++j)
@@ -352,7 +354,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                             pooled[j] = fmaxf(fmaxf(pooled[j], __uint_as_float(t0[j])),
                                               max3(__uint_as_float(t1[j]), __uint_as_float(t2[j]), __uint_as_float(t3[j])));
                     }
-                    const float scale_q = p.gqa_mean_pool ? scale / (float)G : scale;
+                    const float scale_q = !kPlain && p.gqa_mean_pool ? scale / (float)G : scale;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) pooled[j] *= scale_q;
                 } else {
@@ -383,7 +385,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 // partner's value is S = T + h r_i r_j, with the r_j of the tile in shared memory.
                 float removed = 0.f;             // sum of h r_j over the partners found
                 int nhit = 0;
-                int left = row_ok ? p.beta : 0;
+                int left = row_ok ? (kPlain ? 1 : p.beta) : 0;
                 if (rule_on) {
                     bool want = left > 0;
                     const int valid = n - jbase;                  // columns [0, valid) of the tile are candidates
@@ -408,7 +410,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                         // entries with a clear sign bit (h > 0, but also +0 and some NaN patterns of rows that are not
                         // candidates: confirmed one by one below)
                         uint32_t pos = want ? (~neg & colmask) : 0u;
-                        if (p.beta == 1) {
+                        if (kPlain || p.beta == 1) {
                             // one partner at most: the candidate at the highest set bit, its value picked by a select
                             // tree (nearly always a single turn)
                             while (pos != 0u) {
@@ -482,12 +484,12 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 if (lane == 0) mbar_arrive(bar(kBarAccEmpty + grp));
 
                 if (row_ok) {
-                    if (p.alpha == 8) {
+                    if (kPlain || p.alpha == 8) {
 #pragma unroll
                         for (int j = 0; j < 8; ++j) logits[(size_t)j * p.cap_pad + i] = pooled[j];
                     }
                     p.sbar[(size_t)head * p.cap_pad + i] = total - ((float)nhit * p.sim_threshold + removed * ri);
-                    if (p.beta > 1 && rule_on) p.left[(size_t)head * p.cap_pad + i] = left;
+                    if (!kPlain && p.beta > 1 && rule_on) p.left[(size_t)head * p.cap_pad + i] = left;
                 }
                 if (rule_on) {                   // the tokens still short of partners, a bit each
                     const unsigned lacking = __ballot_sync(0xffffffffu, left > 0);
@@ -515,7 +517,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
 
 }  // namespace
 
-template <int D>
+template <int D, bool kPlain>
 static cudaError_t launch_pass1_for(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q, const CUtensorMap &map_hs,
                                     const CUtensorMap &map_ns, const CUtensorMap &map_ts, int q_rows_pad)
 {
@@ -525,22 +527,25 @@ static cudaError_t launch_pass1_for(const Params &p, cudaStream_t s, const CUten
     static std::atomic<unsigned long long> done{0ull};
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D>, kSmemLimit)) != cudaSuccess) return e;
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D, kPlain>, kSmemLimit)) != cudaSuccess) return e;
     const int heads = p.batch * p.hkv;
     // a head is cut into parts when there are too few heads to give every SM several items
     int splits = (4 * sms + heads - 1) / heads;
     splits = splits < 1 ? 1 : (splits > p.tiles ? p.tiles : splits);
     const unsigned long long total_items = (unsigned long long)splits * (unsigned long long)heads;
     const unsigned grid = (unsigned)(total_items < (unsigned long long)sms ? total_items : (unsigned long long)sms);
-    return launch_early(scores_stream_sm100_kernel<D>, grid, kThreadsP1, (size_t)pl.total, s, 1, p, map_k, map_q, map_hs, map_ns, map_ts, splits,
+    return launch_early(scores_stream_sm100_kernel<D, kPlain>, grid, kThreadsP1, (size_t)pl.total, s, 1, p, map_k, map_q, map_hs, map_ns, map_ts, splits,
                         total_items, q_rows_pad);
 }
 
 cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q,
                                       const CUtensorMap &map_hs, const CUtensorMap &map_ns, const CUtensorMap &map_ts, int q_rows_pad)
 {
-    return p.d == 64 ? launch_pass1_for<64>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
-                     : launch_pass1_for<128>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
+    if (p.alpha == 8 && p.beta == 1 && p.sim_threshold < 1.0f && !p.gqa_mean_pool)
+        return p.d == 64 ? launch_pass1_for<64, true>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
+                         : launch_pass1_for<128, true>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
+    return p.d == 64 ? launch_pass1_for<64, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
+                     : launch_pass1_for<128, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
 }
 
 }  // namespace rkv
