@@ -13,7 +13,7 @@
 // Small caches: one kernel, a block per head, with the pooled logits in shared memory.
 // All of them read scratch that the stage before has just written (L2-resident for small batches).  The first two are bound
 // by that memory, the selection by the latency of its barriers: many threads per block and as many blocks as fit.
-// (4096 heads of 4216 tokens: 157 + 162 + 101 us; 147 + 129 + 199 while the selection did Eq. 6 and 7 itself and each of its
+// (4096 heads of 4216 tokens: 144 + 156 + 80 us; 147 + 129 + 199 while the selection did Eq. 6 and 7 itself and each of its
 // threads walked and wrote a run of tokens one by one.  256 heads of 1144 tokens, the single kernel: 31 -> 20 us.)
 #include "rkv_common.cuh"
 
@@ -73,7 +73,7 @@ constexpr int kImpTokens = 1024;     // tokens per importance block
 
 // row_stat[head][j][0] = max of row j, [1] = 1 / sum exp(value - max); row alpha: the column means.  A warp per row, 1024
 // values in flight, the sum kept relative to the running maximum of each lane (a block per row and its barriers: 184 us for
-// 4096 heads of 4216 tokens; 157).
+// 4096 heads of 4216 tokens; 157, and 144 since a last step no longer works on 128-value pieces that lie behind the row).
 __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(Params p)
 {
     pdl_trigger();
@@ -88,7 +88,8 @@ __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(Params p)
     const float *row = means ? p.sbar + (size_t)head * p.cap_pad : p.logits + ((size_t)head * p.alpha + j) * p.cap_pad;
     const float scale = means && p.tri ? (float)n : 1.0f;          // (x / 1 is x)
     float m = -INFINITY, s = 0.f;
-    for (int i0 = lane * 4; i0 < n; i0 += 1024) {
+    for (int at = 0; at < n; at += 1024) {
+        const int i0 = at + lane * 4;
         float4 v[8];
         float top = -INFINITY;
 #pragma unroll
@@ -97,8 +98,10 @@ __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(Params p)
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int i = i0 + u * 128;
+            if (at + u * 128 >= n) break;                          // (the warp as a whole: the rest of a last step is not worked on)
             if (means) v[u] = make_float4(v[u].x / scale, v[u].y / scale, v[u].z / scale, v[u].w / scale);
             if (i + 3 >= n) {
+                if (i >= n) v[u].x = -INFINITY;
                 if (i + 1 >= n) v[u].y = -INFINITY;
                 if (i + 2 >= n) v[u].z = -INFINITY;
                 v[u].w = -INFINITY;
@@ -110,7 +113,10 @@ __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(Params p)
             m = top;
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) s += (expf(v[u].x - m) + expf(v[u].y - m)) + (expf(v[u].z - m) + expf(v[u].w - m));
+        for (int u = 0; u < 8; ++u) {
+            if (at + u * 128 >= n) break;
+            if (i0 + u * 128 < n) s += (expf(v[u].x - m) + expf(v[u].y - m)) + (expf(v[u].z - m) + expf(v[u].w - m));
+        }
     }
     const float mw = warp_max(m);
     s = warp_sum(s == 0.f ? 0.f : s * expf(m - mw));               // (a lane without values: 0)
@@ -210,15 +216,18 @@ __device__ __forceinline__ void window_load(const float *row, int i0, int n, int
 // The default window: eight consecutive tokens per thread, per query row four 16-byte loads for the 16 logits their windows
 // cover (the general kernel above reads each logit nine times).
 constexpr int kImp8Threads = 256;
-constexpr int kImp8Tokens = kImp8Threads * 8;
 
+// Threads go over the groups of eight tokens of all heads in a row (a block per 2048 tokens of a head left every second or third
+// block almost empty: 177 us for 8192 heads of 2168 tokens, 162 now).
 __global__ void __launch_bounds__(kImp8Threads) importance_w4_kernel(Params p)
 {
     pdl_trigger();
     pdl_wait();
-    const int chunks = (p.cap + kImp8Tokens - 1) / kImp8Tokens;
-    const int head = blockIdx.x / chunks;
-    const int i0 = (blockIdx.x % chunks) * kImp8Tokens + threadIdx.x * 8;     // first token of this thread
+    const int groups = (p.cap + 7) / 8;
+    const long long unit = (long long)blockIdx.x * kImp8Threads + threadIdx.x;
+    if (unit >= (long long)p.batch * p.hkv * groups) return;
+    const int head = (int)(unit / groups);
+    const int i0 = (int)(unit % groups) * 8;     // first token of this thread
     const int n = seq_candidates(p, head / p.hkv);
     if (i0 >= n) return;
     const float *logits = p.logits + (size_t)head * p.alpha * p.cap_pad;
@@ -226,6 +235,7 @@ __global__ void __launch_bounds__(kImp8Threads) importance_w4_kernel(Params p)
     float acc[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) acc[t] = 0.f;
+#pragma unroll 2
     for (int j = 0; j < p.alpha; ++j) {
         float x[16], best[8];
         window_load(logits + (size_t)j * p.cap_pad, i0, n, p.cap_pad, x);
@@ -254,16 +264,17 @@ __global__ void __launch_bounds__(kImp8Threads) importance_w4_kernel(Params p)
 // `budget` entries, `budget` apart.
 // The digits are taken from the distance to the smallest key, from its highest bit that occurs: scores of one head lie close
 // together, and their common leading bits would be passes without an effect.
+template <int kThreads>
 __device__ __forceinline__ void radix_select_emit(const uint32_t *keys, uint32_t lo, uint32_t hi, int n, int k, int alpha, int budget,
                                                   int32_t *out, int copies)
 {
-    constexpr int kWarps = kSelThreads / 32;
+    constexpr int kWarps = kThreads / 32;
     __shared__ uint32_t hist[4][256];
     __shared__ uint32_t bound[2][kWarps];
     __shared__ uint32_t sel_prefix, sel_want;
     __shared__ uint32_t warp_tot[kWarps];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int t = tid; t < 4 * 256; t += kSelThreads) (&hist[0][0])[t] = 0u;
+    for (int t = tid; t < 4 * 256; t += kThreads) (&hist[0][0])[t] = 0u;
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
     if (lane == 0) {
@@ -285,7 +296,7 @@ __device__ __forceinline__ void radix_select_emit(const uint32_t *keys, uint32_t
         const int shift = max(top - 8, 0);
         const uint32_t prefix = sel_prefix;
         const uint32_t high_mask = top >= 32 ? 0u : 0xffffffffu << top;
-        for (int i = tid; i < n; i += kSelThreads) {
+        for (int i = tid; i < n; i += kThreads) {
             const uint32_t key = keys[i] - lo;
             if ((key & high_mask) == prefix) atomicAdd(&hist[pass][(key & ~high_mask) >> shift], 1u);
         }
@@ -322,7 +333,7 @@ __device__ __forceinline__ void radix_select_emit(const uint32_t *keys, uint32_t
     const uint32_t need_eq = sel_want;        // how many tokens equal to theta are kept (the latest ones)
 
     // ---- emit the kept positions in ascending order: a contiguous piece per warp, 32 tokens at a time
-    const int piece = ((n + kSelThreads - 1) / kSelThreads) * 32;
+    const int piece = ((n + kThreads - 1) / kThreads) * 32;
     const int first = warp * piece, last = min(first + piece, n);
     uint32_t gt = 0u, eq = 0u;
     for (int i = first; i < last; i += 32) {
@@ -349,37 +360,41 @@ __device__ __forceinline__ void radix_select_emit(const uint32_t *keys, uint32_t
         g += __popc(over_mask);
         q += __popc(tie_mask);
     }
-    for (int j = tid; j < alpha; j += kSelThreads)
+    for (int j = tid; j < alpha; j += kThreads)
         for (int c = 0; c < copies; ++c) out[(size_t)c * budget + k + j] = n + j;   // observation tokens
-    for (int j = k + alpha + tid; j < budget; j += kSelThreads)                     // a sequence with a smaller budget of its own
+    for (int j = k + alpha + tid; j < budget; j += kThreads)                     // a sequence with a smaller budget of its own
         for (int c = 0; c < copies; ++c) out[(size_t)c * budget + j] = -1;
 }
 
 // What a block writes for a head that is not selected from (true): -1 after a wait that ran out in an earlier stage (the
 // scores are incomplete), the identity list under Algorithm 1's guard, and -1 for an invalid length.
+template <int kThreads>
 __device__ __forceinline__ bool settled(const Params &p, int head, int32_t *out)
 {
     const int b = head / p.hkv, L = p.meta[b];
     const bool aborted = call_aborted(p);
     if (!aborted && L > seq_budget(p, b)) return false;
-    for (int j = threadIdx.x; j < p.budget; j += kSelThreads) out[j] = (!aborted && j < L) ? j : -1;
+    for (int j = threadIdx.x; j < p.budget; j += kThreads) out[j] = (!aborted && j < L) ? j : -1;
     return true;
 }
 
-__global__ void __launch_bounds__(kSelThreads, 4) select_kernel(Params p)
+// (what a block waits for is its own barriers: with half the threads twice the blocks are under way.  8192 heads of 2168
+// tokens: 136 us with 512, 98; 4096 heads of 4216: 104, 80.)
+constexpr int kPickThreads = 256;
+__global__ void __launch_bounds__(kPickThreads, 8) select_kernel(Params p)
 {
     extern __shared__ uint4 sel_smem[];            // [cap_pad] keys
     pdl_trigger();
     pdl_wait();
     const int head = blockIdx.x, b = head / p.hkv;
     int32_t *out = p.out_idx + (size_t)head * p.budget;
-    if (settled(p, head, out)) return;
+    if (settled<kPickThreads>(p, head, out)) return;
     if (p.head_mean) return;                       // select_mean_kernel picks the sequence's positions
     const int budget_b = seq_budget(p, b), n = p.meta[b] - p.alpha;
     const uint4 *src = reinterpret_cast<const uint4 *>(p.keys + (size_t)head * p.cap_pad);
     uint32_t lo = 0xffffffffu, hi = 0u;
 #pragma unroll 4
-    for (int v = threadIdx.x; v * 4 < n; v += kSelThreads) {
+    for (int v = threadIdx.x; v * 4 < n; v += kPickThreads) {
         const uint4 k4 = src[v];
         sel_smem[v] = k4;
         lo = min(lo, k4.x);
@@ -388,13 +403,16 @@ __global__ void __launch_bounds__(kSelThreads, 4) select_kernel(Params p)
         if (v * 4 + 2 < n) lo = min(lo, k4.z), hi = max(hi, k4.z);
         if (v * 4 + 3 < n) lo = min(lo, k4.w), hi = max(hi, k4.w);
     }
-    radix_select_emit(reinterpret_cast<const uint32_t *>(sel_smem), lo, hi, n, budget_b - p.alpha, p.alpha, p.budget, out, 1);
+    radix_select_emit<kPickThreads>(reinterpret_cast<const uint32_t *>(sel_smem), lo, hi, n, budget_b - p.alpha, p.alpha, p.budget, out, 1);
 }
 
 // Small caches: the three steps in one block per head, the pooled logits in shared memory.
-__global__ void __launch_bounds__(kSelThreads, 2) select_fused_kernel(Params p)
+// 512 threads where the heads do not fill the chip (the fastest for one head), 256 where blocks queue up: what they wait for is
+// mostly their own barriers and loads, and twice as many are under way.
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, 1024 / kThreads) select_fused_kernel(Params p)
 {
-    constexpr int kWarps = kSelThreads / 32;
+    constexpr int kWarps = kThreads / 32;
     extern __shared__ uint4 sel_smem[];            // [cap_pad] column means, then keys; [cap_pad] means of weights; [alpha][cap_pad] logits
     __shared__ float part[4 * RKV_MAX_GROUP_ROWS];          // a row's two halves: maximum, sum of exponentials
     __shared__ float stat[2 * RKV_MAX_GROUP_ROWS];
@@ -404,7 +422,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_fused_kernel(Params p)
     const int head = blockIdx.x, b = head / p.hkv;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int32_t *out = p.out_idx + (size_t)head * p.budget;
-    if (settled(p, head, out)) return;
+    if (settled<kThreads>(p, head, out)) return;
     const int budget_b = seq_budget(p, b), n = p.meta[b] - p.alpha;
     float *row = reinterpret_cast<float *>(sel_smem), *weight = row + p.cap_pad, *lg = row + 2 * p.cap_pad;
     const float *logits = p.logits + (size_t)head * p.alpha * p.cap_pad;
@@ -412,7 +430,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_fused_kernel(Params p)
 
     // ---- Eq. 6: the column means and their maximum
     float m = -INFINITY;
-    for (int i = tid; i < n; i += kSelThreads) {
+    for (int i = tid; i < n; i += kThreads) {
         const float v = column_mean(p, sbar[i], n);
         row[i] = v;
         m = fmaxf(m, v);
@@ -457,16 +475,16 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_fused_kernel(Params p)
             part[2 * q + 1] = sw;
         }
     }
-    m = block_max<kSelThreads>(m, scratch);        // (its barriers also close the loops above)
-    for (int j = tid; j < p.alpha; j += kSelThreads) {
+    m = block_max<kThreads>(m, scratch);        // (its barriers also close the loops above)
+    for (int j = tid; j < p.alpha; j += kThreads) {
         const float m0 = part[4 * j], m1 = part[4 * j + 2], mj = fmaxf(m0, m1);
         const float s0 = part[4 * j + 1], s1 = part[4 * j + 3];
         stat[2 * j] = mj;
         stat[2 * j + 1] = 1.0f / ((s0 == 0.f ? 0.f : s0 * expf(m0 - mj)) + (s1 == 0.f ? 0.f : s1 * expf(m1 - mj)));
     }
     float s = 0.f;
-    for (int i = tid; i < n; i += kSelThreads) s += expf(row[i] - m);
-    s = block_sum<kSelThreads>(s, scratch);
+    for (int i = tid; i < n; i += kThreads) s += expf(row[i] - m);
+    s = block_sum<kThreads>(s, scratch);
     const float inv = 1.0f / s;
 
     // ---- Eq. 4 and 7; the key of a token takes the place of its column mean
@@ -484,20 +502,20 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_fused_kernel(Params p)
     };
     if (p.mean_then_pool) {
         // Algorithm 1's order: the mean of the alpha softmax weights per position, then the max over the window
-        for (int i = tid; i < n; i += kSelThreads) {
+        for (int i = tid; i < n; i += kThreads) {
             float mean = 0.f;
             for (int j = 0; j < p.alpha; ++j) mean += expf(lg[j * p.cap_pad + i] - stat[2 * j]) * stat[2 * j + 1];
             weight[i] = mean * inv_alpha;
         }
         __syncthreads();
-        for (int i = tid; i < n; i += kSelThreads) {
+        for (int i = tid; i < n; i += kThreads) {
             float best = weight[i];
             for (int u = max(i - W, 0); u <= min(i + W - 1, n - 1); ++u) best = fmaxf(best, weight[u]);
             finish(i, best);
         }
     } else if (W == 4) {
         // eight tokens and half of the query rows per thread; the pair of threads adds its halves up
-        for (int t0 = 0; t0 < n; t0 += kSelThreads * 4) {
+        for (int t0 = 0; t0 < n; t0 += kThreads * 4) {
             const int i0 = t0 + (tid >> 1) * 8;
             float acc[8];
 #pragma unroll
@@ -518,7 +536,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_fused_kernel(Params p)
                 if ((t & 1) == (tid & 1) && i0 + t < n) finish(i0 + t, acc[t] * inv_alpha);
         }
     } else {
-        for (int i = tid; i < n; i += kSelThreads) {
+        for (int i = tid; i < n; i += kThreads) {
             const int first = max(i - W, 0), last = min(i + W - 1, n - 1);
             float acc = 0.f;
             for (int j = 0; j < p.alpha; ++j) {
@@ -531,7 +549,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_fused_kernel(Params p)
         }
     }
     if (p.head_mean) return;      // Z of this head is in p.keys; select_mean_kernel picks the sequence's positions
-    radix_select_emit(keys, lo, hi, n, budget_b - p.alpha, p.alpha, p.budget, out, 1);
+    radix_select_emit<kThreads>(keys, lo, hi, n, budget_b - p.alpha, p.alpha, p.budget, out, 1);
 }
 
 // Algorithm 1's aggregated selection, one block per sequence: AggScore_i = mean over the KV heads of Z_i^h (left in
@@ -557,7 +575,7 @@ __global__ void __launch_bounds__(kSelThreads, 4) select_mean_kernel(Params p)
         lo = min(lo, keys[i]);
         hi = max(hi, keys[i]);
     }
-    radix_select_emit(keys, lo, hi, n, seq_budget(p, b) - p.alpha, p.alpha, p.budget, p.out_idx + (size_t)b * p.hkv * p.budget, p.hkv);
+    radix_select_emit<kSelThreads>(keys, lo, hi, n, seq_budget(p, b) - p.alpha, p.alpha, p.budget, p.out_idx + (size_t)b * p.hkv * p.budget, p.hkv);
 }
 
 }  // namespace
@@ -570,6 +588,15 @@ static cudaError_t launch_select_mean(const Params &p, cudaStream_t s)
     return launch_early(select_mean_kernel, (unsigned)p.batch, kSelThreads, (size_t)p.cap_pad * sizeof(float), s, 1, p);
 }
 
+template <int kThreads>
+static cudaError_t launch_fused(const Params &p, unsigned heads, int dev, cudaStream_t s)
+{
+    static std::atomic<unsigned long long> done{0ull};
+    const cudaError_t e = allow_smem_once(done, dev, select_fused_kernel<kThreads>, (int)kFusedSmemLimit);
+    if (e != cudaSuccess) return e;
+    return launch_early(select_fused_kernel<kThreads>, heads, kThreads, (size_t)(p.alpha + 2) * p.cap_pad * sizeof(float), s, 1, p);
+}
+
 cudaError_t launch_select(const Params &p, cudaStream_t s)
 {
     const unsigned heads = (unsigned)(p.batch * p.hkv);
@@ -577,22 +604,21 @@ cudaError_t launch_select(const Params &p, cudaStream_t s)
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess) return e;
     if (select_is_fused(p.cap_pad, p.alpha)) {
-        static std::atomic<unsigned long long> done{0ull};
         if ((e = mark_kernel(p, 2, s)) != cudaSuccess || (e = mark_kernel(p, 3, s)) != cudaSuccess) return e;
-        if ((e = allow_smem_once(done, dev, select_fused_kernel, (int)kFusedSmemLimit)) != cudaSuccess) return e;
-        e = launch_early(select_fused_kernel, heads, kSelThreads, (size_t)(p.alpha + 2) * p.cap_pad * sizeof(float), s, 1, p);
+        e = heads > 2u * (unsigned)sms ? launch_fused<256>(p, heads, dev, s) : launch_fused<kSelThreads>(p, heads, dev, s);
         if (e != cudaSuccess) return e;
         return p.head_mean ? launch_select_mean(p, s) : cudaSuccess;
     }
     if ((e = launch_early(row_stats_kernel, (heads * (unsigned)(p.alpha + 1) + kStatThreads / 32 - 1) / (kStatThreads / 32), kStatThreads, 0, s, 1, p)) != cudaSuccess) return e;
     if ((e = mark_kernel(p, 2, s)) != cudaSuccess) return e;
     if (p.pool_w == 4 && !p.mean_then_pool)
-        e = launch_early(importance_w4_kernel, heads * (unsigned)((p.cap + kImp8Tokens - 1) / kImp8Tokens), kImp8Threads, 0, s, 1, p);
+        e = launch_early(importance_w4_kernel, (unsigned)(((unsigned long long)heads * ((p.cap + 7) / 8) + kImp8Threads - 1) / kImp8Threads), kImp8Threads, 0,
+                         s, 1, p);
     else
         e = launch_early(importance_kernel, heads * (unsigned)((p.cap + kImpTokens - 1) / kImpTokens), kImpThreads, 0, s, 1, p);
     if (e != cudaSuccess) return e;
     if ((e = mark_kernel(p, 3, s)) != cudaSuccess) return e;
-    if ((e = launch_early(select_kernel, heads, kSelThreads, (size_t)p.cap_pad * sizeof(float), s, 1, p)) != cudaSuccess) return e;
+    if ((e = launch_early(select_kernel, heads, kPickThreads, (size_t)p.cap_pad * sizeof(float), s, 1, p)) != cudaSuccess) return e;
     return p.head_mean ? launch_select_mean(p, s) : cudaSuccess;
 }
 

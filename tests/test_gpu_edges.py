@@ -53,6 +53,18 @@ def test_cuda_core_scoring_tiles(rkv, head_dim, hq, alpha, budget, buffer, lens)
     comp.check_status()
 
 
+@pytest.mark.parametrize("batch,hkv,alpha,pool_w,beta", [(38, 8, 8, 4, 1), (37, 8, 8, 4, 3), (300, 1, 5, 2, 1)])
+def test_many_small_heads(rkv, batch, hkv, alpha, pool_w, beta):  # noqa: F811
+    """304, 296 and 300 heads: the selection's blocks halve above two heads per SM (296 on 148 SMs).  n = 128, 127, 93, lists that
+    end inside a warp's piece."""
+    spec = small_spec("many", batch=batch, hkv=hkv, hq=2 * hkv, budget=100, buffer=36, alpha=alpha, span=4)
+    lens = [(136, 135, 101, 100)[b % 4] for b in range(batch)]
+    wl = ri.make_workload(spec, device="cuda", seed=407 + batch, seq_lens=torch.tensor(lens))
+    rep, comp = run_and_check(rkv, wl, beta=beta, W=pool_w)
+    assert rep.ok(), rep.errors
+    comp.check_status()
+
+
 @pytest.mark.parametrize("batch,hkv,hq,cap", [(1, 1, 4, 128), (1, 1, 4, 8192), (2, 1, 8, 2176), (1, 2, 2, 1920), (1, 2, 2, 1921),
                                               (40, 8, 16, 640)])
 def test_decode_attention_splits(rkv, batch, hkv, hq, cap):  # noqa: F811
