@@ -485,7 +485,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                         // Several partners per token, S = T + h r_i r_j each.  Most 16-column pieces hold none: the others are
                         // loaded again and looked at by one copy of this code (the warps of three roles share the
                         // instruction cache).  4096 heads of 1068 tokens with beta = 4: the pass took 1022 us with every
-                        // chunk of 32 gone through and its r_j loaded where it held a partner, 888 now.
+                        // chunk of 32 gone through and its r_j loaded where it held a partner, 726 now.
 #pragma unroll 1
                         for (unsigned todo = screen128(base, want); todo != 0u;) {
                             const int piece = 31 - __clz((int)todo), c0 = piece * 16;

@@ -308,27 +308,35 @@ __device__ __forceinline__ unsigned screen128(uint32_t base, bool want)
     }
     return __reduce_or_sync(0xffffffffu, want ? neg ^ 255u : 0u);
 }
-// Several partners per token: the entries above zero in the columns of `mask`, cut down to the `left` highest columns; returns how
-// many and adds their sum of h r_j, r_j of column c of the piece in lane `lane0` + c.  mask = 0 for a lane that wants nothing.
-__device__ __forceinline__ int take_many(uint32_t (&g)[16], uint32_t mask, int left, float r_lane, int lane0, float &sum)
+// Several partners per token: the entries above zero in the columns of `mask`, highest column first, at most `left` of them; returns
+// how many and adds their sum of h r_j, r_j of column c of the piece in lane `lane0` + c.  mask = 0 for a lane that wants nothing.
+// A turn per partner, the warp together: most pieces hold one or two per token.  (A clear sign bit may also be +0 or a NaN.)
+__device__ __forceinline__ int take_many(const uint32_t (&g)[16], uint32_t mask, int left, float r_lane, int lane0, float &sum)
 {
-    uint32_t above = 0u;
+    uint32_t n0 = 0u, n1 = 0u;
 #pragma unroll
-    for (int c = 0; c < 16; ++c) above |= (__uint_as_float(g[c]) > 0.f) ? (1u << c) : 0u;
-    uint32_t keep = above & mask;
-    int taken = __popc(keep);
-    for (; taken > left; --taken) keep &= keep - 1u;                   // drop the lowest columns
-    if (__any_sync(0xffffffffu, keep != above && keep != 0u)) {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) g[c] = (keep >> c & 1u) ? g[c] : 0u;
+    for (int c = 7; c >= 0; --c) {
+        n0 = __funnelshift_l(g[c], n0, 1);
+        n1 = __funnelshift_l(g[8 + c], n1, 1);
     }
-    float s0 = 0.f, s1 = 0.f;
+    uint32_t pos = ~(n0 | (n1 << 8)) & mask;
+    int taken = 0;
+    while (__any_sync(0xffffffffu, pos != 0u)) {
+        const int top = 31 - __clz((int)(pos | 1u));
+        const float r = __shfl_sync(0xffffffffu, r_lane, lane0 + top);
+        uint32_t t8[8], t4[4];
 #pragma unroll
-    for (int c = 0; c < 16; c += 2) {
-        s0 = fmaf(fmaxf(__uint_as_float(g[c]), 0.f), __shfl_sync(0xffffffffu, r_lane, lane0 + c), s0);
-        s1 = fmaf(fmaxf(__uint_as_float(g[c + 1]), 0.f), __shfl_sync(0xffffffffu, r_lane, lane0 + c + 1), s1);
+        for (int c = 0; c < 8; ++c) t8[c] = (top & 8) ? g[8 + c] : g[c];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) t4[c] = (top & 4) ? t8[4 + c] : t8[c];
+        const uint32_t u0 = (top & 2) ? t4[2] : t4[0], u1 = (top & 2) ? t4[3] : t4[1];
+        const float v = __uint_as_float((top & 1) ? u1 : u0);
+        if (pos != 0u && v > 0.f) {
+            sum += v * r;
+            ++taken;
+        }
+        pos = taken == left ? 0u : pos & ~(1u << top);
     }
-    if (keep != 0u) sum += s0 + s1;
     return taken;
 }
 
