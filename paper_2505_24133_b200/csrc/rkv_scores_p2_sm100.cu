@@ -421,9 +421,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                     // The accumulator holds h = k_i . k_j - (T / r_i) (||k_j|| + eps): S[j][i] > T exactly when h > 0, so
                     // the screening is a sign test, with nothing to load per column (loads of the r_j were what this
                     // epilogue's time went into: every byte a thread receives, from TMEM or as a shared-memory
-                    // broadcast, passes through the same return path).  32-column chunks, last first; the TMEM load of
-                    // the next chunk is issued before the current one is looked at (two register sets, used alternately).
-                    // (beta = 1, the default: one partner per token)
+                    // broadcast, passes through the same return path).
                     auto chunk = [&](const uint32_t (&g)[32], int ch) {
                         uint32_t colmask = 0xffffffffu;
                         const unsigned own = (unsigned)(i - (jbase + ch * 32));           // zero diagonal (Eq. 5)
@@ -440,20 +438,12 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                         const uint32_t neg = (n0 | (n1 << 8)) | ((n2 << 16) | (n3 << 24));
                         // entries with a clear sign bit (h > 0, but also +0: confirmed one by one below)
                         uint32_t pos = want ? (~neg & colmask) : 0u;
-                        {
+                        if (kOne) {
                             // one partner at most: the candidate at the highest set bit, its value picked by a select
                             // tree (nearly always a single turn); its r_j is fetched once, at the item's end
                             while (pos != 0u) {
                                 const int top = 31 - __clz(pos);
-                                uint32_t t16[16], t8[8], t4[4];
-#pragma unroll
-                                for (int c = 0; c < 16; ++c) t16[c] = (top & 16) ? g[16 + c] : g[c];
-#pragma unroll
-                                for (int c = 0; c < 8; ++c) t8[c] = (top & 8) ? t16[8 + c] : t16[c];
-#pragma unroll
-                                for (int c = 0; c < 4; ++c) t4[c] = (top & 4) ? t8[4 + c] : t8[c];
-                                const uint32_t u0 = (top & 2) ? t4[2] : t4[0], u1 = (top & 2) ? t4[3] : t4[1];
-                                const float hv = __uint_as_float((top & 1) ? u1 : u0);
+                                const float hv = pick32(g, top);
                                 if (hv > 0.f) {
                                     hit_h = hv;
                                     hit_j = jbase + ch * 32 + top;
@@ -463,43 +453,41 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                                 }
                                 pos &= ~(1u << top);
                             }
+                        } else {
+                            // several: S = T + h r_i r_j each, a turn per partner, the warp together (4096 heads of 1068 tokens with
+                            // beta = 4: the pass took 1020 us while every column of a chunk that holds a partner was compared,
+                            // multiplied by an r_j loaded then and summed; 603 now)
+                            while (__any_sync(0xffffffffu, pos != 0u)) {
+                                const int top = 31 - __clz((int)(pos | 1u));
+                                const float r = __shfl_sync(0xffffffffu, rj[ch], top);
+                                const float hv = pick32(g, top);
+                                if (pos != 0u && hv > 0.f) {
+                                    removed += hv * r;
+                                    ++nhit;
+                                    --left;
+                                }
+                                pos = left == 0 ? 0u : pos & ~(1u << top);
+                            }
+                            want = left > 0;
                         }
                     };
-                    if (kOne) {
-                        if (__any_sync(0xffffffffu, want)) {
-                            uint32_t ga[32], gb[32];
-                            tmem_ld32(base + 96, ga);
-                            tmem_wait32(ga);
-                            tmem_ld32(base + 64, gb);
-                            chunk(ga, 3);
-                            tmem_wait32(gb);
-                            tmem_ld32(base + 32, ga);
-                            chunk(gb, 2);
-                            tmem_wait32(ga);
-                            tmem_ld32(base, gb);
-                            chunk(ga, 1);
-                            tmem_wait32(gb);
-                            chunk(gb, 0);
-                        }
-                    } else if (__any_sync(0xffffffffu, want)) {
-                        // Several partners per token, S = T + h r_i r_j each.  Most 16-column pieces hold none: the others are
-                        // loaded again and looked at by one copy of this code (the warps of three roles share the
-                        // instruction cache).  4096 heads of 1068 tokens with beta = 4: the pass took 1022 us with every
-                        // chunk of 32 gone through and its r_j loaded where it held a partner, 726 now.
-#pragma unroll 1
-                        for (unsigned todo = screen128(base, want); todo != 0u;) {
-                            const int piece = 31 - __clz((int)todo), c0 = piece * 16;
-                            todo &= ~(1u << piece);
-                            uint32_t g[16];
-                            tmem_get16(base + c0, g);
-                            uint32_t mask = left > 0 ? 0xffffu : 0u;
-                            const unsigned own = (unsigned)(i - (jbase + c0));                // zero diagonal (Eq. 5)
-                            if (own < 16u) mask &= ~(1u << own);
-                            const float r_lane = piece >= 6 ? rj[3] : piece >= 4 ? rj[2] : piece >= 2 ? rj[1] : rj[0];
-                            const int taken = take_many(g, mask, left, r_lane, (piece & 1) * 16, removed);
-                            nhit += taken;
-                            left -= taken;
-                        }
+                    // 32-column chunks, last first; the TMEM load of the next chunk is issued before the current one is looked at (two
+                    // register sets, used alternately).  What this takes is integer instructions (two cycles each) and their fetch:
+                    // longer loads, or a conjunction of signs first and the chunks it names loaded again, were slower with beta = 1.
+                    if (__any_sync(0xffffffffu, want)) {
+                        uint32_t ga[32], gb[32];
+                        tmem_ld32(base + 96, ga);
+                        tmem_wait32(ga);
+                        tmem_ld32(base + 64, gb);
+                        chunk(ga, 3);
+                        tmem_wait32(gb);
+                        tmem_ld32(base + 32, ga);
+                        chunk(gb, 2);
+                        tmem_wait32(ga);
+                        tmem_ld32(base, gb);
+                        chunk(ga, 1);
+                        tmem_wait32(gb);
+                        chunk(gb, 0);
                     }
                     tc_fence_before();
                     __syncwarp();

@@ -217,37 +217,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
         : "r"(taddr)
         : "memory");
 }
-// 64 columns, loaded and waited for in one statement: where the registers pass through a statement of their own for the wait,
-// each of them is copied (32 columns at a time that way, a tile's screening below took 740 cycles instead of 480).
-__device__ __forceinline__ void tmem_get64(uint32_t taddr, uint32_t (&r)[64])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, "
-        "%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
-        "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
-          "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
-          "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
-          "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
-          "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_get16(uint32_t taddr, uint32_t (&r)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
 {
     asm volatile(
@@ -288,58 +257,19 @@ __device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32])
                  :: "memory");
 }
 
-__device__ __forceinline__ uint32_t and16(const uint32_t (&g)[64], int at)
+// Entry `at` of 32 registers, by a select tree
+__device__ __forceinline__ float pick32(const uint32_t (&g)[32], int at)
 {
-    const uint32_t a = (g[at] & g[at + 1] & g[at + 2]) & g[at + 3] & g[at + 4], b = (g[at + 5] & g[at + 6] & g[at + 7]) & g[at + 8] & g[at + 9];
-    return (a & g[at + 10] & g[at + 11]) & (b & g[at + 12] & g[at + 13]) & (g[at + 14] & g[at + 15]);
-}
-// Which 16-column pieces of a 128-column accumulator row hold an entry with a clear sign bit for some lane that wants to know
-// (bit c: piece c).  A conjunction of sign bits, half an instruction per entry, is all that is done with most entries: what a
-// tile's screening takes is its integer instructions (64 per warp and 128 columns, two cycles each; a funnel shift per entry
-// took twice that).  The pieces it names are loaded once more and looked at by one copy of the code that does so.
-__device__ __forceinline__ unsigned screen128(uint32_t base, bool want)
-{
-    unsigned neg = 0u;
-#pragma unroll 1                            // (the two loads then use the same registers: unrolled, they spilled)
-    for (int half = 1; half >= 0; --half) {
-        uint32_t g[64];
-        tmem_get64(base + 64 * half, g);
-        neg = neg << 4 | and16(g, 48) >> 31 << 3 | and16(g, 32) >> 31 << 2 | and16(g, 16) >> 31 << 1 | and16(g, 0) >> 31;
-    }
-    return __reduce_or_sync(0xffffffffu, want ? neg ^ 255u : 0u);
-}
-// Several partners per token: the entries above zero in the columns of `mask`, highest column first, at most `left` of them; returns
-// how many and adds their sum of h r_j, r_j of column c of the piece in lane `lane0` + c.  mask = 0 for a lane that wants nothing.
-// A turn per partner, the warp together: most pieces hold one or two per token.  (A clear sign bit may also be +0 or a NaN.)
-__device__ __forceinline__ int take_many(const uint32_t (&g)[16], uint32_t mask, int left, float r_lane, int lane0, float &sum)
-{
-    uint32_t n0 = 0u, n1 = 0u;
+    uint32_t t16[16], t8[8], t4[4];
 #pragma unroll
-    for (int c = 7; c >= 0; --c) {
-        n0 = __funnelshift_l(g[c], n0, 1);
-        n1 = __funnelshift_l(g[8 + c], n1, 1);
-    }
-    uint32_t pos = ~(n0 | (n1 << 8)) & mask;
-    int taken = 0;
-    while (__any_sync(0xffffffffu, pos != 0u)) {
-        const int top = 31 - __clz((int)(pos | 1u));
-        const float r = __shfl_sync(0xffffffffu, r_lane, lane0 + top);
-        uint32_t t8[8], t4[4];
+    for (int c = 0; c < 16; ++c) t16[c] = (at & 16) ? g[16 + c] : g[c];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) t8[c] = (top & 8) ? g[8 + c] : g[c];
+    for (int c = 0; c < 8; ++c) t8[c] = (at & 8) ? t16[8 + c] : t16[c];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) t4[c] = (top & 4) ? t8[4 + c] : t8[c];
-        const uint32_t u0 = (top & 2) ? t4[2] : t4[0], u1 = (top & 2) ? t4[3] : t4[1];
-        const float v = __uint_as_float((top & 1) ? u1 : u0);
-        if (pos != 0u && v > 0.f) {
-            sum += v * r;
-            ++taken;
-        }
-        pos = taken == left ? 0u : pos & ~(1u << top);
-    }
-    return taken;
+    for (int c = 0; c < 4; ++c) t4[c] = (at & 4) ? t8[4 + c] : t8[c];
+    const uint32_t u0 = (at & 2) ? t4[2] : t4[0], u1 = (at & 2) ? t4[3] : t4[1];
+    return __uint_as_float((at & 1) ? u1 : u0);
 }
-
 // max(a, b, c), NaN operands ignored
 __device__ __forceinline__ float max3(float a, float b, float c)
 {
