@@ -361,33 +361,32 @@ def kernel_table(rkv, timed: Timed, kw, KB, peaks):
     n = spec.cap - spec.alpha
     esz = wl.k_cache.element_size()
     row = spec.head_dim * esz
-    wide_row = max(spec.head_dim, 128 if spec.head_dim == 64 else 0) * 2       # a row of the bf16 scoring copy (8-bit caches, d = 64)
+    wide_row = spec.head_dim * 2                       # a row of the bf16 scoring copy (8-bit caches)
     P = spec.head_problems
     T = (n + 127) // 128
     q_cols = -(-(spec.n_q_heads // spec.n_kv_heads) * spec.alpha // 16) * 16 + 16
     # one tile product = 128 x 128 outputs over K = 128 + 16: the head dimension plus the one extra K = 16 step that
     # folds the threshold test into the accumulator (both scoring passes issue it for every key tile)
-    # (head dimension 64 runs on keys padded to 128: the padding's products are not counted as work)
     tile_flops = 2.0 * 128 * 128 * (spec.head_dim + 16)
     rule_on = comp_ev.desc.beta > 0 and comp_ev.desc.sim_threshold < 1.0
     pass1_tiles = P * T if rule_on else 0              # every row tile meets the last key tile once
     pass1_flops = pass1_tiles * tile_flops + P * T * 2.0 * 128 * q_cols * spec.head_dim
     pass2_flops = max(tiles_executed - pass1_tiles, 0) * tile_flops
-    pass2_useful = pairs2 * 2.0 * 128 * (128 + 16)     # listed tokens x keys of the streamed tiles x 2 (d + 16)
+    pass2_useful = pairs2 * 2.0 * 128 * (spec.head_dim + 16)     # listed tokens x keys of the streamed tiles x 2 (d + 16)
     # algorithmic work per launch: bytes a kernel has to move / flops it has to execute, nothing it merely could
     work = {
-        # K once; r_i, Kbar_i.Kbar_i and the 16-byte slice out.  8-bit caches and d = 64: the stored keys in and their bf16 /
-        # padded copy out (written by the prep kernel itself when a stored row is 128 bytes and the capacity a whole
-        # number of tiles; else by a pass of its own, and read back)
-        "prep": ("hbm", P * (n * row + spec.cap * (8 + 16)) if (esz > 1 and spec.head_dim != 64) else
+        # K once; r_i, Kbar_i.Kbar_i and the 16-byte slice out.  8-bit caches: the stored keys in and their bf16 copy out
+        # (written by the prep kernel itself when a stored row is 128 bytes and the capacity a whole number of tiles;
+        # else by a pass of its own, and read back)
+        "prep": ("hbm", P * (n * row + spec.cap * (8 + 16)) if esz > 1 else
                  (P * (n * row + n * wide_row + spec.cap * (8 + 16)) if (row == 128 and spec.cap % 128 == 0) else
                   P * (spec.cap * row + spec.cap * wide_row + n * wide_row + spec.cap * (8 + 16)))),
         "scores_pass1": ("tensor", pass1_flops),
-        "scores_list": ("hbm", P * n * 8),
+        "scores_list": ("hbm", P * n / 8),                 # a bit per token (and what it lists)
         "scores_pass2": ("tensor", pass2_flops),
-        "row_stats": ("hbm", P * spec.alpha * n * 4),
-        "importance": ("hbm", P * (spec.alpha + 1) * n * 4),
-        "select": ("hbm", P * (2 * n * 4 + spec.budget * 4)),
+        "row_stats": ("hbm", P * (spec.alpha + 1) * n * 4),      # pooled logits and column means
+        "importance": ("hbm", P * (spec.alpha + 2) * n * 4),     # both once more, the keys out
+        "select": ("hbm", P * (n * 4 + spec.budget * 4)),
         "gather": ("hbm", moved_rows * row * 2 * 2 + P * spec.budget * 4),      # K and V rows that move: read + write
     }
     kernels = {}

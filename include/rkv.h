@@ -319,8 +319,7 @@ RKV_API int rkv_decode_attention(const rkv_desc_t *desc, const void *k_cache, co
 RKV_API int rkv_selftest_wait_expiry(int32_t *device_status, unsigned long long *report_words, int64_t limit_cycles,
                                      void *stream);
 
-/* Number of kernels a call launches (for launch accounting; the memset that precedes the prep kernel is not
- * counted).  rkv_launch_count_for() is exact for the given sizes; rkv_launch_count(), which does not know them, gives
+/* Number of kernels a call launches (for launch accounting).  rkv_launch_count_for() is exact for the given sizes; rkv_launch_count(), which does not know them, gives
  * the count for large caches (small ones run the select stage as one kernel instead of three). */
 RKV_API int rkv_launch_count(const rkv_desc_t *desc, uint32_t stage_mask);
 RKV_API int rkv_launch_count_for(const rkv_desc_t *desc, int32_t budget, int32_t buffer, int32_t alpha,
