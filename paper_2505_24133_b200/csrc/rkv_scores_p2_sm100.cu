@@ -545,94 +545,127 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 }
 
 // ---- before every round: list, per head, the tokens still short of partners, and cut the list into work items ----
-constexpr int kCompactWarps = 8;         // a warp per head
-constexpr int kWordsPerLane = RKV_MAX_CAP / 32 / 32;
+constexpr int kCompactWarps = 8;         // of a block; one or four per head
 constexpr int kDenseMinTiles = 12;       // caches of fewer key tiles never take the symmetric route (two more launches)
 
 // The tokens are given as one bit each, 32 to a word, so a list costs a head's 33 words per 1024 tokens and what it writes.
-// (Read from a word per token by a block per head, a listing of 4096 heads of 4216 tokens took 81 us; 37 now.)
+// (Read from a word per token by a block per head, a listing of 4096 heads of 4216 tokens took 81 us; 37 with bits.  The counters
+// took part of that: three atomics per head on one line of memory.  A block adds its heads' up first: 33; 8192 heads of 2168
+// tokens 35 -> 25.)  kHeadWarps: four warps share the words of a head where there are few heads -- one warp's turns over them are
+// then what a call waits for (256 heads of 1144 tokens: 12 -> 8 us) --, one takes them all where blocks with more heads, and
+// so fewer atomics, count for more (with two heads a block 8192 took 50 us).
 // `below`: key tiles under the first pass's part that earlier rounds have covered; `width`: tiles of this round's
 // window (the last round passes a width that reaches tile 0 whatever the cache size).
+template <int kHeadWarps>
 __global__ void __launch_bounds__(kCompactWarps * 32) strag_compact_kernel(Params p, int round, int below, int width)
 {
+    constexpr int kCompactHeads = kCompactWarps / kHeadWarps, kWordsPerLane = RKV_MAX_CAP / 32 / (32 * kHeadWarps);
     pdl_trigger();
     pdl_wait();
-    const int head = blockIdx.x * kCompactWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (head >= p.batch * p.hkv) return;
-    const int n = seq_candidates(p, head / p.hkv);
-    const uint32_t *bits = p.lacking + (size_t)head * (p.cap_pad / 32);
+    __shared__ int warp_count[kCompactWarps], block_chunks[kCompactHeads];
+    __shared__ unsigned long long block_pairs[kCompactHeads], block_slot;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int mate = warp / kHeadWarps, part = warp % kHeadWarps;        // which head of the block, which part of its words
+    const int head = blockIdx.x * kCompactHeads + mate;
+    const bool head_ok = head < p.batch * p.hkv;
+    const int n = head_ok ? seq_candidates(p, head / p.hkv) : 0;
     int32_t *list = p.strag + (size_t)head * p.cap_pad;
     // the first pass scanned every token against the last kPass1Depth key tiles; this round starts `below` tiles
     // under that
     const int n_tiles = (n + kTile - 1) / kTile;
-    const int first_tile = n_tiles - kPass1Depth - 1 - below;
-    if (first_tile < 0 || call_aborted(p) || (round > 0 && p.dense[head])) {
-        // nothing left to scan for this head, the call has given up, or the head went to the symmetric route
-        if (lane == 0 && round == 0) p.dense[head] = 0;
-        return;
-    }
-    const int words = (n + 31) / 32;
+    const int first_tile = n_tiles - kPass1Depth - 1 - below, n_iter = min(width, first_tile + 1);
+    // a head without anything left to scan, or one that went to the symmetric route, lists nothing; nor does a call that has given up
+    const bool scans = head_ok && first_tile >= 0 && !call_aborted(p) && !(round > 0 && p.dense[head]);
+    const int words = scans ? (n + 31) / 32 : 0, per_warp = (words + kHeadWarps - 1) / kHeadWarps, word0 = part * per_warp;
+    const int my_words = min(per_warp, words - word0);
+    const uint32_t *bits = p.lacking + (size_t)head * (p.cap_pad / 32) + word0;
     uint32_t word[kWordsPerLane];
-    int count = 0;
+    int my_count = 0;
 #pragma unroll
     for (int k = 0; k < kWordsPerLane; ++k) {
-        word[k] = k * 32 + lane < words ? bits[k * 32 + lane] : 0u;
-        count += __popc(word[k]);
+        word[k] = k * 32 + lane < my_words ? bits[k * 32 + lane] : 0u;
+        my_count += __popc(word[k]);
     }
-    count = __reduce_add_sync(0xffffffffu, count);
-    if (round == 0) {
+    my_count = __reduce_add_sync(0xffffffffu, my_count);
+    if (lane == 0) warp_count[warp] = my_count;
+    __syncthreads();
+    int count = 0, at = 0;                   // the head's listed tokens; those of the parts before this one
+#pragma unroll
+    for (int w = 0; w < kHeadWarps; ++w) {
+        count += warp_count[mate * kHeadWarps + w];
+        at += w < part ? warp_count[mate * kHeadWarps + w] : 0;
+    }
+    const bool speaks = head_ok && part == 0 && lane == 0;               // for its head
+    if (speaks && !scans && round == 0) p.dense[head] = 0;
+    if (scans && round == 0) {
         // Most tokens still lack a partner (few pairs exceed T): the rounds would form nearly the whole matrix for this
         // head.  It goes to the symmetric route instead, which forms each tile pair once.
         const bool dense = p.dense_ok && n_tiles >= kDenseMinTiles && 5 * count > 4 * n;
-        if (lane == 0) p.dense[head] = dense ? 1 : 0;
+        if (speaks) p.dense[head] = dense ? 1 : 0;
         if (dense) {
             uint4 *best = reinterpret_cast<uint4 *>(p.best + (size_t)head * p.cap_pad);
-            for (int i = lane; i < p.cap_pad / 4; i += 32) best[i] = make_uint4(0u, 0u, 0u, 0u);
+            for (int i = part * 32 + lane; i < p.cap_pad / 4; i += 32 * kHeadWarps) best[i] = make_uint4(0u, 0u, 0u, 0u);
             const int pairs_of_tiles = (n_tiles + 1) / 2;
-            unsigned long long at = 0ull;
-            if (lane == 0) {
-                at = atomicAdd(&p.counters[kDenseWords], (unsigned long long)pairs_of_tiles);
-                // useful work: every unordered pair of the listed tokens' tiles once
-                atomicAdd(&p.counters[kPairsWord], (unsigned long long)count * (unsigned long long)(n_tiles + 1) / 2ull);
+            if (part == 0) {
+                unsigned long long slot = 0ull;
+                if (lane == 0) {
+                    slot = atomicAdd(&p.counters[kDenseWords], (unsigned long long)pairs_of_tiles);
+                    // useful work: every unordered pair of the listed tokens' tiles once
+                    atomicAdd(&p.counters[kPairsWord], (unsigned long long)count * (unsigned long long)(n_tiles + 1) / 2ull);
+                }
+                slot = __shfl_sync(0xffffffffu, slot, 0);
+                for (int q = lane; q < pairs_of_tiles; q += 32) p.dense_items[slot + q] = make_int4(head, q, n, 0);   // longest first
             }
-            at = __shfl_sync(0xffffffffu, at, 0);
-            for (int q = lane; q < pairs_of_tiles; q += 32) p.dense_items[at + q] = make_int4(head, q, n, 0);   // longest first
-            return;
+            count = 0;                       // nothing for the rounds
         }
     }
-    if (count == 0) return;
-    int at = 0;                              // ascending positions
+    const int chunks = (count + kRowsPerItem - 1) / kRowsPerItem;
+    if (part == 0 && lane == 0) {
+        block_chunks[mate] = chunks;
+        block_pairs[mate] = (unsigned long long)count * (unsigned long long)n_iter;    // the work the round cannot avoid
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {                  // the block's place in the work list, under way while the lists are written
+        int total = 0;
+        unsigned long long pairs = 0ull;
 #pragma unroll
-    for (int k = 0; k < kWordsPerLane; ++k) {
-        if (k * 32 >= words) break;
-        const int mine = __popc(word[k]);
-        int incl = mine;
+        for (int w = 0; w < kCompactHeads; ++w) {
+            total += block_chunks[w];
+            pairs += block_chunks[w] > 0 ? block_pairs[w] : 0ull;
+        }
+        if (total > 0) {
+            block_slot = atomicAdd(&p.counters[kRoundWords + 2 * round], (unsigned long long)total);
+            atomicAdd(&p.counters[2], (unsigned long long)total);
+            atomicAdd(&p.counters[kPairsWord], pairs);
+        }
+    }
+    if (count > 0) {                         // ascending positions
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int o = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += o;
+        for (int k = 0; k < kWordsPerLane; ++k) {
+            if (k * 32 >= my_words) break;
+            const int mine = __popc(word[k]);
+            int incl = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += o;
+            }
+            const int first = at + incl - mine;
+            for (unsigned todo = __ballot_sync(0xffffffffu, mine > 0); todo != 0u; todo &= todo - 1u) {
+                const int src = __ffs(todo) - 1;
+                const uint32_t w = __shfl_sync(0xffffffffu, word[k], src);
+                const int f = __shfl_sync(0xffffffffu, first, src);
+                if (w >> lane & 1u) list[f + __popc(w & ((1u << lane) - 1u))] = (word0 + k * 32 + src) * 32 + lane;
+            }
+            at += __shfl_sync(0xffffffffu, incl, 31);
         }
-        const int first = at + incl - mine;
-        for (unsigned todo = __ballot_sync(0xffffffffu, mine > 0); todo != 0u; todo &= todo - 1u) {
-            const int src = __ffs(todo) - 1;
-            const uint32_t w = __shfl_sync(0xffffffffu, word[k], src);
-            const int f = __shfl_sync(0xffffffffu, first, src);
-            if (w >> lane & 1u) list[f + __popc(w & ((1u << lane) - 1u))] = (k * 32 + src) * 32 + lane;
-        }
-        at += __shfl_sync(0xffffffffu, incl, 31);
     }
-    const int chunks = (count + kRowsPerItem - 1) / kRowsPerItem, n_iter = min(width, first_tile + 1);
-    unsigned long long slot = 0ull;
-    if (lane == 0) {
-        slot = atomicAdd(&p.counters[kRoundWords + 2 * round], (unsigned long long)chunks);
-        atomicAdd(&p.counters[2], (unsigned long long)chunks);
-        // listed tokens x key tiles: the work the round cannot avoid
-        atomicAdd(&p.counters[kPairsWord], (unsigned long long)count * (unsigned long long)n_iter);
-    }
-    slot = __shfl_sync(0xffffffffu, slot, 0);
-    for (int q = lane; q < chunks; q += 32) {
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < mate; ++w) before += block_chunks[w];
+    for (int q = part * 32 + lane; q < chunks; q += 32 * kHeadWarps) {
         const int k0 = q * kRowsPerItem;
-        p.strag_items[slot + q] = make_int4(head, k0, min(count - k0, kRowsPerItem) | (n_iter << 16), first_tile);
+        p.strag_items[block_slot + before + q] = make_int4(head, k0, min(count - k0, kRowsPerItem) | (n_iter << 16), first_tile);
     }
 }
 
@@ -678,7 +711,9 @@ static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
     int below = 0;
     for (int r = 0; r < rounds; ++r) {
         const int width = r == rounds - 1 ? (1 << 20) : kRoundTiles[r];
-        if ((e = launch_early(strag_compact_kernel, (unsigned)((heads + kCompactWarps - 1) / kCompactWarps), kCompactWarps * 32, 0, s, 1, p, r, below, width)) != cudaSuccess) return e;
+        e = heads <= 4 * sms ? launch_early(strag_compact_kernel<4>, (unsigned)((heads + kCompactWarps / 4 - 1) / (kCompactWarps / 4)), kCompactWarps * 32, 0, s, 1, p, r, below, width)
+                             : launch_early(strag_compact_kernel<1>, (unsigned)((heads + kCompactWarps - 1) / kCompactWarps), kCompactWarps * 32, 0, s, 1, p, r, below, width);
+        if (e != cudaSuccess) return e;
         if (r == 0 && (e = mark_kernel(p, 1, s)) != cudaSuccess) return e;
         if ((e = launch_early(scores_pass2_sm100_kernel<D, kOne>, grid2, kThreads, Lay<D>::kSmemBytes, s, 1, p, map_k, map_ns, r)) != cudaSuccess) return e;
         // the heads the first listing sent to the symmetric route (none on inputs where similar keys are common:

@@ -53,6 +53,18 @@ def test_cuda_core_scoring_tiles(rkv, head_dim, hq, alpha, budget, buffer, lens)
     comp.check_status()
 
 
+@pytest.mark.parametrize("batch,hkv", [(74, 8), (75, 8), (593, 1)])
+def test_lists_of_many_heads(rkv, batch, hkv):  # noqa: F811
+    """592, 600 and 593 heads (four per SM on 148): above that a warp lists a head alone.  Two key tiles, a last block of the listing
+    that is not full, sequences without anything below their last tile."""
+    spec = small_spec("lists", batch=batch, hkv=hkv, hq=hkv, budget=150, buffer=42, span=4, copy_frac=0.2)
+    lens = [(192, 191, 151, 150)[b % 4] for b in range(batch)]
+    wl = ri.make_workload(spec, device="cuda", seed=408 + batch, seq_lens=torch.tensor(lens))
+    rep, comp = run_and_check(rkv, wl)
+    assert rep.ok(), rep.errors
+    comp.check_status()
+
+
 @pytest.mark.parametrize("batch,hkv,alpha,pool_w,beta", [(38, 8, 8, 4, 1), (37, 8, 8, 4, 3), (300, 1, 5, 2, 1)])
 def test_many_small_heads(rkv, batch, hkv, alpha, pool_w, beta):  # noqa: F811
     """304, 296 and 300 heads: the selection's blocks halve above two heads per SM (296 on 148 SMs).  n = 128, 127, 93, lists that
