@@ -83,7 +83,6 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
     auto bar = [bar0](int idx) -> uint32_t { return bar0 + 8u * (uint32_t)idx; };
 
     const ErrSink sink = make_sink(p);
-    pdl_trigger();
     pdl_wait();
     if (threadIdx.x == 0) *bail = (call_aborted(p) || *item_count == 0ull) ? 1 : 0;     // nothing listed for this route
     __syncthreads();
@@ -137,6 +136,7 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 mbar_arrive(bar(L::kBarQFull + qs));
                 ++k_item;
             }
+            pdl_trigger();                  // no item is left: the next kernel may be let in
             if (!*abort_flag) {             // terminator (skipped when the block is aborting)
                 const uint32_t qs = k_item % kItemSlotsD;
                 if (mbar_wait(bar(L::kBarQEmpty + qs), ((k_item / kItemSlotsD) & 1) ^ 1, abort_flag, sink)) {
@@ -391,6 +391,7 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 // the partner's similarity off its column sum, S = Kbar_i . Kbar_j, recomputed from the two key rows in fp32.
 constexpr int kFinishThreads = 256;
 
+template <int D>
 __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
 {
     // work unit = (head, chunk of 256 tokens), handed out with the grid as stride.  When no head took the route (the
@@ -411,11 +412,11 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
     const uint32_t b = p.best[hoff + i];
     if (b == 0u) continue;
     const int j = (int)b - 1;
-    const uint4 *ki = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, i) * p.d);
-    const uint4 *kj = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, j) * p.d);
+    const uint4 *ki = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, i) * D);
+    const uint4 *kj = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, j) * D);
     float dot = 0.f;
 #pragma unroll 4
-    for (int c = 0; c < p.d / 8; ++c) {
+    for (int c = 0; c < D / 8; ++c) {
         float a[8], bb[8];
         Elem<__nv_bfloat16>::unpack(__ldg(ki + c), a);
         Elem<__nv_bfloat16>::unpack(__ldg(kj + c), bb);
@@ -452,7 +453,9 @@ cudaError_t launch_dense_finish(const Params &p, cudaStream_t s)
     if (e != cudaSuccess) return e;
     const unsigned long long units = (unsigned long long)(p.batch * p.hkv) * (unsigned long long)((p.cap + kFinishThreads - 1) / kFinishThreads);
     const unsigned long long wave = 8ull * (unsigned long long)sms;             // resident blocks of this size
-    return launch_early(dense_finish_kernel, (unsigned)(units < wave ? units : wave), kFinishThreads, 0, s, 1, p);
+    const unsigned grid = (unsigned)(units < wave ? units : wave);
+    return p.d == 64 ? launch_early(dense_finish_kernel<64>, grid, kFinishThreads, 0, s, 1, p)
+                     : launch_early(dense_finish_kernel<128>, grid, kFinishThreads, 0, s, 1, p);
 }
 
 }  // namespace rkv

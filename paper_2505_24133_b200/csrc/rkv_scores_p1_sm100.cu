@@ -111,7 +111,6 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
 
     // Once a bounded wait of this call has run out, the blocks still to start return at once.
     const ErrSink sink = make_sink(p);
-    pdl_trigger();
     pdl_wait();
     if (threadIdx.x == 0) *bail = call_aborted(p) ? 1 : 0;
     __syncthreads();
@@ -213,6 +212,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 }
                 ++k_item;
             }
+            pdl_trigger();                  // no item is left: the next kernel may be let in
             // terminator: tells the other roles that no item follows (skipped when the block is aborting)
             if (!*abort_flag) {
                 const uint32_t slot = k_item & 1;

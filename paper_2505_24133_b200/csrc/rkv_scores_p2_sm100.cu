@@ -115,7 +115,6 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
     // invalid length does not stop the others: it just has no candidates).  Pass 2 has nothing to do when the list
     // is empty.
     const ErrSink sink = make_sink(p);
-    pdl_trigger();
     pdl_wait();
     if (threadIdx.x == 0) {
         int b = call_aborted(p) ? 1 : 0;
@@ -212,6 +211,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 mbar_arrive(bar.at(L::kBarQFull + qs));
                 ++k_item;
             }
+            pdl_trigger();                  // no item is left: the next kernel may be let in
             // terminator: tells the other roles that no item follows (skipped when the block is aborting)
             if (!*abort_flag) {
                 const uint32_t qs = k_item % kItemSlots;
