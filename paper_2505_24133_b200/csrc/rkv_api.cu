@@ -116,6 +116,14 @@ int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout 
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// What a compression asks of its descriptor and lambda beside the shapes and the tensors.
+int check_settings(const rkv_desc_t *d, float lambda)
+{
+    if (reinterpret_cast<uintptr_t>(d->budgets) & 3u) return RKV_ERR_INVALID_ARG;
+    if (!(lambda >= 0.f && lambda <= 1.f)) return RKV_ERR_INVALID_ARG;
+    return use_simt(d) || scores_sm100_available() ? RKV_OK : RKV_ERR_UNSUPPORTED;
+}
+
 int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window, int32_t *seq_lens, int budget,
         int buffer, int alpha, float lambda, int32_t *out_idx, void *stream, uint32_t stages)
 {
@@ -124,14 +132,12 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
     if (rc != RKV_OK) return rc;
     if (!k_cache || !v_cache || !q_window || !seq_lens || !out_idx) return RKV_ERR_INVALID_ARG;
     if (!aligned16(k_cache) || !aligned16(v_cache) || !aligned16(q_window)) return RKV_ERR_INVALID_ARG;
-    if ((reinterpret_cast<uintptr_t>(seq_lens) & 3u) || (reinterpret_cast<uintptr_t>(out_idx) & 3u) ||
-        (reinterpret_cast<uintptr_t>(d->budgets) & 3u))
-        return RKV_ERR_INVALID_ARG;
-    if (!(lambda >= 0.f && lambda <= 1.f)) return RKV_ERR_INVALID_ARG;
+    if ((reinterpret_cast<uintptr_t>(seq_lens) & 3u) || (reinterpret_cast<uintptr_t>(out_idx) & 3u)) return RKV_ERR_INVALID_ARG;
+    if ((rc = check_settings(d, lambda)) == RKV_ERR_INVALID_ARG) return rc;
     if ((stages & ~RKV_STAGE_ALL) != 0u || stages == 0u) return RKV_ERR_INVALID_ARG;
     if (!d->workspace || d->workspace_bytes < lay.total) return RKV_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(d->workspace) & 255u) return RKV_ERR_WORKSPACE;
-    if (!use_simt(d) && !scores_sm100_available()) return RKV_ERR_UNSUPPORTED;
+    if (rc != RKV_OK) return rc;
 
     Params p;
     memset(&p, 0, sizeof(p));
@@ -409,6 +415,7 @@ int rkv_compress_host(const rkv_desc_t *desc, void *host_k_cache, void *host_v_c
         return RKV_ERR_INVALID_ARG;      // (the host-buffer form takes contiguous caches only)
     if (!desc->workspace || desc->workspace_bytes < h.total) return RKV_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(desc->workspace) & 255u) return RKV_ERR_WORKSPACE;
+    if ((rc = check_settings(desc, lambda)) != RKV_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // Pieces of whole sequences: while one is compressed, the next comes in and the one before goes out (the link carries both
     // directions at once).  A copy costs about 5 us beside its bytes, so a piece has 16 MB or more, and the small arrays cross
@@ -481,7 +488,16 @@ int rkv_compress_host(const rkv_desc_t *desc, void *host_k_cache, void *host_v_c
         copy(host_out_idx, ws + h.idx, h.idx_bytes, cudaMemcpyDeviceToHost, down);
         link(3 * kMaxPieces + 1, down, s);
     }
-    if (pipe) pipe_pool().give(std::move(pipe));
+    if (pipe) {
+        // an error on the way: what is under way in the copy streams still reads and writes the caller's buffers and workspace,
+        // so the caller's stream waits for it as it does after a call that succeeds
+        if (rc != RKV_OK || e != cudaSuccess)
+            for (cudaStream_t x : {up, down})
+                if (cudaEventRecord(pipe->ev[3 * kMaxPieces + 1], x) != cudaSuccess ||
+                    cudaStreamWaitEvent(s, pipe->ev[3 * kMaxPieces + 1], 0) != cudaSuccess)
+                    cudaStreamSynchronize(x);
+        pipe_pool().give(std::move(pipe));
+    }
     return rc != RKV_OK ? rc : (e == cudaSuccess ? RKV_OK : cuda_fail(e, where));
 }
 

@@ -169,3 +169,17 @@ def test_eight_bit_cache_type_sizes_and_counts(rkv):
     assert rkv.rkv_workspace_bytes(_desc(rkv, dtype=3), 1024, 128, alpha) == 0
     assert rkv.rkv_decode_workspace_bytes(_desc(rkv, dtype=rkv.RKV_FP8_E4M3), 1024, 128) == \
         rkv.rkv_decode_workspace_bytes(_desc(rkv), 1024, 128) > 0       # the attention takes 8-bit caches like bf16 ones
+
+
+@pytest.mark.parametrize("case,want", [("lambda", 1), ("lambda_nan", 1), ("budgets", 1), ("no_workspace", 3)])
+def test_host_buffer_form_checks_everything_before_the_first_copy(rkv, case, want):
+    """A call of several pieces: what the compression of a piece would refuse is refused before any copy is enqueued (no CUDA call is
+    made, so this runs without a GPU, and the fake pointers are never read)."""
+    d = _desc(rkv, batch=16)
+    d.workspace, d.workspace_bytes = 0x10000, 1 << 40
+    lam = {"lambda": 2.0, "lambda_nan": float("nan")}.get(case, 0.1)
+    if case == "budgets":
+        d.budgets = 0x30002
+    elif case == "no_workspace":
+        d.workspace = None
+    assert rkv.rkv_compress_host(d, 0x20000, 0x20000, 0x20000, 0x30000, 1024, 128, 8, lam, 0x30000, 0) == want
