@@ -4,6 +4,7 @@
 #include <cstring>
 #include <memory>
 #include <mutex>
+#include <thread>
 
 #include "rkv_common.cuh"
 
@@ -281,13 +282,18 @@ int host_layout(const rkv_desc_t *d, int budget, int buffer, int alpha, HostLayo
 }
 
 // Two copy streams and the events between them and the caller's stream, for the host-buffer form.  A call takes one from the
-// pool while it enqueues and gives it back then; the next taker's copies queue up behind what is still in the streams.
-// Creating the two streams for each call took 250 us.
+// pool while it enqueues and gives it back then.  The next taker gets one whose work is done, or the one that its own stream
+// used last: behind another stream's copies a call would wait for work that it has no part in.  Creating the two streams
+// for each call took 250 us.
 constexpr int kMaxPieces = 8;
 struct HostPipe {
     int dev = -1;
     cudaStream_t up = nullptr, down = nullptr;
     cudaEvent_t ev[3 * kMaxPieces + 2] = {};
+    cudaStream_t user = nullptr;            // the stream of the call that used it last, and that call's thread (the handles of the
+    std::thread::id thread;                 // legacy and the per-thread default stream stand for a stream per thread)
+    bool last_used_by(cudaStream_t s) const { return user == s && thread == std::this_thread::get_id(); }
+    bool idle() const { return cudaStreamQuery(up) == cudaSuccess && cudaStreamQuery(down) == cudaSuccess; }
     bool open(int device)
     {
         dev = device;
@@ -307,19 +313,25 @@ struct HostPipe {
 };
 class PipePool {
 public:
-    std::unique_ptr<HostPipe> take(int dev)
+    std::unique_ptr<HostPipe> take(int dev, cudaStream_t s)
     {
-        {
-            std::lock_guard<std::mutex> guard(lock_);
-            for (auto &x : free_)
-                if (x && x->dev == dev) return std::move(x);
+        // (queries and new streams are no part of a capture that another thread may have under way)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        std::unique_ptr<HostPipe> x = find(dev, s);
+        if (!x) {
+            x.reset(new HostPipe);
+            if (!x->open(dev)) {
+                cudaGetLastError();         // (the call then goes through the caller's stream alone)
+                x.reset();
+            }
         }
-        std::unique_ptr<HostPipe> made(new HostPipe);
-        if (!made->open(dev)) {
-            cudaGetLastError();             // (the call then goes through the caller's stream alone)
-            made.reset();
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (x) {
+            x->user = s;
+            x->thread = std::this_thread::get_id();
         }
-        return made;
+        return x;
     }
     void give(std::unique_ptr<HostPipe> x)
     {
@@ -332,6 +344,15 @@ public:
     }                                       // (no slot left: destroyed when its work is done)
 
 private:
+    std::unique_ptr<HostPipe> find(int dev, cudaStream_t s)
+    {
+        std::lock_guard<std::mutex> guard(lock_);
+        for (auto &x : free_)
+            if (x && x->dev == dev && x->last_used_by(s)) return std::move(x);
+        for (auto &x : free_)
+            if (x && x->dev == dev && x->idle()) return std::move(x);
+        return nullptr;
+    }
     std::mutex lock_;
     std::unique_ptr<HostPipe> free_[16];
 };
@@ -428,7 +449,7 @@ int rkv_compress_host(const rkv_desc_t *desc, void *host_k_cache, void *host_v_c
     if (capturing != cudaStreamCaptureStatusNone || desc->stage_events || desc->kernel_events || desc->dbg_counters) pieces = 1;
     int dev = 0;
     std::unique_ptr<HostPipe> pipe;
-    if (pieces > 1 && cudaGetDevice(&dev) == cudaSuccess) pipe = pipe_pool().take(dev);
+    if (pieces > 1 && cudaGetDevice(&dev) == cudaSuccess) pipe = pipe_pool().take(dev, s);
     if (!pipe) pieces = 1;
     cudaStream_t up = pipe ? pipe->up : s, down = pipe ? pipe->down : s;
     cudaError_t e = cudaSuccess;

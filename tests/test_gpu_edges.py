@@ -159,6 +159,34 @@ def test_host_buffers_in_pieces(rkv, batch):  # noqa: F811
             assert torch.equal(hv[b, :, :n].view(torch.int16), wl.v_cache[b, :, :n].cpu().view(torch.int16))
 
 
+def test_host_buffers_on_independent_streams(rkv):  # noqa: F811
+    """A call in pieces on one stream does not wait for the copies of a call whose own stream is busy with something else."""
+    batch = 9                                            # 42 MB of caches: two pieces
+    spec = small_spec("streams", batch=batch, hkv=8, hq=16, budget=1024, buffer=128, span=32)
+    wl = ri.make_workload(spec, device="cuda", seed=433)
+    sets = []
+    for _ in range(3):
+        comp = rkv.Compressor(batch, 8, 16, spec.budget, spec.buffer, 8, 0.1, host_staging=True)
+        sets.append((comp, [t.cpu().pin_memory() for t in (wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens)],
+                     torch.empty(batch, 8, spec.budget, dtype=torch.int32).pin_memory()))
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    for (comp, host, hidx), stream in zip(sets, (a, a, b)):
+        with torch.cuda.stream(stream):
+            if comp is sets[1][0]:
+                torch.cuda._sleep(1_000_000_000)         # about half a second of the first stream, on which its second call waits
+            comp.compress_host(*host, hidx, stream)
+    b.synchronize()
+    assert not a.query()
+    a.synchronize()
+    want = sets[0]
+    for comp, host, hidx in sets:
+        comp.check_status()
+        assert torch.equal(hidx, want[2]) and torch.equal(host[3], want[1][3])
+        for x, y in zip(host[:2], want[1][:2]):
+            assert torch.equal(x[:, :, :spec.budget].view(torch.int16), y[:, :, :spec.budget].view(torch.int16))
+
+
 @pytest.mark.parametrize("head_dim,dtype", [(64, "fp8"), (64, "bf16"), (128, "bf16"), (256, "bf16"), (256, "f32")])
 @pytest.mark.parametrize("pattern", ["runs", "last_k", "sparse", "identity"])
 def test_compaction_by_bulk_copies(rkv, head_dim, dtype, pattern):  # noqa: F811
