@@ -212,6 +212,10 @@ __device__ __forceinline__ void widen16(const uint4 &codes, uint4 *lo, uint4 *hi
 // A kernel launched through launch_early() may become resident while its predecessor in the stream is still running: it
 // lets its own successor in (pdl_trigger) and waits for the predecessor's results (pdl_wait) before it touches global
 // memory.  Between the short kernels of a decode step the launch gap, 2-3 us, is most of the time.
+// Such a kernel is on the GPU while its inputs are still being written, so it reads them with ordinary loads: the read-only
+// path (__ldg) asks for data that nothing writes from the kernel's first block to its last.  The second pass, the symmetric
+// scan and its finish may use it for keys and norms: they are launched after a listing kernel, which is launched when
+// every block of the first pass is out of items, and the first pass waited for all that was written before it.
 // The persistent scoring kernels let it in when they are out of items: blocks that wait through a long kernel take from it (the
 // symmetric scan of 2048 heads of 4216 tokens, T = 0.9: 5105 us beside waiting blocks, 4764 without).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -309,14 +309,14 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                     ri = ri_next;
                     self = self_next;
                 } else {
-                    ri = row_ok ? __ldg(inv_norm + i) : 0.f;
-                    self = row_ok ? __ldg(self_dot + i) : 0.f;
+                    ri = row_ok ? inv_norm[i] : 0.f;
+                    self = row_ok ? self_dot[i] : 0.f;
                 }
                 if (t + 2 < d.z) {               // this group's next tile of the item: its factors arrive while this one is drained
                     const int i2 = i + 2 * kTile;
                     t_next = t + 2;
-                    ri_next = i2 < n ? __ldg(inv_norm + i2) : 0.f;
-                    self_next = i2 < n ? __ldg(self_dot + i2) : 0.f;
+                    ri_next = i2 < n ? inv_norm[i2] : 0.f;
+                    self_next = i2 < n ? self_dot[i2] : 0.f;
                 }
                 if (!mbar_wait(bar(kBarAccFull + grp), (ccount >> 1) & 1, abort_flag, sink)) {
                     ok = false;

@@ -46,7 +46,7 @@ __device__ __forceinline__ void load_rows(const T *src, int first_row, int valid
     for (int v = threadIdx.x; v < kRows * kVecPerRow; v += kSimtThreads) {
         const int r = v / kVecPerRow, c = (v % kVecPerRow) * kPerVec;
         uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-        if (first_row + r < valid_rows) raw = __ldg(reinterpret_cast<const uint4 *>(src + (size_t)r * D + c));
+        if (first_row + r < valid_rows) raw = *reinterpret_cast<const uint4 *>(src + (size_t)r * D + c);
         float f[kPerVec];
         Elem<T>::unpack(raw, f);
 #pragma unroll

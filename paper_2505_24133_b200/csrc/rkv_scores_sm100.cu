@@ -206,8 +206,15 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
         if (!is_q) {
             // inverse norms of the whole head and sum_j Kbar_j into shared memory
             const float *inv_norm = p.inv_norm + (size_t)head * p.cap_pad;
-            for (int v = et; v < n_tiles * (kTile / 4); v += 256)
-                reinterpret_cast<float4 *>(r_s)[v] = __ldg(reinterpret_cast<const float4 *>(inv_norm) + v);
+            for (int v0 = et; v0 < n_tiles * (kTile / 4); v0 += 4 * 256) {        // loads of four steps ahead of their stores
+                float4 r4[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (v0 + 256 * u < n_tiles * (kTile / 4)) r4[u] = reinterpret_cast<const float4 *>(inv_norm)[v0 + 256 * u];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (v0 + 256 * u < n_tiles * (kTile / 4)) reinterpret_cast<float4 *>(r_s)[v0 + 256 * u] = r4[u];
+            }
             if (et < kDim) {                 // the tile sums added up in tile order
                 const float *ts = p.tile_sum + (size_t)head * p.tiles * kDim + et;
                 float sum = 0.f;

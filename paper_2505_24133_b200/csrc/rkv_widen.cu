@@ -26,7 +26,6 @@ widen_keys_kernel(Params p, int key_blocks, __nv_bfloat16 *wide, int src_vecs, i
                   int q_rows)
 {
     pdl_trigger();
-    pdl_wait();
     if ((int)blockIdx.x >= key_blocks) {
         // queries: rows of src_q_vecs = dst_vecs / 2 vectors (bf16, 64 dimensions) -> rows of dst_vecs, zero-padded
         const int q_vecs = dst_vecs / 2;
@@ -77,8 +76,11 @@ cudaError_t launch_widen_keys(const Params &stored, __nv_bfloat16 *wide, int wid
     const unsigned key_blocks = keys ? (unsigned)stored.tiles * (unsigned)(stored.batch * stored.hkv) : 0u;
     const unsigned grid = key_blocks + (unsigned)((q_rows + kTile - 1) / kTile);
     if (grid == 0u) return cudaSuccess;
-    return launch_early(widen_keys_kernel, grid, kWidenThreads, 0, s, 1, stored, (int)key_blocks, wide, stored.store_row_bytes / 16,
-                        wide_d * 2 / 16, codes, static_cast<const uint4 *>(q_src), static_cast<uint4 *>(q_dst), q_rows);
+    // (not launched early: it reads the keys through the read-only path, and a kernel in front of it may still be appending to
+    // them.  With ordinary loads 1024 heads of 4123 tokens of 128 codes took 476-494 us instead of 457.)
+    widen_keys_kernel<<<grid, kWidenThreads, 0, s>>>(stored, (int)key_blocks, wide, stored.store_row_bytes / 16, wide_d * 2 / 16, codes,
+                                                     static_cast<const uint4 *>(q_src), static_cast<uint4 *>(q_dst), q_rows);
+    return cudaGetLastError();
 }
 
 }  // namespace rkv

@@ -183,3 +183,18 @@ def test_host_buffer_form_checks_everything_before_the_first_copy(rkv, case, wan
     elif case == "no_workspace":
         d.workspace = None
     assert rkv.rkv_compress_host(d, 0x20000, 0x20000, 0x20000, 0x30000, 1024, 128, 8, lam, 0x30000, 0) == want
+
+
+def test_early_launched_kernels_use_ordinary_loads():
+    """A kernel that may be on the GPU before its predecessors have written its inputs must not read them through the read-only data
+    path, which is defined for data that does not change during the kernel's whole lifetime.  Those of the second scoring pass
+    start only when the first has waited for all that they read that way."""
+    csrc = os.path.join(ROOT, "paper_2505_24133_b200", "csrc")
+    later = ("rkv_scores_p2_sm100.cu", "rkv_scores_dense_sm100.cu")
+    seen = 0
+    for f in sorted(os.listdir(csrc)):
+        text = re.sub(r"//.*", "", open(os.path.join(csrc, f)).read())
+        if "pdl_wait" in text and f not in later:
+            seen += 1
+            assert not re.search(r"__ldg\s*\(|ld\.global\.nc|__restrict__", text), f
+    assert seen >= 7
