@@ -102,7 +102,8 @@ def _load_fast(L) -> None:
         raw, device = (lambda _: _stream(None)), (lambda: 0)
     address = [ctypes.cast(f, ctypes.c_void_p).value for f in (L.rkv_push_query, L.rkv_append, L.rkv_decode_attention,
                                                                L.rkv_compress_stages)]
-    module.bind(*address, torch.cuda.is_initialized, device, raw, lambda: _stream(None))
+    module.bind(*address, torch.cuda.is_initialized, device, raw, lambda: _stream(None), RkvDesc,
+                ctypes.sizeof(RkvDesc))
     _fast = module
 
 
@@ -166,7 +167,7 @@ def rkv_compress_stages(desc, k_cache, v_cache, q_window, seq_lens, budget, buff
                         stream=None, stage_mask: int = RKV_STAGE_ALL) -> int:
     if _fast is None:
         lib()
-    return _fast.compress_stages(desc, k_cache, v_cache, q_window, seq_lens, budget, buffer, alpha, lam, out_idx, stream,
+    return _fast.compress_stages(desc, k_cache, v_cache, q_window, seq_lens, budget, buffer, alpha, float(lam), out_idx, stream,
                                  stage_mask)
 
 

@@ -22,6 +22,8 @@ static PyObject *g_device, *g_raw_stream;    /* current device; its current stre
 static PyObject *g_slow_stream;              /* the binding's own answer, asked until CUDA is initialised */
 static PyObject *g_initialised;
 static int g_ready;
+static PyObject *g_desc_type;                /* the binding's descriptor structure, and its size */
+static Py_ssize_t g_desc_size;
 static PyObject *s_contiguous, *s_data_ptr, *s_cuda_stream;
 
 static int get_ptr(PyObject *o, void **out)
@@ -96,8 +98,21 @@ static int get_int(PyObject *o, int32_t *out)
     return PyErr_Occurred() ? -1 : 0;
 }
 
-/* the descriptor (a ctypes structure) stays where it is while `view` is held */
-static int get_desc(PyObject *o, Py_buffer *view) { return PyObject_GetBuffer(o, view, PyBUF_SIMPLE); }
+/* the descriptor (a ctypes structure of the binding's type, nothing else that has bytes) stays where it is while `view` is held */
+static int get_desc(PyObject *o, Py_buffer *view)
+{
+    const int is = PyObject_IsInstance(o, g_desc_type);
+    if (is < 0) return -1;
+    if (!is) {
+        PyErr_Format(PyExc_TypeError, "expected an RkvDesc, got %s", Py_TYPE(o)->tp_name);
+        return -1;
+    }
+    if (PyObject_GetBuffer(o, view, PyBUF_SIMPLE)) return -1;
+    if (view->len >= g_desc_size) return 0;
+    PyBuffer_Release(view);
+    PyErr_SetString(PyExc_TypeError, "the descriptor is too small");
+    return -1;
+}
 
 static int want(Py_ssize_t n, Py_ssize_t expected)
 {
@@ -173,12 +188,12 @@ static PyObject *compress_stages(PyObject *self, PyObject *const *a, Py_ssize_t 
 }
 
 /* (addresses of rkv_push_query, rkv_append, rkv_decode_attention, rkv_compress_stages; is_initialised, current_device,
- *  raw_stream(device), slow_stream) */
+ *  raw_stream(device), slow_stream; the descriptor's type and size) */
 static PyObject *bind(PyObject *self, PyObject *args)
 {
     unsigned long long f[4];
-    PyObject *o[4];
-    if (!PyArg_ParseTuple(args, "KKKKOOOO", &f[0], &f[1], &f[2], &f[3], &o[0], &o[1], &o[2], &o[3])) return NULL;
+    PyObject *o[5];
+    if (!PyArg_ParseTuple(args, "KKKKOOOOOn", &f[0], &f[1], &f[2], &f[3], &o[0], &o[1], &o[2], &o[3], &o[4], &g_desc_size)) return NULL;
     g_push = (push_fn)(uintptr_t)f[0];
     g_append = (append_fn)(uintptr_t)f[1];
     g_attend = (attend_fn)(uintptr_t)f[2];
@@ -187,6 +202,7 @@ static PyObject *bind(PyObject *self, PyObject *args)
     Py_XSETREF(g_device, Py_NewRef(o[1]));
     Py_XSETREF(g_raw_stream, Py_NewRef(o[2]));
     Py_XSETREF(g_slow_stream, Py_NewRef(o[3]));
+    Py_XSETREF(g_desc_type, Py_NewRef(o[4]));
     Py_RETURN_NONE;
 }
 

@@ -198,3 +198,28 @@ def test_early_launched_kernels_use_ordinary_loads():
             seen += 1
             assert not re.search(r"__ldg\s*\(|ld\.global\.nc|__restrict__", text), f
     assert seen >= 7
+
+
+@pytest.mark.parametrize("bad", [b"\x02\x00\x00\x00", bytearray(4096), None, 7, (ctypes.c_char * 4)()])
+def test_only_a_descriptor_is_taken_as_one(rkv, bad):
+    """The calls marshalled in C read the descriptor's fields from its memory: any other object is refused, however many bytes it has."""
+    calls = [lambda d: rkv.rkv_compress_stages(d, None, None, None, None, 64, 32, 8, 0.1, None, 0),
+             lambda d: rkv.rkv_append(d, None, None, None, None, None, 64, 32, 0),
+             lambda d: rkv.rkv_push_query(d, None, None, 8, 0, 0),
+             lambda d: rkv.rkv_decode_attention(d, None, None, None, None, None, 64, 32, 0)]
+    for call in calls:
+        with pytest.raises(TypeError):
+            call(bad)
+        assert call(_desc(rkv)) in (1, 3)                  # null tensors
+
+
+def test_arguments_are_taken_as_before(rkv):
+    """Integers are what Python takes as an index, lambda is whatever float() takes."""
+    import numpy as np
+    d = _desc(rkv)
+    assert rkv.rkv_append(d, None, None, None, None, None, np.int64(64), 32, 0) == 1
+    for bad in (64.0, "64", None):
+        with pytest.raises((TypeError, ctypes.ArgumentError)):
+            rkv.rkv_append(d, None, None, None, None, None, bad, 32, 0)
+    for lam in (0, 1, "0.5", np.float32(0.1)):
+        assert rkv.rkv_compress_stages(d, None, None, None, None, 64, 32, 8, lam, None, 0) == 1
