@@ -8,13 +8,14 @@ from __future__ import annotations
 import ctypes
 import importlib.util
 import os
+import sysconfig
 from typing import Optional, Sequence
 
 import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_PKG, "librkv_b200.so")
-_CALL_PATH = os.path.join(_PKG, "_rkv_call.so")
+_CALL_PATH = os.path.join(_PKG, "_rkv_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 _lib = None
 _fast = None        # the calls made per layer and step, marshalled in C (csrc/pycall.c)
 

@@ -11,7 +11,8 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "librkv_b200.so")
-CALL = os.path.join(PKG, "_rkv_call.so")            # argument marshalling of the per-layer calls
+# argument marshalling of the per-layer calls; built against one interpreter's C API, so the file is that interpreter's
+CALL = os.path.join(PKG, "_rkv_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-shared",

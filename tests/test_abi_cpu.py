@@ -223,3 +223,11 @@ def test_arguments_are_taken_as_before(rkv):
             rkv.rkv_append(d, None, None, None, None, None, bad, 32, 0)
     for lam in (0, 1, "0.5", np.float32(0.1)):
         assert rkv.rkv_compress_stages(d, None, None, None, None, 64, 32, 8, lam, None, 0) == 1
+
+
+def test_marshalling_module_belongs_to_this_interpreter(rkv):
+    """It uses an interpreter's full C API: one built for another interpreter must not be picked up under the same name."""
+    import sysconfig
+    from paper_2505_24133_b200 import binding, build
+    assert build.CALL == binding._CALL_PATH and os.path.exists(build.CALL)
+    assert build.CALL.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
