@@ -47,7 +47,7 @@ struct Params {
     int mean_then_pool;             // importance in Algorithm 1's order (mean over query rows, then pooling)
     float sim_threshold, eps, lambda;
     // workspace carve-up
-    float *inv_norm;     // [P][cap_pad]         r_i = 1 / (||k_i|| + eps); 0 for i >= n
+    float *inv_norm;     // [P][cap_pad]         r_i = 1 / (||k_i|| + eps); 0 for i >= n; kGaveUp first in a tile: not finished
     __nv_bfloat16 *norm_split;    // [P][cap_pad][8]   (n1, n2, n3, n1, n2, n1, 0, 0): 1 / r_i as three bf16 parts, laid
                                   // out (zeros up to 16 are added on the way) as the extra K = 16 slice the scoring passes append to a key row
     __nv_bfloat16 *thr_split;     // [P][128][8]       (-t1, -t1, -t1, -t2, -t2, -t3, 0, 0): -T / r_j of the keys of the
@@ -136,6 +136,10 @@ __device__ __forceinline__ bool call_aborted(const Params &p)
 {
     return *reinterpret_cast<volatile unsigned long long *>(p.counters + kAbortWord) != 0ull;
 }
+
+// What a prep block that gave up on a wait leaves as the first r of the tiles it has not finished (an r is never negative).
+constexpr float kGaveUp = -1.f;
+__device__ __forceinline__ bool prep_gave_up(float r) { return r < 0.f; }
 
 // Number of candidates of a sequence of length L with the given budget: 0 = nothing to compress.
 __device__ __forceinline__ int candidates_from_meta(int L, int budget, int alpha)

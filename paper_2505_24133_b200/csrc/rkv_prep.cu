@@ -5,8 +5,10 @@
 // scoring stage obtain sum_j S[j][i] = Kbar_i . (sum_j Kbar_j) - Kbar_i . Kbar_i (Eq. 6 before the
 // retention rule) without accumulating the n x n matrix element by element.
 // Rows i >= n (observation tokens, unused capacity) get r_i = 0 and contribute nothing.
-// The call's counters start at zero: the first block clears them (a memset in front of this kernel cost a small call 3 us;
-// the first of a block's waits could record that it ran out many microseconds later at the earliest).
+// The call's counters start at zero: the first block clears them (a memset in front of this kernel cost a small call 3 us).
+// The abort word is among them, so no block of these kernels sets it: nothing would order that against the first block's
+// store.  A block that gives up on a wait leaves kGaveUp as the first r of every tile that it has not finished instead, and
+// the kernel that reads the norms next (head_sum_kernel, the CUDA-core kernel, the row-block kernel) records the abort.
 // Kbar_i . Kbar_i is kept per row as well (self_dot).
 //
 // HBM-bound: each block brings its tile of K into shared memory with one bulk copy (cp.async.bulk, bounded wait
@@ -25,6 +27,18 @@ __device__ __forceinline__ void clear_counters(const Params &p)
     if (blockIdx.x == 0 && threadIdx.x < kCounterWords) p.counters[threadIdx.x] = 0ull;
 }
 
+// Where the waits of the prep kernels record that they ran out: the caller's status, but not the abort word (see above).
+__device__ __forceinline__ ErrSink prep_sink(const Params &p) { return ErrSink{p.status, nullptr, p.wait_cycles}; }
+
+// Error path: one thread waits for what its block still has under way before the block's memory is given up, however short the
+// caller's own limit is.
+__device__ __forceinline__ void drain(uint32_t bar, uint32_t parity)
+{
+    const long long start = clock64();
+    while (!sm100::mbar_try_wait_asleep(bar, parity))
+        if (clock64() - start > sm100::kWaitCycles) return;
+}
+
 constexpr int kPrepThreads = 256;
 constexpr int kPrepWarps = kPrepThreads / 32;
 
@@ -35,7 +49,7 @@ __global__ void __launch_bounds__(kPrepThreads, D <= 128 ? 5 : 2) prep_kernel(Pa
     extern __shared__ __align__(128) uint8_t prep_smem[];       // the tile's candidate rows, then one mbarrier
     constexpr int kTileBytesT = kTile * D * (int)sizeof(T);
     __shared__ int abort_flag;
-    const ErrSink sink = make_sink(p);
+    const ErrSink sink = prep_sink(p);
     pdl_trigger();
     pdl_wait();
     clear_counters(p);
@@ -91,7 +105,10 @@ __global__ void __launch_bounds__(kPrepThreads, D <= 128 ? 5 : 2) prep_kernel(Pa
     __syncthreads();
     const bool landed = rows_here == 0 || mbar_wait(bar, 0, &abort_flag, sink);
     if (!__syncthreads_and(landed)) {      // the block leaves as a whole, or not at all
-        __nanosleep(200000);               // error path only: let the copy land before the block's memory is reused
+        if (threadIdx.x == 0) {
+            inv_norm[tile * kTile] = kGaveUp;
+            drain(bar, 0);
+        }
         return;
     }
     const uint4 *tile_s = reinterpret_cast<const uint4 *>(prep_smem);
@@ -283,7 +300,7 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
     __shared__ __align__(8) unsigned long long bars[kPrepTcBufs + 1];      // tile landed (per buffer); product done
     __shared__ uint32_t tmem_holder;
     __shared__ int abort_flag;
-    const ErrSink sink = make_sink(p);
+    const ErrSink sink = prep_sink(p);
     const int t = threadIdx.x, warp = t >> 5;
     const uint32_t bar_tile0 = smem_u32(&bars[0]), bar_mma = smem_u32(&bars[kPrepTcBufs]);
 
@@ -331,8 +348,8 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
     if (t == 0)
         for (int q = 0; q < kPrepTcBufs - 1; ++q) issue_copy(q);
 
-    int k = 0;
-    for (int idx = (int)blockIdx.x; idx < total; idx += (int)gridDim.x, ++k) {
+    int k = 0, idx = (int)blockIdx.x;
+    for (; idx < total; idx += (int)gridDim.x, ++k) {
         const PrepUnit w = prep_unit_at<kSub>(p, idx, t == 0 && !p.lengths_done);
         const int head = w.head, n = w.n, rows_here = w.rows_here;
         const int buf = k % kPrepTcBufs;
@@ -472,10 +489,18 @@ __global__ void __launch_bounds__(kPrepTcThreads, kPrepTcBlocks) prep_tc_kernel(
         if (!done) break;
     }
 
+    if (t == 0 && idx < total) {            // error path: units from this one on are given up
+        for (int e = k; e < k + kPrepTcBufs; ++e)
+            if ((long long)blockIdx.x + (long long)e * gridDim.x < total) drain(bar_tile0 + 8u * (e % kPrepTcBufs), (uint32_t)(e / kPrepTcBufs) & 1u);
+        drain(bar_mma, mma_parity ^ 1u);
+        for (; idx < total; idx += (int)gridDim.x) {
+            const PrepUnit w = prep_unit_at<kSub>(p, idx, !p.lengths_done);
+            for (int u = 0; u < kSub && w.tile + u < p.tiles; ++u) p.inv_norm[(size_t)w.head * p.cap_pad + (w.tile + u) * kTile] = kGaveUp;
+        }
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
-        if (abort_flag) __nanosleep(200000);       // error path only: let the copies in flight land
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kPrepTcTmemCols) : "memory");
     }
@@ -508,7 +533,7 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
     __shared__ __align__(8) unsigned long long bars[3];      // stored tile landed (per stage); product done
     __shared__ uint32_t tmem_holder;
     __shared__ int abort_flag;
-    const ErrSink sink = make_sink(p);
+    const ErrSink sink = prep_sink(p);
     const int t = threadIdx.x, warp = t >> 5;
     const uint32_t bar_raw0 = smem_u32(&bars[0]), bar_mma = smem_u32(&bars[2]);
 
@@ -551,8 +576,8 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
     clear_counters(p);
     if (t == 0) issue_copy(0);
 
-    int k = 0;
-    for (int idx = (int)blockIdx.x; idx < total; idx += (int)gridDim.x, ++k) {
+    int k = 0, idx = (int)blockIdx.x;
+    for (; idx < total; idx += (int)gridDim.x, ++k) {
         const PrepUnit w = prep_unit_at<1>(p, idx, t == 0);
         const int head = w.head, tile = w.tile, n = w.n, rows_here = w.rows_here;
         const int buf = k & 1;
@@ -692,10 +717,18 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
     }
 
     if (t == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");      // the stores are through before the block leaves
+    if (t == 0 && idx < total) {            // error path: tiles from this one on are given up
+        for (int e = k; e < k + 2; ++e)
+            if ((long long)blockIdx.x + (long long)e * gridDim.x < total) drain(bar_raw0 + 8u * (e & 1), (uint32_t)(e >> 1) & 1u);
+        drain(bar_mma, mma_parity ^ 1u);
+        for (; idx < total; idx += (int)gridDim.x) {
+            const PrepUnit w = prep_unit_at<1>(p, idx, true);
+            p.inv_norm[(size_t)w.head * p.cap_pad + w.tile * kTile] = kGaveUp;
+        }
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
-        if (abort_flag) __nanosleep(200000);       // error path only: let the copies in flight land
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kPrepTcTmemCols) : "memory");
     }
@@ -704,12 +737,13 @@ prep_fused_kernel(Params p, const __grid_constant__ CUtensorMap map_src, const _
 // The tile sums of a head added up in tile order (a launch of its own behind prep_tc_kernel: no tickets, no fences in
 // the streaming kernel), also as three bf16 rows whose sum is s to fp32 accuracy (rows 3..15 of the 16-row block are
 // zero): appended to the query rows, they let the tensor cores form Kbar_i . s along with the logits.
-template <int D>
+template <int D>                             // (D >= 64, the most tiles that a head can have)
 __global__ void __launch_bounds__(D) head_sum_kernel(Params p)
 {
     pdl_trigger();
     pdl_wait();
     const int head = blockIdx.x, t = threadIdx.x;
+    const float first_r = t < p.tiles ? p.inv_norm[(size_t)head * p.cap_pad + t * kTile] : 0.f;
     const float *ts = p.tile_sum + (size_t)head * p.tiles * D + t;
     float s = 0.f;
     for (int q = 0; q < p.tiles; ++q) s += ts[(size_t)q * D];
@@ -722,6 +756,7 @@ __global__ void __launch_bounds__(D) head_sum_kernel(Params p)
         rest -= __bfloat162float(h16);
     }
     for (int z = 3; z < 16; ++z) hs[z * D] = __float2bfloat16_rn(0.f);
+    if (prep_gave_up(first_r)) report_timeout(make_sink(p));
 }
 
 }  // namespace

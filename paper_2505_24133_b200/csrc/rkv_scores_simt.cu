@@ -127,7 +127,11 @@ __global__ void __launch_bounds__(kSimtThreads, D <= 128 ? 3 : 2) scores_simt_ke
         for (int j0 = (n - 1) / kCols * kCols; j0 >= 0; j0 -= kCols) {          // descending j: "largest positions first"
             __syncthreads();
             load_rows<T, D, kCols>(key_rows(j0), j0, n, tileB);
-            if (t < kCols) rB[t] = j0 + t < n ? inv_norm[j0 + t] : 0.f;
+            if (t < kCols) {
+                const float r = j0 + t < n ? inv_norm[j0 + t] : 0.f;
+                if (prep_gave_up(r)) report_timeout(make_sink(p));
+                rB[t] = r;
+            }
             __syncthreads();
             float s[kRowsT][kC];
             tile_product<D, kRowsT>(tileA, tileB, s);

@@ -212,8 +212,11 @@ scores_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const _
                 for (int u = 0; u < 4; ++u)
                     if (v0 + 256 * u < n_tiles * (kTile / 4)) r4[u] = reinterpret_cast<const float4 *>(inv_norm)[v0 + 256 * u];
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (v0 + 256 * u < n_tiles * (kTile / 4)) reinterpret_cast<float4 *>(r_s)[v0 + 256 * u] = r4[u];
+                for (int u = 0; u < 4; ++u) {
+                    if (v0 + 256 * u >= n_tiles * (kTile / 4)) break;
+                    if (prep_gave_up(r4[u].x)) report_timeout(sink);
+                    reinterpret_cast<float4 *>(r_s)[v0 + 256 * u] = r4[u];
+                }
             }
             if (et < kDim) {                 // the tile sums added up in tile order
                 const float *ts = p.tile_sum + (size_t)head * p.tiles * kDim + et;

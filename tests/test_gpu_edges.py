@@ -227,3 +227,22 @@ def test_compaction_by_bulk_copies(rkv, head_dim, dtype, pattern):  # noqa: F811
     assert torch.equal(u8(wl.k_cache)[:, :, :budget], k0.gather(2, take))
     assert torch.equal(u8(wl.v_cache)[:, :, :budget], v0.gather(2, take))
     assert wl.seq_lens.tolist() == [min(int(x), budget) for x in lens]
+
+
+@pytest.mark.parametrize("dtype,head_dim,tile", [("f32", 128, 0), ("f32", 64, 2), ("bf16", 256, 0), ("bf16", 256, 2)])
+def test_norms_of_a_tile_given_up_abort_the_call(rkv, dtype, head_dim, tile):  # noqa: F811
+    """What a prep block that gave up leaves behind (-1 as the first norm of a tile), put there by hand between the stages: the
+    scoring kernel records the abort."""
+    spec = small_spec("mark", batch=3, hkv=2, hq=4, budget=300, buffer=84, head_dim=head_dim, dtype=dtype, span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=453)
+    k0, s0 = wl.k_cache.clone(), wl.seq_lens.clone()
+    comp = rkv.Compressor(3, 2, 4, spec.budget, spec.buffer, spec.alpha, 0.1, dtype=spec.torch_dtype, head_dim=head_dim)
+    comp.compress(wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens, stages=rkv.RKV_STAGE_PREP)
+    norms = comp.workspace[:6 * 384 * 4].view(torch.float32).view(6, 384)       # no copy of the keys: they come first
+    assert bool((norms[:, :300] > 0).all())
+    norms[4, 128 * tile] = -1.0
+    rest = rkv.RKV_STAGE_SCORES | rkv.RKV_STAGE_SELECT | rkv.RKV_STAGE_GATHER
+    comp.compress(wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens, stages=rest)
+    torch.cuda.synchronize()
+    assert int(comp.status.item()) == 5
+    assert torch.equal(wl.k_cache, k0) and torch.equal(wl.seq_lens, s0) and bool((comp.out_idx == -1).all())
