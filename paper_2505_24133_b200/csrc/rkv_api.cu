@@ -559,7 +559,7 @@ static int attend_plan(const rkv_desc_t *d, int32_t budget, int32_t buffer, int 
     if (device_sms(&dev, &sms) != cudaSuccess)
         sms = 148;       // sizing only (no device here): the B200's count
     *splits = attend_splits(d->batch * d->n_kv_heads, budget + buffer, sms, G, d->dtype);
-    *bytes = attend_partial_bytes(d->batch * d->n_kv_heads, *splits, G);
+    *bytes = attend_workspace_bytes(d->batch * d->n_kv_heads, budget + buffer, sms, G, d->dtype);
     return RKV_OK;
 }
 

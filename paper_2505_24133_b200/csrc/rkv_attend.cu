@@ -365,8 +365,9 @@ int attend_splits(int heads, int cap, int sms, int G, int dtype)
     return splits > tiles ? tiles : splits;
 }
 
-size_t attend_partial_bytes(int heads, int splits, int G)
+size_t attend_workspace_bytes(int heads, int cap, int sms, int G, int dtype)
 {
+    const int splits = attend_uses_tc(G, dtype) ? attend_tc_workspace_splits(heads, cap, sms) : attend_splits(heads, cap, sms, G, dtype);
     return splits > 1 ? (size_t)heads * splits * G * (kHeadDim + 2) * sizeof(float) : 0;
 }
 

@@ -487,6 +487,17 @@ int attend_tc_splits(int heads, int cap, int sms)
     return best;
 }
 
+// Splits that the size of the workspace is counted by: the fewest that give two waves of resident blocks.  The clusters need none
+// of it; the size has always been this, and callers that needed no workspace still need none.
+int attend_tc_workspace_splits(int heads, int cap, int sms)
+{
+    const int tiles = (cap + kTile - 1) / kTile;
+    int splits = (4 * sms + heads - 1) / heads;
+    const int least = (tiles + kTcMaxTiles - 1) / kTcMaxTiles;
+    splits = splits < least ? least : splits;
+    return splits > tiles ? tiles : splits;
+}
+
 cudaError_t launch_attend_tc(const void *k_cache, const void *v_cache, const void *q_new, const int32_t *seq_lens, float *out,
                              int batch, int hkv, int hq, int cap, int splits, int32_t *status, long long wait_cycles,
                              const int32_t *block_table, long long pool_pages, int src, cudaStream_t s)

@@ -294,7 +294,8 @@ int attend_tc_splits(int heads, int cap, int sms);
 int attend_max_group();
 int attend_splits(int heads, int cap, int sms, int G, int dtype);
 bool attend_supported(int G, int dtype, int head_dim);
-size_t attend_partial_bytes(int heads, int splits, int G);
+int attend_tc_workspace_splits(int heads, int cap, int sms);
+size_t attend_workspace_bytes(int heads, int cap, int sms, int G, int dtype);      // for the partial results of the splits
 bool scores_sm100_available();
 long long sm100_default_wait_cycles();          // default limit of the kernels' bounded waits (about two seconds)
 bool scores_dense_possible(int tiles, int beta);   // the symmetric route of the second pass may be taken (two more launches)

@@ -231,3 +231,17 @@ def test_marshalling_module_belongs_to_this_interpreter(rkv):
     from paper_2505_24133_b200 import binding, build
     assert build.CALL == binding._CALL_PATH and os.path.exists(build.CALL)
     assert build.CALL.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+@pytest.mark.parametrize("dtype,head_dim", [("RKV_BF16", 128), ("RKV_FP8_E4M3", 128), ("RKV_BF16", 64)])
+def test_decode_attention_workspace_depends_on_the_shape_alone(rkv, dtype, head_dim):
+    """What the tensor-core attention asks for (on 148 SMs): nothing where the heads give two waves of blocks by themselves and a block
+    holds a head's scores (15 key tiles), whatever split the kernel takes; otherwise the partial results of the fewest splits
+    that give two waves."""
+    for heads in (1, 8, 100, 128, 300, 591, 592, 600, 800, 1024, 4096):
+        for tiles in (1, 2, 9, 13, 15, 16, 33, 64):
+            for group in (1, 4, 8):
+                d = _desc(rkv, batch=heads, n_kv_heads=1, n_q_heads=group, head_dim=head_dim, dtype=getattr(rkv, dtype))
+                splits = min(max(-(-4 * 148 // heads), -(-tiles // 15)), tiles)
+                want = heads * splits * group * 130 * 4 if splits > 1 else 0
+                assert rkv.rkv_decode_workspace_bytes(d, 128 * tiles - 20, 20) == want, (heads, tiles, group)
