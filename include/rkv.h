@@ -166,7 +166,8 @@ typedef struct rkv_desc {
 /* Fill *desc with the defaults above (pool_w 4, beta 1, T 0.5, eps 1e-8, head_dim 128, bf16), zero elsewhere. */
 RKV_API void rkv_desc_default(rkv_desc_t *desc);
 
-/* Bytes of device scratch a call with this descriptor and these sizes needs (0 if the arguments are invalid). */
+/* Bytes of device scratch that serve a compression and the decode attention of this descriptor and these sizes (0 if the
+ * arguments are invalid). */
 RKV_API size_t rkv_workspace_bytes(const rkv_desc_t *desc, int32_t budget, int32_t buffer, int32_t alpha);
 
 /* Install *desc (copied) as the calling thread's current descriptor, used by rkv_compress(). */
@@ -239,8 +240,8 @@ RKV_API int rkv_compress_host(const rkv_desc_t *desc, void *host_k_cache, void *
  *
  * Arguments, layouts, results and error codes are those of rkv_compress_ex; desc->workspace and
  * desc->workspace_bytes are ignored.  In addition:
- *   - a shape whose rkv_workspace_bytes() exceeds RKV_STATIC_SCRATCH_BYTES is refused with RKV_ERR_WORKSPACE
- *     before anything is launched (rkv_workspace_bytes() tells what a shape needs).  32 MiB covers, for example,
+ *   - a shape whose compression needs more than RKV_STATIC_SCRATCH_BYTES (rkv_workspace_bytes() where the decode
+ *     attention does not need more) is refused with RKV_ERR_WORKSPACE before anything is launched.  32 MiB covers, for example,
  *     256 head-problems at budget 1024 + buffer 128 (all 32 layers of an 8-KV-head model, batch 1);
  *     larger batches are split into several calls over sub-ranges of the batch dimension, one after the other.
  *   - the call makes no cudaMalloc / cudaFree and calls no allocating library routine.

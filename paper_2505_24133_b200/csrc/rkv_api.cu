@@ -1,5 +1,6 @@
 // C ABI of the R-KV compression library: argument checks, workspace carve-up, stage launches.
 // See include/rkv.h for the contract of every entry point.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <memory>
@@ -363,6 +364,13 @@ PipePool &pipe_pool()
 }
 
 }  // namespace
+
+size_t compression_bytes(const rkv_desc_t *d, int budget, int buffer, int alpha)
+{
+    Layout lay;
+    return check_shapes(d, budget, buffer, alpha, &lay) == RKV_OK ? lay.total : 0;
+}
+
 }  // namespace rkv
 
 using namespace rkv;
@@ -383,8 +391,10 @@ void rkv_desc_default(rkv_desc_t *desc)
 
 size_t rkv_workspace_bytes(const rkv_desc_t *desc, int32_t budget, int32_t buffer, int32_t alpha)
 {
-    Layout lay;
-    return check_shapes(desc, budget, buffer, alpha, &lay) == RKV_OK ? lay.total : 0;
+    // (one workspace serves a compression and the decode attention of its shape: with fp32 caches and large query groups the latter
+    // may need more)
+    const size_t scoring = compression_bytes(desc, budget, buffer, alpha);
+    return scoring ? std::max(scoring, rkv_decode_workspace_bytes(desc, budget, buffer)) : 0;
 }
 
 int rkv_set_desc(const rkv_desc_t *desc)

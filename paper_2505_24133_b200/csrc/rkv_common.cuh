@@ -271,6 +271,8 @@ inline cudaError_t allow_smem_once(std::atomic<unsigned long long> &done, int de
     return e;
 }
 
+size_t compression_bytes(const rkv_desc_t *d, int budget, int buffer, int alpha);     // scratch of a compression alone; 0: invalid
+
 // launchers (one per stage); each returns cudaGetLastError() of its launch
 cudaError_t launch_prep(const Params &p, cudaStream_t s);
 cudaError_t launch_widen_keys(const Params &stored, __nv_bfloat16 *wide, int wide_d, const void *q_src, void *q_dst,

@@ -57,7 +57,7 @@ int rkv_compress_static(const rkv_desc_t *desc, void *k_cache, void *v_cache, co
 {
     if (!desc) return RKV_ERR_INVALID_ARG;
     // size check first: a shape that does not fit is refused without touching the device
-    const size_t need = rkv_workspace_bytes(desc, budget, buffer, alpha);
+    const size_t need = compression_bytes(desc, budget, buffer, alpha);
     if (need == 0) {
         // bad shape: the ordinary argument checks name the problem (invalid or unsupported) before any launch
         rkv_desc_t probe = *desc;

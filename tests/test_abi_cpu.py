@@ -245,3 +245,17 @@ def test_decode_attention_workspace_depends_on_the_shape_alone(rkv, dtype, head_
                 splits = min(max(-(-4 * 148 // heads), -(-tiles // 15)), tiles)
                 want = heads * splits * group * 130 * 4 if splits > 1 else 0
                 assert rkv.rkv_decode_workspace_bytes(d, 128 * tiles - 20, 20) == want, (heads, tiles, group)
+
+
+def test_one_workspace_serves_the_compression_and_the_attention(rkv):
+    """rkv_workspace_bytes() covers rkv_decode_workspace_bytes() for every shape (fp32 caches, large groups and few query rows are
+    the shapes where the attention's partial results are the larger part)."""
+    for dtype in (rkv.RKV_BF16, rkv.RKV_F32, rkv.RKV_FP8_E4M3):
+        for batch, hkv in ((1, 1), (1, 4), (2, 1), (3, 8), (16, 2), (32, 2), (75, 8), (128, 4)):
+            for group in (1, 4, 5, 7, 8):
+                for budget, buffer in ((5, 512), (100, 28), (1024, 32), (2048, 32), (4096, 128), (7600, 512)):
+                    for alpha in (1, 4, 8):
+                        if alpha >= budget:
+                            continue
+                        d = _desc(rkv, batch=batch, n_kv_heads=hkv, n_q_heads=hkv * group, dtype=dtype)
+                        assert rkv.rkv_workspace_bytes(d, budget, buffer, alpha) >= rkv.rkv_decode_workspace_bytes(d, budget, buffer)
