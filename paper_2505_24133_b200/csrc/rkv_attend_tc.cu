@@ -404,7 +404,8 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
             } else {
                 part[g * kStride + r] = num;
                 if (r == 0) {
-                    part[g * kStride + kHeadDim] = ok ? m[g] : -INFINITY;
+                    // -inf stands for a split without rows; one whose scores are all NaN (or -inf: the sum is NaN too) takes part
+                    part[g * kStride + kHeadDim] = !ok ? -INFINITY : m[g] == -INFINITY ? 0.f : m[g];
                     part[g * kStride + kHeadDim + 1] = den;
                 }
             }

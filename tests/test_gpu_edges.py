@@ -105,6 +105,28 @@ def test_decode_attention_splits(rkv, batch, hkv, hq, cap):  # noqa: F811
     assert (np.abs(got - ref) <= 1e-3 * scale + 1e-7).all(), float((np.abs(got - ref) / scale).max())
 
 
+@pytest.mark.parametrize("cap,nan_rows", [(1920, (0, 128)), (1920, (0, 1920)), (1920, (1152, 1280)), (1280, (5, 6))])
+def test_decode_attention_over_nan_keys(rkv, cap, nan_rows):  # noqa: F811
+    """Keys of NaN give the output row that they give when one block holds the head (zeros: no sum of weights), also when they are
+    all that a block of the cluster holds; a sequence without any is not touched by them."""
+    batch, hkv, hq = 2, 1, 4
+    g = torch.Generator(device="cuda").manual_seed(9)
+    k, v = (torch.randn(batch, hkv, cap, 128, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    q_new = torch.randn(batch, hq, 128, generator=g, device="cuda").to(torch.bfloat16)
+    k[0, :, nan_rows[0]:nan_rows[1]] = float("nan")
+    comp = rkv.Compressor(batch, hkv, hq, cap - 64, 64, 8, 0.1)
+    lens = torch.full((batch,), cap, dtype=torch.int32, device="cuda")
+    out = torch.full((batch, hq, 128), 7.0, device="cuda")
+    assert rkv.rkv_decode_attention(comp.desc, k, v, q_new, lens, out, cap - 64, 64) == 0
+    torch.cuda.synchronize()
+    comp.check_status()
+    assert not out[0].any()
+    ref = oracle.oracle_decode_attention(k[1:].float().cpu().numpy(), v[1:].float().cpu().numpy(), q_new[1:].float().cpu().numpy(),
+                                         np.array([cap], dtype=np.int32))
+    got = out[1:].cpu().numpy().astype(np.float64)
+    assert (np.abs(got - ref) <= 1e-3 * np.abs(ref).max(axis=-1, keepdims=True) + 1e-7).all()
+
+
 @pytest.mark.parametrize("hkv,head_dim,dtype", [(1, 64, torch.bfloat16), (32, 128, torch.float32)])
 def test_append_rows_of_one_block(rkv, hkv, head_dim, dtype):  # noqa: F811
     """A sequence's new rows are moved by one block: 8 vectors and 1024 (several per thread); appends in a row, the last one
