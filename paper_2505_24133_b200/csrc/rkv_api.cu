@@ -559,7 +559,7 @@ int rkv_push_query(const rkv_desc_t *d, void *q_window, const void *q_new, int32
     return e == cudaSuccess ? RKV_OK : cuda_fail(e, "push_query launch");
 }
 
-static int attend_plan(const rkv_desc_t *d, int32_t budget, int32_t buffer, int *splits, size_t *bytes)
+static int attend_plan(const rkv_desc_t *d, int32_t budget, int32_t buffer, int *splits, size_t *bytes, int *sm_count)
 {
     int rc = check_shapes(d, budget, buffer, 1, nullptr);
     if (rc != RKV_OK) return rc;
@@ -568,6 +568,7 @@ static int attend_plan(const rkv_desc_t *d, int32_t budget, int32_t buffer, int 
     int dev = 0, sms = 0;
     if (device_sms(&dev, &sms) != cudaSuccess)
         sms = 148;       // sizing only (no device here): the B200's count
+    *sm_count = sms;
     *splits = attend_splits(d->batch * d->n_kv_heads, budget + buffer, sms, G, d->dtype);
     *bytes = attend_workspace_bytes(d->batch * d->n_kv_heads, budget + buffer, sms, G, d->dtype);
     return RKV_OK;
@@ -575,17 +576,17 @@ static int attend_plan(const rkv_desc_t *d, int32_t budget, int32_t buffer, int 
 
 size_t rkv_decode_workspace_bytes(const rkv_desc_t *desc, int32_t budget, int32_t buffer)
 {
-    int splits = 1;
+    int splits = 1, sms = 0;
     size_t bytes = 0;
-    return attend_plan(desc, budget, buffer, &splits, &bytes) == RKV_OK ? bytes : 0;
+    return attend_plan(desc, budget, buffer, &splits, &bytes, &sms) == RKV_OK ? bytes : 0;
 }
 
 int rkv_decode_attention(const rkv_desc_t *d, const void *k_cache, const void *v_cache, const void *q_new,
                          const int32_t *seq_lens, float *out, int32_t budget, int32_t buffer, void *stream)
 {
-    int splits = 1;
+    int splits = 1, sms = 0;
     size_t bytes = 0;
-    int rc = attend_plan(d, budget, buffer, &splits, &bytes);
+    int rc = attend_plan(d, budget, buffer, &splits, &bytes, &sms);
     if (rc != RKV_OK) return rc;
     if (!k_cache || !v_cache || !q_new || !seq_lens || !out) return RKV_ERR_INVALID_ARG;
     if (!aligned16(k_cache) || !aligned16(v_cache) || !aligned16(q_new) || !aligned16(out)) return RKV_ERR_INVALID_ARG;
@@ -597,7 +598,7 @@ int rkv_decode_attention(const rkv_desc_t *d, const void *k_cache, const void *v
     const long long wait = d->wait_limit_cycles > 0 ? (long long)d->wait_limit_cycles : sm100_default_wait_cycles();
     const cudaError_t e = launch_attend(k_cache, v_cache, q_new, seq_lens, out, static_cast<float *>(d->workspace), d->batch,
                                         d->n_kv_heads, d->n_q_heads, budget + buffer, splits, d->dtype, d->device_status,
-                                        wait, d->block_table, d->pool_pages, d->head_dim, static_cast<cudaStream_t>(stream));
+                                        wait, d->block_table, d->pool_pages, d->head_dim, sms, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? RKV_OK : cuda_fail(e, "decode attention launch");
 }
 

@@ -373,7 +373,7 @@ size_t attend_workspace_bytes(int heads, int cap, int sms, int G, int dtype)
 
 cudaError_t launch_attend(const void *k_cache, const void *v_cache, const void *q_new, const int32_t *seq_lens, float *out,
                           float *partial, int batch, int hkv, int hq, int cap, int splits, int dtype, int32_t *status,
-                          long long wait_cycles, const int32_t *block_table, long long pool_pages, int head_dim, cudaStream_t s)
+                          long long wait_cycles, const int32_t *block_table, long long pool_pages, int head_dim, int sms, cudaStream_t s)
 {
     const int G = hq / hkv;
     AttendParams p;
@@ -393,10 +393,15 @@ cudaError_t launch_attend(const void *k_cache, const void *v_cache, const void *
     p.block_table = block_table;
     p.d_out = head_dim;
     cudaError_t e;
-    if (attend_uses_tc(G, dtype))           // (merges its splits itself)
-        return launch_attend_tc(k_cache, v_cache, q_new, seq_lens, out, batch, hkv, hq, cap, splits, status, wait_cycles,
-                                block_table, pool_pages, dtype == RKV_FP8_E4M3 ? 1 : (head_dim == 64 ? 2 : 0), s);
-    e = launch_dtype<float>(p, G, s);
+    if (attend_uses_tc(G, dtype)) {
+        const int src = dtype == RKV_FP8_E4M3 ? 1 : (head_dim == 64 ? 2 : 0);
+        const bool separate = attend_tc_separate(batch * hkv, cap, splits, sms, src);
+        e = launch_attend_tc(k_cache, v_cache, q_new, seq_lens, out, separate ? partial : nullptr, batch, hkv, hq, cap, splits, status,
+                             wait_cycles, block_table, pool_pages, src, s);
+        if (!separate) return e;             // (a cluster merges its splits itself)
+    } else {
+        e = launch_dtype<float>(p, G, s);
+    }
     if (e != cudaSuccess || splits == 1) return e;
     attend_merge_kernel<<<(unsigned)(batch * hkv * G), kHeadDim, 0, s>>>(p, G);
     return cudaGetLastError();

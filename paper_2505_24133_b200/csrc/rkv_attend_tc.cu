@@ -19,7 +19,11 @@
 // is split into two bf16 parts (rows g and 8 + g of P: N = 16 has the room), so the products carry fp32-accurate
 // weights; the sum of the weights is taken from the same parts.  The splits of a head are one thread-block cluster: each
 // leaves its partial result in its shared memory, then every block merges a share of the outputs from all of them (a merge
-// kernel of its own behind this one took 4 us of a decode step's 33 per layer).
+// kernel of its own behind this one took 4 us of a decode step's 33 per layer).  Where the tiles pass through the softmax threads
+// (8-bit caches, 64 dimensions) and the blocks queue up, the splits are blocks of their own all the same and leave their
+// partial results in the workspace for that kernel: a cluster holds its SMs until its slowest block is done, and starts when all
+// of its blocks fit (4096 heads of 4224 tokens, 3 splits: 8-bit 1267 us as clusters, 1116 as blocks; 64 dimensions 1065, 925; bf16 of
+// 128 dimensions, whose blocks end together, 1204, 1243).
 //
 // Warps 0..3: softmax (thread = TMEM lane = key row of a tile, later = output dimension), warp 4: TMA producer,
 // warp 5: MMA issuer and TMEM owner.
@@ -75,10 +79,11 @@ constexpr int kTcSmem = kOffMisc + 16 + 1024;        // + slack for the 1024-byt
 static_assert(2 * (kTcSmem + 1024) <= 227 * 1024, "two blocks per SM");
 static_assert(16 + 16 * kTcMaxTiles <= (int)kTcTmemCols, "TMEM columns");
 
-struct AttendTcParams {
+struct AttendTcParams {          // (64 bytes: the tensor maps behind it start at the next multiple of 64)
     const int32_t *seq_lens;
-    float *out;                 // [batch][hq][d]
-    int batch, hkv, hq, cap, splits, tiles_per_split;
+    float *out;                 // [batch][hq][d]; separate: [P][splits][G][d + 2], the splits' partial results
+    int separate;               // the splits are blocks of their own, not a cluster
+    int hkv, hq, cap, splits, tiles_per_split;
     int32_t *status;
     long long wait_cycles;
     const int32_t *block_table; // paged caches: [P][cap / 128] page ids, else null
@@ -192,7 +197,8 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     const int t0 = split * p.tiles_per_split;                       // first key tile of this block
     const int T = min(min(p.tiles_per_split, kTcMaxTiles), (L + kTile - 1) / kTile - t0);      // its tiles (<= 0: none)
     constexpr int kStride = kHeadDim + 2;
-    float *part = reinterpret_cast<float *>(smem + kOffP);          // [G][d + 2]: unnormalised output, maximum (base-2 domain), sum of weights
+    // [G][d + 2]: unnormalised output, maximum (base-2 domain), sum of weights
+    float *part = kFp8 && p.separate ? p.out + ((size_t)head * p.splits + split) * G * kStride : reinterpret_cast<float *>(smem + kOffP);
     static_assert(G * kStride * 4 <= 2 * kTcSmall, "the partial result takes the room of P");
     float *out = p.out + ((size_t)b * p.hq + (size_t)h * G) * kDim;
 
@@ -204,9 +210,15 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     if (T <= 0) {       // no cached row falls into this split (uniform for the block)
         if (p.splits == 1) {
             for (int x = threadIdx.x; x < G * kDim; x += kTcThreads) out[x] = 0.f;
-        } else if (threadIdx.x < G) {
-            part[threadIdx.x * kStride + kHeadDim] = -INFINITY;
-            part[threadIdx.x * kStride + kHeadDim + 1] = 0.f;
+        } else {
+            if (kFp8 && p.separate) {                    // (what the merge kernel multiplies by 0 must not be NaN)
+                for (int x = threadIdx.x; x < G * kStride; x += kTcThreads) part[x] = 0.f;
+                __syncthreads();
+            }
+            if (threadIdx.x < G) {
+                part[threadIdx.x * kStride + kHeadDim] = -INFINITY;
+                part[threadIdx.x * kStride + kHeadDim + 1] = 0.f;
+            }
         }
     } else if (warp == 4) {
         // ------------------------------------------------------------------ TMA producer
@@ -315,7 +327,7 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
         if (ok) ok = mbar_wait(bar(kBarScores), 0, abort_flag, sink);
         float m[G], l[G];
 #pragma unroll
-        for (int g = 0; g < G; ++g) m[g] = -INFINITY, l[g] = 0.f;
+        for (int g = 0; g < G; ++g) m[g] = -3.402823466e38f, l[g] = 0.f;      // (-inf stands for a split without rows in the merge)
         if (ok) {
             tc_fence_after();
             for (int t = 0; t < T; ++t) {
@@ -404,8 +416,7 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
             } else {
                 part[g * kStride + r] = num;
                 if (r == 0) {
-                    // -inf stands for a split without rows; one whose scores are all NaN (or -inf: the sum is NaN too) takes part
-                    part[g * kStride + kHeadDim] = !ok ? -INFINITY : m[g] == -INFINITY ? 0.f : m[g];
+                    part[g * kStride + kHeadDim] = ok ? m[g] : -INFINITY;
                     part[g * kStride + kHeadDim + 1] = den;
                 }
             }
@@ -413,10 +424,10 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     }
 
     // ---- merge the splits: out = sum_s 2^(m_s - m) num_s / sum_s 2^(m_s - m) l_s, block r of the cluster taking its share
-    if (p.splits > 1) {
+    if (p.splits > 1 && !(kFp8 && p.separate)) {
         __syncwarp();
         cluster_sync();
-        const uint32_t base = smem_u32(part);
+        const uint32_t base = sbase + kOffP;
         for (int x = split * kTcThreads + threadIdx.x; x < G * kDim; x += p.splits * kTcThreads) {
             const int g = x / kDim, c = x % kDim;
             const uint32_t row = base + (uint32_t)(g * kStride) * 4u;
@@ -449,22 +460,22 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
 }
 
 template <int G, int kSrc>
-cudaError_t launch_tc_one(const AttendTcParams &p, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
+cudaError_t launch_tc_one(const AttendTcParams &p, int heads, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
                           cudaStream_t s)
 {
     static std::atomic<unsigned long long> done{0ull};
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess || (e = allow_smem_once(done, dev, attend_tc_kernel<G, kSrc>, kTcSmem, true)) != cudaSuccess) return e;
-    return launch_early(attend_tc_kernel<G, kSrc>, (unsigned)(p.batch * p.hkv * p.splits), kTcThreads, kTcSmem, s,
-                        (unsigned)p.splits, p, mk, mv, mq);
+    return launch_early(attend_tc_kernel<G, kSrc>, (unsigned)(heads * p.splits), kTcThreads, kTcSmem, s,
+                        p.separate ? 1u : (unsigned)p.splits, p, mk, mv, mq);
 }
 template <int G>
-cudaError_t launch_tc_for(const AttendTcParams &p, int src, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
+cudaError_t launch_tc_for(const AttendTcParams &p, int heads, int src, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
                           cudaStream_t s)
 {
-    return src == 1 ? launch_tc_one<G, 1>(p, mk, mv, mq, s) : src == 2 ? launch_tc_one<G, 2>(p, mk, mv, mq, s)
-                                                                          : launch_tc_one<G, 0>(p, mk, mv, mq, s);
+    return src == 1 ? launch_tc_one<G, 1>(p, heads, mk, mv, mq, s) : src == 2 ? launch_tc_one<G, 2>(p, heads, mk, mv, mq, s)
+                                                                          : launch_tc_one<G, 0>(p, heads, mk, mv, mq, s);
 }
 
 }  // namespace
@@ -499,15 +510,22 @@ int attend_tc_workspace_splits(int heads, int cap, int sms)
     return splits > tiles ? tiles : splits;
 }
 
+// The splits are blocks of their own: more than two waves of them, of a kind that clusters slow down, and the workspace holds their
+// partial results.  (Up to two waves clusters are the faster, by 10-30 % below one; from there on blocks are, by 1 to 17 %.)
+bool attend_tc_separate(int heads, int cap, int splits, int sms, int src)
+{
+    return splits > 1 && src != 0 && (long long)heads * splits > 4ll * sms && splits <= attend_tc_workspace_splits(heads, cap, sms);
+}
+
 cudaError_t launch_attend_tc(const void *k_cache, const void *v_cache, const void *q_new, const int32_t *seq_lens, float *out,
-                             int batch, int hkv, int hq, int cap, int splits, int32_t *status, long long wait_cycles,
+                             float *partial, int batch, int hkv, int hq, int cap, int splits, int32_t *status, long long wait_cycles,
                              const int32_t *block_table, long long pool_pages, int src, cudaStream_t s)
 {
     const int tiles = (cap + kTile - 1) / kTile;
     AttendTcParams p;
     p.seq_lens = seq_lens;
-    p.out = out;
-    p.batch = batch;
+    p.out = partial ? partial : out;
+    p.separate = partial ? 1 : 0;
     p.hkv = hkv;
     p.hq = hq;
     p.cap = cap;
@@ -525,14 +543,14 @@ cudaError_t launch_attend_tc(const void *k_cache, const void *v_cache, const voi
     const bool q_ok = src == 2 ? sm100::make_map_rows(&mq, q_new, (uint64_t)batch * hq, 64, 16) : sm100::make_map(&mq, q_new, (uint64_t)batch * hq, 16);
     if (!maps_ok || !q_ok) return cudaErrorInvalidValue;
     switch (hq / hkv) {
-        case 1: return launch_tc_for<1>(p, src, mk, mv, mq, s);
-        case 2: return launch_tc_for<2>(p, src, mk, mv, mq, s);
-        case 3: return launch_tc_for<3>(p, src, mk, mv, mq, s);
-        case 4: return launch_tc_for<4>(p, src, mk, mv, mq, s);
-        case 5: return launch_tc_for<5>(p, src, mk, mv, mq, s);
-        case 6: return launch_tc_for<6>(p, src, mk, mv, mq, s);
-        case 7: return launch_tc_for<7>(p, src, mk, mv, mq, s);
-        case 8: return launch_tc_for<8>(p, src, mk, mv, mq, s);
+        case 1: return launch_tc_for<1>(p, batch * hkv, src, mk, mv, mq, s);
+        case 2: return launch_tc_for<2>(p, batch * hkv, src, mk, mv, mq, s);
+        case 3: return launch_tc_for<3>(p, batch * hkv, src, mk, mv, mq, s);
+        case 4: return launch_tc_for<4>(p, batch * hkv, src, mk, mv, mq, s);
+        case 5: return launch_tc_for<5>(p, batch * hkv, src, mk, mv, mq, s);
+        case 6: return launch_tc_for<6>(p, batch * hkv, src, mk, mv, mq, s);
+        case 7: return launch_tc_for<7>(p, batch * hkv, src, mk, mv, mq, s);
+        case 8: return launch_tc_for<8>(p, batch * hkv, src, mk, mv, mq, s);
         default: return cudaErrorInvalidValue;
     }
 }

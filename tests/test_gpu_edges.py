@@ -105,6 +105,38 @@ def test_decode_attention_splits(rkv, batch, hkv, hq, cap):  # noqa: F811
     assert (np.abs(got - ref) <= 1e-3 * scale + 1e-7).all(), float((np.abs(got - ref) / scale).max())
 
 
+@pytest.mark.parametrize("dtype,head_dim", [("fp8", 128), ("bf16", 64), ("bf16", 128)])
+@pytest.mark.parametrize("heads,cap", [(296, 2176), (297, 2176), (200, 4224)])
+def test_decode_attention_splits_as_blocks(rkv, dtype, head_dim, heads, cap):  # noqa: F811
+    """Two waves of blocks on 148 SMs (two splits of 296 heads: clusters) and more (8-bit caches and 64 dimensions: blocks of their
+    own, partial results in the workspace, here full of NaN): lengths that leave the last splits without a row, none at all."""
+    group = 4
+    g = torch.Generator(device="cuda").manual_seed(heads)
+    k, v = (torch.randn(heads, 1, cap, head_dim, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    dt = torch.float8_e4m3fn if dtype == "fp8" else torch.bfloat16
+    k, v = k.to(dt), v.to(dt)
+    q_new = torch.randn(heads, group, head_dim, generator=g, device="cuda").to(torch.bfloat16)
+    lens = torch.tensor([(cap, cap - 1, 1, 130, 0, cap // 2)[b % 6] for b in range(heads)], dtype=torch.int32)
+    for b, L in enumerate(lens.tolist()):
+        for t in (k, v):
+            t.view(torch.uint8 if dtype == "fp8" else torch.int16)[b, :, L:] = 0x7F if dtype == "fp8" else 0x7FC0
+    comp = rkv.Compressor(heads, 1, group, cap - 64, 64, 8, 0.1, dtype=dt, head_dim=head_dim)
+    comp.workspace.fill_(0xFF)
+    out = torch.full((heads, group, head_dim), 7.0, device="cuda")
+    for _ in range(2):
+        assert rkv.rkv_decode_attention(comp.desc, k, v, q_new, lens.cuda(), out, cap - 64, 64) == 0
+    torch.cuda.synchronize()
+    comp.check_status()
+    rows = [0, 1, 2, 3, 4, 5, heads - 6, heads - 5, heads - 4, heads - 3, heads - 2, heads - 1]
+    K, V = (torch.nan_to_num(t.view(torch.uint8)[rows].view(t.dtype).float() if dtype == "fp8" else t[rows].float(), nan=0.0).cpu().numpy()
+            for t in (k, v))
+    ref = oracle.oracle_decode_attention(K, V, q_new[rows].float().cpu().numpy(), lens[rows].numpy())
+    got = out[rows].cpu().numpy().astype(np.float64)
+    assert np.isfinite(out.cpu().numpy()).all()
+    scale = np.maximum(np.abs(ref).max(axis=-1, keepdims=True), 1e-30)
+    assert (np.abs(got - ref) <= 1e-3 * scale + 1e-7).all(), float((np.abs(got - ref) / scale).max())
+
+
 @pytest.mark.parametrize("cap,nan_rows", [(1920, (0, 128)), (1920, (0, 1920)), (1920, (1152, 1280)), (1280, (5, 6))])
 def test_decode_attention_over_nan_keys(rkv, cap, nan_rows):  # noqa: F811
     """Keys of NaN give the output row that they give when one block holds the head (zeros: no sum of weights), also when they are
