@@ -7,13 +7,20 @@
 // reallocation.  HBM-bound: kept rows read and written once.
 // The stream of (KV head 0, K) also stores the new length, seq_lens[b] = budget.
 //
-// Two kernels.  gather_bulk_kernel (more streams than SMs): bulk copies through shared memory, eight streams per block, a
-// loading and a storing warp each.  What is kept comes in runs (a few per cent of the rows are dropped), so a chunk is one
-// to three copies in and one copy out, and the bytes in flight cost neither registers nor issue slots.  Measured against
-// 16-byte loads and stores by threads, the form that all sizes had: 8192 streams of 4096 rows of 256 bytes 2779 -> 2535 us,
-// of 128 bytes 1591 -> 1317 us; 512 streams of 1024 rows of 512 bytes 119 -> 72 us.  gather_kernel (fewer streams): threads,
-// a row cut into four column slices with a block each (128 streams of 4096 rows: 56 us; 74 with the bulk kernel, whose one
-// stream per block keeps too little in flight).
+// Two kernels.  gather_bulk_kernel: bulk copies through shared memory, eight streams per block, a loading and a storing warp
+// each, a block per SM.  What is kept comes in runs (a few per cent of the rows are dropped), so a chunk is one to three copies in
+// and one copy out, and the bytes in flight cost neither registers nor issue slots.  gather_kernel: 16-byte loads and stores by
+// threads, a block per stream, or four that take a column slice of its rows each.  Which one a call takes is a matter of how
+// many streams there are and how long a row is (launch_gather_for; us for 1024 to 4096 rows per stream, in the call):
+//   streams x rows of bytes    160 x 2048 x 256   160 x 2048 x 128   512 x 4096 x 256   4096 x 2048 x 256   8192 x 4096 x 256
+//   bulk                              45                 33               168                 694               2800
+//   threads, four slices              35                 25               207                 837               3486
+//   threads, a block per stream       72                 39               213                 698               2768
+//                            24576 x 4096 x 256   8192 x 4096 x 128  16384 x 2048 x 128   8192 x 1024 x 512
+//   bulk                            8490               1400                1408                1386
+//   threads, a block per stream     8090               1563                1519                1792
+// (The bulk kernel on fewer SMs: up to 116 blocks moved 8192 streams of 256-byte rows in 2720-2790 us, 118 to 136 in 2880-3020.  A count
+// between those would do on one GPU and lie on the wrong side of the step on another.)
 #include <algorithm>
 
 #include "rkv_sm100.cuh"
@@ -132,12 +139,13 @@ __global__ void __launch_bounds__(kBulkThreads, 1) gather_bulk_kernel(Params p, 
 
 // ---- threads -----------------------------------------------------------------------------------------------------------
 constexpr int kGatherThreads = 256;
-constexpr int kSplit = 4;                           // column slices of a row (disjoint bytes: no ordering among them)
-constexpr int kChunkRows = 64 * kSplit;             // 16 KB in flight per block
 
-template <int kVecPerRow>                           // 16-byte vectors per row: 4 (8-bit, d = 64) .. 64 (fp32, d = 256)
+// kVecPerRow: 16-byte vectors per row: 4 (8-bit, d = 64) .. 64 (fp32, d = 256).  kSplit: column slices of a row (disjoint bytes: no
+// ordering among them).
+template <int kVecPerRow, int kSplit>
 __global__ void __launch_bounds__(kGatherThreads) gather_kernel(Params p)
 {
+    constexpr int kChunkRows = 64 * kSplit;             // of 256 bytes: 16 KB in flight per block
     constexpr int kVecPerSlice = kVecPerRow / kSplit;
     constexpr int kVecPerThread = kChunkRows * kVecPerSlice / kGatherThreads;
     constexpr int kRowsPerStep = kGatherThreads / kVecPerSlice;
@@ -186,13 +194,18 @@ cudaError_t launch_gather_for(const Params &p, cudaStream_t s)
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess) return e;
-    if (streams <= (unsigned)sms) return launch_early(gather_kernel<kVecPerRow>, streams * kSplit, kGatherThreads, 0, s, 1, p);
-    // With every SM at work the memory turns between reading and writing more often: where there are streams enough, 13
-    // blocks per 16 SMs move 3-5 % more than one per SM (8192 and 14336 streams; half as many move less).
+    // Few streams: what a block of either kernel keeps in flight does not fill the chip, so a row is cut into slices (wide rows fill
+    // a slice's chunk by themselves: from a stream per SM on they are the bulk kernel's).
+    if (streams <= (unsigned)(kVecPerRow <= 16 ? sms * 3 / 2 : sms))
+        return launch_early(gather_kernel<kVecPerRow, 4>, streams * 4, kGatherThreads, 0, s, 1, p);
+    // Rows of 256 bytes in many streams: the thread kernel keeps as much in flight as the bulk kernel, and turns between reading and
+    // writing less often.
+    if constexpr (kVecPerRow == 16)
+        if (streams >= 4096u) return launch_early(gather_kernel<kVecPerRow, 1>, streams, kGatherThreads, 0, s, 1, p);
     static std::atomic<unsigned long long> done{0ull};
     if ((e = allow_smem_once(done, dev, gather_bulk_kernel<kVecPerRow * 16>, kBulkSmem)) != cudaSuccess) return e;
-    const unsigned blocks = streams >= 4096u ? (unsigned)(sms * 13 / 16) : std::min(streams, (unsigned)sms);
-    return launch_early(gather_bulk_kernel<kVecPerRow * 16>, blocks, kBulkThreads, (size_t)kBulkSmem, s, 1, p, (int)streams);
+    return launch_early(gather_bulk_kernel<kVecPerRow * 16>, std::min(streams, (unsigned)sms), kBulkThreads, (size_t)kBulkSmem, s, 1, p,
+                        (int)streams);
 }
 
 }  // namespace

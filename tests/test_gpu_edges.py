@@ -241,12 +241,15 @@ def test_host_buffers_on_independent_streams(rkv):  # noqa: F811
             assert torch.equal(x[:, :, :spec.budget].view(torch.int16), y[:, :, :spec.budget].view(torch.int16))
 
 
-@pytest.mark.parametrize("head_dim,dtype", [(64, "fp8"), (64, "bf16"), (128, "bf16"), (256, "bf16"), (256, "f32")])
+@pytest.mark.parametrize("head_dim,dtype,batch", [(64, "fp8", 19), (64, "bf16", 19), (128, "bf16", 19), (256, "bf16", 19), (256, "f32", 19),
+                                                  (64, "fp8", 28), (64, "bf16", 28), (128, "bf16", 28), (128, "bf16", 27), (256, "bf16", 18),
+                                                  (128, "bf16", 511), (128, "bf16", 512)])
 @pytest.mark.parametrize("pattern", ["runs", "last_k", "sparse", "identity"])
-def test_compaction_by_bulk_copies(rkv, head_dim, dtype, pattern):  # noqa: F811
-    """More streams than SMs: the gather stage alone on hand-made ascending lists, every row width; runs that cross chunks,
+def test_compaction_by_bulk_copies(rkv, head_dim, dtype, batch, pattern):  # noqa: F811
+    """The gather stage alone on hand-made ascending lists, every row width, eight streams per sequence on both sides of the lines between its
+    kernels (222 streams on 148 SMs, 148 for rows of 512 bytes and more, 4096 for rows of 256); runs that cross chunks,
     single rows, a long shift, a list in place already, a budget that is not a whole number of chunks; ragged lengths."""
-    batch, hkv, budget, buffer, alpha = 19, 4, 333, 83, 8
+    hkv, budget, buffer, alpha = 4, 333, 83, 8
     spec = small_spec("bulk", batch=batch, hkv=hkv, hq=hkv, budget=budget, buffer=buffer, head_dim=head_dim, dtype=dtype)
     cap = spec.cap
     lens = torch.tensor([budget - 5 if b % 7 == 3 else cap - b % 5 for b in range(batch)])
