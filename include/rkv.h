@@ -262,8 +262,8 @@ RKV_API int rkv_compress_static(const rkv_desc_t *desc, void *k_cache, void *v_c
 
 /* The two cache updates of a decode step that surround the compression, so that a whole decode segment (buffer
  * appends, then rkv_compress when seq_lens reaches budget + buffer: Section 3.1) can be enqueued, or captured in a
- * CUDA graph, through this library alone.  Both only enqueue work on `stream` (two launches / one launch) and use no
- * workspace.
+ * CUDA graph, through this library alone.  Both only enqueue work on `stream` (one launch, two for the appends of very many
+ * heads) and use no workspace.
  *
  * rkv_append: the newly generated token of every sequence enters the buffer part of its cache.
  *   k_new, v_new [batch, n_kv_heads, head_dim] (device, dtype of the cache, 16-byte aligned) are copied to row

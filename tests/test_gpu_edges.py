@@ -159,10 +159,11 @@ def test_decode_attention_over_nan_keys(rkv, cap, nan_rows):  # noqa: F811
     assert (np.abs(got - ref) <= 1e-3 * np.abs(ref).max(axis=-1, keepdims=True) + 1e-7).all()
 
 
-@pytest.mark.parametrize("hkv,head_dim,dtype", [(1, 64, torch.bfloat16), (32, 128, torch.float32)])
+@pytest.mark.parametrize("hkv,head_dim,dtype", [(1, 64, torch.bfloat16), (32, 128, torch.float32), (512, 128, torch.bfloat16),
+                                                (513, 128, torch.bfloat16)])
 def test_append_rows_of_one_block(rkv, hkv, head_dim, dtype):  # noqa: F811
-    """A sequence's new rows are moved by one block: 8 vectors and 1024 (several per thread); appends in a row, the last one
-    into a cache that is full by then."""
+    """A sequence's new rows are moved by one block: 8 vectors and 1024 (several per thread), up to 8192; by several from there on; appends
+    in a row, the last one into a cache that is full by then."""
     batch, budget, buffer = 3, 24, 8
     cap = budget + buffer
     comp = rkv.Compressor(batch, hkv, hkv, budget, buffer, 8, 0.1, dtype=dtype, head_dim=head_dim)
