@@ -101,7 +101,7 @@ static int get_int(PyObject *o, int32_t *out)
 /* the descriptor (a ctypes structure of the binding's type, nothing else that has bytes) stays where it is while `view` is held */
 static int get_desc(PyObject *o, Py_buffer *view)
 {
-    const int is = PyObject_IsInstance(o, g_desc_type);
+    const int is = (PyObject *)Py_TYPE(o) == g_desc_type ? 1 : PyObject_IsInstance(o, g_desc_type);
     if (is < 0) return -1;
     if (!is) {
         PyErr_Format(PyExc_TypeError, "expected an RkvDesc, got %s", Py_TYPE(o)->tp_name);
