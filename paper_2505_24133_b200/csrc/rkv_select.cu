@@ -63,6 +63,10 @@ __device__ __forceinline__ float block_sum(float v, float *scratch)
     return warp_sum((threadIdx.x & 31) < kThreads / 32 ? scratch[threadIdx.x & 31] : 0.f);
 }
 
+// What a lane takes its exponentials relative to: its running maximum, unless it has met nothing above -inf yet (a logit may be
+// that low: it weighs nothing, where -inf - -inf would make the row's sum NaN).
+__device__ __forceinline__ float finite_ref(float m) { return m == -INFINITY ? 0.f : m; }
+
 // Eq. 6's column mean of a token: the two-pass scoring kernels leave the column sum minus the removed entries.
 __device__ __forceinline__ float column_mean(const Params &p, float v, int n) { return p.tri ? v / (float)n : v; }
 
@@ -112,10 +116,11 @@ __global__ void __launch_bounds__(kStatThreads) row_stats_kernel(Params p)
             s *= expf(m - top);
             m = top;
         }
+        const float ref = finite_ref(m);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             if (at + u * 128 >= n) break;
-            if (i0 + u * 128 < n) s += (expf(v[u].x - m) + expf(v[u].y - m)) + (expf(v[u].z - m) + expf(v[u].w - m));
+            if (i0 + u * 128 < n) s += (expf(v[u].x - ref) + expf(v[u].y - ref)) + (expf(v[u].z - ref) + expf(v[u].w - ref));
         }
     }
     const float mw = warp_max(m);
@@ -462,10 +467,11 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) select_fused_kernel
                 sj *= expf(mj - top);
                 mj = top;
             }
+            const float ref = finite_ref(mj);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (i0 + u * 128 >= end) break;
-                sj += (expf(v[u].x - mj) + expf(v[u].y - mj)) + (expf(v[u].z - mj) + expf(v[u].w - mj));
+                sj += (expf(v[u].x - ref) + expf(v[u].y - ref)) + (expf(v[u].z - ref) + expf(v[u].w - ref));
             }
         }
         const float mw = warp_max(mj);

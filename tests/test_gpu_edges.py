@@ -304,3 +304,31 @@ def test_norms_of_a_tile_given_up_abort_the_call(rkv, dtype, head_dim, tile):  #
     torch.cuda.synchronize()
     assert int(comp.status.item()) == 5
     assert torch.equal(wl.k_cache, k0) and torch.equal(wl.seq_lens, s0) and bool((comp.out_idx == -1).all())
+
+
+@pytest.mark.parametrize("budget,buffer", [(600, 100), (1900, 100)])
+def test_logits_of_minus_infinity(rkv, budget, buffer):  # noqa: F811
+    """Products that overflow to -inf weigh nothing in the softmax of Eq. 3, also where they are all that a lane sees (the lanes of the
+    row statistics take four of every 128 tokens): single-kernel and three-kernel selection."""
+    spec = small_spec("inf", batch=1, hkv=1, hq=1, budget=budget, buffer=buffer, span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=461)
+    pos = torch.arange(spec.cap, device="cuda")
+    low = (pos % 128 >= 40) & (pos % 128 < 48)
+    wl.q_window.fill_(1e30)
+    wl.k_cache[:] = torch.where(low[:, None], -1e10, 0.0).to(torch.bfloat16)
+    wl.k_cache[0, 0, :, 0] += torch.where(low, 0.0, (pos % 7).float() * 1e-30).to(torch.bfloat16)
+    rep, comp = run_and_check(rkv, wl)
+    assert rep.ok(), rep.errors
+    comp.check_status()
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("beta,T", [(4, 0.5), (5, 0.5), (8, 0.3), (40, 0.2)])
+def test_first_pass_partners_of_a_chunk(rkv, head_dim, beta, T):  # noqa: F811
+    """Up to four partners of a chunk are taken out one by one, more in one sum: copies in abundance, counts on both sides within a
+    warp, partners that run out in the middle of a chunk."""
+    spec = small_spec("chunk", batch=2, hkv=2, hq=4, budget=150, buffer=100, head_dim=head_dim, span=2, copy_frac=0.7)
+    wl = ri.make_workload(spec, device="cuda", seed=463 + beta, seq_lens=torch.tensor([250, 201]))
+    rep, comp = run_and_check(rkv, wl, beta=beta, T=T)
+    assert rep.ok(), rep.errors
+    comp.check_status()
