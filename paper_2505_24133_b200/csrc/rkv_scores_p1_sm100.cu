@@ -38,6 +38,7 @@ constexpr int kThreadsP1 = 320;
 constexpr int kHalfBytes = kTile * 64 * 2;       // one TMA box: 128 rows x 64 bf16 (128-byte swizzled rows)
 constexpr int kSliceBytes = kTile * 32;          // the extra K = 16 slice of an operand: 128 rows x 32 bytes (32-byte swizzle)
 constexpr int kMaxStagesA = 8;
+constexpr int kMostTurns = 4;                    // partners of a chunk that are taken out one by one
 constexpr uint32_t kTmemColsP1 = 512;            // 2 buffers x (128 key columns + up to 128 query columns)
 constexpr int kSmemLimit = 227 * 1024;
 
@@ -88,8 +89,9 @@ __host__ __device__ inline SmemPlan make_plan(int q_rows_pad)
 // Item descriptor (int4): {head, first row tile, one past the last row tile, n}.  x < 0: no more items.
 // kPlain: alpha = 8, the maximum over the group, the retention rule on -- the defaults -- without the code of the other
 // forms: the roles share the instruction cache (4096 heads of 4216 tokens: 1036 us with it, 992 without).
-// kOne: beta = 1 as well.
-template <int D, bool kPlain, bool kOne>
+// kOne: beta = 1 as well.  kMany: beta > kMostTurns, the form that can also take a chunk's partners out in one sum (4096 heads of 4216
+// tokens: beta = 8 1960 us without it, beta = 16 2200; beta = 2 and 3, which never need it, 1238 and 1424, 1320 and 1492 with it).
+template <int D, bool kPlain, bool kOne, bool kMany>
 __global__ void __launch_bounds__(kThreadsP1, 1)
 scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,
                            const __grid_constant__ CUtensorMap map_hs, const __grid_constant__ CUtensorMap map_ns,
@@ -426,6 +428,31 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                             }
                             return;
                         }
+                        // Several partners: a turn each, or, where some lane has many, one sum over the columns for all lanes (a
+                        // warp takes as many turns as the lane with most).
+                        const int turns = !kMany ? 0 : (int)__reduce_max_sync(0xffffffffu, pos != 0u ? (unsigned)min(__popc(pos), left) : 0u);
+                        if (kMany && turns > kMostTurns) {
+                            uint32_t hits = 0u;
+#pragma unroll
+                            for (int c = 0; c < 32; ++c) hits |= (__uint_as_float(g[c]) > 0.f) ? (1u << c) : 0u;
+                            hits &= pos;
+                            int taken = __popc(hits);
+                            for (; taken > left; --taken) hits &= hits - 1u;                   // drop the lowest positions
+                            float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                const float4 R = reinterpret_cast<const float4 *>(rj)[ch * 8 + q];
+                                s0 += (hits >> (4 * q) & 1u) ? __uint_as_float(g[4 * q]) * R.x : 0.f;
+                                s1 += (hits >> (4 * q + 1) & 1u) ? __uint_as_float(g[4 * q + 1]) * R.y : 0.f;
+                                s2 += (hits >> (4 * q + 2) & 1u) ? __uint_as_float(g[4 * q + 2]) * R.z : 0.f;
+                                s3 += (hits >> (4 * q + 3) & 1u) ? __uint_as_float(g[4 * q + 3]) * R.w : 0.f;
+                            }
+                            removed += (s0 + s1) + (s2 + s3);
+                            nhit += taken;
+                            left -= taken;
+                            want = left > 0;
+                            return;
+                        }
                         while (pos != 0u) {
                             const int top = 31 - __clz((int)pos);
                             const float hv = pick32(g, top);
@@ -499,7 +526,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
 
 }  // namespace
 
-template <int D, bool kPlain, bool kOne>
+template <int D, bool kPlain, bool kOne, bool kMany>
 static cudaError_t launch_pass1_for(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q, const CUtensorMap &map_hs,
                                     const CUtensorMap &map_ns, const CUtensorMap &map_ts, int q_rows_pad)
 {
@@ -509,14 +536,14 @@ static cudaError_t launch_pass1_for(const Params &p, cudaStream_t s, const CUten
     static std::atomic<unsigned long long> done{0ull};
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D, kPlain, kOne>, kSmemLimit)) != cudaSuccess) return e;
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D, kPlain, kOne, kMany>, kSmemLimit)) != cudaSuccess) return e;
     const int heads = p.batch * p.hkv;
     // a head is cut into parts when there are too few heads to give every SM several items
     int splits = (4 * sms + heads - 1) / heads;
     splits = splits < 1 ? 1 : (splits > p.tiles ? p.tiles : splits);
     const unsigned long long total_items = (unsigned long long)splits * (unsigned long long)heads;
     const unsigned grid = (unsigned)(total_items < (unsigned long long)sms ? total_items : (unsigned long long)sms);
-    return launch_early(scores_stream_sm100_kernel<D, kPlain, kOne>, grid, kThreadsP1, (size_t)pl.total, s, 1, p, map_k, map_q, map_hs, map_ns, map_ts, splits,
+    return launch_early(scores_stream_sm100_kernel<D, kPlain, kOne, kMany>, grid, kThreadsP1, (size_t)pl.total, s, 1, p, map_k, map_q, map_hs, map_ns, map_ts, splits,
                         total_items, q_rows_pad);
 }
 
@@ -525,9 +552,13 @@ static cudaError_t launch_pass1_form(const Params &p, cudaStream_t s, const CUte
                                      const CUtensorMap &map_ns, const CUtensorMap &map_ts, int q_rows_pad)
 {
     const bool plain = p.alpha == 8 && p.beta > 0 && p.sim_threshold < 1.0f && !p.gqa_mean_pool;
-    return !plain        ? launch_pass1_for<D, false, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
-           : p.beta == 1 ? launch_pass1_for<D, true, true>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
-                         : launch_pass1_for<D, true, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
+    const bool many = p.beta > kMostTurns;
+    if (!plain)
+        return many ? launch_pass1_for<D, false, false, true>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
+                    : launch_pass1_for<D, false, false, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
+    return p.beta == 1 ? launch_pass1_for<D, true, true, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
+           : many      ? launch_pass1_for<D, true, false, true>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
+                       : launch_pass1_for<D, true, false, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
 }
 
 cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q,
