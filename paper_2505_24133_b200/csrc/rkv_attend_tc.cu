@@ -482,18 +482,21 @@ cudaError_t launch_tc_for(const AttendTcParams &p, int heads, int src, const CUt
 
 // Splits of a head's key tiles (blocks of a cluster) for the tensor-core kernel: at most kTcMaxTiles tiles per block, and
 // among those the number with the shortest run: waves of resident blocks (2 per SM) times what a block spends, its tiles and
-// about two tiles' worth of set-up and merge.  (128 heads of 33 tiles: 4 splits, two waves of 9 tiles, where the earlier rule,
-// the fewest splits that give two waves of blocks, took three waves of 7.)
+// about three tiles' worth of set-up and merge.  (128 heads of 33 tiles: 4 splits, two waves of 9 tiles, 49 us; 5, the fewest that give
+// two waves of blocks, 54.  With two tiles' worth 600 heads of 15 tiles were cut in three, 98 us and 114 for 8-bit caches, 93
+// and 97 uncut; 512 heads of 33 tiles in four, 167 and 192, 163 and 172 in three.)  The fewest splits where they give four
+// waves: a part of the last one counts for little then (256 heads of 64 tiles: 159 us with 5 splits, 165 with 8).
 int attend_tc_splits(int heads, int cap, int sms)
 {
-    const int tiles = (cap + kTile - 1) / kTile;
+    const int tiles = (cap + kTile - 1) / kTile, least = (tiles + kTcMaxTiles - 1) / kTcMaxTiles;
+    if ((long long)heads * least >= 8ll * sms) return least;
     int best = 0;
     long long best_cost = 0;
-    for (int s = (tiles + kTcMaxTiles - 1) / kTcMaxTiles; s <= tiles && s <= kTcMaxSplits; ++s) {
+    for (int s = least; s <= tiles && s <= kTcMaxSplits; ++s) {
         const int per = (tiles + s - 1) / s;
         if (s > 1 && (tiles + per - 1) / per < s) continue;          // the last blocks would have no tile
         const long long waves = ((long long)heads * s + 2 * sms - 1) / (2 * sms);
-        const long long cost = waves * (per + 2);
+        const long long cost = waves * (per + 3);
         if (best == 0 || cost < best_cost) best = s, best_cost = cost;
     }
     return best;
