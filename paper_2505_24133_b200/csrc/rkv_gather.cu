@@ -19,8 +19,9 @@
 //                            24576 x 4096 x 256   8192 x 4096 x 128  16384 x 2048 x 128   8192 x 1024 x 512
 //   bulk                            8490               1400                1408                1386
 //   threads, a block per stream     8090               1563                1519                1792
-// (The bulk kernel on fewer SMs: up to 116 blocks moved 8192 streams of 256-byte rows in 2720-2790 us, 118 to 136 in 2880-3020.  A count
-// between those would do on one GPU and lie on the wrong side of the step on another.)
+// The bulk kernel on fewer SMs is no rule to go by: somewhere between 100 and 122 blocks, differently on different GPUs of the type,
+// lies a step of 10 % (8192 streams of 256-byte rows with 120 blocks: 2620, 2760, 2875 and 2940 us on four of them, with 111 blocks 2725 on
+// one and 2940 on another; by threads 2768-2772 on all).
 #include <algorithm>
 
 #include "rkv_sm100.cuh"
