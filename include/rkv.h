@@ -59,7 +59,7 @@ typedef enum {
  *     no infinities; one byte per element, rows of head_dim bytes); q_window (and q_new of rkv_push_query) is bf16.
  *     Eq. 1-7 are evaluated on the values the codes stand for: the keys are widened to bf16 (exactly; every E4M3 value
  *     is a bf16 value) into the workspace, which grows by (batch * n_kv_heads * (budget + buffer) + 128) * head_dim * 2
- *     bytes (nothing more for head_dim 64, whose padded copy exists anyway), and every scoring stage runs on that copy as for a bf16 cache.  The compaction moves the stored bytes; no
+ *     bytes (nothing more for head_dim 64, whose workspace has room for a copy in any case), and every scoring stage runs on that copy as for a bf16 cache.  The compaction moves the stored bytes; no
  *     scale factor is applied or needed (cosine similarity does not see a per-tensor scale; fold a key scale into
  *     the queries for Eq. 2).  rkv_decode_attention takes this type too (q_new bf16): the codes are widened on their
  *     way to the tensor cores, no copy is kept. */
@@ -106,11 +106,9 @@ typedef struct rkv_desc {
     int32_t batch;       /* sequences; layers that fire together are folded into this dimension */
     int32_t n_kv_heads;  /* KV heads per sequence */
     int32_t n_q_heads;   /* query heads; G = n_q_heads / n_kv_heads must be integral (G = 1: Eq. 1) */
-    int32_t head_dim;    /* d: 64, 128 or 256.  The tensor-core scoring kernels are built for bf16 keys with d = 128;
-                            bf16 and 8-bit caches with d = 64 are scored by them on a copy of the keys (and of the
-                            observation queries) padded with zeros to 128 in the workspace -- dot products and norms do
-                            not see the padding --; d = 256 by a tensor-core kernel that forms the whole similarity
-                            matrix; fp32 caches by the CUDA-core kernel (fp32 arithmetic, slower) */
+    int32_t head_dim;    /* d: 64, 128 or 256.  bf16 caches with d = 64 and 128 are scored by the two-pass tensor-core kernels
+                            as they lie, 8-bit caches on a bf16 copy of their keys in the workspace; d = 256 by a
+                            tensor-core kernel that forms the whole similarity matrix; fp32 caches by the CUDA-core kernel (fp32 arithmetic, slower) */
     int32_t dtype;       /* rkv_dtype_t of k_cache and v_cache (and of q_window, except for 8-bit caches: bf16) */
     int32_t pool_w;      /* W of Eq. 4; 0 = no pooling.  Range [0, 64].  Default 4 (the paper prints no value) */
     int32_t beta;        /* beta of Section 3.3; 0 = rule off.  Default 1 (the paper prints no value) */
@@ -193,7 +191,8 @@ RKV_API int rkv_set_desc(const rkv_desc_t *desc);
  * of the batch is compressed as usual.
  * If a bounded wait inside a kernel runs out (RKV_ERR_TIMEOUT in device_status), the scores of the call are
  * incomplete: the remaining kernels then leave ALL caches and lengths of the batch unmodified and set every
- * entry of out_idx to -1.  The state that carries this between the kernels lives in the workspace and is reset by
+ * entry of out_idx to -1.  (The compaction itself waits for its own copies, with the default limit whatever
+ * wait_limit_cycles says: should the memory not answer for that long, the caches it was moving are lost.)  The state that carries this between the kernels lives in the workspace and is reset by
  * each call, so nothing has to be cleared before the next one.
  * Requires 1 <= alpha < budget, buffer >= 1, cap <= RKV_MAX_CAP, G * alpha <= RKV_MAX_GROUP_ROWS,
  * lambda in [0, 1].  Host-detectable errors return before anything is launched.
@@ -296,9 +295,10 @@ RKV_API int rkv_push_query(const rkv_desc_t *desc, void *q_window, const void *q
  * cache type) or 64 (bf16 caches: tiles padded to 128 on their way to the tensor cores), and G = n_q_heads /
  * n_kv_heads up to 8 (RKV_ERR_UNSUPPORTED otherwise).  The rows of a head are cut into splits (with
  * few head-problems, to fill the GPU; for bf16 and 8-bit caches also whenever budget + buffer exceeds 1920 rows, what one block
- * holds scores for) whose partial results go through desc->workspace: rkv_decode_workspace_bytes() says how much that
- * needs (0 when there is a single split; never more than a compression of the same shape needs, so one workspace
- * serves both).  Enqueues one or two kernels on `stream`; return codes as for rkv_compress_ex.
+ * holds scores for).  Their partial results may go through desc->workspace (always with fp32 caches; with 8-bit caches and
+ * head_dim 64 where there are many blocks; otherwise they stay in shared memory): rkv_decode_workspace_bytes() says how
+ * much a call asks for (0 when the head-problems fill the GPU by themselves and a block holds a head's scores; never more than
+ * rkv_workspace_bytes() of the same shape, so one workspace serves both).  Enqueues one or two kernels on `stream`; return codes as for rkv_compress_ex.
  */
 RKV_API size_t rkv_decode_workspace_bytes(const rkv_desc_t *desc, int32_t budget, int32_t buffer);
 RKV_API int rkv_decode_attention(const rkv_desc_t *desc, const void *k_cache, const void *v_cache, const void *q_new,

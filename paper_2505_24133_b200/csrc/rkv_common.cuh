@@ -13,7 +13,7 @@
 
 namespace rkv {
 
-constexpr int kHeadDim = 128;   // d of the tensor-core kernels (other head dimensions go through the CUDA-core kernels)
+constexpr int kHeadDim = 128;   // columns of a full operand block of the tensor-core kernels (64 dimensions: half a block, 256: two)
 constexpr int kTile = 128;      // keys per tile (rows of one tensor-core operand tile)
 
 // meta[b] values

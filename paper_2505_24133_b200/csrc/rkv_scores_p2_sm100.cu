@@ -9,7 +9,7 @@
 //
 //   list    The tokens still short of partners (a bit each, kept by the scans) are listed per head, ascending, in chunks of 256 (strag_compact_kernel).
 //   scan    Work item = (head, chunk of 256 listed tokens, window of key tiles): the chunk's key rows are gathered
-//           into two resident operand tiles by the epilogue warps; the window's key tiles stream through a ring, last
+//           into two resident operand tiles by the gather warps; the window's key tiles stream through a ring, last
 //           to first.  The removed entries are subtracted from what the first pass stored, `left` is updated.
 //
 // The first round's window is a few tiles only (kRoundTiles); the tokens that found their partners in it drop out of the next

@@ -1,8 +1,8 @@
 // Stage "select": finishes the scores and picks the kept tokens.  Larger caches, three kernels:
 //
-//   row_stats   one block per (head, row): the maximum and the sum of exponentials of the row's n values, i.e. a softmax in
+//   row_stats   one warp per (head, row): the maximum and the sum of exponentials of the row's n values, i.e. a softmax in
 //               two numbers -- the alpha rows of pooled logits (Eq. 3) and the row of column means (Eq. 6)
-//   importance  one block per (head, 1024 or 2048 tokens): Eq. 4's sliding max over {i-W .. i+W-1} per row (taken on the
+//   importance  eight consecutive tokens per thread (other windows than the default: a block per 1024 tokens of a head): Eq. 4's sliding max over {i-W .. i+W-1} per row (taken on the
 //               logits: exp is monotone, so the max of the weights is the weight of the max), the softmax weight of
 //               that maximum, mean over the alpha rows  -> I;  R of Eq. 6;  Eq. 7  Z = lambda I - (1 - lambda) R, left as
 //               an order-preserving integer key

@@ -186,9 +186,9 @@ def test_append_rows_of_one_block(rkv, hkv, head_dim, dtype):  # noqa: F811
     assert int(comp.status.item()) == 1              # the full cache was reported
 
 
-@pytest.mark.parametrize("batch", [7, 17])
+@pytest.mark.parametrize("batch", [7, 9, 17])
 def test_host_buffers_in_pieces(rkv, batch):  # noqa: F811
-    """The host-buffer form cuts larger batches into pieces of whole sequences: uneven pieces (33 and 80 MB of caches), two
+    """The host-buffer form cuts larger batches into pieces of whole sequences: one piece (33 MB of caches), uneven ones (42 and 80), two
     calls in a row on the same buffers' copies, ragged lengths, per-sequence budgets."""
     spec = small_spec("pieces", batch=batch, hkv=8, hq=16, budget=1024, buffer=128, span=32)
     lens = [spec.cap - 9 * (b % 5) for b in range(batch)]
@@ -196,12 +196,12 @@ def test_host_buffers_in_pieces(rkv, batch):  # noqa: F811
     budgets = torch.tensor([spec.budget - 13 * (b % 3) for b in range(batch)])
     wl = ri.make_workload(spec, device="cuda", seed=431, seq_lens=torch.tensor(lens))
     ch = rkv.Compressor(batch, 8, 16, spec.budget, spec.buffer, 8, 0.1, host_staging=True, budgets=budgets)
+    sets = [[t.cpu().pin_memory() for t in (wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens)] for _ in range(2)]
     got = []
-    for _ in range(2):
-        hk, hv, hq, hs = (t.cpu().pin_memory() for t in (wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens))
-        hidx = torch.empty(batch, 8, spec.budget, dtype=torch.int32).pin_memory()
+    for hk, hv, hq, hs in sets:                     # (nothing between the calls waits for the GPU)
+        got.append((hk, hv, hs, torch.empty(batch, 8, spec.budget, dtype=torch.int32, pin_memory=True)))
+    for (hk, hv, hq, hs), (_, _, _, hidx) in zip(sets, got):
         ch.compress_host(hk, hv, hq, hs, hidx)
-        got.append((hk, hv, hs, hidx))
     cd = rkv.Compressor(batch, 8, 16, spec.budget, spec.buffer, 8, 0.1, budgets=budgets)
     idx = cd.compress(wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens)
     torch.cuda.synchronize()
