@@ -289,6 +289,7 @@ int host_layout(const rkv_desc_t *d, int budget, int buffer, int alpha, HostLayo
 constexpr int kMaxPieces = 8;
 struct HostPipe {
     int dev = -1;
+    unsigned long long context = 0ull;      // its streams live and die with it
     cudaStream_t up = nullptr, down = nullptr;
     cudaEvent_t ev[3 * kMaxPieces + 2] = {};
     cudaStream_t user = nullptr;            // the stream of the call that used it last, and that call's thread (the handles of the
@@ -298,6 +299,7 @@ struct HostPipe {
     bool open(int device)
     {
         dev = device;
+        context = context_id();
         bool ok = cudaStreamCreateWithFlags(&up, cudaStreamNonBlocking) == cudaSuccess &&
                   cudaStreamCreateWithFlags(&down, cudaStreamNonBlocking) == cudaSuccess;
         for (cudaEvent_t &x : ev)
@@ -347,11 +349,12 @@ public:
 private:
     std::unique_ptr<HostPipe> find(int dev, cudaStream_t s)
     {
+        const unsigned long long context = context_id();
         std::lock_guard<std::mutex> guard(lock_);
         for (auto &x : free_)
-            if (x && x->dev == dev && x->last_used_by(s)) return std::move(x);
+            if (x && x->dev == dev && x->context == context && x->last_used_by(s)) return std::move(x);
         for (auto &x : free_)
-            if (x && x->dev == dev && x->idle()) return std::move(x);
+            if (x && x->dev == dev && x->context == context && x->idle()) return std::move(x);
         return nullptr;
     }
     std::mutex lock_;

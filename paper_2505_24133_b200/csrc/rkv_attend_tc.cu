@@ -463,7 +463,7 @@ template <int G, int kSrc>
 cudaError_t launch_tc_one(const AttendTcParams &p, int heads, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
                           cudaStream_t s)
 {
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess || (e = allow_smem_once(done, dev, attend_tc_kernel<G, kSrc>, kTcSmem, true)) != cudaSuccess) return e;

@@ -2,6 +2,7 @@
 // Nothing here is part of the public ABI (see include/rkv.h).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 #include <cuda_runtime.h>
@@ -258,16 +259,34 @@ inline cudaError_t device_sms(int *dev, int *sms)
     if (e == cudaSuccess && slot) known[*dev].store(*sms, std::memory_order_relaxed);
     return e;
 }
-// The kernel's dynamic shared memory limit (and clusters of more than 8 blocks), set once per device.  `done`: the caller's
-// bit per device.
-template <class Kernel>
-inline cudaError_t allow_smem_once(std::atomic<unsigned long long> &done, int dev, Kernel kernel, int bytes, bool wide_cluster = false)
+// The id of the calling thread's current context, 0 where the driver cannot tell.  Ids are never used again, unlike handles: what
+// belongs to a context (function attributes, streams) is kept under its id.
+inline unsigned long long context_id()
 {
-    const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
-    if (bit && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
+    typedef CUresult (*GetId)(CUcontext, unsigned long long *);
+    static const GetId get = []() -> GetId {
+        void *sym = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const bool ok = cudaGetDriverEntryPoint("cuCtxGetId", &sym, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess;
+        return ok ? reinterpret_cast<GetId>(sym) : nullptr;
+    }();
+    unsigned long long id = 0ull;
+    return get && get(nullptr, &id) == CUDA_SUCCESS ? id : 0ull;
+}
+// The kernel's dynamic shared memory limit (and clusters of more than 8 blocks), set once per context.  `done`: the context that the
+// caller's kernel was last prepared for, per device.
+struct PerDevice {
+    std::atomic<unsigned long long> context[kDeviceSlots] = {};
+};
+template <class Kernel>
+inline cudaError_t allow_smem_once(PerDevice &done, int dev, Kernel kernel, int bytes, bool wide_cluster = false)
+{
+    const bool slot = dev >= 0 && dev < kDeviceSlots;
+    const unsigned long long context = slot ? context_id() : 0ull;
+    if (context && done.context[dev].load(std::memory_order_relaxed) == context) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess && wide_cluster) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    if (e == cudaSuccess && context) done.context[dev].store(context, std::memory_order_relaxed);
     return e;
 }
 

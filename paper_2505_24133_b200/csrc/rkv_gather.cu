@@ -203,7 +203,7 @@ cudaError_t launch_gather_for(const Params &p, cudaStream_t s)
     // writing less often.
     if constexpr (kVecPerRow == 16)
         if (streams >= 4096u) return launch_early(gather_kernel<kVecPerRow, 1>, streams, kGatherThreads, 0, s, 1, p);
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     if ((e = allow_smem_once(done, dev, gather_bulk_kernel<kVecPerRow * 16>, kBulkSmem)) != cudaSuccess) return e;
     return launch_early(gather_bulk_kernel<kVecPerRow * 16>, std::min(streams, (unsigned)sms), kBulkThreads, (size_t)kBulkSmem, s, 1, p,
                         (int)streams);

@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(D) head_sum_kernel(Params p)
 template <typename T, int D>
 static cudaError_t launch_prep_for(const Params &p, int dev, cudaStream_t s)
 {
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     const unsigned grid = (unsigned)p.tiles * (unsigned)(p.batch * p.hkv);
     const int smem = kTile * D * (int)sizeof(T) + 16;
     const cudaError_t e = allow_smem_once(done, dev, prep_kernel<T, D>, smem);
@@ -740,7 +740,7 @@ static cudaError_t launch_prep_for(const Params &p, int dev, cudaStream_t s)
 template <int D>
 static cudaError_t launch_prep_tc_for(const Params &p, int dev, int sms, cudaStream_t s)
 {
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     CUtensorMap map_k;
     if (!sm100::make_map_rows(&map_k, p.k_cache, sm100::key_rows_total(p), D, kTile)) return cudaErrorInvalidValue;
     cudaError_t e = allow_smem_once(done, dev, prep_tc_kernel<D>, kPrepTcSmem);
@@ -762,7 +762,7 @@ cudaError_t launch_prep(const Params &p, cudaStream_t s)
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess) return e;
     if (p.fused_codes) {                    // the tensor-core form that also writes the scoring copy
-        static std::atomic<unsigned long long> done{0ull};
+        static PerDevice done;
         const int total = p.tiles * p.batch * p.hkv;
         const uint64_t wide_rows = (uint64_t)p.batch * p.hkv * p.cap + kTile;
         const uint64_t src_rows = p.fuse_table ? (uint64_t)p.pool_pages * kTile : (uint64_t)p.batch * p.hkv * p.cap;

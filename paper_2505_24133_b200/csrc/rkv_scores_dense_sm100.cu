@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
 template <int D>
 static cudaError_t launch_dense_for(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns)
 {
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_dense_sm100_kernel<D>, LayD<D>::kSmemBytesD)) != cudaSuccess) return e;

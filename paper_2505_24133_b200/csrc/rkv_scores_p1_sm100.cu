@@ -533,7 +533,7 @@ static cudaError_t launch_pass1_for(const Params &p, cudaStream_t s, const CUten
     const SmemPlan pl = make_plan<D>(q_rows_pad);
     if (pl.stages < 2) return cudaErrorInvalidConfiguration;
     // (how much shared memory a call needs depends on its query group: the most that any may need is allowed once)
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D, kPlain, kOne, kMany>, kSmemLimit)) != cudaSuccess) return e;

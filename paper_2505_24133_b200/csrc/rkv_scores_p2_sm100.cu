@@ -692,7 +692,7 @@ static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
         !make_map_k16(&map_ts, p.thr_split, (uint64_t)p.batch * p.hkv * kTile))
         return cudaErrorInvalidValue;
     cudaError_t e;
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     int dev = 0, sms = 0;
     if ((e = device_sms(&dev, &sms)) != cudaSuccess || (e = allow_smem_once(done, dev, scores_pass2_sm100_kernel<D, kOne>, Lay<D>::kSmemBytes)) != cudaSuccess)
         return e;

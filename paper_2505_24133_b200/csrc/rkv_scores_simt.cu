@@ -213,7 +213,7 @@ template <typename T, int D, int kRowsT>
 cudaError_t launch_simt_rows(const Params &p, int dev, cudaStream_t s)
 {
     using S = SimtShape<D, kRowsT>;
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     const int row_blocks = (p.cap + S::kRowsA - 1) / S::kRowsA, key_blocks = (p.cap + S::kCols - 1) / S::kCols;
     const unsigned grid = (unsigned)(row_blocks + key_blocks) * (unsigned)(p.batch * p.hkv);
     const cudaError_t e = allow_smem_once(done, dev, scores_simt_kernel<T, D, kRowsT>, S::kBytes);

@@ -357,7 +357,7 @@ template <int kBlocks>
 cudaError_t launch_blocks(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q, unsigned grid,
                           int row_blocks, int q_rows_pad)
 {
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_sm100_kernel<kBlocks>, Smem<kBlocks>::kBytes)) != cudaSuccess) return e;

@@ -597,7 +597,7 @@ static cudaError_t launch_select_mean(const Params &p, cudaStream_t s)
 template <int kThreads>
 static cudaError_t launch_fused(const Params &p, unsigned heads, int dev, cudaStream_t s)
 {
-    static std::atomic<unsigned long long> done{0ull};
+    static PerDevice done;
     const cudaError_t e = allow_smem_once(done, dev, select_fused_kernel<kThreads>, (int)kFusedSmemLimit);
     if (e != cudaSuccess) return e;
     return launch_early(select_fused_kernel<kThreads>, heads, kThreads, (size_t)(p.alpha + 2) * p.cap_pad * sizeof(float), s, 1, p);

@@ -332,3 +332,52 @@ def test_first_pass_partners_of_a_chunk(rkv, head_dim, beta, T):  # noqa: F811
     rep, comp = run_and_check(rkv, wl, beta=beta, T=T)
     assert rep.ok(), rep.errors
     comp.check_status()
+
+
+SECOND_CONTEXT = """
+import ctypes, sys
+import torch
+import paper_2505_24133_b200 as rkv
+cu = ctypes.CDLL("libcuda.so.1")
+P = ctypes.c_void_p
+
+def call():
+    d = rkv.rkv_desc_default()
+    d.batch, d.n_kv_heads, d.n_q_heads = 2, 4, 8
+    need, cap = rkv.rkv_workspace_bytes(d, 300, 84, 8), 384
+
+    def device(nbytes, fill=0x3f):
+        p = P()
+        assert cu.cuMemAlloc_v2(ctypes.byref(p), ctypes.c_size_t(nbytes)) == 0 and cu.cuMemsetD8_v2(p, ctypes.c_ubyte(fill), ctypes.c_size_t(nbytes)) == 0
+        return p.value
+    d.workspace, d.workspace_bytes = device(need, 0), need
+    k, v, q, idx = device(8 * cap * 256), device(8 * cap * 256), device(2 * 8 * 8 * 256), device(8 * 300 * 4)
+    lens = device(8, 0)
+    assert cu.cuMemsetD32_v2(P(lens), ctypes.c_uint(cap), ctypes.c_size_t(2)) == 0
+    out = device(2 * 8 * 128 * 4)
+    rc = rkv.rkv_compress_stages(d, k, v, q, lens, 300, 84, 8, 0.1, idx, 0)
+    rc2 = rkv.rkv_decode_attention(d, k, v, q, lens, out, 300, 84, 0)
+    assert cu.cuCtxSynchronize() == 0
+    got = (ctypes.c_int * 2)()
+    assert cu.cuMemcpyDtoH_v2(got, P(lens), ctypes.c_size_t(8)) == 0
+    return rc, rc2, list(got)
+
+torch.zeros(1, device="cuda")                       # the primary context
+first = call()
+ctx, dev = P(), ctypes.c_int()
+assert cu.cuDeviceGet(ctypes.byref(dev), 0) == 0 and cu.cuCtxCreate_v2(ctypes.byref(ctx), 0, dev) == 0
+second = call()
+print(first, second)
+sys.exit(0 if first == second == (0, 0, [300, 300]) else 1)
+"""
+
+
+def test_calls_in_a_second_context_of_the_device(rkv):  # noqa: F811
+    """Function attributes belong to a context: kernels prepared in one are prepared again in another."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", SECOND_CONTEXT], cwd=root, capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, PYTHONPATH=root))
+    assert r.returncode == 0, r.stdout + r.stderr[-2000:]
