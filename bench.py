@@ -38,8 +38,7 @@ UNIT = "tokens/s"
 # workloads of that cache size; the capture has G = 4, other group sizes differ only in the few KB of queries per head).
 # None = the kernel has changed since the counters were taken.
 NCU_TRAFFIC_PER_HEAD_N4216 = {
-    "prep": 304.14e6 / 256,                   # prep kernel + the per-head key sums
-    "scores_pass1": 336.94e6 / 256, "scores_list": 0.16e6 / 256,
+    "prep": None, "scores_pass1": None, "scores_list": 0.16e6 / 256,
     "scores_pass2": 348.08e6 / 256,           # both scans, the second listing and the symmetric route's two launches, as bench.py's interval has them
     "row_stats": 38.95e6 / 256, "importance": 38.98e6 / 256, "select": 4.35e6 / 256, "gather": 1006.17e6 / 256,
 }
@@ -364,23 +363,22 @@ def kernel_table(rkv, timed: Timed, kw, KB, peaks):
     wide_row = spec.head_dim * 2                       # a row of the bf16 scoring copy (8-bit caches)
     P = spec.head_problems
     T = (n + 127) // 128
-    q_cols = -(-(spec.n_q_heads // spec.n_kv_heads) * spec.alpha // 16) * 16 + 16
     # one tile product = 128 x 128 outputs over K = 128 + 16: the head dimension plus the one extra K = 16 step that
     # folds the threshold test into the accumulator (both scoring passes issue it for every key tile)
     tile_flops = 2.0 * 128 * 128 * (spec.head_dim + 16)
     rule_on = comp_ev.desc.beta > 0 and comp_ev.desc.sim_threshold < 1.0
     pass1_tiles = P * T if rule_on else 0              # every row tile meets the last key tile once
-    pass1_flops = pass1_tiles * tile_flops + P * T * 2.0 * 128 * q_cols * spec.head_dim
+    pass1_flops = pass1_tiles * tile_flops + P * T * 2.0 * 128 * 16 * spec.head_dim       # and the key sum's columns
     pass2_flops = max(tiles_executed - pass1_tiles, 0) * tile_flops
     pass2_useful = pairs2 * 2.0 * 128 * (spec.head_dim + 16)     # listed tokens x keys of the streamed tiles x 2 (d + 16)
     # algorithmic work per launch: bytes a kernel has to move / flops it has to execute, nothing it merely could
     work = {
-        # K once; r_i, Kbar_i.Kbar_i and the 16-byte slice out.  8-bit caches: the stored keys in and their bf16 copy out
+        # K once; r_i, Kbar_i.Kbar_i, the 16-byte slice and the pooled logits out.  8-bit caches: the stored keys in and their bf16 copy out
         # (written by the prep kernel itself when a stored row is 128 bytes and the capacity a whole number of tiles;
         # else by a pass of its own, and read back)
-        "prep": ("hbm", P * (n * row + spec.cap * (8 + 16)) if esz > 1 else
-                 (P * (n * row + n * wide_row + spec.cap * (8 + 16)) if (row == 128 and spec.cap % 128 == 0) else
-                  P * (spec.cap * row + spec.cap * wide_row + n * wide_row + spec.cap * (8 + 16)))),
+        "prep": ("hbm", P * (n * row + spec.cap * (24 + 4 * spec.alpha)) if esz > 1 else
+                 (P * (n * row + n * wide_row + spec.cap * (24 + 4 * spec.alpha)) if (row == 128 and spec.cap % 128 == 0) else
+                  P * (spec.cap * row + spec.cap * wide_row + n * wide_row + spec.cap * (24 + 4 * spec.alpha)))),
         "scores_pass1": ("tensor", pass1_flops),
         "scores_list": ("hbm", P * n / 8),                 # a bit per token (and what it lists)
         "scores_pass2": ("tensor", pass2_flops),
@@ -429,7 +427,7 @@ def rooflines(spec, kernels, scoring, peaks):
                     "unit": "TFLOP/s", "frac": k["frac_of_bf16_peak"],
                     "peak_source": f"{peaks['source']} burst cuBLAS bf16",
                     "traffic": traffic(nm), "flops_per_launch": k["flops_per_launch"],
-                    "counts": "128x128x(128+16) tile products the kernel executed (counted by the kernel) + its query products",
+                    "counts": "128x128x(128+16) tile products the kernel executed (counted by the kernel) + the key sum's columns of the first pass",
                     "full_matrix_equivalent_tflops": scoring["full_matrix_equivalent_tflops"],
                     "other_pass": {c: kernels[c]["frac_of_bf16_peak"] for c in cands if c != nm}}
     hbm = {}

@@ -89,8 +89,9 @@ typedef enum { RKV_BF16 = 0, RKV_F32 = 1, RKV_FP8_E4M3 = 2 } rkv_dtype_t;
                                    scored by forming each pair of key tiles once; beta = 1 only).  A cross-check. */
 
 /* stage bits for rkv_compress_stages */
-#define RKV_STAGE_PREP 1u    /* key inverse norms and per-tile sums of normalised keys */
-#define RKV_STAGE_SCORES 2u  /* Eq. 2-3 pooled logits; Eq. 5 matrix + retention rule + Eq. 6 column means */
+#define RKV_STAGE_PREP 1u    /* key inverse norms and per-tile sums of normalised keys; on the two-pass tensor-core route, which reads
+                              * the keys here anyway, Eq. 2-3 pooled logits as well */
+#define RKV_STAGE_SCORES 2u  /* Eq. 2-3 pooled logits (other routes); Eq. 5 matrix + retention rule + Eq. 6 column means */
 #define RKV_STAGE_SELECT 4u  /* Eq. 3 softmax, Eq. 4, Eq. 6 softmax, Eq. 7, top-k, index list */
 #define RKV_STAGE_GATHER 8u  /* in-place compaction of K and V, seq_lens update */
 #define RKV_STAGE_ALL 15u

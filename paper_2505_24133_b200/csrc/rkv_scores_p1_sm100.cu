@@ -1,29 +1,30 @@
-// Stage "scores", first pass, for bf16 caches: every candidate token against the observation queries (Eq. 2-3) and
-// against the LAST key tile of its head (Eq. 5 and the start of Section 3.3's scan, which runs from the last position
-// downwards).  tcgen05.mma with TMEM accumulators, fed by TMA, one persistent block per SM.
+// Stage "scores", first pass, for bf16 caches of 64 and 128 dimensions: every candidate token against the LAST key tile of its head
+// (Eq. 5 and the start of Section 3.3's scan, which runs from the last position downwards) and against the head's key sum (Eq. 6).
+// tcgen05.mma with TMEM accumulators, fed by TMA, one persistent block per SM.
 //
 // The pass is a single sweep over the keys, so it is organised as a stream: the 128-row key tiles of a head flow
 // through a ring of shared-memory stages as the A operand (one token per TMEM lane), while ONE B operand block of the
-// head stays put: the rows of its last key tile, then its G * alpha query rows, then 16 rows that hold sum_j Kbar_j
-// split into bf16 parts.  Per streamed tile the tensor cores form one product of N = 128 + query rows + 16 (a product
-// with few columns costs nearly as much as one with 128), plus one K = 16 step on the key columns that folds the
+// head stays put: the rows of its last key tile, then 16 rows that hold sum_j Kbar_j split into bf16 parts.  Per streamed tile the
+// tensor cores form one product of N = 128 + 16, plus one K = 16 step on the key columns that folds the
 // threshold test into the accumulator (slices of both operands written by the prep stage):
 //
 //   columns [0, 128)         h = k_i . k_j - T / (r_i r_j) for the 128 keys j of the last tile: S[j][i] > T exactly
 //                            when h > 0.  The thread that owns token i scans them from the last position downwards,
 //                            "the first beta hits" are Section 3.3's partners; a partner's value is T + h r_i r_j
-//   columns [128, 128 + q)   k_i . q for every query row (a thread ends up with all logits of its key and takes the max,
-//                            or the mean, over the group: Eq. 3), then k_i . s in three parts, which gives
-//                            sum_j S[j][i] = Kbar_i . (sum_j Kbar_j) - Kbar_i . Kbar_i without forming the matrix
+//   columns [128, 144)       k_i . s in three parts, which gives sum_j S[j][i] = Kbar_i . (sum_j Kbar_j) - Kbar_i . Kbar_i without
+//                            forming the matrix
 //
-// Out, per token: the pooled logits, the column sum minus the removed entries (sbar), the partners still lacking (a bit, and for beta > 1 how many).
+// Out, per token: the column sum minus the removed entries (sbar), the partners still lacking (a bit, and for beta > 1 how many).
+//
+// What bounds it: with 128 dimensions the keys' bytes (4096 heads of 4216 tokens: 792 us for 5.0 GB), with 64 the integer instructions
+// of the screening (8192 heads of 2168 tokens: 573).  While the query rows rode in the B block too (the logits are the prep stage's
+// now) the product had 128 + G alpha + 16 columns, so that only two accumulators fitted, and the epilogue formed the logits: 994 and 786.
 //
 // Work item = (head, range of row tiles); items are handed out by a global ticket counter, head-major.  The operands
-// that stay put are double-buffered across items, so the next item's arrive while the current one is streamed, and
-// the ring never drains at an item boundary.
-// Warp roles (320 threads): warp 0 = tickets + TMA producer, warp 1 = MMA issuer and TMEM owner, warps 2..9 = epilogue
-// in two groups of four (warp w may touch TMEM lanes 32 (w % 4) .. +31); group g drains accumulator buffer g, i.e.
-// every second tile of the stream.  Every wait on an mbarrier is bounded; on expiry the block records
+// that stay put are double-buffered across items, so the next item's copies run under the current item's products.
+// Warp roles (448 threads): warp 0 = tickets + TMA producer, warp 1 = MMA issuer and TMEM owner, warps 2..13 = epilogue
+// in three groups of four (warp w may touch TMEM lanes 32 (w % 4) .. +31); group g drains accumulator buffer g, i.e.
+// every third tile of the stream.  Every wait on an mbarrier is bounded; on expiry the block records
 // RKV_ERR_TIMEOUT, stops issuing work and leaves through the common exit that frees TMEM.  No TMA multicast, no
 // cluster launch.
 #include "rkv_sm100.cuh"
@@ -34,82 +35,68 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kThreadsP1 = 320;
 constexpr int kHalfBytes = kTile * 64 * 2;       // one TMA box: 128 rows x 64 bf16 (128-byte swizzled rows)
 constexpr int kSliceBytes = kTile * 32;          // the extra K = 16 slice of an operand: 128 rows x 32 bytes (32-byte swizzle)
 constexpr int kMaxStagesA = 8;
 constexpr int kMostTurns = 4;                    // partners of a chunk that are taken out one by one
-constexpr uint32_t kTmemColsP1 = 512;            // 2 buffers x (128 key columns + up to 128 query columns)
+constexpr uint32_t kGroups = 3;                  // accumulator buffers, and the groups of four epilogue warps that drain one each
+constexpr uint32_t kAccCols = 160;               // 128 key columns + 16, up to a multiple of 32
+constexpr uint32_t kTmemColsP1 = 512;
+static_assert(kGroups * kAccCols <= kTmemColsP1, "TMEM columns");
+constexpr int kThreadsP1 = 64 + 128 * (int)kGroups;
 constexpr int kSmemLimit = 227 * 1024;
 
 enum {
     kBarSlotFull = 0,                            // [2] item descriptor written and its resident operands landed
-    kBarSlotEmpty = kBarSlotFull + 2,            // [2] ... no longer read: the MMA thread and the 8 epilogue warps
+    kBarSlotEmpty = kBarSlotFull + 2,            // [2] ... no longer read: the MMA thread and the epilogue warps
     kBarAFull = kBarSlotEmpty + 2,               // [kMaxStagesA] streamed tile landed
     kBarAEmpty = kBarAFull + kMaxStagesA,        // [kMaxStagesA] ... and consumed by the products
-    kBarAccFull = kBarAEmpty + kMaxStagesA,      // [2] accumulator buffer written
-    kBarAccEmpty = kBarAccFull + 2,              // [2] ... and drained by its 4 epilogue warps
-    kNumBarsP1 = kBarAccEmpty + 2
+    kBarAccFull = kBarAEmpty + kMaxStagesA,      // [kGroups] accumulator buffer written
+    kBarAccEmpty = kBarAccFull + 3,              // [kGroups] ... and drained by its 4 epilogue warps
+    kNumBarsP1 = kBarAccEmpty + 3
 };
 
-// Shared-memory carve-up, offsets from a 1024-byte aligned base.
-struct SmemPlan {
-    int stages;          // ring depth
-    int q_bytes;         // bytes of the query block: (q_rows_pad + 16) rows
-    int off_aug;         // stages x slice of a streamed tile
-    int off_slot;        // 2 x [B block: rows [0, 128) the last key tile, then the query block; as 64-column boxes, one
-                         //      behind the other | slice of the last key tile]
-    int slot_bytes;      // (128 + q_rows_pad + 16) rows; with 128 dimensions a 64-column half is slot_bytes / 2
-    int slot_stride;     // slot_bytes + kSliceBytes
-    int off_rj;          // 2 x 128 floats: r_j of the last key tile
-    int off_bar, off_items, off_misc, total;
-};
-
+// Shared memory (offsets from a 1024-byte aligned base).
 template <int D>
-__host__ __device__ inline SmemPlan make_plan(int q_rows_pad)
-{
-    constexpr int kTileBytes = kTile * D * 2;
-    SmemPlan pl;
-    pl.q_bytes = (q_rows_pad + 16) * D * 2;
-    pl.slot_bytes = kTileBytes + pl.q_bytes;
-    pl.slot_stride = pl.slot_bytes + kSliceBytes;
-    const int fixed = 2 * pl.slot_stride + 2 * kTile * 4 + kNumBarsP1 * 8 + 2 * 16 + 16 + 1024;   // + alignment slack
-    int stages = (kSmemLimit - fixed) / (kTileBytes + kSliceBytes);
-    pl.stages = stages > kMaxStagesA ? kMaxStagesA : stages;
-    pl.off_aug = pl.stages * kTileBytes;
-    pl.off_slot = pl.off_aug + pl.stages * kSliceBytes;
-    pl.off_rj = pl.off_slot + 2 * pl.slot_stride;
-    pl.off_bar = pl.off_rj + 2 * kTile * 4;
-    pl.off_items = pl.off_bar + kNumBarsP1 * 8;
-    pl.off_misc = pl.off_items + 2 * 16;
-    pl.total = pl.off_misc + 16 + 1024;
-    return pl;
-}
+struct Lay {
+    static constexpr int kTileBytes = kTile * D * 2;                   // an operand tile: one 64-column box or two
+    // B block: rows [0, 128) the last key tile, then 16 rows of the key sum; as 64-column boxes, one behind the other; then the slice
+    // of the last key tile
+    static constexpr int kSumBytes = 16 * D * 2, kSlotBytes = kTileBytes + kSumBytes, kBoxBytes = kSlotBytes / (D / 64);
+    static constexpr int kSlotStride = kSlotBytes + kSliceBytes;
+    static constexpr int kFixed = 2 * (kSlotStride + kTile * 4) + kNumBarsP1 * 8 + 2 * 16 + 32 + 1024;      // + alignment slack
+    static constexpr int kFit = (kSmemLimit - kFixed) / (kTileBytes + kSliceBytes);
+    static constexpr int kStages = kFit > kMaxStagesA ? kMaxStagesA : kFit;                                // ring depth
+    static constexpr int kOffAug = kStages * kTileBytes;               // a slice per stage
+    static constexpr int kOffSlot = kOffAug + kStages * kSliceBytes;   // 2 B blocks
+    static constexpr int kOffRj = kOffSlot + 2 * kSlotStride;          // 2 x 128 floats: r_j of the last key tile
+    static constexpr int kOffBar = kOffRj + 2 * kTile * 4;
+    static constexpr int kOffItems = (kOffBar + kNumBarsP1 * 8 + 15) / 16 * 16;
+    static constexpr int kOffMisc = kOffItems + 2 * 16;
+    static constexpr int kBytes = kOffMisc + 16 + 1024;
+    static_assert(kBoxBytes % 1024 == 0 && kBytes <= kSmemLimit, "shared memory");
+};
 
 // Item descriptor (int4): {head, first row tile, one past the last row tile, n}.  x < 0: no more items.
-// kPlain: alpha = 8, the maximum over the group, the retention rule on -- the defaults -- without the code of the other
-// forms: the roles share the instruction cache (4096 heads of 4216 tokens: 1036 us with it, 992 without).
-// kOne: beta = 1 as well.  kMany: beta > kMostTurns, the form that can also take a chunk's partners out in one sum (4096 heads of 4216
-// tokens: beta = 8 1960 us without it, beta = 16 2200; beta = 2 and 3, which never need it, 1238 and 1424, 1320 and 1492 with it).
-template <int D, bool kPlain, bool kOne, bool kMany>
+// kRule: the retention rule is on.  kOne: beta = 1.  kMany: beta > kMostTurns, the form that can also take a chunk's partners out in one sum
+// (each without the others' code: the roles share the instruction cache).
+template <int D, bool kRule, bool kOne, bool kMany>
 __global__ void __launch_bounds__(kThreadsP1, 1)
-scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,
-                           const __grid_constant__ CUtensorMap map_hs, const __grid_constant__ CUtensorMap map_ns,
-                           const __grid_constant__ CUtensorMap map_ts, int splits, unsigned long long total_items,
-                           int q_rows_pad)
+scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_hs,
+                           const __grid_constant__ CUtensorMap map_ns, const __grid_constant__ CUtensorMap map_ts, int splits,
+                           unsigned long long total_items)
 {
+    using L = Lay<D>;
+    constexpr uint32_t kStages = L::kStages;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = align_smem(smem_raw);
     const uint32_t sbase = smem_u32(smem);
-    constexpr int kTileBytes = kTile * D * 2;        // an operand tile: one 64-column box or two
-    const SmemPlan pl = make_plan<D>(q_rows_pad);
-    int4 *items = reinterpret_cast<int4 *>(smem + pl.off_items);
-    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + pl.off_misc);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + pl.off_misc + 4);
-    volatile int *bail = reinterpret_cast<volatile int *>(smem + pl.off_misc + 8);
-    const uint32_t bar0 = sbase + pl.off_bar;
-    auto bar = [bar0](int idx) -> uint32_t { return bar0 + 8u * (uint32_t)idx; };
-    const int stages = pl.stages;
+    int4 *items = reinterpret_cast<int4 *>(smem + L::kOffItems);
+    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + L::kOffMisc);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L::kOffMisc + 4);
+    volatile int *bail = reinterpret_cast<volatile int *>(smem + L::kOffMisc + 8);
+    const uint32_t bar0 = sbase + L::kOffBar;
+    auto bar = [bar0](uint32_t idx) -> uint32_t { return bar0 + 8u * idx; };
 
     // Once a bounded wait of this call has run out, the blocks still to start return at once.
     const ErrSink sink = make_sink(p);
@@ -119,12 +106,12 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
     if (*bail) return;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool rule_on = kPlain || (p.beta > 0 && p.sim_threshold < 1.0f);
-
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
             mbar_init(bar(kBarSlotFull + s), 1);
-            mbar_init(bar(kBarSlotEmpty + s), 9);
+            mbar_init(bar(kBarSlotEmpty + s), 1 + 4 * kGroups);
+        }
+        for (uint32_t s = 0; s < kGroups; ++s) {
             mbar_init(bar(kBarAccFull + s), 1);
             mbar_init(bar(kBarAccEmpty + s), 4);
         }
@@ -168,47 +155,38 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 const uint32_t slot = k_item & 1;
                 if (!mbar_wait(bar(kBarSlotEmpty + slot), ((k_item >> 1) & 1) ^ 1, abort_flag, sink)) break;
                 items[slot] = make_int4(head, t0, t1, n);
-                const uint32_t slot_addr = sbase + pl.off_slot + slot * pl.slot_stride;
+                const uint32_t slot_addr = sbase + L::kOffSlot + slot * L::kSlotStride;
                 const uint32_t full = bar(kBarSlotFull + slot);
                 // the descriptor is published by this arrival; the barrier completes when the operands have landed too
-                mbar_expect_tx(full, (uint32_t)pl.q_bytes + (rule_on ? (uint32_t)(kTileBytes + kSliceBytes + kTile * 4) : 0u));
-                {
-                    const int b = head / p.hkv, h = head % p.hkv;
-                    const int q_row = (b * p.hq + h * p.group) * p.alpha;
-                    const uint32_t half = (uint32_t)pl.slot_bytes / 2, qdst = slot_addr + kTile * 128;
-                    // behind the key tile's rows: the query rows, then 16 rows holding sum_j Kbar_j split into bf16
-                    // parts; every 64-column box
+                mbar_expect_tx(full, (uint32_t)L::kSumBytes + (kRule ? (uint32_t)(L::kTileBytes + kSliceBytes + kTile * 4) : 0u));
+                // behind the key tile's rows: 16 rows holding sum_j Kbar_j split into bf16 parts; every 64-column box
 #pragma unroll
-                    for (int x = 0; x < D / 64; ++x) {
-                        tma_load_2d(qdst + x * half, &map_q, x * 64, q_row, full);
-                        tma_load_2d(qdst + x * half + q_rows_pad * 128, &map_hs, x * 64, head * 16, full);
-                    }
-                }
-                if (rule_on) {
+                for (int x = 0; x < D / 64; ++x) tma_load_2d(slot_addr + x * L::kBoxBytes + kTile * 128, &map_hs, x * 64, head * 16, full);
+                if (kRule) {
                     const int y = (int)tile_row0(p, head, n_tiles - 1);
-                    tma_load_2d(slot_addr, &map_k, 0, y, full);
-                    if (D == 128) tma_load_2d(slot_addr + (uint32_t)pl.slot_bytes / 2, &map_k, 64, y, full);
+#pragma unroll
+                    for (int x = 0; x < D / 64; ++x) tma_load_2d(slot_addr + x * L::kBoxBytes, &map_k, x * 64, y, full);
                     // the tile's extra slice: -T / r_j of its keys in three bf16 parts
-                    tma_load_2d(slot_addr + (uint32_t)pl.slot_bytes, &map_ts, 0, head * kTile, full);
+                    tma_load_2d(slot_addr + L::kSlotBytes, &map_ts, 0, head * kTile, full);
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(sbase + pl.off_rj + slot * kTile * 4),
+                                 ::"r"(sbase + L::kOffRj + slot * kTile * 4),
                                    "l"(p.inv_norm + (size_t)head * p.cap_pad + (size_t)(n_tiles - 1) * kTile),
                                    "r"((uint32_t)(kTile * 4)), "r"(full)
                                  : "memory");
                 }
                 for (int t = t0; t < t1; ++t) {
-                    const uint32_t s = acount % (uint32_t)stages;
-                    if (!mbar_wait(bar(kBarAEmpty + s), ((acount / (uint32_t)stages) & 1) ^ 1, abort_flag, sink)) {
+                    const uint32_t s = acount % kStages;
+                    if (!mbar_wait(bar(kBarAEmpty + s), ((acount / kStages) & 1) ^ 1, abort_flag, sink)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t dst = sbase + s * kTileBytes;
+                    const uint32_t dst = sbase + s * L::kTileBytes;
                     const int y = (int)tile_row0(p, head, t);
-                    mbar_expect_tx(bar(kBarAFull + s), kTileBytes + (rule_on ? kSliceBytes : 0));
+                    mbar_expect_tx(bar(kBarAFull + s), L::kTileBytes + (kRule ? kSliceBytes : 0));
                     tma_load_2d(dst, &map_k, 0, y, bar(kBarAFull + s));
                     if (D == 128) tma_load_2d(dst + kHalfBytes, &map_k, 64, y, bar(kBarAFull + s));
-                    if (rule_on)    // the tile's extra slice: 1 / r_i of its keys in three bf16 parts
-                        tma_load_2d(sbase + pl.off_aug + s * kSliceBytes, &map_ns, 0, head * p.cap_pad + t * kTile,
+                    if (kRule)      // the tile's extra slice: 1 / r_i of its keys in three bf16 parts
+                        tma_load_2d(sbase + L::kOffAug + s * kSliceBytes, &map_ns, 0, head * p.cap_pad + t * kTile,
                                     bar(kBarAFull + s));
                     ++acount;
                 }
@@ -228,9 +206,8 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            // one product per streamed tile: N = the 128 keys of the last tile + the query block (the query block alone
-            // while the retention rule is off)
-            const uint32_t idesc_kq = instr_desc(kTile, kTile + q_rows_pad + 16), idesc_q = instr_desc(kTile, q_rows_pad + 16);
+            // one product per streamed tile: N = the 128 keys of the last tile + the key sum (that alone while the rule is off)
+            const uint32_t idesc_ks = instr_desc(kTile, kTile + 16), idesc_s = instr_desc(kTile, 16);
             const uint32_t idesc_k = instr_desc(kTile, kTile);
             uint32_t k_item = 0, acount = 0;
             bool ok = true;
@@ -239,30 +216,30 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 if (!mbar_wait(bar(kBarSlotFull + slot), (k_item >> 1) & 1, abort_flag, sink)) break;
                 const int4 d = items[slot];
                 if (d.x < 0) break;
-                const uint32_t b_block = sbase + pl.off_slot + slot * pl.slot_stride, b_half = (uint32_t)pl.slot_bytes / 2;
+                const uint32_t b_block = sbase + L::kOffSlot + slot * L::kSlotStride;
                 for (int t = d.y; t < d.z; ++t) {
-                    const uint32_t s = acount % (uint32_t)stages;
-                    if (!mbar_wait(bar(kBarAFull + s), (acount / (uint32_t)stages) & 1, abort_flag, sink)) {
+                    const uint32_t s = acount % kStages;
+                    if (!mbar_wait(bar(kBarAFull + s), (acount / kStages) & 1, abort_flag, sink)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t a = acount & 1;                 // tile c of the stream uses accumulator buffer c & 1
-                    if (!mbar_wait(bar(kBarAccEmpty + a), ((acount >> 1) & 1) ^ 1, abort_flag, sink)) {
+                    const uint32_t a = acount % kGroups;           // tile c of the stream uses accumulator buffer c % kGroups
+                    if (!mbar_wait(bar(kBarAccEmpty + a), ((acount / kGroups) & 1) ^ 1, abort_flag, sink)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t tile = sbase + s * kTileBytes;
-                    const uint32_t d_tmem = tmem_base + a * 256;
-                    if (rule_on) {
-                        if (D == 128) umma_tile_k128_halves(d_tmem, tile, kHalfBytes, b_block, b_half, idesc_kq);
-                        else umma_tile_k64(d_tmem, tile, b_block, idesc_kq);
+                    const uint32_t tile = sbase + s * L::kTileBytes;
+                    const uint32_t d_tmem = tmem_base + a * kAccCols;
+                    if (kRule) {
+                        if (D == 128) umma_tile_k128_halves(d_tmem, tile, kHalfBytes, b_block, L::kBoxBytes, idesc_ks);
+                        else umma_tile_k64(d_tmem, tile, b_block, idesc_ks);
                         // ... - T / (r_i r_j) onto the key columns: the accumulator's sign is the threshold test
-                        umma_k16_sw32(d_tmem, sbase + pl.off_aug + s * kSliceBytes, b_block + (uint32_t)pl.slot_bytes, idesc_k);
+                        umma_k16_sw32(d_tmem, sbase + L::kOffAug + s * kSliceBytes, b_block + L::kSlotBytes, idesc_k);
                         ++tiles_done;
                     } else {
-                        if (D == 128) umma_tile_k128_halves(d_tmem + 128, tile, kHalfBytes, b_block + kTile * 128, b_half, idesc_q);
-                        else umma_tile_k64(d_tmem + 128, tile, b_block + kTile * 128, idesc_q);
+                        if (D == 128) umma_tile_k128_halves(d_tmem + 128, tile, kHalfBytes, b_block + kTile * 128, L::kBoxBytes, idesc_s);
+                        else umma_tile_k64(d_tmem + 128, tile, b_block + kTile * 128, idesc_s);
                     }
                     umma_commit(bar(kBarAccFull + a));
                     umma_commit(bar(kBarAEmpty + s));              // the stage may be refilled once these products have read it
@@ -276,14 +253,10 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
         __syncwarp();
     } else {
         // ------------------------------------------------------------------ epilogue warps
-        const int ew = warp - 2;                 // 0..7
-        const int grp = ew >> 2;                 // accumulator buffer this warp drains
+        const uint32_t grp = (uint32_t)(warp - 2) >> 2;      // accumulator buffer this warp drains
         const int quad = warp & 3;               // TMEM lane quadrant this warp may access
         const int lrow = quad * 32 + lane;       // row within the 128-row tile
-        const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)grp * 256;
-        const float kInf = __int_as_float(0x7f800000);
-        const float scale = p.logit_scale;                    // 1 / sqrt(d)
-        const int G = p.group;
+        const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + grp * kAccCols;
         uint32_t k_item = 0, ccount = 0;         // ccount: tiles of the stream so far (all of them, not only this group's)
         bool ok = true;
 
@@ -296,14 +269,12 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
             const int last_tile = (n + kTile - 1) / kTile - 1;
             const int jbase = last_tile * kTile;
             const float *inv_norm = p.inv_norm + (size_t)head * p.cap_pad;
-            const float *rj = reinterpret_cast<const float *>(smem + pl.off_rj + slot * kTile * 4);
-            float *logits = p.logits + (size_t)head * p.alpha * p.cap_pad;
-
+            const float *rj = reinterpret_cast<const float *>(smem + L::kOffRj + slot * kTile * 4);
             const float *self_dot = p.self_dot + (size_t)head * p.cap_pad;
             float ri_next = 0.f, self_next = 0.f;
             int t_next = -1;                     // the tile ri_next / self_next were fetched for
             for (int t = d.y; t < d.z; ++t, ++ccount) {
-                if ((int)(ccount & 1) != grp) continue;
+                if (ccount % kGroups != grp) continue;
                 const int i = t * kTile + lrow;
                 const bool row_ok = i < n;
                 float ri, self;
@@ -314,73 +285,22 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                     ri = row_ok ? inv_norm[i] : 0.f;
                     self = row_ok ? self_dot[i] : 0.f;
                 }
-                if (t + 2 < d.z) {               // this group's next tile of the item: its factors arrive while this one is drained
-                    const int i2 = i + 2 * kTile;
-                    t_next = t + 2;
+                if (t + (int)kGroups < d.z) {    // this group's next tile of the item: its factors arrive while this one is drained
+                    const int i2 = i + (int)kGroups * kTile;
+                    t_next = t + (int)kGroups;
                     ri_next = i2 < n ? inv_norm[i2] : 0.f;
                     self_next = i2 < n ? self_dot[i2] : 0.f;
                 }
-                if (!mbar_wait(bar(kBarAccFull + grp), (ccount >> 1) & 1, abort_flag, sink)) {
+                if (!mbar_wait(bar(kBarAccFull + grp), (ccount / kGroups) & 1, abort_flag, sink)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
 
-                // ---- Eq. 2-3: all G * alpha logits of this key in its accumulator row, then k_i . s in three parts
-                const uint32_t qbase = lane_base + 128;
+                // ---- Eq. 6 before the retention rule, sum_j S[j][i]: Kbar_i . s (in three parts) - Kbar_i . Kbar_i
                 uint32_t sp[8];
-                tmem_ld8(qbase + q_rows_pad, sp);
-                float pooled[8];
-                if (kPlain || p.alpha == 8) {
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) pooled[j] = !kPlain && p.gqa_mean_pool ? 0.f : -kInf;
-                    for (int g0 = 0; g0 < G; g0 += 4) {       // four query heads per round trip to TMEM
-                        uint32_t t0[8], t1[8], t2[8], t3[8];
-                        tmem_ld8(qbase + g0 * 8, t0);
-                        tmem_ld8(qbase + min(g0 + 1, G - 1) * 8, t1);     // heads beyond the group re-read its last one
-                        tmem_ld8(qbase + min(g0 + 2, G - 1) * 8, t2);
-                        tmem_ld8(qbase + min(g0 + 3, G - 1) * 8, t3);
-                        tmem_wait8(t0);
-                        tmem_wait8(t1);
-                        tmem_wait8(t2);
-                        tmem_wait8(t3);
-                        if (!kPlain && p.gqa_mean_pool) {        // the variant: sum over the group (scaled to the mean below)
-                            const bool h1 = g0 + 1 < G, h2 = g0 + 2 < G, h3 = g0 + 3 < G;
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                pooled[j] += (__uint_as_float(t0[j]) + (h1 ? __uint_as_float(t1[j]) : 0.f)) +
-                                             ((h2 ? __uint_as_float(t2[j]) : 0.f) + (h3 ? __uint_as_float(t3[j]) : 0.f));
-                            continue;
-                        }
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            pooled[j] = fmaxf(fmaxf(pooled[j], __uint_as_float(t0[j])),
-                                              max3(__uint_as_float(t1[j]), __uint_as_float(t2[j]), __uint_as_float(t3[j])));
-                    }
-                    const float scale_q = !kPlain && p.gqa_mean_pool ? scale / (float)G : scale;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) pooled[j] *= scale_q;
-                } else {
-                    for (int j = 0; j < p.alpha; ++j) {
-                        float best = -kInf, sum = 0.f;
-                        for (int g0 = 0; g0 < G; g0 += 4) {
-                            uint32_t tq[4];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) tmem_ld1(qbase + min(g0 + u, G - 1) * p.alpha + j, tq[u]);
-                            asm volatile("tcgen05.wait::ld.sync.aligned;"
-                                         : "+r"(tq[0]), "+r"(tq[1]), "+r"(tq[2]), "+r"(tq[3]) :: "memory");
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                best = fmaxf(best, __uint_as_float(tq[u]));
-                                sum += (g0 + u < G) ? __uint_as_float(tq[u]) : 0.f;
-                            }
-                        }
-                        if (row_ok)      // (written here: alpha is not known at compile time on this path)
-                            logits[(size_t)j * p.cap_pad + i] = p.gqa_mean_pool ? sum * scale / (float)G : best * scale;
-                    }
-                }
+                tmem_ld8(lane_base + 128, sp);
                 tmem_wait8(sp);
-                // sum_j S[j][i] before the retention rule: Kbar_i . s - Kbar_i . Kbar_i
                 const float total = ri * ((__uint_as_float(sp[0]) + __uint_as_float(sp[1])) + __uint_as_float(sp[2])) - self;
 
                 // ---- the last key tile, last position first.  The accumulator holds h = k_i . k_j - T / (r_i r_j):
@@ -389,7 +309,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 float removed = 0.f;             // sum of h r_j over the partners found
                 int nhit = 0;
                 int left = row_ok ? (kOne ? 1 : p.beta) : 0;
-                if (rule_on) {
+                if (kRule) {
                     bool want = left > 0;
                     const int valid = n - jbase;                  // columns [0, valid) of the tile are candidates
                     // 32-column chunks, last first.  The TMEM load of the next chunk is issued before the current one is
@@ -493,14 +413,10 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 if (lane == 0) mbar_arrive(bar(kBarAccEmpty + grp));
 
                 if (row_ok) {
-                    if (kPlain || p.alpha == 8) {
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) logits[(size_t)j * p.cap_pad + i] = pooled[j];
-                    }
                     p.sbar[(size_t)head * p.cap_pad + i] = total - ((float)nhit * p.sim_threshold + removed * ri);
-                    if (!kOne && p.beta > 1 && rule_on) p.left[(size_t)head * p.cap_pad + i] = left;
+                    if (kRule && !kOne && p.beta > 1) p.left[(size_t)head * p.cap_pad + i] = left;
                 }
-                if (rule_on) {                   // the tokens still short of partners, a bit each
+                if (kRule) {                     // the tokens still short of partners, a bit each
                     const unsigned lacking = __ballot_sync(0xffffffffu, left > 0);
                     if (lane == 0) p.lacking[(size_t)head * (p.cap_pad / 32) + t * 4 + quad] = lacking;
                 }
@@ -526,46 +442,38 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
 
 }  // namespace
 
-template <int D, bool kPlain, bool kOne, bool kMany>
-static cudaError_t launch_pass1_for(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q, const CUtensorMap &map_hs,
-                                    const CUtensorMap &map_ns, const CUtensorMap &map_ts, int q_rows_pad)
+template <int D, bool kRule, bool kOne, bool kMany>
+static cudaError_t launch_pass1_for(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_hs, const CUtensorMap &map_ns,
+                                    const CUtensorMap &map_ts)
 {
-    const SmemPlan pl = make_plan<D>(q_rows_pad);
-    if (pl.stages < 2) return cudaErrorInvalidConfiguration;
-    // (how much shared memory a call needs depends on its query group: the most that any may need is allowed once)
     static PerDevice done;
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D, kPlain, kOne, kMany>, kSmemLimit)) != cudaSuccess) return e;
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D, kRule, kOne, kMany>, Lay<D>::kBytes)) != cudaSuccess) return e;
     const int heads = p.batch * p.hkv;
     // a head is cut into parts when there are too few heads to give every SM several items
     int splits = (4 * sms + heads - 1) / heads;
     splits = splits < 1 ? 1 : (splits > p.tiles ? p.tiles : splits);
     const unsigned long long total_items = (unsigned long long)splits * (unsigned long long)heads;
     const unsigned grid = (unsigned)(total_items < (unsigned long long)sms ? total_items : (unsigned long long)sms);
-    return launch_early(scores_stream_sm100_kernel<D, kPlain, kOne, kMany>, grid, kThreadsP1, (size_t)pl.total, s, 1, p, map_k, map_q, map_hs, map_ns, map_ts, splits,
-                        total_items, q_rows_pad);
+    return launch_early(scores_stream_sm100_kernel<D, kRule, kOne, kMany>, grid, kThreadsP1, (size_t)Lay<D>::kBytes, s, 1, p, map_k, map_hs, map_ns, map_ts,
+                        splits, total_items);
 }
 
 template <int D>
-static cudaError_t launch_pass1_form(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q, const CUtensorMap &map_hs,
-                                     const CUtensorMap &map_ns, const CUtensorMap &map_ts, int q_rows_pad)
+static cudaError_t launch_pass1_form(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_hs, const CUtensorMap &map_ns,
+                                     const CUtensorMap &map_ts)
 {
-    const bool plain = p.alpha == 8 && p.beta > 0 && p.sim_threshold < 1.0f && !p.gqa_mean_pool;
-    const bool many = p.beta > kMostTurns;
-    if (!plain)
-        return many ? launch_pass1_for<D, false, false, true>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
-                    : launch_pass1_for<D, false, false, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
-    return p.beta == 1 ? launch_pass1_for<D, true, true, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
-           : many      ? launch_pass1_for<D, true, false, true>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
-                       : launch_pass1_for<D, true, false, false>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
+    if (p.beta < 1 || !(p.sim_threshold < 1.0f)) return launch_pass1_for<D, false, false, false>(p, s, map_k, map_hs, map_ns, map_ts);
+    return p.beta == 1           ? launch_pass1_for<D, true, true, false>(p, s, map_k, map_hs, map_ns, map_ts)
+           : p.beta > kMostTurns ? launch_pass1_for<D, true, false, true>(p, s, map_k, map_hs, map_ns, map_ts)
+                                 : launch_pass1_for<D, true, false, false>(p, s, map_k, map_hs, map_ns, map_ts);
 }
 
-cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q,
-                                      const CUtensorMap &map_hs, const CUtensorMap &map_ns, const CUtensorMap &map_ts, int q_rows_pad)
+cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_hs,
+                                      const CUtensorMap &map_ns, const CUtensorMap &map_ts)
 {
-    return p.d == 64 ? launch_pass1_form<64>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)
-                     : launch_pass1_form<128>(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad);
+    return p.d == 64 ? launch_pass1_form<64>(p, s, map_k, map_hs, map_ns, map_ts) : launch_pass1_form<128>(p, s, map_k, map_hs, map_ns, map_ts);
 }
 
 }  // namespace rkv

@@ -682,11 +682,8 @@ int scores_pass2_rounds(int tiles)
 template <int D, bool kOne>
 static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
 {
-    const int q_rows = p.group * p.alpha;
-    const int q_rows_pad = (q_rows + 15) / 16 * 16;
-    CUtensorMap map_k, map_q, map_hs, map_ns, map_ts;
+    CUtensorMap map_k, map_hs, map_ns, map_ts;
     if (!make_map_rows(&map_k, p.k_cache, key_rows_total(p), D, kTile) ||
-        !make_map_rows(&map_q, p.q_window, (uint64_t)p.batch * p.hq * p.alpha, D, (uint32_t)q_rows_pad) ||
         !make_map_rows(&map_hs, p.head_sum_bf16, (uint64_t)p.batch * p.hkv * 16, D, 16u) ||
         !make_map_k16(&map_ns, p.norm_split, (uint64_t)p.batch * p.hkv * p.cap_pad) ||
         !make_map_k16(&map_ts, p.thr_split, (uint64_t)p.batch * p.hkv * kTile))
@@ -697,7 +694,7 @@ static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
     if ((e = device_sms(&dev, &sms)) != cudaSuccess || (e = allow_smem_once(done, dev, scores_pass2_sm100_kernel<D, kOne>, Lay<D>::kSmemBytes)) != cudaSuccess)
         return e;
     const int heads = p.batch * p.hkv;
-    if ((e = launch_scores_pass1_sm100(p, s, map_k, map_q, map_hs, map_ns, map_ts, q_rows_pad)) != cudaSuccess) return e;
+    if ((e = launch_scores_pass1_sm100(p, s, map_k, map_hs, map_ns, map_ts)) != cudaSuccess) return e;
     if ((e = mark_kernel(p, 0, s)) != cudaSuccess) return e;
     const bool rule_on = p.beta > 0 && p.sim_threshold < 1.0f;
     if (!rule_on || p.tiles < 2) return mark_kernel(p, 1, s);       // nobody can lack partners / the first pass has seen everything

@@ -82,6 +82,12 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+// The tensor map is on its way to where the copies look for it, while the kernel waits for the one before it.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap *map)
+{
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows 128 bytes apart, 8-row groups
 // 1024 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
@@ -378,9 +384,8 @@ inline bool make_map_k16(CUtensorMap *map, const void *base, uint64_t rows)
 }  // namespace sm100
 
 // first scoring pass of the two-pass tensor-core route (its own file); the maps are built by the caller
-cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_q,
-                                      const CUtensorMap &map_hs, const CUtensorMap &map_ns, const CUtensorMap &map_ts,
-                                      int q_rows_pad);
+cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_hs,
+                                      const CUtensorMap &map_ns, const CUtensorMap &map_ts);
 
 // symmetric route of the second pass (its own file)
 cudaError_t launch_scores_dense_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns);
