@@ -373,12 +373,10 @@ def kernel_table(rkv, timed: Timed, kw, KB, peaks):
     pass2_useful = pairs2 * 2.0 * 128 * (spec.head_dim + 16)     # listed tokens x keys of the streamed tiles x 2 (d + 16)
     # algorithmic work per launch: bytes a kernel has to move / flops it has to execute, nothing it merely could
     work = {
-        # K once; r_i, Kbar_i.Kbar_i, the 16-byte slice and the pooled logits out.  8-bit caches: the stored keys in and their bf16 copy out
-        # (written by the prep kernel itself when a stored row is 128 bytes and the capacity a whole number of tiles;
-        # else by a pass of its own, and read back)
-        "prep": ("hbm", P * (n * row + spec.cap * (24 + 4 * spec.alpha)) if esz > 1 else
-                 (P * (n * row + n * wide_row + spec.cap * (24 + 4 * spec.alpha)) if (row == 128 and spec.cap % 128 == 0) else
-                  P * (spec.cap * row + spec.cap * wide_row + n * wide_row + spec.cap * (24 + 4 * spec.alpha)))),
+        # K once; r_i, Kbar_i.Kbar_i, the 16-byte slice and the pooled logits out.  8-bit caches of other than 128 dimensions: their bf16
+        # copy by a pass of its own, which is read back
+        "prep": ("hbm", P * (n * row + spec.cap * (24 + 4 * spec.alpha)) if esz > 1 or spec.head_dim == 128 else
+                 P * (spec.cap * row + spec.cap * wide_row + n * wide_row + spec.cap * (24 + 4 * spec.alpha))),
         "scores_pass1": ("tensor", pass1_flops),
         "scores_list": ("hbm", P * n / 8),                 # a bit per token (and what it lists)
         "scores_pass2": ("tensor", pass2_flops),

@@ -57,9 +57,10 @@ typedef enum {
  *   RKV_BF16, RKV_F32: k_cache, v_cache and q_window all hold that type.
  *   RKV_FP8_E4M3: k_cache and v_cache hold 8-bit E4M3 codes (1 sign bit, 4 exponent bits with bias 7, 3 mantissa bits,
  *     no infinities; one byte per element, rows of head_dim bytes); q_window (and q_new of rkv_push_query) is bf16.
- *     Eq. 1-7 are evaluated on the values the codes stand for: the keys are widened to bf16 (exactly; every E4M3 value
- *     is a bf16 value) into the workspace, which grows by (batch * n_kv_heads * (budget + buffer) + 128) * head_dim * 2
- *     bytes (nothing more for head_dim 64, whose workspace has room for a copy in any case), and every scoring stage runs on that copy as for a bf16 cache.  The compaction moves the stored bytes; no
+ *     Eq. 1-7 are evaluated on the values the codes stand for.  With head_dim 128 the two-pass tensor-core kernels score the codes
+ *     as they are stored; otherwise the keys are widened to bf16 (exactly; every E4M3 value is a bf16 value) into the workspace and
+ *     scored there as for a bf16 cache.  The workspace has room for that copy in either case, (batch * n_kv_heads * (budget + buffer)
+ *     + 128) * head_dim * 2 bytes (for head_dim 64 it has so for bf16 caches too).  The compaction moves the stored bytes; no
  *     scale factor is applied or needed (cosine similarity does not see a per-tensor scale; fold a key scale into
  *     the queries for Eq. 2).  rkv_decode_attention takes this type too (q_new bf16): the codes are widened on their
  *     way to the tensor cores, no copy is kept. */
@@ -108,7 +109,7 @@ typedef struct rkv_desc {
     int32_t n_kv_heads;  /* KV heads per sequence */
     int32_t n_q_heads;   /* query heads; G = n_q_heads / n_kv_heads must be integral (G = 1: Eq. 1) */
     int32_t head_dim;    /* d: 64, 128 or 256.  bf16 caches with d = 64 and 128 are scored by the two-pass tensor-core kernels
-                            as they lie, 8-bit caches on a bf16 copy of their keys in the workspace; d = 256 by a
+                            as they lie, 8-bit caches with d = 128 as well, others on a bf16 copy of their keys in the workspace; d = 256 by a
                             tensor-core kernel that forms the whole similarity matrix; fp32 caches by the CUDA-core kernel (fp32 arithmetic, slower) */
     int32_t dtype;       /* rkv_dtype_t of k_cache and v_cache (and of q_window, except for 8-bit caches: bf16) */
     int32_t pool_w;      /* W of Eq. 4; 0 = no pooling.  Range [0, 64].  Default 4 (the paper prints no value) */

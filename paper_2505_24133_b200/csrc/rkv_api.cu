@@ -28,12 +28,11 @@ struct Layout {
     int cap, cap_pad, tiles, tri;
 };
 
-// The two-pass tensor-core scoring kernels are built for bf16 keys of 64 and 128 dimensions; 8-bit caches use them on a
-// widened copy.  The row-block tensor-core kernel, which forms the whole similarity matrix, takes 256 dimensions, and
+// The two-pass tensor-core scoring kernels are built for bf16 keys of 64 and 128 dimensions and for E4M3 codes of 128; other 8-bit
+// caches use them on a widened copy.  The row-block tensor-core kernel, which forms the whole similarity matrix, takes 256 dimensions, and
 // the others where it is asked for (64 on a copy padded with zeros to 128: dot products and norms do not see the padding);
 // fp32 caches, or a request for it, the CUDA-core kernel.
-// Bytes of a cache element and of a query element.  8-bit caches (E4M3 codes) are scored on a bf16 copy of their keys
-// in the workspace (every E4M3 value is a bf16 value), with bf16 queries.
+// Bytes of a cache element and of a query element.  8-bit caches (E4M3 codes) have bf16 queries.
 size_t cache_esz(const rkv_desc_t *d) { return d->dtype == RKV_BF16 ? 2 : d->dtype == RKV_F32 ? 4 : 1; }
 size_t query_esz(const rkv_desc_t *d) { return d->dtype == RKV_F32 ? 4 : 2; }
 
@@ -54,9 +53,10 @@ bool lengths_ahead(const rkv_desc_t *d) { return d->head_dim == 64 && use_tri(d)
 // Tensor-core scoring of 64 dimensions, by either route.  Its workspace has room for the padded copy, used or not: callers
 // have relied on the size.
 bool tensor64(const rkv_desc_t *d) { return d->head_dim == 64 && !use_simt(d); }
-// The prep kernel writes the copy of the keys itself (instead of a widening pass in front of it): rows of 128 E4M3 codes in
-// caches whose capacity is a whole number of 128-row tiles.
-bool fused_codes(const rkv_desc_t *d, long long cap) { return d->dtype == RKV_FP8_E4M3 && d->head_dim == kHeadDim && cap % kTile == 0; }
+// Rows of 128 E4M3 codes are scored as they are stored on the two-pass route.  For the other routes the prep kernel writes the widened
+// copy itself (instead of a widening pass in front of it) where the capacity is a whole number of 128-row tiles.
+bool direct_codes(const rkv_desc_t *d) { return d->dtype == RKV_FP8_E4M3 && d->head_dim == kHeadDim && use_tri(d); }
+bool whole_tiles_of_codes(const rkv_desc_t *d, long long cap) { return d->dtype == RKV_FP8_E4M3 && d->head_dim == kHeadDim && cap % kTile == 0; }
 
 // Returns RKV_OK and fills *lay when the shape arguments are usable.
 int check_shapes(const rkv_desc_t *d, int budget, int buffer, int alpha, Layout *lay)
@@ -212,22 +212,25 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
         return ev && ev[i] ? cudaEventRecord(static_cast<cudaEvent_t>(ev[i]), s) : cudaSuccess;
     };
     if ((e = mark(0)) != cudaSuccess) return cuda_fail(e, "cudaEventRecord");
-    // What the gather moves is the caller's caches as they are stored; for 8-bit caches every stage before it reads the
+    // What the gather moves is the caller's caches as they are stored; where a copy is scored every stage before it reads the
     // bf16 copy of the keys (contiguous: the block table, if any, is followed once, by the widening kernel).
     Params stored = p;
-    if (needs_copy(d)) {
+    p.codes = direct_codes(d) ? 1 : 0;
+    const bool copies = needs_copy(d) && !p.codes;
+    if (copies) {
         p.k_cache = ws + lay.k_wide;
         p.block_table = nullptr;
         p.dtype = RKV_BF16;
         p.d = scoring_dim(d);
         if (pads_dim(d)) p.q_window = ws + lay.q_wide;
-        p.fused_codes = fused_codes(d, lay.cap) ? 1 : 0;
+        p.fused_codes = whole_tiles_of_codes(d, lay.cap) ? 1 : 0;
         p.fuse_src = stored.k_cache;
         p.fuse_table = stored.block_table;
     }
-    p.lengths_done = lengths_ahead(d) ? 1 : 0;
+    // (launches that callers count on: a kernel of its own records the lengths where the capacity is not a whole number of tiles)
+    p.lengths_done = lengths_ahead(d) || (p.codes && lay.cap % kTile != 0) ? 1 : 0;
     if (stages & RKV_STAGE_PREP) {
-        if (needs_copy(d) &&
+        if (copies &&
             (e = launch_widen_keys(stored, static_cast<__nv_bfloat16 *>(p.k_cache), p.d, pads_dim(d) ? stored.q_window : nullptr,
                                    pads_dim(d) ? ws + lay.q_wide : nullptr, !p.fused_codes, s)) != cudaSuccess)
             return cuda_fail(e, "widen launch");
@@ -632,7 +635,7 @@ int rkv_launch_count_for(const rkv_desc_t *desc, int32_t budget, int32_t buffer,
     if (check_shapes(desc, budget, buffer, alpha, &lay) != RKV_OK) return 0;
     int c = rkv_launch_count(desc, stage_mask);
     // the prep kernel writes the copy of the keys itself and nothing else needs a pass of its own
-    if ((stage_mask & RKV_STAGE_PREP) && fused_codes(desc, lay.cap)) c -= 1;
+    if ((stage_mask & RKV_STAGE_PREP) && whole_tiles_of_codes(desc, lay.cap)) c -= 1;
     if ((stage_mask & RKV_STAGE_SELECT) && select_is_fused(lay.cap_pad, alpha)) c -= 2;
     if ((stage_mask & RKV_STAGE_SCORES) && use_tri(desc) && desc->beta > 0 && desc->sim_threshold < 1.0f)
     {

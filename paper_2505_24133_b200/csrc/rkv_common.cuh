@@ -33,10 +33,11 @@ struct Params {
     int d;                          // head dimension: 64, 128 or 256
     int cap, cap_pad, tiles;        // cap_pad = tiles * kTile
     int budget, buffer, alpha;
-    int dtype;                      // of the keys the scoring stages read (bf16 for 8-bit caches: their widened copy)
+    int dtype;                      // of the keys the scoring stages read (bf16 where a widened copy of 8-bit caches is scored)
     int store_row_bytes;            // bytes of a row of the caches as stored (what the gather moves)
     float logit_scale;              // Eq. 2's 1 / sqrt(d) with the caches' own head dimension (d above may be a padded one)
     int lengths_done;               // 1: a kernel of its own records the lengths and clears the counters ahead of prep
+    int codes;                      // 1: the keys are scored as they are stored, E4M3 codes of 128 dimensions
     int fused_codes;                // 1: prep writes the scoring copy itself (k_cache above) from stored rows of 128 E4M3 codes
     const void *fuse_src;           // the stored keys
     const int32_t *fuse_table;      // their block table (paged caches), else null

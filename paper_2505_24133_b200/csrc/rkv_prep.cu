@@ -168,7 +168,9 @@ __global__ void __launch_bounds__(kPrepThreads, D <= 128 ? 5 : 2) prep_kernel(Pa
 // The tile sums of a head added up in tile order (a launch of its own behind the streaming kernel: no tickets, no fences in
 // the streaming kernel), also as three bf16 rows whose sum is s to fp32 accuracy (rows 3..15 of the 16-row block are
 // zero): behind the rows of the last key tile they let the first scoring pass form Kbar_i . s in its own product.
-template <int D>                             // (D >= 64, the most tiles that a head can have)
+// kCodes: as E4M3 codes, for keys that are.  A part holds what the parts before it left, 16 times as large: four more bits of the
+// sum each, so that seven hold all that fp32 does, down to components 2^-24 of the largest.
+template <int D, bool kCodes = false>        // (D >= 64, the most tiles that a head can have)
 __global__ void __launch_bounds__(D) head_sum_kernel(Params p)
 {
     pdl_trigger();
@@ -178,6 +180,29 @@ __global__ void __launch_bounds__(D) head_sum_kernel(Params p)
     const float *ts = p.tile_sum + (size_t)head * p.tiles * D + t;
     float s = 0.f;
     for (int q = 0; q < p.tiles; ++q) s += ts[(size_t)q * D];
+    if constexpr (kCodes) {
+        __shared__ float top[D / 32];
+        float m = fabsf(s);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        if ((t & 31) == 0) top[t / 32] = m;
+        __syncthreads();
+        for (int w = 0; w < D / 32; ++w) m = fmaxf(m, top[w]);
+        int e = 0;
+        if (m > 0.f && m < 1e30f) frexpf(m, &e);                       // m < 2^e
+        e = max(-100, min(100, 8 - e));                                // the largest component into [128, 256)
+        uint8_t *rows = reinterpret_cast<uint8_t *>(p.head_sum_bf16) + (size_t)head * kSumHeadBytes;
+        float rest = ldexpf(s, e);
+        for (int part = 0; part < 16; ++part) {
+            const __nv_fp8_storage_t code = part < kSumParts ? __nv_cvt_float_to_fp8(rest, __NV_SATFINITE, __NV_E4M3) : 0;
+            const __half_raw h = __nv_cvt_fp8_to_halfraw(code, __NV_E4M3);
+            rows[part * D + t] = code;
+            rest = (rest - __half2float(*reinterpret_cast<const __half *>(&h))) * 16.f;
+        }
+        if (t == 0) *reinterpret_cast<float *>(rows + kSumScaleAt) = ldexpf(1.f, -e);
+        if (prep_gave_up(first_r)) report_timeout(make_sink(p));
+        return;
+    }
     __nv_bfloat16 *hs = p.head_sum_bf16 + (size_t)head * 16 * D + t;
     float rest = s;
 #pragma unroll
@@ -195,7 +220,9 @@ __global__ void __launch_bounds__(D) head_sum_kernel(Params p)
 cudaError_t launch_head_sum(const Params &p, cudaStream_t s)
 {
     const unsigned heads = (unsigned)(p.batch * p.hkv);
-    return p.d == 64 ? launch_early(head_sum_kernel<64>, heads, 64, 0, s, 1, p) : launch_early(head_sum_kernel<128>, heads, 128, 0, s, 1, p);
+    return p.codes     ? launch_early(head_sum_kernel<128, true>, heads, 128, 0, s, 1, p)
+           : p.d == 64 ? launch_early(head_sum_kernel<64>, heads, 64, 0, s, 1, p)
+                       : launch_early(head_sum_kernel<128>, heads, 128, 0, s, 1, p);
 }
 
 template <typename T, int D>
@@ -215,7 +242,7 @@ cudaError_t launch_prep(const Params &p, cudaStream_t s)
     int dev = 0, sms = 0;
     const cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess) return e;
-    if (p.fused_codes || (bf16 && (p.d == 128 || (p.d == 64 && p.tri)))) return launch_prep_sm100(p, s);          // the tensor-core form
+    if (p.fused_codes || p.codes || (bf16 && (p.d == 128 || (p.d == 64 && p.tri)))) return launch_prep_sm100(p, s);          // the tensor-core form
     switch (p.d) {
         case 64: return bf16 ? launch_prep_for<__nv_bfloat16, 64>(p, dev, s) : launch_prep_for<float, 64>(p, dev, s);
         case 128: return launch_prep_for<float, 128>(p, dev, s);

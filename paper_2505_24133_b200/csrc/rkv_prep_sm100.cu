@@ -17,7 +17,8 @@
 // 64 dimensions: a unit of work is two tiles of a head, one behind the other in the same 32 KB: the two halves of the key sums' M, with
 // their r_i as rows 0..2 and 3..5 of the B operand.  Codes: the tile arrives as stored (16 KB) and the thread that owns a row
 // widens it into one of the groups' bf16 operand tiles, taking the norm on the way; with `copy` the same tile goes out by a TMA
-// store as the head's part of the scoring copy, which the later stages then read.
+// store as the head's part of the scoring copy, for the scoring kernels that need one (4096 heads of 4216 tokens: 779 us, 1381 with the
+// copy).
 //
 // The threshold test of Section 3.3, S[j][i] > T, as the sign of k_i . k_j - T / (r_i r_j): the scoring kernels append one K = 16
 // step to a tile product whose operands are the slices.  1 / r = ||k|| + eps in three bf16 parts (their sum has fp32 accuracy) as
@@ -583,11 +584,11 @@ cudaError_t launch_for(const Params &p, cudaStream_t s)
     if (e != cudaSuccess || (e = allow_smem_once(done, dev, prep_sm100_kernel<D, kCodes>, kSmemLimit)) != cudaSuccess) return e;
     // the logits are left to the other scoring kernels where those form them
     const int q_rows_pad = p.tri ? (p.group * p.alpha + 15) / 16 * 16 : 0;
-    const int copy = kCodes ? 1 : 0;
-    const int32_t *table = kCodes ? p.fuse_table : p.block_table;
+    const int copy = kCodes ? p.fused_codes : 0;
+    const int32_t *table = copy ? p.fuse_table : p.block_table;
     const uint64_t rows = table ? (uint64_t)p.pool_pages * kTile : (uint64_t)p.batch * p.hkv * p.cap;
     CUtensorMap map_k, map_q, map_wide;
-    const bool ok = (kCodes ? make_map_row128(&map_k, p.fuse_src, rows, true) : make_map_rows(&map_k, p.k_cache, rows, D, kTile)) &&
+    const bool ok = (kCodes ? make_map_row128(&map_k, copy ? p.fuse_src : p.k_cache, rows, true) : make_map_rows(&map_k, p.k_cache, rows, D, kTile)) &&
                     make_map_rows(&map_q, p.q_window, (uint64_t)p.batch * p.hq * p.alpha, D, (uint32_t)std::max(q_rows_pad, 16)) &&
                     (!copy || make_map(&map_wide, p.k_cache, (uint64_t)p.batch * p.hkv * p.cap + kTile, kTile));
     if (!ok) return cudaErrorInvalidValue;
@@ -605,7 +606,7 @@ cudaError_t launch_for(const Params &p, cudaStream_t s)
 
 cudaError_t launch_prep_sm100(const Params &p, cudaStream_t s)
 {
-    const cudaError_t e = p.fused_codes ? launch_for<128, true>(p, s) : p.d == 64 ? launch_for<64, false>(p, s) : launch_for<128, false>(p, s);
+    const cudaError_t e = p.fused_codes || p.codes ? launch_for<128, true>(p, s) : p.d == 64 ? launch_for<64, false>(p, s) : launch_for<128, false>(p, s);
     return e == cudaSuccess ? launch_head_sum(p, s) : e;
 }
 

@@ -66,7 +66,7 @@ struct LayD {                                    // see the second pass's Lay
 };
 
 // Item descriptor (int4): {head, pair of row tiles p, n, -}.  x < 0: no more items.
-template <int D>
+template <int D, bool kCodes>
 __global__ void __launch_bounds__(kThreadsD, 1)
 scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_ns)
 {
@@ -191,7 +191,7 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
         // ------------------------------------------------------------------ MMA issuers (one per row tile of the item)
         if (lane == 0) {
             const int m = warp == 1 ? 0 : 1;
-            const uint32_t idesc_k = instr_desc(kTile, kTile);
+            const uint32_t idesc_s = instr_desc(kTile, kTile), idesc_k = kCodes ? instr_desc_codes(kTile, kTile) : idesc_s;
             uint32_t k_item = 0, bcount = 0, cnt = 0;
             bool ok = true;
             while (ok) {
@@ -224,8 +224,8 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                         tc_fence_after();
                         const uint32_t d_tmem = tmem_base + a * 256 + m * 128;
                         if (D == 128) umma_tile_k128(d_tmem, resident, stage, idesc_k);
-                        else umma_tile_k64(d_tmem, resident, stage, idesc_k);
-                        umma_k16_sw32(d_tmem, res_slice, sbase + L::kOffAugB + s * kSliceBytes, idesc_k);
+                        else umma_tile_row128<kCodes>(d_tmem, resident, stage, idesc_k);
+                        umma_k16_sw32(d_tmem, res_slice, sbase + L::kOffAugB + s * kSliceBytes, idesc_s);
                         umma_commit(bar(L::kBarAccFull + a * 2 + m));
                         ++cnt;
                         ++tiles_done;
@@ -391,7 +391,7 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
 // the partner's similarity off its column sum, S = Kbar_i . Kbar_j, recomputed from the two key rows in fp32.
 constexpr int kFinishThreads = 256;
 
-template <int D>
+template <int D, bool kCodes>
 __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
 {
     // work unit = (head, chunk of 256 tokens), handed out with the grid as stride.  When no head took the route (the
@@ -417,11 +417,20 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
     float dot = 0.f;
 #pragma unroll 4
     for (int c = 0; c < D / 8; ++c) {
-        float a[8], bb[8];
-        Elem<__nv_bfloat16>::unpack(__ldg(ki + c), a);
-        Elem<__nv_bfloat16>::unpack(__ldg(kj + c), bb);
+        const uint4 vi = __ldg(ki + c), vj = __ldg(kj + c);
+        uint4 wi[2] = {vi, vi}, wj[2] = {vj, vj};
+        if (kCodes) {
+            widen16(vi, &wi[0], &wi[1]);
+            widen16(vj, &wj[0], &wj[1]);
+        }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) dot = fmaf(a[e], bb[e], dot);
+        for (int half = 0; half < (kCodes ? 2 : 1); ++half) {
+            float a[8], bb[8];
+            Elem<__nv_bfloat16>::unpack(wi[half], a);
+            Elem<__nv_bfloat16>::unpack(wj[half], bb);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) dot = fmaf(a[e], bb[e], dot);
+        }
     }
     p.sbar[hoff + i] -= dot * p.inv_norm[hoff + i] * p.inv_norm[hoff + j];
     }
@@ -429,21 +438,22 @@ __global__ void __launch_bounds__(kFinishThreads) dense_finish_kernel(Params p)
 
 }  // namespace
 
-template <int D>
+template <int D, bool kCodes>
 static cudaError_t launch_dense_for(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns)
 {
     static PerDevice done;
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_dense_sm100_kernel<D>, LayD<D>::kSmemBytesD)) != cudaSuccess) return e;
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_dense_sm100_kernel<D, kCodes>, LayD<D>::kSmemBytesD)) != cudaSuccess) return e;
     const unsigned long long max_items = (unsigned long long)(p.batch * p.hkv) * (unsigned long long)((p.tiles + 1) / 2);
     const unsigned grid = (unsigned)(max_items < (unsigned long long)sms ? max_items : (unsigned long long)sms);
-    return launch_early(scores_dense_sm100_kernel<D>, grid, kThreadsD, LayD<D>::kSmemBytesD, s, 1, p, map_k, map_ns);
+    return launch_early(scores_dense_sm100_kernel<D, kCodes>, grid, kThreadsD, LayD<D>::kSmemBytesD, s, 1, p, map_k, map_ns);
 }
 
 cudaError_t launch_scores_dense_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_ns)
 {
-    return p.d == 64 ? launch_dense_for<64>(p, s, map_k, map_ns) : launch_dense_for<128>(p, s, map_k, map_ns);
+    return p.codes ? launch_dense_for<64, true>(p, s, map_k, map_ns) : p.d == 64 ? launch_dense_for<64, false>(p, s, map_k, map_ns)
+                                                                              : launch_dense_for<128, false>(p, s, map_k, map_ns);
 }
 
 cudaError_t launch_dense_finish(const Params &p, cudaStream_t s)
@@ -454,8 +464,9 @@ cudaError_t launch_dense_finish(const Params &p, cudaStream_t s)
     const unsigned long long units = (unsigned long long)(p.batch * p.hkv) * (unsigned long long)((p.cap + kFinishThreads - 1) / kFinishThreads);
     const unsigned long long wave = 8ull * (unsigned long long)sms;             // resident blocks of this size
     const unsigned grid = (unsigned)(units < wave ? units : wave);
-    return p.d == 64 ? launch_early(dense_finish_kernel<64>, grid, kFinishThreads, 0, s, 1, p)
-                     : launch_early(dense_finish_kernel<128>, grid, kFinishThreads, 0, s, 1, p);
+    return p.codes   ? launch_early(dense_finish_kernel<64, true>, grid, kFinishThreads, 0, s, 1, p)
+         : p.d == 64 ? launch_early(dense_finish_kernel<64, false>, grid, kFinishThreads, 0, s, 1, p)
+                     : launch_early(dense_finish_kernel<128, false>, grid, kFinishThreads, 0, s, 1, p);
 }
 
 }  // namespace rkv

@@ -1,4 +1,4 @@
-// Stage "scores", first pass, for bf16 caches of 64 and 128 dimensions: every candidate token against the LAST key tile of its head
+// Stage "scores", first pass, for bf16 caches of 64 and 128 dimensions and E4M3 codes of 128: every candidate token against the LAST key tile of its head
 // (Eq. 5 and the start of Section 3.3's scan, which runs from the last position downwards) and against the head's key sum (Eq. 6).
 // tcgen05.mma with TMEM accumulators, fed by TMA, one persistent block per SM.
 //
@@ -17,7 +17,7 @@
 // Out, per token: the column sum minus the removed entries (sbar), the partners still lacking (a bit, and for beta > 1 how many).
 //
 // What bounds it: with 128 dimensions the keys' bytes (4096 heads of 4216 tokens: 792 us for 5.0 GB), with 64 the integer instructions
-// of the screening (8192 heads of 2168 tokens: 573).  While the query rows rode in the B block too (the logits are the prep stage's
+// of the screening (8192 heads of 2168 tokens: 573; 4096 of 4216 in 8 bits: 615, and 765 on their widened copy).  While the query rows rode in the B block too (the logits are the prep stage's
 // now) the product had 128 + G alpha + 16 columns, so that only two accumulators fitted, and the epilogue formed the logits: 994 and 786.
 //
 // Work item = (head, range of row tiles); items are handed out by a global ticket counter, head-major.  The operands
@@ -78,9 +78,9 @@ struct Lay {
 };
 
 // Item descriptor (int4): {head, first row tile, one past the last row tile, n}.  x < 0: no more items.
-// kRule: the retention rule is on.  kOne: beta = 1.  kMany: beta > kMostTurns, the form that can also take a chunk's partners out in one sum
+// kCodes: E4M3 codes of 128 dimensions, whose rows are as long as those of 64 dimensions in bf16 (D = 64).  kRule: the retention rule is on.  kOne: beta = 1.  kMany: beta > kMostTurns, the form that can also take a chunk's partners out in one sum
 // (each without the others' code: the roles share the instruction cache).
-template <int D, bool kRule, bool kOne, bool kMany>
+template <int D, bool kCodes, bool kRule, bool kOne, bool kMany>
 __global__ void __launch_bounds__(kThreadsP1, 1)
 scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_hs,
                            const __grid_constant__ CUtensorMap map_ns, const __grid_constant__ CUtensorMap map_ts, int splits,
@@ -161,7 +161,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 mbar_expect_tx(full, (uint32_t)L::kSumBytes + (kRule ? (uint32_t)(L::kTileBytes + kSliceBytes + kTile * 4) : 0u));
                 // behind the key tile's rows: 16 rows holding sum_j Kbar_j split into bf16 parts; every 64-column box
 #pragma unroll
-                for (int x = 0; x < D / 64; ++x) tma_load_2d(slot_addr + x * L::kBoxBytes + kTile * 128, &map_hs, x * 64, head * 16, full);
+                for (int x = 0; x < D / 64; ++x) tma_load_2d(slot_addr + x * L::kBoxBytes + kTile * 128, &map_hs, x * 64, head * (kCodes ? kSumHeadBytes / 128 : 16), full);
                 if (kRule) {
                     const int y = (int)tile_row0(p, head, n_tiles - 1);
 #pragma unroll
@@ -207,7 +207,8 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             // one product per streamed tile: N = the 128 keys of the last tile + the key sum (that alone while the rule is off)
-            const uint32_t idesc_ks = instr_desc(kTile, kTile + 16), idesc_s = instr_desc(kTile, 16);
+            const uint32_t idesc_ks = kCodes ? instr_desc_codes(kTile, kTile + 16) : instr_desc(kTile, kTile + 16);
+            const uint32_t idesc_s = kCodes ? instr_desc_codes(kTile, 16) : instr_desc(kTile, 16);
             const uint32_t idesc_k = instr_desc(kTile, kTile);
             uint32_t k_item = 0, acount = 0;
             bool ok = true;
@@ -233,13 +234,13 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                     const uint32_t d_tmem = tmem_base + a * kAccCols;
                     if (kRule) {
                         if (D == 128) umma_tile_k128_halves(d_tmem, tile, kHalfBytes, b_block, L::kBoxBytes, idesc_ks);
-                        else umma_tile_k64(d_tmem, tile, b_block, idesc_ks);
+                        else umma_tile_row128<kCodes>(d_tmem, tile, b_block, idesc_ks);
                         // ... - T / (r_i r_j) onto the key columns: the accumulator's sign is the threshold test
                         umma_k16_sw32(d_tmem, sbase + L::kOffAug + s * kSliceBytes, b_block + L::kSlotBytes, idesc_k);
                         ++tiles_done;
                     } else {
                         if (D == 128) umma_tile_k128_halves(d_tmem + 128, tile, kHalfBytes, b_block + kTile * 128, L::kBoxBytes, idesc_s);
-                        else umma_tile_k64(d_tmem + 128, tile, b_block + kTile * 128, idesc_s);
+                        else umma_tile_row128<kCodes>(d_tmem + 128, tile, b_block + kTile * 128, idesc_s);
                     }
                     umma_commit(bar(kBarAccFull + a));
                     umma_commit(bar(kBarAEmpty + s));              // the stage may be refilled once these products have read it
@@ -271,6 +272,7 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
             const float *inv_norm = p.inv_norm + (size_t)head * p.cap_pad;
             const float *rj = reinterpret_cast<const float *>(smem + L::kOffRj + slot * kTile * 4);
             const float *self_dot = p.self_dot + (size_t)head * p.cap_pad;
+            const float sum_scale = kCodes ? *reinterpret_cast<const float *>(reinterpret_cast<const uint8_t *>(p.head_sum_bf16) + (size_t)head * kSumHeadBytes + kSumScaleAt) : 1.f;
             float ri_next = 0.f, self_next = 0.f;
             int t_next = -1;                     // the tile ri_next / self_next were fetched for
             for (int t = d.y; t < d.z; ++t, ++ccount) {
@@ -297,11 +299,19 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 }
                 tc_fence_after();
 
-                // ---- Eq. 6 before the retention rule, sum_j S[j][i]: Kbar_i . s (in three parts) - Kbar_i . Kbar_i
+                // ---- Eq. 6 before the retention rule, sum_j S[j][i]: Kbar_i . s (in parts) - Kbar_i . Kbar_i
                 uint32_t sp[8];
                 tmem_ld8(lane_base + 128, sp);
                 tmem_wait8(sp);
-                const float total = ri * ((__uint_as_float(sp[0]) + __uint_as_float(sp[1])) + __uint_as_float(sp[2])) - self;
+                float sum = __uint_as_float(sp[kCodes ? kSumParts - 1 : 0]);
+                if (kCodes) {
+#pragma unroll
+                    for (int part = kSumParts - 2; part >= 0; --part) sum = fmaf(sum, 0.0625f, __uint_as_float(sp[part]));
+                    sum *= sum_scale;
+                } else {
+                    sum = (sum + __uint_as_float(sp[1])) + __uint_as_float(sp[2]);
+                }
+                const float total = ri * sum - self;
 
                 // ---- the last key tile, last position first.  The accumulator holds h = k_i . k_j - T / (r_i r_j):
                 // S[j][i] > T exactly when h > 0, so the screening is a sign test with nothing to load per column; a
@@ -442,38 +452,40 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
 
 }  // namespace
 
-template <int D, bool kRule, bool kOne, bool kMany>
+template <int D, bool kCodes, bool kRule, bool kOne, bool kMany>
 static cudaError_t launch_pass1_for(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_hs, const CUtensorMap &map_ns,
                                     const CUtensorMap &map_ts)
 {
     static PerDevice done;
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D, kRule, kOne, kMany>, Lay<D>::kBytes)) != cudaSuccess) return e;
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, scores_stream_sm100_kernel<D, kCodes, kRule, kOne, kMany>, Lay<D>::kBytes)) != cudaSuccess) return e;
     const int heads = p.batch * p.hkv;
     // a head is cut into parts when there are too few heads to give every SM several items
     int splits = (4 * sms + heads - 1) / heads;
     splits = splits < 1 ? 1 : (splits > p.tiles ? p.tiles : splits);
     const unsigned long long total_items = (unsigned long long)splits * (unsigned long long)heads;
     const unsigned grid = (unsigned)(total_items < (unsigned long long)sms ? total_items : (unsigned long long)sms);
-    return launch_early(scores_stream_sm100_kernel<D, kRule, kOne, kMany>, grid, kThreadsP1, (size_t)Lay<D>::kBytes, s, 1, p, map_k, map_hs, map_ns, map_ts,
+    return launch_early(scores_stream_sm100_kernel<D, kCodes, kRule, kOne, kMany>, grid, kThreadsP1, (size_t)Lay<D>::kBytes, s, 1, p, map_k, map_hs, map_ns, map_ts,
                         splits, total_items);
 }
 
-template <int D>
+template <int D, bool kCodes>
 static cudaError_t launch_pass1_form(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_hs, const CUtensorMap &map_ns,
                                      const CUtensorMap &map_ts)
 {
-    if (p.beta < 1 || !(p.sim_threshold < 1.0f)) return launch_pass1_for<D, false, false, false>(p, s, map_k, map_hs, map_ns, map_ts);
-    return p.beta == 1           ? launch_pass1_for<D, true, true, false>(p, s, map_k, map_hs, map_ns, map_ts)
-           : p.beta > kMostTurns ? launch_pass1_for<D, true, false, true>(p, s, map_k, map_hs, map_ns, map_ts)
-                                 : launch_pass1_for<D, true, false, false>(p, s, map_k, map_hs, map_ns, map_ts);
+    if (p.beta < 1 || !(p.sim_threshold < 1.0f)) return launch_pass1_for<D, kCodes, false, false, false>(p, s, map_k, map_hs, map_ns, map_ts);
+    return p.beta == 1           ? launch_pass1_for<D, kCodes, true, true, false>(p, s, map_k, map_hs, map_ns, map_ts)
+           : p.beta > kMostTurns ? launch_pass1_for<D, kCodes, true, false, true>(p, s, map_k, map_hs, map_ns, map_ts)
+                                 : launch_pass1_for<D, kCodes, true, false, false>(p, s, map_k, map_hs, map_ns, map_ts);
 }
 
 cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_hs,
                                       const CUtensorMap &map_ns, const CUtensorMap &map_ts)
 {
-    return p.d == 64 ? launch_pass1_form<64>(p, s, map_k, map_hs, map_ns, map_ts) : launch_pass1_form<128>(p, s, map_k, map_hs, map_ns, map_ts);
+    return p.codes     ? launch_pass1_form<64, true>(p, s, map_k, map_hs, map_ns, map_ts)
+           : p.d == 64 ? launch_pass1_form<64, false>(p, s, map_k, map_hs, map_ns, map_ts)
+                       : launch_pass1_form<128, false>(p, s, map_k, map_hs, map_ns, map_ts);
 }
 
 }  // namespace rkv

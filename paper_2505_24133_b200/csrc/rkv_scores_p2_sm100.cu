@@ -95,7 +95,7 @@ struct Bars {
 // first (highest) streamed tile}.  x < 0: no more items.  `round` selects the round's counters.
 // kOne: beta = 1 (each form without the other's code: the roles share the instruction cache.  1433 -> 1401 us
 // for 4096 heads of 4216 tokens, 591 -> 516 for the 64 dimensions above).
-template <int D, bool kOne>
+template <int D, bool kCodes, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1)
 scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_ns,
                           int round)
@@ -231,7 +231,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
         // arrival otherwise.
         if (lane == 0) {
             const int m = warp == 1 ? 0 : 1;
-            const uint32_t idesc_k = instr_desc(kTile, kTile);
+            const uint32_t idesc_s = instr_desc(kTile, kTile), idesc_k = kCodes ? instr_desc_codes(kTile, kTile) : idesc_s;
             uint32_t k_item = 0, bcount = 0, cnt = 0;
             bool ok = true;
             while (ok) {
@@ -265,9 +265,9 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                         tc_fence_after();
                         const uint32_t d_tmem = tmem_base + a * 256 + m * 128;
                         if (D == 128) umma_tile_k128(d_tmem, resident, stage, idesc_k);
-                        else umma_tile_k64(d_tmem, resident, stage, idesc_k);
+                        else umma_tile_row128<kCodes>(d_tmem, resident, stage, idesc_k);
                         // ... - (T / r_i) (||k_j|| + eps): the accumulator's sign is the threshold test
-                        umma_k16_sw32(d_tmem, res_slice, sbase + L::kOffAugB + s * kSliceBytes, idesc_k);
+                        umma_k16_sw32(d_tmem, res_slice, sbase + L::kOffAugB + s * kSliceBytes, idesc_s);
                         umma_commit(bar.at(L::kBarAccFull + a * 2 + m));
                         ++cnt;
                         ++tiles_done;
@@ -679,19 +679,22 @@ int scores_pass2_rounds(int tiles)
     return below <= 8 ? 1 : 2;
 }
 
-template <int D, bool kOne>
+template <int D, bool kCodes, bool kOne>
 static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
 {
     CUtensorMap map_k, map_hs, map_ns, map_ts;
-    if (!make_map_rows(&map_k, p.k_cache, key_rows_total(p), D, kTile) ||
-        !make_map_rows(&map_hs, p.head_sum_bf16, (uint64_t)p.batch * p.hkv * 16, D, 16u) ||
+    const uint64_t sum_rows = (uint64_t)p.batch * p.hkv * (kCodes ? kSumHeadBytes / 128 : 16);
+    const bool keys_ok = kCodes ? make_map_row128(&map_k, p.k_cache, key_rows_total(p), true) &&
+                                      encode_map(&map_hs, MapKey{p.head_sum_bf16, sum_rows, CU_TENSOR_MAP_DATA_TYPE_UINT8, 128u, 128u, 128u, 16u, CU_TENSOR_MAP_SWIZZLE_128B})
+                                : make_map_rows(&map_k, p.k_cache, key_rows_total(p), D, kTile) && make_map_rows(&map_hs, p.head_sum_bf16, sum_rows, D, 16u);
+    if (!keys_ok ||
         !make_map_k16(&map_ns, p.norm_split, (uint64_t)p.batch * p.hkv * p.cap_pad) ||
         !make_map_k16(&map_ts, p.thr_split, (uint64_t)p.batch * p.hkv * kTile))
         return cudaErrorInvalidValue;
     cudaError_t e;
     static PerDevice done;
     int dev = 0, sms = 0;
-    if ((e = device_sms(&dev, &sms)) != cudaSuccess || (e = allow_smem_once(done, dev, scores_pass2_sm100_kernel<D, kOne>, Lay<D>::kSmemBytes)) != cudaSuccess)
+    if ((e = device_sms(&dev, &sms)) != cudaSuccess || (e = allow_smem_once(done, dev, scores_pass2_sm100_kernel<D, kCodes, kOne>, Lay<D>::kSmemBytes)) != cudaSuccess)
         return e;
     const int heads = p.batch * p.hkv;
     if ((e = launch_scores_pass1_sm100(p, s, map_k, map_hs, map_ns, map_ts)) != cudaSuccess) return e;
@@ -712,7 +715,7 @@ static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
                              : launch_early(strag_compact_kernel<1>, (unsigned)((heads + kCompactWarps - 1) / kCompactWarps), kCompactWarps * 32, 0, s, 1, p, r, below, width);
         if (e != cudaSuccess) return e;
         if (r == 0 && (e = mark_kernel(p, 1, s)) != cudaSuccess) return e;
-        if ((e = launch_early(scores_pass2_sm100_kernel<D, kOne>, grid2, kThreads, Lay<D>::kSmemBytes, s, 1, p, map_k, map_ns, r)) != cudaSuccess) return e;
+        if ((e = launch_early(scores_pass2_sm100_kernel<D, kCodes, kOne>, grid2, kThreads, Lay<D>::kSmemBytes, s, 1, p, map_k, map_ns, r)) != cudaSuccess) return e;
         // the heads the first listing sent to the symmetric route (none on inputs where similar keys are common:
         // the kernel then returns at once)
         if (r == 0 && dense_possible && (e = launch_scores_dense_sm100(p, s, map_k, map_ns)) != cudaSuccess) return e;
@@ -723,8 +726,10 @@ static cudaError_t launch_tri_for(const Params &p, cudaStream_t s)
 
 cudaError_t launch_scores_tri_sm100(const Params &p, cudaStream_t s)
 {
-    if (p.d == 64) return p.beta == 1 ? launch_tri_for<64, true>(p, s) : launch_tri_for<64, false>(p, s);
-    return p.beta == 1 ? launch_tri_for<128, true>(p, s) : launch_tri_for<128, false>(p, s);
+    const bool one = p.beta == 1;
+    if (p.codes) return one ? launch_tri_for<64, true, true>(p, s) : launch_tri_for<64, true, false>(p, s);
+    if (p.d == 64) return one ? launch_tri_for<64, false, true>(p, s) : launch_tri_for<64, false, false>(p, s);
+    return one ? launch_tri_for<128, false, true>(p, s) : launch_tri_for<128, false, false>(p, s);
 }
 
 }  // namespace rkv

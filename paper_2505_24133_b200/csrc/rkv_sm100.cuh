@@ -187,6 +187,26 @@ __device__ __forceinline__ void umma_tile_k64(uint32_t d_tmem, uint32_t a_addr, 
 #pragma unroll
     for (int ks = 0; ks < 4; ++ks) umma(d_tmem, smem_desc(a_addr + 32 * ks), smem_desc(b_addr + 32 * ks), idesc, ks > 0 ? 1u : 0u);
 }
+// Instruction descriptor of kind::f8f6f4: E4M3 x E4M3 -> fp32, both operands K-major, M x N tile.
+__host__ __device__ constexpr uint32_t instr_desc_codes(int M, int N) { return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24); }
+// The product of keys whose rows are 128 bytes: 64 dimensions in bf16, or 128 E4M3 codes (four K = 32 steps of the 8-bit kind; products
+// of codes are exact, the accumulator is the same fp32 one that bf16 steps add to).
+template <bool kCodes>
+__device__ __forceinline__ void umma_tile_row128(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc)
+{
+    if (!kCodes) {
+        umma_tile_k64(d_tmem, a_addr, b_addr, idesc);
+        return;
+    }
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(smem_desc(a_addr + 32 * ks)), "l"(smem_desc(b_addr + 32 * ks)), "r"(idesc), "r"(ks)
+            : "memory");
+}
 // One more K = 16 step onto the accumulator at d_tmem: both operands are 128 rows x 16 bf16 (32-byte rows, 32-byte
 // swizzle, 8-row groups 256 bytes apart, 256-byte aligned).
 __device__ __forceinline__ void umma_k16_sw32(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc)
@@ -382,6 +402,10 @@ inline bool make_map_k16(CUtensorMap *map, const void *base, uint64_t rows)
 }
 
 }  // namespace sm100
+
+// The key sum of a head as the first scoring pass reads it beside 8-bit keys: 16 rows of 128 codes, the first kSumParts of which are
+// s 2^e in parts that are a 16th of the one before each; then 2^-e.  (The rows take the first half of the head's room for bf16 rows.)
+constexpr int kSumParts = 7, kSumHeadBytes = 16 * kHeadDim * 2, kSumScaleAt = 16 * kHeadDim;
 
 // first scoring pass of the two-pass tensor-core route (its own file); the maps are built by the caller
 cudaError_t launch_scores_pass1_sm100(const Params &p, cudaStream_t s, const CUtensorMap &map_k, const CUtensorMap &map_hs,

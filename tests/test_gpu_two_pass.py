@@ -33,3 +33,50 @@ def test_logits_where_blocks_take_many_units(rkv, head_dim, dtype):  # noqa: F81
     rep, comp = run_and_check(rkv, wl, check_rows=[0, 1, 2, 98, 99, 100, 101, 197, 198])
     assert rep.ok(), rep.errors
     comp.check_status()
+
+
+@pytest.mark.parametrize("beta,T", [(1, 0.5), (1, 0.95), (3, 0.5), (1, 1.0)])
+@pytest.mark.parametrize("budget,buffer,lens", [(100, 28, [128, 127, 101]), (100, 36, [136, 135, 101]), (1500, 164, [1664, 1545, 1501])])
+def test_codes_scored_as_they_are_stored(rkv, beta, T, budget, buffer, lens):  # noqa: F811
+    """E4M3 codes of 128 dimensions: capacities of a whole number of tiles and others, one tile, both rounds, the symmetric route (T =
+    0.95, 13 tiles), several partners, the rule off; the values the codes stand for span eight octaves."""
+    spec = small_spec("codes", batch=3, hkv=2, hq=8, budget=budget, buffer=buffer, dtype="fp8", span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=561 + budget, seq_lens=torch.tensor(lens))
+    scale = torch.exp2(torch.randint(-4, 4, (spec.cap, 1), generator=torch.Generator().manual_seed(5)).float()).cuda()
+    wl.k_cache.copy_((wl.k_cache.float() * scale).clamp(-448, 448).to(torch.float8_e4m3fn))
+    for b, L in enumerate(lens):
+        wl.k_cache.view(torch.uint8)[b, :, L:] = 0x7F      # NaN
+    rep, comp = run_and_check(rkv, wl, beta=beta, T=T)
+    assert rep.ok(), rep.errors
+    assert rep.compressed_heads == 2 * sum(L > budget for L in lens)
+    comp.check_status()
+
+
+@pytest.mark.parametrize("budget,buffer", [(500, 140), (500, 150)])
+def test_codes_by_either_route(rkv, budget, buffer):  # noqa: F811
+    """The codes as they are against their widened copy (row-block kernel), both kinds of capacity: the same lists."""
+    spec = small_spec("routes8", batch=2, hkv=2, hq=8, budget=budget, buffer=buffer, dtype="fp8", span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=571, seq_lens=torch.tensor([640, 601]))
+    got = []
+    for flags in (0, rkv.RKV_FLAG_ROWBLOCK_SCORES):
+        k, v, lens = wl.k_cache.clone(), wl.v_cache.clone(), wl.seq_lens.clone()
+        comp = rkv.Compressor(2, 2, 8, budget, buffer, 8, 0.1, dtype=torch.float8_e4m3fn, flags=flags)
+        idx = comp.compress(k, v, wl.q_window, lens)
+        torch.cuda.synchronize()
+        comp.check_status()
+        got.append(idx.clone())
+    assert torch.equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("size", [0.0, 1e-3, 1.0, 400.0])
+def test_key_sums_of_codes(rkv, size):  # noqa: F811
+    """The head's key sum travels as codes in parts of falling weight: keys of one value, of the smallest and of the largest codes, none."""
+    spec = small_spec("sums", batch=1, hkv=1, hq=1, budget=300, buffer=100, dtype="fp8", span=1, copy_frac=0.0)
+    wl = ri.make_workload(spec, device="cuda", seed=581)
+    k = wl.k_cache.float()
+    k[..., :64] *= size
+    k[..., 64:] *= 0.0 if size == 0.0 else 1.0
+    wl.k_cache.copy_(k.clamp(-448, 448).to(torch.float8_e4m3fn))
+    rep, comp = run_and_check(rkv, wl)
+    assert rep.ok(), rep.errors
+    comp.check_status()
