@@ -17,7 +17,7 @@
 // 64 dimensions: a unit of work is two tiles of a head, one behind the other in the same 32 KB: the two halves of the key sums' M, with
 // their r_i as rows 0..2 and 3..5 of the B operand.  Codes: the tile arrives as stored (16 KB) and the thread that owns a row
 // widens it into one of the groups' bf16 operand tiles, taking the norm on the way; with `copy` the same tile goes out by a TMA
-// store as the head's part of the scoring copy, for the scoring kernels that need one (4096 heads of 4216 tokens: 779 us, 1381 with the
+// store as the head's part of the scoring copy, for the scoring kernels that need one (4096 heads of 4216 tokens: 743 us, 1381 with the
 // copy).
 //
 // The threshold test of Section 3.3, S[j][i] > T, as the sign of k_i . k_j - T / (r_i r_j): the scoring kernels append one K = 16
@@ -29,7 +29,8 @@
 // block.  Warp 0 = TMA producer (a ring of up to six tiles: what bounds the kernel is how many bytes an SM has under way); it hands
 // each unit's descriptor on with its data.  Warp 1 = issuer of the logits' products and TMEM owner, warp 2 = issuer of the key sums', then
 // groups of four warps that take the units in turn: a unit's time is a chain of latencies (landing, norms, product, TMEM loads), which
-// three groups overlap.
+// four groups overlap (with three 4096 heads of 4216 tokens in 8 bits took 779 us, 743 with four; 8192 of 2168 tokens of 64 dimensions 574,
+// 550; with 128 dimensions in bf16, at its bytes, no difference).
 #include <algorithm>
 
 #include "rkv_prep.cuh"
@@ -40,7 +41,7 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kMaxGroups = 3;
+constexpr int kMaxGroups = 4;
 constexpr int kGroupWarp0 = 3;
 constexpr int kThreads = (kGroupWarp0 + 4 * kMaxGroups) * 32;
 constexpr int kBoxBytes = kTile * 64 * 2;                  // one TMA box: 128 rows of 128 bytes
@@ -246,7 +247,7 @@ __device__ __forceinline__ void pool_logits(const Params &p, uint32_t qbase, boo
 }
 
 // map_k: the stored keys.  map_wide, copy: see above.  q_rows_pad: 0 where another kernel forms the logits.  table: the block table of
-// the stored keys.  groups: as many as have room for their accumulators (64 dimensions and more than 72 query rows: two).
+// the stored keys.  groups: as many as have room for their accumulators (64 dimensions: three from 64 query rows on, two from 80).
 template <int D, bool kCodes>
 __global__ void __launch_bounds__(kThreads, 1)
 prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,

@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("head_dim,dtype", [(64, "bf16"), (128, "bf16"), (128, "fp8")])
 @pytest.mark.parametrize("hq,alpha,mean", [(1, 8, False), (7, 8, False), (14, 8, False), (14, 8, True), (9, 12, False), (3, 5, True)])
 def test_logits_of_the_prep_stage(rkv, head_dim, dtype, hq, alpha, mean):  # noqa: F811
-    """Query blocks of 16 to 112 rows (64 dimensions: three groups' accumulators up to 72 rows, two above), other window lengths than
+    """Query blocks of 16 to 112 rows (64 dimensions: four groups' accumulators up to 48 rows, three at 64, two above), other window lengths than
     eight, the mean over the group; units without a candidate, heads that change inside a block's range (24 heads of four tiles)."""
     lens = [(512, 385, 384, 257, 300, 400)[b % 6] for b in range(12)]
     spec = small_spec("logits", batch=12, hkv=2, hq=2 * hq, budget=300, buffer=212, alpha=alpha, head_dim=head_dim, dtype=dtype, span=8)
