@@ -29,7 +29,7 @@
 // Items are handed out by a global ticket counter, longest first within a head, so neighbouring blocks work on
 // the same head while its keys are in L2.
 // Warp roles (512 threads): warp 15 = tickets (publishes item descriptors up to three items ahead), warps 11..14 =
-// gather (fill the resident tiles of the NEXT item while the current one is scanned: two buffers), warp 0 = TMA
+// gather (fill the resident tiles of the NEXT item while the current one is scanned), warp 0 = TMA
 // producer of the streamed key tiles, warp 1 = MMA issuer of row tile 0 and TMEM owner, warp 10 = MMA issuer of row
 // tile 1, warps 2..9 = epilogue (warp w may touch TMEM lanes 32 (w % 4) .. +31; warps 2-5 serve row tile 0, warps 6-9
 // row tile 1).
@@ -55,34 +55,41 @@ constexpr int kPass1Depth = 1;                   // key tiles every token is sca
 constexpr int kRoundWords = 8;                   // Params::counters[kRoundWords + 2 r], [.. + 1]: items and ticket of round r
 
 // The operand tiles of D-dimensional keys and where everything lies in shared memory (offsets from a 1024-byte aligned base).
+// The streamed tiles' copies take about 2 us under load, so as many of them as fit are under way: with 128 dimensions three resident
+// tiles instead of four make room for a third stage (4096 heads of 4216 tokens: 1439 us with four and two, 1384; 7168 of 2168: 973, 903;
+// 4096 of 1144, beta = 4: 605, 589; with 64 dimensions six stages instead of four make no difference).  The second tile of the next
+// item then waits, in registers, for the present item's end.
 // The extra K = 16 slices of the operands: 128 rows x 32 bytes each (32-byte swizzle), one per resident tile and one
 // per stage of the ring.
 constexpr int kSliceBytes = kTile * 32;
 template <int D>
 struct Lay {
     static constexpr int kTileBytes = kTile * D * 2;                  // one 64-column box (16 KB) or two
-    static constexpr int kStagesB = D == 64 ? 4 : 2;                  // ring depth of streamed tiles
-    static constexpr int kOffA = 0;                                   // 2 buffers x 2 resident tiles (the gathered rows of an item)
-    static constexpr int kOffB = kOffA + 2 * 2 * kTileBytes;          // kStagesB streamed tiles
-    static constexpr int kOffAugA = kOffB + kStagesB * kTileBytes;    // 2 buffers x 2 slices
-    static constexpr int kOffAugB = kOffAugA + 2 * 2 * kSliceBytes;   // kStagesB slices
-    // what the epilogue needs to know about an item's tokens, left by the gather warps: position, r_i, partners lacking
-    static constexpr int kOffStash = kOffAugB + kStagesB * kSliceBytes;            // 2 buffers x 3 arrays x kRowsPerItem words
-    static constexpr int kOffBar = kOffStash + 2 * 3 * kRowsPerItem * 4;           // mbarriers
+    static constexpr int kResident = D == 64 ? 4 : 3;                 // resident tiles (128 gathered rows each), taken in turn
+    static constexpr int kStagesB = D == 64 ? 6 : 3;                  // ring depth of streamed tiles
+    static constexpr int kOffA = 0;
+    static constexpr int kOffB = kOffA + kResident * kTileBytes;
+    static constexpr int kOffAugA = kOffB + kStagesB * kTileBytes;
+    static constexpr int kOffAugB = kOffAugA + kResident * kSliceBytes;
+    // what the epilogue needs to know about a tile's tokens, left by the gather warps: position, r_i, partners lacking
+    static constexpr int kOffStash = kOffAugB + kStagesB * kSliceBytes;            // kResident x 3 arrays x kTile words
+    static constexpr int kOffMerge = kOffStash + kResident * 3 * kTile * 4;        // kResident x {position, accumulator value} x kTile: see kBarMerge
+    static constexpr int kOffBar = kOffMerge + kResident * 2 * kTile * 4;          // mbarriers
     static constexpr int kBarQFull = 0;                          // [kItemSlots] item descriptor written
     static constexpr int kBarQEmpty = kBarQFull + kItemSlots;    // [kItemSlots] read by the producer, the 2 MMA threads, the 8 epilogue and the 4 gather warps
-    static constexpr int kBarAFull = kBarQEmpty + kItemSlots;    // [2] resident tiles, slices and stash of the item in place (4 gather warps)
-    static constexpr int kBarAEmpty = kBarAFull + 2;             // [2] ... no longer read (2 MMA threads, 8 epilogue warps)
-    static constexpr int kBarBFull = kBarAEmpty + 2;             // [kStagesB]
+    static constexpr int kBarAFull = kBarQEmpty + kItemSlots;    // [kResident] resident tile, slice and stash in place (4 gather warps)
+    static constexpr int kBarAEmpty = kBarAFull + kResident;     // [kResident] ... no longer read (2 MMA threads, 8 epilogue warps)
+    static constexpr int kBarBFull = kBarAEmpty + kResident;     // [kStagesB]
     static constexpr int kBarBEmpty = kBarBFull + kStagesB;      // [kStagesB]
     static constexpr int kBarAccFull = kBarBEmpty + kStagesB;    // [2 buffers][2 row tiles]
     static constexpr int kBarAccEmpty = kBarAccFull + 4;         // [2][2], 4 warps each
-    static constexpr int kBarMerge = kBarAccEmpty + 4;           // [2] findings of the second half in the stash (its 4 epilogue warps)
-    static constexpr int kNumBars = kBarMerge + 2;
-    static constexpr int kOffItems = kOffBar + kNumBars * 8;          // kItemSlots x int4
+    // [kResident] findings of the second half of an item of one row tile (its 4 epilogue warps).  As many as resident tiles: the second
+    // half can be that many items ahead before it waits for a tile that the first has to give back
+    static constexpr int kBarMerge = kBarAccEmpty + 4;
+    static constexpr int kNumBars = kBarMerge + kResident;
+    static constexpr int kOffItems = (kOffBar + kNumBars * 8 + 15) / 16 * 16;      // kItemSlots x int4
     static constexpr int kOffMisc = kOffItems + kItemSlots * 16;      // tmem base, abort flag, bail flag
     static constexpr int kSmemBytes = kOffMisc + 16 + 1024;           // + slack for the manual 1024-byte alignment
-    static_assert(kOffItems % 16 == 0, "item descriptors are read as int4");
     static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 };
 
@@ -132,7 +139,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             mbar_init(bar.at(L::kBarQFull + s), 1);
             mbar_init(bar.at(L::kBarQEmpty + s), 15);
         }
-        for (int s = 0; s < 2; ++s) {
+        for (int s = 0; s < L::kResident; ++s) {
             // the 4 gather warps fill the resident tiles; the MMA threads and the epilogue warps read them and the stash
             mbar_init(bar.at(L::kBarAFull + s), 4);
             mbar_init(bar.at(L::kBarAEmpty + s), 10);
@@ -159,6 +166,16 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
     unsigned long long tiles_done = 0ull;
+    // The u-th use of a resident tile: its buffer, and the parity of its barriers' phase.  Whoever waits for these barriers meets every
+    // phase in order (a parity tells two neighbouring phases apart, no more).
+    auto buf_of = [](uint32_t u) -> uint32_t { return u % L::kResident; };
+    auto phase_of = [](uint32_t u) -> uint32_t { return u / L::kResident & 1u; };
+    auto prefetch_tile = [&](int head, int jt) {
+        const int y = (int)tile_row0(p, head, jt);
+#pragma unroll
+        for (int x = 0; x < D; x += 64)
+            asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(reinterpret_cast<uint64_t>(&map_k)), "r"(x), "r"(y) : "memory");
+    };
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -209,6 +226,10 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 if (!mbar_wait(bar.at(L::kBarQEmpty + qs), ((k_item / kItemSlots) & 1) ^ 1, abort_flag, sink)) break;
                 items[qs] = desc;
                 mbar_arrive(bar.at(L::kBarQFull + qs));
+                // The first tiles of the block's first two items are asked into L2 while their tokens are gathered: nothing else is
+                // under way yet.  (256 heads of 1144 tokens, all of whose items these are: the pass 36 -> 32 us; for all items of a
+                // large call it costs, 7168 heads of 2168 tokens 895 -> 1041.)
+                for (int it = 0; k_item < 2 && it < min(desc.z >> 16, 4); ++it) prefetch_tile(desc.x, desc.w - it);
                 ++k_item;
             }
             pdl_trigger();                  // no item is left: the next kernel may be let in
@@ -232,7 +253,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
         if (lane == 0) {
             const int m = warp == 1 ? 0 : 1;
             const uint32_t idesc_s = instr_desc(kTile, kTile), idesc_k = kCodes ? instr_desc_codes(kTile, kTile) : idesc_s;
-            uint32_t k_item = 0, bcount = 0, cnt = 0;
+            uint32_t k_item = 0, bcount = 0, cnt = 0, use = 0;       // use: uses of resident tiles before this item
             bool ok = true;
             while (ok) {
                 const uint32_t qs = k_item % kItemSlots;
@@ -244,11 +265,14 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 const int n_iter = d.z >> 16;
                 const bool split = kOne && num_m == 1;    // one row tile, its key tiles dealt out to both issuers
                 const bool mine = m < num_m || split;
-                const uint32_t ab = k_item & 1;                  // resident buffer of this item
-                if (!mbar_wait(bar.at(L::kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink)) break;     // the gathered rows are in place
+                // the gathered rows are in place (of the second row tile: the first issuer asks at the item's end, to stay in step)
+                const uint32_t own = use + (num_m == 2 && m == 1 ? 1u : 0u);
+                if (!mbar_wait(bar.at(L::kBarAFull + buf_of(use)), phase_of(use), abort_flag, sink) ||
+                    (own != use && !mbar_wait(bar.at(L::kBarAFull + buf_of(own)), phase_of(own), abort_flag, sink)))
+                    break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t resident = sbase + L::kOffA + (ab * 2 + (split ? 0 : m)) * L::kTileBytes;
-                const uint32_t res_slice = sbase + L::kOffAugA + (ab * 2 + (split ? 0 : m)) * kSliceBytes;
+                const uint32_t resident = sbase + L::kOffA + buf_of(own) * L::kTileBytes;
+                const uint32_t res_slice = sbase + L::kOffAugA + buf_of(own) * kSliceBytes;
                 for (int it = 0; it < n_iter; ++it) {
                     const uint32_t s = bcount % L::kStagesB;
                     if (!mbar_wait(bar.at(L::kBarBFull + s), (bcount / L::kStagesB) & 1, abort_flag, sink)) {
@@ -278,20 +302,26 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                     ++bcount;
                 }
                 if (!ok) break;
-                if (mine) umma_commit(bar.at(L::kBarAEmpty + ab));   // so may the resident tiles
-                else mbar_arrive(bar.at(L::kBarAEmpty + ab));
+                for (int x = 0; x < num_m; ++x) {                    // so may the resident tiles
+                    const uint32_t u = use + (uint32_t)x;
+                    if (u > own && !mbar_wait(bar.at(L::kBarAFull + buf_of(u)), phase_of(u), abort_flag, sink)) ok = false;
+                    if (mine && u == own) umma_commit(bar.at(L::kBarAEmpty + buf_of(u)));
+                    else mbar_arrive(bar.at(L::kBarAEmpty + buf_of(u)));
+                }
+                use += (uint32_t)num_m;
                 ++k_item;
             }
         }
         __syncwarp();
     } else if (warp >= kGatherWarp0) {
         // ------------------------------------------------------------------ gather warps
-        // They run one item ahead of the scan: the listed tokens' key rows go into the resident tiles of the buffer
-        // the scan is not using (same swizzled layout as a TMA load), each row's extra slice beside them, and what the
-        // epilogue needs to know about the token into the stash.  Thread g serves rows g and g + 128 of the item.
+        // They run as far ahead of the scan as there are resident tiles that it does not use: the listed tokens' key rows go into
+        // the next of them (same swizzled layout as a TMA load), each row's extra slice beside them, and what the epilogue needs
+        // to know about the token into the stash.  Thread g serves rows g and g + 128 of the item.
         const int gt = (warp - kGatherWarp0) * 32 + lane;      // 0..127
-        uint32_t k_item = 0;
-        while (true) {
+        uint32_t k_item = 0, use = 0;
+        bool ok = true;
+        while (ok) {
             const uint32_t qs = k_item % kItemSlots;
             if (!mbar_wait(bar.at(L::kBarQFull + qs), (k_item / kItemSlots) & 1, abort_flag, sink)) break;
             const int4 d = items[qs];
@@ -299,8 +329,6 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             if (lane == 0) mbar_arrive(bar.at(L::kBarQEmpty + qs));
             if (d.x < 0) break;
             const int head = d.x, k0 = d.y, rows = d.z & 0xffff;
-            const uint32_t ab = k_item & 1;
-            if (!mbar_wait(bar.at(L::kBarAEmpty + ab), ((k_item >> 1) & 1) ^ 1, abort_flag, sink)) break;
             const int num_m = rows > kTile ? 2 : 1;
             const size_t hoff = (size_t)head * p.cap_pad;
             int pos[2];
@@ -313,19 +341,19 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 rr[m] = pos[m] >= 0 ? __ldg(p.inv_norm + hoff + pos[m]) : 0.f;
                 lf[m] = pos[m] >= 0 ? (kOne ? 1 : p.left[hoff + pos[m]]) : 0;
             }
-            int32_t *stash_i = reinterpret_cast<int32_t *>(smem + L::kOffStash + ab * 3 * kRowsPerItem * 4);
-            float *stash_r = reinterpret_cast<float *>(stash_i + kRowsPerItem);
-            int32_t *stash_left = stash_i + 2 * kRowsPerItem;
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
-                if (m >= num_m) break;
+                if (m >= num_m || !ok) break;
                 const bool row_ok = pos[m] >= 0;
-                uint8_t *tile = smem + L::kOffA + (ab * 2 + m) * L::kTileBytes;
                 const uint4 *src = reinterpret_cast<const uint4 *>(
                     static_cast<const __nv_bfloat16 *>(p.k_cache) + (size_t)row_index(p, head, row_ok ? pos[m] : 0) * D);
-                uint4 v[D / 8];
+                uint4 v[D / 8];                      // under way while the tile is still in use
 #pragma unroll
                 for (int c = 0; c < D / 8; ++c) v[c] = row_ok ? __ldg(src + c) : make_uint4(0u, 0u, 0u, 0u);
+                const uint32_t ab = buf_of(use);
+                if (!(ok = mbar_wait(bar.at(L::kBarAEmpty + ab), phase_of(use) ^ 1u, abort_flag, sink))) break;
+                ++use;
+                uint8_t *tile = smem + L::kOffA + ab * L::kTileBytes;
 #pragma unroll
                 for (int hb = 0; hb < D / 64; ++hb) {
 #pragma unroll
@@ -342,18 +370,19 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                     part[c] = (uint32_t)__bfloat16_as_ushort(h16);
                     rest -= __bfloat162float(h16);
                 }
-                uint8_t *slice = smem + L::kOffAugA + (ab * 2 + m) * kSliceBytes + gt * 32;
+                uint8_t *slice = smem + L::kOffAugA + ab * kSliceBytes + gt * 32;
                 const int sw = (gt >> 2) & 1;
                 *reinterpret_cast<uint4 *>(slice + (sw << 4)) =
                     make_uint4(part[0] | (part[0] << 16), part[0] | (part[1] << 16), part[1] | (part[2] << 16), 0u);
                 *reinterpret_cast<uint4 *>(slice + ((sw ^ 1) << 4)) = make_uint4(0u, 0u, 0u, 0u);
-                stash_i[m * kTile + gt] = row_ok ? pos[m] : 0;
-                stash_r[m * kTile + gt] = rr[m];
-                stash_left[m * kTile + gt] = lf[m];
+                int32_t *stash = reinterpret_cast<int32_t *>(smem + L::kOffStash + ab * 3 * kTile * 4);
+                stash[gt] = row_ok ? pos[m] : 0;
+                reinterpret_cast<float *>(stash)[kTile + gt] = rr[m];
+                stash[2 * kTile + gt] = lf[m];
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor-core reads
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar.at(L::kBarAFull + ab));
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor-core reads
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar.at(L::kBarAFull + ab));
             ++k_item;
         }
     } else {
@@ -363,7 +392,7 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
         const int quad = warp & 3;               // TMEM lane quadrant this warp may access
         const int lrow = quad * 32 + lane;       // row within the 128-row tile
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
-        uint32_t k_item = 0, cnt = 0, merge_parity = 0;      // merge_parity: bit b: phase of the merging barrier of buffer b
+        uint32_t k_item = 0, cnt = 0, use = 0, merges = 0;      // merges: items of one row tile so far
 
         while (true) {
             const uint32_t qs = k_item % kItemSlots;
@@ -374,8 +403,6 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             if (d.x < 0) break;
             const int head = d.x;
             const float *inv_norm = p.inv_norm + (size_t)head * p.cap_pad;
-            const uint32_t ab = k_item & 1;          // resident buffer (and stash) of this item
-
             // ---- per item: which token this thread owns (left in the stash by the gather warps), where the scan
             // starts and ends
             const int rows = d.z & 0xffff, first_tile = d.w, last_tile = d.w - (d.z >> 16) + 1;
@@ -383,15 +410,17 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
             const bool active = (m == 0) || (rows > kTile) || split;
             const int r_item = split ? lrow : m * kTile + lrow;               // row of the item
             const bool row_ok = active && r_item < rows;
-            bool item_ok = mbar_wait(bar.at(L::kBarAFull + ab), (k_item >> 1) & 1, abort_flag, sink);
-            int32_t *stash_i = reinterpret_cast<int32_t *>(smem + L::kOffStash + ab * 3 * kRowsPerItem * 4);
-            float *stash_r = reinterpret_cast<float *>(stash_i + kRowsPerItem);
+            // the resident tile (and stash) whose rows these warps look after; the other one's barrier is met at the item's end, or here
+            const uint32_t num_m = rows > kTile ? 2u : 1u, own = use + (num_m == 2u && m == 1 ? 1u : 0u);
+            bool item_ok = mbar_wait(bar.at(L::kBarAFull + buf_of(use)), phase_of(use), abort_flag, sink);
+            if (own != use && item_ok) item_ok = mbar_wait(bar.at(L::kBarAFull + buf_of(own)), phase_of(own), abort_flag, sink);
+            const int32_t *stash = reinterpret_cast<const int32_t *>(smem + L::kOffStash + buf_of(own) * 3 * kTile * 4);
             int i = 0, left = 0;
             float ri = 0.f;
             if (row_ok && item_ok) {
-                i = stash_i[r_item];
-                ri = stash_r[r_item];
-                left = stash_i[2 * kRowsPerItem + r_item];
+                i = stash[lrow];
+                ri = reinterpret_cast<const float *>(stash)[kTile + lrow];
+                left = stash[2 * kTile + lrow];
             }
 
             float removed = 0.f;
@@ -496,24 +525,29 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 item_ok = ok;
             }
             if (split && item_ok) {
-                // the second half leaves its findings where the stash of a second row tile would be
-                if (m == 1) {
-                    stash_i[kTile + lrow] = hit_j;
-                    stash_r[kTile + lrow] = hit_h;
+                int32_t *found_j = reinterpret_cast<int32_t *>(smem + L::kOffMerge + buf_of(merges) * 2 * kTile * 4);
+                float *found_h = reinterpret_cast<float *>(found_j + kTile);
+                const uint32_t merge = bar.at(L::kBarMerge + (int)buf_of(merges));
+                if (m == 1) {                        // the second half leaves its findings
+                    found_j[lrow] = hit_j;
+                    found_h[lrow] = hit_h;
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar.at(L::kBarMerge + ab));
+                    if (lane == 0) mbar_arrive(merge);
                 } else {
-                    item_ok = mbar_wait(bar.at(L::kBarMerge + ab), merge_parity >> ab & 1u, abort_flag, sink);
-                    merge_parity ^= 1u << ab;
-                    if (item_ok && stash_i[kTile + lrow] > hit_j) {
-                        hit_j = stash_i[kTile + lrow];
-                        hit_h = stash_r[kTile + lrow];
+                    item_ok = mbar_wait(merge, phase_of(merges), abort_flag, sink);
+                    if (item_ok && found_j[lrow] > hit_j) {
+                        hit_j = found_j[lrow];
+                        hit_h = found_h[lrow];
                     }
                 }
             }
-            // the item's resident buffer and stash are no longer read by this warp
+            if (split) ++merges;
+            if (own == use && num_m == 2u && item_ok) item_ok = mbar_wait(bar.at(L::kBarAFull + buf_of(use + 1u)), phase_of(use + 1u), abort_flag, sink);
+            // the item's resident tiles and stash are no longer read by this warp
             __syncwarp();
-            if (lane == 0 && item_ok) mbar_arrive(bar.at(L::kBarAEmpty + ab));
+            if (lane == 0 && item_ok)
+                for (uint32_t x = 0; x < num_m; ++x) mbar_arrive(bar.at(L::kBarAEmpty + buf_of(use + x)));
+            use += num_m;
             if (!item_ok) break;              // (the epilogue warps meet at no barrier of their own: each may leave alone)
             if (row_ok && !(split && m == 1)) {
                 // S = T + h r_i r_j for every partner found here

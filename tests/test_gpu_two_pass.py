@@ -80,3 +80,22 @@ def test_key_sums_of_codes(rkv, size):  # noqa: F811
     rep, comp = run_and_check(rkv, wl)
     assert rep.ok(), rep.errors
     comp.check_status()
+
+
+@pytest.mark.parametrize("head_dim,dtype", [(64, "bf16"), (128, "bf16"), (128, "fp8")])
+@pytest.mark.parametrize("beta,T,span", [(1, 0.95, 1), (1, 0.5, 1), (2, 0.5, 16)])
+@pytest.mark.parametrize("budget,buffer,batch", [(120, 40, 40), (250, 150, 25), (1300, 100, 13)])
+def test_second_pass_items_in_a_row(rkv, head_dim, dtype, beta, T, span, budget, buffer, batch):  # noqa: F811
+    """Items of one and of two row tiles behind one another on every SM (resident tiles are taken in turn, three or four of them): T =
+    0.95 lists nearly every token (129 to 152 of them, 384 to 392: two items, of two row tiles and of one or two; 1392: six), T = 0.5
+    few (one row tile, its key tiles dealt out to both halves)."""
+    some = [budget + buffer, budget + buffer - 15, budget + 17, budget + 9]
+    lens = [some[b % 4] for b in range(batch)]
+    spec = small_spec("items", batch=batch, hkv=8, hq=8, budget=budget, buffer=buffer, head_dim=head_dim, dtype=dtype, span=span, copy_frac=0.5)
+    wl = ri.make_workload(spec, device="cuda", seed=501 + budget, seq_lens=torch.tensor(lens))
+    for b, L in enumerate(lens):
+        wl.k_cache.view(torch.int16 if dtype == "bf16" else torch.uint8)[b, :, L:] = 0x7FC0 if dtype == "bf16" else 0x7F      # NaN
+    rows = sorted({0, 1, 2, 3, batch // 2, batch - 2, batch - 1})
+    rep, comp = run_and_check(rkv, wl, beta=beta, T=T, flags=rkv.RKV_FLAG_NO_SYMMETRIC, check_rows=rows)
+    assert rep.ok(), rep.errors
+    comp.check_status()
