@@ -12,7 +12,8 @@
 //   values   O^T [d x 16] += V_tile^T [d x 128 keys] . P [128 keys x 16]   (the V tile as TMA leaves it, used transposed:
 //            MN-major A operand; P = the softmax weights in bf16, written to shared memory by the softmax threads)
 //
-// A block owns one (KV head, split of the key tiles) with at most 15 tiles.  First all its K tiles stream through the
+// A block owns one (KV head, split of the key tiles) with at most 15 tiles, or two chunks of up to 14 that go through the following
+// one after the other.  First all its K tiles stream through the
 // ring and leave their scores in TMEM (16 columns each, 240 at most, beside the 16 output columns); then the exact
 // maximum per query over the whole split is taken, so the weights need no running rescale; then the V tiles stream
 // through the same ring while the softmax threads turn score columns into P tiles (double-buffered).  Every weight
@@ -45,12 +46,13 @@ using namespace sm100;
 
 constexpr int kTcThreads = 192;
 constexpr int kTcStages = 3;                         // ring of key / value tiles
-constexpr int kTcMaxTiles = 15;                      // key tiles per block
+constexpr int kTcMaxTiles = 15;                      // key tiles per block in one chunk
+constexpr int kTcChunkTiles = 14;                    // ... and in each of two
 constexpr int kTcMaxSplits = 16;                     // blocks of a cluster
 constexpr int kTcHalf = kTile * 64 * 2;              // one TMA box: 128 rows x 64 bf16
 constexpr int kTcTileBytes = 2 * kTcHalf;            // 32 KB
 constexpr int kTcSmall = 16 * kHeadDim * 2;          // a [16 x 128] bf16 operand (Q^T or P): two [16 x 64] halves of 2 KB
-constexpr uint32_t kTcTmemCols = 256;                // 16 (output) + 16 per key tile
+constexpr uint32_t kTcTmemCols = 256;                // 16 (output) per chunk + 16 per key tile of a chunk
 
 constexpr int kOffRing = 0;                          // bf16 caches: kTcStages tiles.  8-bit caches: kConvBufs widened tiles,
 constexpr int kConvBufs = 2;
@@ -77,7 +79,7 @@ enum {
 constexpr int kOffMisc = kOffBars + kTcNumBars * 8;  // TMEM base, abort flag
 constexpr int kTcSmem = kOffMisc + 16 + 1024;        // + slack for the 1024-byte alignment
 static_assert(2 * (kTcSmem + 1024) <= 227 * 1024, "two blocks per SM");
-static_assert(16 + 16 * kTcMaxTiles <= (int)kTcTmemCols, "TMEM columns");
+static_assert(16 + 16 * kTcMaxTiles <= (int)kTcTmemCols && 32 + 16 * kTcChunkTiles <= (int)kTcTmemCols, "TMEM columns");
 
 struct AttendTcParams {          // (64 bytes: the tensor maps behind it start at the next multiple of 64)
     const int32_t *seq_lens;
@@ -130,10 +132,11 @@ __device__ __forceinline__ uint32_t small_off(int g, int k)
 }
 
 // With kFp8, kBarFull / kBarEmpty [0 .. kConvBufs) stand for the widened tiles (filled by the softmax threads, 128 arrivals).
+// kTwo: blocks of more tiles than one chunk takes (an instance of its own: small calls are latency, 6.3 us without this code, 6.5 with it).
 // kSrc: 0 = bf16 caches of 128 dimensions (tiles go to the tensor cores as they land), 1 = E4M3 codes of 128 dimensions,
 // 2 = bf16 caches of 64 dimensions (both: rows of 128 bytes, widened / padded with zeros into bf16 operand tiles of
 // 128 dimensions; the queries of the 64-dimension case fill the first half of their operand, the rest stays zero).
-template <int G, int kSrc>
+template <int G, int kSrc, bool kTwo>
 __global__ void __launch_bounds__(kTcThreads, 2)
 attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                  const __grid_constant__ CUtensorMap map_q)
@@ -225,7 +228,15 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
         report(p.status, RKV_ERR_INVALID_ARG);
         L = 0;
     }
-    const int T = min(min(p.tiles_per_split, kTcMaxTiles), (L + kTile - 1) / kTile - t0);      // its tiles (<= 0: none)
+    const int T = min(p.tiles_per_split, (L + kTile - 1) / kTile - t0);      // its tiles (<= 0: none)
+    // more than a block's columns hold the scores of: two chunks, one after the other, each with its own maximum and output columns
+    const int chunks = kTwo && T > kTcMaxTiles ? 2 : 1, T0 = chunks == 2 ? (T + 1) / 2 : T;        // T0: tiles of the first chunk
+    // in the order of the ring -- the first chunk's K tiles, its V tiles, the second's -- tile i is this one of the block, of K or of V
+    auto source = [&](int i, bool *value) -> int {
+        const int c = kTwo && i >= 2 * T0, j = c ? i - 2 * T0 : i, n = c ? T - T0 : T0;
+        *value = j >= n;
+        return (c ? T0 : 0) + (j >= n ? j - n : j);
+    };
     constexpr int kStride = kHeadDim + 2;
     // [G][d + 2]: unnormalised output, maximum (base-2 domain), sum of weights
     float *part = kFp8 && p.separate ? p.out + ((size_t)head * p.splits + split) * G * kStride : reinterpret_cast<float *>(smem + kOffP);
@@ -256,7 +267,9 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
             constexpr int kRing = kFp8 ? kRawStages : kTcStages, kEmpty = kFp8 ? kBarRawEmpty : kBarEmpty;
             for (int i = 1; i < 2 * T; ++i) {                // the other K tiles, then the V tiles
                 if (!mbar_wait(bar(kEmpty + i % kRing), ((i / kRing) & 1) ^ 1, abort_flag, sink)) break;
-                fetch_tile(i < T ? &map_k : &map_v, i, t0 + (i < T ? i : i - T));
+                bool value;
+                const int t = source(i, &value);
+                fetch_tile(value ? &map_v : &map_k, i, t0 + t);
             }
         }
         __syncwarp();
@@ -266,36 +279,41 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
             bool ok = mbar_wait(bar(kBarQ), 0, abort_flag, sink);
             const uint32_t idesc_s = instr_desc(kTile, 16);
             constexpr int kBufs = kFp8 ? kConvBufs : kTcStages;      // operand tiles the tensor cores read from
-            for (int t = 0; t < T && ok; ++t) {              // scores of key tile t into its own 16 columns
-                const int s = t % kBufs;
-                ok = mbar_wait(bar(kBarFull + s), (t / kBufs) & 1, abort_flag, sink);
-                if (!ok) break;
-                tc_fence_after();
-                umma_tile_k128_halves(tmem + 16 + 16 * t, sbase + kOffRing + s * kTcTileBytes, kTcHalf, sbase + kOffQ,
-                                      kTcSmall / 2, idesc_s);
-                umma_commit(bar(kBarEmpty + s));
-            }
-            if (ok) umma_commit(bar(kBarScores));
             // f32 accumulate, bf16 x bf16, A MN-major (bit 15), B K-major, M = 128, N = 16
             const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
-            for (int t = 0; t < T && ok; ++t) {              // O^T += V_t^T . P_t
-                const int i = T + t, s = i % kBufs, pb = t & 1;
-                ok = mbar_wait(bar(kBarFull + s), (i / kBufs) & 1, abort_flag, sink) &&
-                     mbar_wait(bar(kBarPFull + pb), (t >> 1) & 1, abort_flag, sink);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t v_tile = sbase + kOffRing + s * kTcTileBytes, p_tile = sbase + kOffP + pb * kTcSmall;
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {             // 16 keys per step
-                    const uint32_t a_addr = v_tile + ks * 2048;             // 16 rows of 128 bytes further
-                    const uint32_t b_addr = p_tile + (ks >> 2) * (kTcSmall / 2) + (ks & 3) * 32;
-                    // A: 64-element (128-byte) atoms along M 16 KB apart (the second TMA box), 8-row groups along K 1 KB apart
-                    const uint64_t da = (uint64_t)((a_addr & 0x3FFFFu) >> 4) | ((uint64_t)(16384u >> 4) << 16) |
-                                        ((uint64_t)(1024u >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-                    umma(tmem, da, smem_desc(b_addr), idesc_o, (t > 0 || ks > 0) ? 1u : 0u);
+            int i = 0;                                       // tiles of the ring so far
+            for (int c = 0; c < (kTwo ? chunks : 1) && ok; ++c) {
+                const int n = c ? T - T0 : T0, done = c ? T0 : 0;
+                // (the second chunk's scores take the columns of the first's: the last of its weights have been waited for)
+                for (int t = 0; t < n && ok; ++t, ++i) {     // scores of key tile t into its own 16 columns
+                    const int s = i % kBufs;
+                    ok = mbar_wait(bar(kBarFull + s), (i / kBufs) & 1, abort_flag, sink);
+                    if (!ok) break;
+                    tc_fence_after();
+                    umma_tile_k128_halves(tmem + 16 * (chunks + t), sbase + kOffRing + s * kTcTileBytes, kTcHalf, sbase + kOffQ,
+                                          kTcSmall / 2, idesc_s);
+                    umma_commit(bar(kBarEmpty + s));
                 }
-                umma_commit(bar(kBarEmpty + s));
-                umma_commit(bar(kBarPEmpty + pb));
+                if (ok) umma_commit(bar(kBarScores));
+                for (int t = 0; t < n && ok; ++t, ++i) {     // O^T += V_t^T . P_t
+                    const int s = i % kBufs, pt = done + t, pb = pt & 1;
+                    ok = mbar_wait(bar(kBarFull + s), (i / kBufs) & 1, abort_flag, sink) &&
+                         mbar_wait(bar(kBarPFull + pb), (pt >> 1) & 1, abort_flag, sink);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t v_tile = sbase + kOffRing + s * kTcTileBytes, p_tile = sbase + kOffP + pb * kTcSmall;
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks) {         // 16 keys per step
+                        const uint32_t a_addr = v_tile + ks * 2048;             // 16 rows of 128 bytes further
+                        const uint32_t b_addr = p_tile + (ks >> 2) * (kTcSmall / 2) + (ks & 3) * 32;
+                        // A: 64-element (128-byte) atoms along M 16 KB apart (the second TMA box), 8-row groups along K 1 KB apart
+                        const uint64_t da = (uint64_t)((a_addr & 0x3FFFFu) >> 4) | ((uint64_t)(16384u >> 4) << 16) |
+                                            ((uint64_t)(1024u >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+                        umma(tmem + 16 * c, da, smem_desc(b_addr), idesc_o, (t > 0 || ks > 0) ? 1u : 0u);
+                    }
+                    umma_commit(bar(kBarEmpty + s));
+                    umma_commit(bar(kBarPEmpty + pb));
+                }
             }
             if (ok) umma_commit(bar(kBarOut));
         }
@@ -311,7 +329,8 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
             const int s = i % kRawStages, cb = i % kConvBufs;
             if (!mbar_wait(bar(kBarRawFull + s), (i / kRawStages) & 1, abort_flag, sink)) return false;
             if (!mbar_wait(bar(kBarEmpty + cb), ((i / kConvBufs) & 1) ^ 1, abort_flag, sink)) return false;
-            const bool row_valid = (t0 + (i < T ? i : i - T)) * kTile + r < L;
+            bool value;
+            const bool row_valid = (t0 + source(i, &value)) * kTile + r < L;
             const uint8_t *raw = smem + kOffRaw + s * kRawBytes + r * 128;
             uint8_t *dst = smem + kOffRing + cb * kTcTileBytes + r * 128;
             uint4 codes[8];                                  // the whole row first: the loads must not wait for the stores
@@ -336,71 +355,90 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
             return true;
         };
         bool ok = true;
-        if (kFp8)
-            for (int t = 0; t < T && ok; ++t) ok = widen_tile(t);
-        if (ok) ok = mbar_wait(bar(kBarScores), 0, abort_flag, sink);
-        float m[G], l[G];
+        float m[G], l[G], m0[G], l0[G];              // of the present chunk, and of the first
 #pragma unroll
-        for (int g = 0; g < G; ++g) m[g] = -3.402823466e38f, l[g] = 0.f;      // (-inf stands for a split without rows in the merge)
-        if (ok) {
-            tc_fence_after();
-            for (int t = 0; t < T; ++t) {
-                uint32_t acc[16];
-                tmem_ld16(lane_base + 16 + 16 * t, acc);
-                tmem_wait16(acc);
-                const bool valid = (t0 + t) * kTile + r < L;
-#pragma unroll
-                for (int g = 0; g < G; ++g)
-                    if (valid) m[g] = fmaxf(m[g], __uint_as_float(acc[g]) * c2);
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) m[g] = fmaxf(m[g], __shfl_xor_sync(0xffffffffu, m[g], off));
-            if (lane == 0) red[warp * 8 + g] = m[g];
-        }
-        softmax_sync();
-#pragma unroll
-        for (int g = 0; g < G; ++g) m[g] = fmaxf(fmaxf(red[g], red[8 + g]), fmaxf(red[16 + g], red[24 + g]));
-        softmax_sync();                                  // `red` is used again for the sums
-
-        for (int t = 0; t < T && ok; ++t) {
-            const int pb = t & 1;
-            if (kFp8) ok = widen_tile(T + t);
-            if (ok) ok = mbar_wait(bar(kBarPEmpty + pb), ((t >> 1) & 1) ^ 1, abort_flag, sink);
-            if (!ok) break;
-            uint32_t acc[16];
-            tmem_ld16(lane_base + 16 + 16 * t, acc);
-            tmem_wait16(acc);
-            const bool valid = (t0 + t) * kTile + r < L;
-            uint8_t *pt = smem + kOffP + pb * kTcSmall;
+        for (int g = 0; g < G; ++g) m0[g] = -INFINITY, l0[g] = 0.f;
+        for (int c = 0; c < (kTwo ? chunks : 1); ++c) {
+            const int n = c ? T - T0 : T0, done = c ? T0 : 0;
+            if (kFp8)
+                for (int t = 0; t < n && ok; ++t) ok = widen_tile(2 * done + t);
+            if (ok) ok = mbar_wait(bar(kBarScores), c, abort_flag, sink);
 #pragma unroll
             for (int g = 0; g < G; ++g) {
-                // (a NaN or infinite score of a row that is not cached never gets here: `valid` decides)
-                const float w = valid ? exp2f(__uint_as_float(acc[g]) * c2 - m[g]) : 0.f;
-                const __nv_bfloat16 hi = __float2bfloat16_rn(w);
-                const __nv_bfloat16 lo = __float2bfloat16_rn(w - __bfloat162float(hi));
-                l[g] += __bfloat162float(hi) + __bfloat162float(lo);
-                *reinterpret_cast<__nv_bfloat16 *>(pt + small_off(g, r)) = hi;
-                *reinterpret_cast<__nv_bfloat16 *>(pt + small_off(8 + g, r)) = lo;
+                if (c > 0) m0[g] = m[g], l0[g] = l[g];
+                m[g] = -3.402823466e38f, l[g] = 0.f;      // (-inf stands for a split without rows in the merge)
             }
-            if (!kFp8 && !valid) {
-                // a row beyond the sequence's length may hold anything, and 0 x NaN would spoil the product: its V row
-                // is cleared in shared memory (only the split's last tile has such rows)
-                const int i = T + t, s = i % kTcStages;
-                ok = mbar_wait(bar(kBarFull + s), (i / kTcStages) & 1, abort_flag, sink);
-                if (ok) {
-                    uint8_t *vt = smem + kOffRing + s * kTcTileBytes;
+            if (ok) {
+                tc_fence_after();
+                for (int t = 0; t < n; ++t) {
+                    uint32_t acc[16];
+                    tmem_ld16(lane_base + 16 * (chunks + t), acc);
+                    tmem_wait16(acc);
+                    const bool valid = (t0 + done + t) * kTile + r < L;
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        *reinterpret_cast<uint4 *>(vt + r * 128 + c * 16) = make_uint4(0u, 0u, 0u, 0u);
-                        *reinterpret_cast<uint4 *>(vt + kTcHalf + r * 128 + c * 16) = make_uint4(0u, 0u, 0u, 0u);
-                    }
+                    for (int g = 0; g < G; ++g)
+                        if (valid) m[g] = fmaxf(m[g], __uint_as_float(acc[g]) * c2);
                 }
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // generic writes -> tensor-core reads
-            mbar_arrive(bar(kBarPFull + pb));
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) m[g] = fmaxf(m[g], __shfl_xor_sync(0xffffffffu, m[g], off));
+                if (lane == 0) red[warp * 8 + g] = m[g];
+            }
+            softmax_sync();
+#pragma unroll
+            for (int g = 0; g < G; ++g) m[g] = fmaxf(fmaxf(red[g], red[8 + g]), fmaxf(red[16 + g], red[24 + g]));
+            softmax_sync();                              // `red` is used again
+
+            for (int t = 0; t < n && ok; ++t) {
+                const int pt = done + t, pb = pt & 1, i = 2 * done + n + t;
+                if (kFp8) ok = widen_tile(i);
+                if (ok) ok = mbar_wait(bar(kBarPEmpty + pb), ((pt >> 1) & 1) ^ 1, abort_flag, sink);
+                if (!ok) break;
+                uint32_t acc[16];
+                tmem_ld16(lane_base + 16 * (chunks + t), acc);
+                tmem_wait16(acc);
+                tc_fence_before();                       // (the second chunk's scores are written behind this thread's arrival below)
+                const bool valid = (t0 + done + t) * kTile + r < L;
+                uint8_t *pt_smem = smem + kOffP + pb * kTcSmall;
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    // (a NaN or infinite score of a row that is not cached never gets here: `valid` decides)
+                    const float w = valid ? exp2f(__uint_as_float(acc[g]) * c2 - m[g]) : 0.f;
+                    const __nv_bfloat16 hi = __float2bfloat16_rn(w);
+                    const __nv_bfloat16 lo = __float2bfloat16_rn(w - __bfloat162float(hi));
+                    l[g] += __bfloat162float(hi) + __bfloat162float(lo);
+                    *reinterpret_cast<__nv_bfloat16 *>(pt_smem + small_off(g, r)) = hi;
+                    *reinterpret_cast<__nv_bfloat16 *>(pt_smem + small_off(8 + g, r)) = lo;
+                }
+                if (!kFp8 && !valid) {
+                    // a row beyond the sequence's length may hold anything, and 0 x NaN would spoil the product: its V row
+                    // is cleared in shared memory (only the split's last tile has such rows)
+                    const int s = i % kTcStages;
+                    ok = mbar_wait(bar(kBarFull + s), (i / kTcStages) & 1, abort_flag, sink);
+                    if (ok) {
+                        uint8_t *vt = smem + kOffRing + s * kTcTileBytes;
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) {
+                            *reinterpret_cast<uint4 *>(vt + r * 128 + x * 16) = make_uint4(0u, 0u, 0u, 0u);
+                            *reinterpret_cast<uint4 *>(vt + kTcHalf + r * 128 + x * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // generic writes -> tensor-core reads
+                mbar_arrive(bar(kBarPFull + pb));
+            }
+        }
+        // the chunks relative to the larger of their maxima (one chunk: w0 = 0, w1 = 1)
+        float w0[G], w1[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const float top = fmaxf(m0[g], m[g]);
+            w0[g] = chunks > 1 ? exp2f(m0[g] - top) : 0.f;
+            w1[g] = chunks > 1 ? exp2f(m[g] - top) : 1.f;
+            l[g] = chunks > 1 ? l0[g] * w0[g] + l[g] * w1[g] : l[g];
+            m[g] = top;
         }
 
         // ---- the sums of the weights over the 128 key rows, then the output columns
@@ -412,18 +450,23 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
         }
         softmax_sync();
         if (ok) ok = mbar_wait(bar(kBarOut), 0, abort_flag, sink);
-        uint32_t o[16];
+        uint32_t o[16], o0[16];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) o[c] = 0u;
+        for (int c = 0; c < 16; ++c) o[c] = o0[c] = 0u;
         if (ok) {
             tc_fence_after();
-            tmem_ld16(lane_base, o);
+            tmem_ld16(lane_base + 16 * (chunks - 1), o);
             tmem_wait16(o);
+            if (chunks > 1) {
+                tmem_ld16(lane_base, o0);
+                tmem_wait16(o0);
+            }
         }
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             const float den = ok ? (red[g] + red[8 + g]) + (red[16 + g] + red[24 + g]) : 0.f;     // error path: zeros
-            const float num = __uint_as_float(o[g]) + __uint_as_float(o[8 + g]);
+            float num = __uint_as_float(o[g]) + __uint_as_float(o[8 + g]);
+            if (chunks > 1) num = (__uint_as_float(o0[g]) + __uint_as_float(o0[8 + g])) * w0[g] + num * w1[g];
             if (r >= kDim) continue;                          // (64 dimensions: the padded half of the output)
             if (p.splits == 1) {
                 out[(size_t)g * kDim + r] = den > 0.f ? num / den : 0.f;
@@ -481,44 +524,48 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     }
 }
 
-template <int G, int kSrc>
+template <int G, int kSrc, bool kTwo>
 cudaError_t launch_tc_one(const AttendTcParams &p, int heads, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
                           cudaStream_t s)
 {
     static PerDevice done;
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, attend_tc_kernel<G, kSrc>, kTcSmem, true)) != cudaSuccess) return e;
-    return launch_early(attend_tc_kernel<G, kSrc>, (unsigned)(heads * p.splits), kTcThreads, kTcSmem, s,
+    if (e != cudaSuccess || (e = allow_smem_once(done, dev, attend_tc_kernel<G, kSrc, kTwo>, kTcSmem, true)) != cudaSuccess) return e;
+    return launch_early(attend_tc_kernel<G, kSrc, kTwo>, (unsigned)(heads * p.splits), kTcThreads, kTcSmem, s,
                         p.separate ? 1u : (unsigned)p.splits, p, mk, mv, mq);
 }
 template <int G>
 cudaError_t launch_tc_for(const AttendTcParams &p, int heads, int src, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
                           cudaStream_t s)
 {
-    return src == 1 ? launch_tc_one<G, 1>(p, heads, mk, mv, mq, s) : src == 2 ? launch_tc_one<G, 2>(p, heads, mk, mv, mq, s)
-                                                                          : launch_tc_one<G, 0>(p, heads, mk, mv, mq, s);
+    const bool two = p.tiles_per_split > kTcMaxTiles;
+    if (src == 1) return two ? launch_tc_one<G, 1, true>(p, heads, mk, mv, mq, s) : launch_tc_one<G, 1, false>(p, heads, mk, mv, mq, s);
+    if (src == 2) return two ? launch_tc_one<G, 2, true>(p, heads, mk, mv, mq, s) : launch_tc_one<G, 2, false>(p, heads, mk, mv, mq, s);
+    return two ? launch_tc_one<G, 0, true>(p, heads, mk, mv, mq, s) : launch_tc_one<G, 0, false>(p, heads, mk, mv, mq, s);
 }
 
 }  // namespace
 
-// Splits of a head's key tiles (blocks of a cluster) for the tensor-core kernel: at most kTcMaxTiles tiles per block, and
-// among those the number with the shortest run: waves of resident blocks (2 per SM) times what a block spends, its tiles and
-// about three tiles' worth of set-up and merge.  (128 heads of 33 tiles: 4 splits, two waves of 9 tiles, 49 us; 5, the fewest that give
-// two waves of blocks, 54.  With two tiles' worth 600 heads of 15 tiles were cut in three, 98 us and 114 for 8-bit caches, 93
-// and 97 uncut; 512 heads of 33 tiles in four, 167 and 192, 163 and 172 in three.)  The fewest splits where they give four
-// waves: a part of the last one counts for little then (256 heads of 64 tiles: 159 us with 5 splits, 165 with 8).
+// Splits of a head's key tiles (blocks of a cluster) for the tensor-core kernel: at most 28 tiles per block, and among those the number
+// with the shortest run: waves of resident blocks (2 per SM) times what a block spends, its tiles and about three tiles' worth of
+// set-up and merge, and one and a half more for a second chunk.  (128 heads of 33 tiles: 4 splits, two waves of 9 tiles, 49 us; 5, the
+// fewest that give two waves of blocks, 54.  With two tiles' worth 600 heads of 15 tiles were cut in three, 98 us and 114 for 8-bit
+// caches, 93 and 97 uncut; 512 heads of 33 tiles in four, 167 and 192, 163 and 172 in three.  Two chunks, where one block of 16 to 28
+// tiles takes the place of two: 200 heads of 16 tiles 49.7 us with two splits, 39.0; 512 of 16 99.7, 84.1; 296 of 20 70.4, 63.7; 148 of
+// 33 60.7, 54.7; 8-bit 296 of 17 52.2, 42.9; where the rule keeps one chunk nothing moved.)  The fewest splits of one chunk where
+// they give four waves: a part of the last one counts for little then (256 heads of 64 tiles: 159 us with 5 splits, 165 with 8).
 int attend_tc_splits(int heads, int cap, int sms)
 {
     const int tiles = (cap + kTile - 1) / kTile, least = (tiles + kTcMaxTiles - 1) / kTcMaxTiles;
     if ((long long)heads * least >= 8ll * sms) return least;
     int best = 0;
     long long best_cost = 0;
-    for (int s = least; s <= tiles && s <= kTcMaxSplits; ++s) {
+    for (int s = (tiles + 2 * kTcChunkTiles - 1) / (2 * kTcChunkTiles); s <= tiles && s <= kTcMaxSplits; ++s) {
         const int per = (tiles + s - 1) / s;
         if (s > 1 && (tiles + per - 1) / per < s) continue;          // the last blocks would have no tile
         const long long waves = ((long long)heads * s + 2 * sms - 1) / (2 * sms);
-        const long long cost = waves * (per + 3);
+        const long long cost = waves * (2 * (per + 3) + (per > kTcMaxTiles ? 3 : 0));
         if (best == 0 || cost < best_cost) best = s, best_cost = cost;
     }
     return best;
@@ -559,7 +606,7 @@ cudaError_t launch_attend_tc(const void *k_cache, const void *v_cache, const voi
     p.status = status;
     p.wait_cycles = wait_cycles;
     p.block_table = block_table;
-    if (p.tiles_per_split > kTcMaxTiles) return cudaErrorInvalidValue;
+    if (p.tiles_per_split > 2 * kTcChunkTiles) return cudaErrorInvalidValue;
     const uint64_t rows = block_table ? (uint64_t)pool_pages * kTile : (uint64_t)batch * hkv * cap;
     CUtensorMap mk, mv, mq;
     // src: 0 = bf16 caches of 128 dimensions, 1 = E4M3 codes of 128 dimensions, 2 = bf16 caches of 64 dimensions

@@ -99,3 +99,33 @@ def test_second_pass_items_in_a_row(rkv, head_dim, dtype, beta, T, span, budget,
     rep, comp = run_and_check(rkv, wl, beta=beta, T=T, flags=rkv.RKV_FLAG_NO_SYMMETRIC, check_rows=rows)
     assert rep.ok(), rep.errors
     comp.check_status()
+
+
+@pytest.mark.parametrize("dtype,head_dim,hq", [("bf16", 128, 4), ("bf16", 128, 8), ("fp8", 128, 3), ("bf16", 64, 1)])
+@pytest.mark.parametrize("heads,cap", [(148, 4224), (296, 2176), (148, 7040)])
+def test_decode_attention_in_two_chunks(rkv, dtype, head_dim, hq, heads, cap):  # noqa: F811
+    """Blocks of more key tiles than their columns hold the scores of (17 and 28 tiles, two to a head; 17, one): lengths that end in the
+    first chunk, at its last row, in the second, at a block's first row; logits far apart between the chunks."""
+    import numpy as np
+    import oracle
+    spec = ri.CacheSpec("chunks", 1, heads, 1, hq, head_dim, cap - 64, 64, 8, 0.1, dtype, 16, 0.3, 0.05, 4, 8.0)
+    per = -(-cap // 128) // (1 if heads == 296 else 2) * 128
+    some = [cap, cap - 1, 1, 9 * 128, 9 * 128 + 1, 15 * 128, 15 * 128 + 1, 16 * 128 + 5, per, per + 1, 130]
+    lens = [min(some[b % len(some)], cap) for b in range(heads)]
+    wl = ri.make_workload(spec, device="cuda", seed=611, seq_lens=torch.tensor(lens))
+    wl.k_cache[1::3, :, 1500:] = (wl.k_cache[1::3, :, 1500:].float() * 8).clamp(-448, 448).to(wl.k_cache.dtype)
+    for b, L in enumerate(lens):
+        for t in (wl.k_cache, wl.v_cache):
+            t.view(torch.int16 if dtype == "bf16" else torch.uint8)[b, :, L:] = 0x7FC0 if dtype == "bf16" else 0x7F      # NaN
+    q_new = torch.randn(heads, hq, head_dim, generator=torch.Generator(device="cuda").manual_seed(7), device="cuda").to(torch.bfloat16)
+    comp = rkv.Compressor(heads, 1, hq, spec.budget, spec.buffer, spec.alpha, 0.1, dtype=spec.torch_dtype, head_dim=head_dim)
+    out = torch.full((heads, hq, head_dim), 7.0, device="cuda")
+    assert rkv.rkv_decode_attention(comp.desc, wl.k_cache, wl.v_cache, q_new, wl.seq_lens, out, spec.budget, spec.buffer) == 0
+    torch.cuda.synchronize()
+    comp.check_status()
+    rows = list(range(0, heads, 13)) + list(range(11))
+    K, V = (torch.nan_to_num(t[rows].float(), nan=0.0).cpu().numpy() for t in (wl.k_cache, wl.v_cache))
+    ref = oracle.oracle_decode_attention(K, V, q_new[rows].float().cpu().numpy(), np.array([lens[r] for r in rows], dtype=np.int32))
+    got = out[rows].cpu().numpy().astype(np.float64)
+    scale = np.maximum(np.abs(ref).max(axis=-1, keepdims=True), 1e-30)
+    assert (np.abs(got - ref) <= 1e-3 * scale + 1e-7).all(), float((np.abs(got - ref) / scale).max())
