@@ -74,19 +74,22 @@ enum {
 struct Plan {
     int stages, q_bytes, off_own, off_q, off_sum, off_bar, off_units, off_misc, total;
 };
+// groups: as many as there are stages at most.  A group waits for unit k by the parity of its stage's phase, which is exact once the unit
+// before in that stage, k - stages, has landed; what a group knows to have landed is everything up to its own unit before, k - groups
+// (its key sums were issued in order).
 template <int D, bool kCodes>
-__host__ __device__ inline Plan make_plan(int q_rows_pad)
+__host__ __device__ inline Plan make_plan(int q_rows_pad, int groups)
 {
     Plan pl;
     pl.q_bytes = q_rows_pad * D * 2;
-    const int own = kCodes ? kMaxGroups * kOperandBytes : 0;
-    const int fixed = own + 2 * pl.q_bytes + kMaxGroups * kSumB + kNumBars * 8 + 16 + (kMaxStages + kMaxGroups) * 16 + 32 + 1024;      // + alignment slack
+    const int own = kCodes ? groups * kOperandBytes : 0;
+    const int fixed = own + 2 * pl.q_bytes + groups * kSumB + kNumBars * 8 + 16 + (kMaxStages + kMaxGroups) * 16 + 32 + 1024;      // + alignment slack
     const int stages = (kSmemLimit - fixed) / Form<D, kCodes>::kStageBytes;
     pl.stages = stages > kMaxStages ? kMaxStages : stages;
     pl.off_own = pl.stages * Form<D, kCodes>::kStageBytes;
     pl.off_q = pl.off_own + own;
     pl.off_sum = pl.off_q + 2 * pl.q_bytes;
-    pl.off_bar = pl.off_sum + kMaxGroups * kSumB;
+    pl.off_bar = pl.off_sum + groups * kSumB;
     pl.off_units = pl.off_bar + (kNumBars * 8 + 15) / 16 * 16;
     pl.off_misc = pl.off_units + (kMaxStages + kMaxGroups) * 16;
     pl.total = pl.off_misc + 32 + 1024;
@@ -259,7 +262,7 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
     extern __shared__ uint8_t prep_raw[];
     uint8_t *smem = align_smem(prep_raw);
     const uint32_t sbase = smem_u32(smem);
-    const Plan pl = make_plan<D, kCodes>(q_rows_pad);
+    const Plan pl = make_plan<D, kCodes>(q_rows_pad, groups);
     const uint32_t stages = (uint32_t)pl.stages;
     int *misc = reinterpret_cast<int *>(smem + pl.off_misc);           // TMEM base, abort flag, units and query blocks asked for
     volatile int *abort_flag = misc + 1;
@@ -299,7 +302,7 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     // rows 3 kSub..15 of the key sums' B operands stay zero; the others are rewritten in full for every unit
-    for (int x = threadIdx.x; x < kMaxGroups * kSumB / 16; x += kThreads) reinterpret_cast<uint4 *>(smem + pl.off_sum)[x] = make_uint4(0u, 0u, 0u, 0u);
+    for (int x = threadIdx.x; x < groups * kSumB / 16; x += kThreads) reinterpret_cast<uint4 *>(smem + pl.off_sum)[x] = make_uint4(0u, 0u, 0u, 0u);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -598,8 +601,9 @@ cudaError_t launch_for(const Params &p, cudaStream_t s)
         (e = launch_early(lengths_kernel, (unsigned)((p.batch + kLengthThreads - 1) / kLengthThreads), kLengthThreads, 0, s, 1, p)) != cudaSuccess)
         return e;
     const int total = (p.tiles + F::kSub - 1) / F::kSub * p.batch * p.hkv;
-    const int groups = std::min(kMaxGroups, (int)kTmemCols / (16 + F::kSub * q_rows_pad));
-    return launch_early(prep_sm100_kernel<D, kCodes>, (unsigned)std::min(total, sms), kThreads, (size_t)make_plan<D, kCodes>(q_rows_pad).total, s, 1, p,
+    int groups = std::min(kMaxGroups, (int)kTmemCols / (16 + F::kSub * q_rows_pad));
+    while (groups > 1 && make_plan<D, kCodes>(q_rows_pad, groups).stages < groups) --groups;
+    return launch_early(prep_sm100_kernel<D, kCodes>, (unsigned)std::min(total, sms), kThreads, (size_t)make_plan<D, kCodes>(q_rows_pad, groups).total, s, 1, p,
                         map_k, map_q, map_wide, table, copy, total, q_rows_pad, groups);
 }
 

@@ -24,10 +24,12 @@ def test_logits_of_the_prep_stage(rkv, head_dim, dtype, hq, alpha, mean):  # noq
     comp.check_status()
 
 
+@pytest.mark.parametrize("hq", [16, 64, 112])
 @pytest.mark.parametrize("head_dim,dtype", [(64, "bf16"), (128, "bf16"), (128, "fp8")])
-def test_logits_where_blocks_take_many_units(rkv, head_dim, dtype):  # noqa: F811
-    """1600 heads of two tiles: every block's range runs over many heads, so query blocks and ring stages are used over and over."""
-    spec = small_spec("range", batch=200, hkv=8, hq=16, budget=150, buffer=42, head_dim=head_dim, dtype=dtype, span=8)
+def test_logits_where_blocks_take_many_units(rkv, head_dim, dtype, hq):  # noqa: F811
+    """1600 heads of two tiles: every block's range runs over many heads, so query blocks and ring stages are used over and over; with 16,
+    64 and 112 query rows the ring has more stages than there are groups, and as many."""
+    spec = small_spec("range", batch=200, hkv=8, hq=hq, budget=150, buffer=42, head_dim=head_dim, dtype=dtype, span=8)
     lens = [(192, 191, 151, 150)[b % 4] for b in range(200)]
     wl = ri.make_workload(spec, device="cuda", seed=551, seq_lens=torch.tensor(lens))
     rep, comp = run_and_check(rkv, wl, check_rows=[0, 1, 2, 98, 99, 100, 101, 197, 198])
