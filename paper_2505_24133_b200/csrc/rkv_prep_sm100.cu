@@ -292,7 +292,8 @@ __device__ __forceinline__ void pool_logits(const Params &p, uint32_t qbase, boo
 }
 
 // map_k: the stored keys.  map_wide, copy: see above.  q_rows_pad: 0 where another kernel forms the logits.  table: the block table of
-// the stored keys.  groups: as many as have room for their accumulators (64 dimensions: three from 64 query rows on, two from 80).
+// the stored keys.  groups: as many as have room for their accumulators (64 dimensions: three from 64 query rows on, two from 80), and for
+// no fewer ring stages (codes: three from 48 query rows on).
 template <int D, bool kCodes>
 __global__ void __launch_bounds__(kThreads, 1)
 prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,
