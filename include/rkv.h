@@ -58,7 +58,7 @@ typedef enum {
  *   RKV_FP8_E4M3: k_cache and v_cache hold 8-bit E4M3 codes (1 sign bit, 4 exponent bits with bias 7, 3 mantissa bits,
  *     no infinities; one byte per element, rows of head_dim bytes); q_window (and q_new of rkv_push_query) is bf16.
  *     Eq. 1-7 are evaluated on the values the codes stand for.  With head_dim 128 the two-pass tensor-core kernels score the codes
- *     as they are stored; otherwise the keys are widened to bf16 (exactly; every E4M3 value is a bf16 value) into the workspace and
+ *     as they are stored (where one call preps and scores them); otherwise the keys are widened to bf16 (exactly; every E4M3 value is a bf16 value) into the workspace and
  *     scored there as for a bf16 cache.  The workspace has room for that copy in either case, (batch * n_kv_heads * (budget + buffer)
  *     + 128) * head_dim * 2 bytes (for head_dim 64 it has so for bf16 caches too).  The compaction moves the stored bytes; no
  *     scale factor is applied or needed (cosine similarity does not see a per-tensor scale; fold a key scale into
@@ -90,9 +90,8 @@ typedef enum { RKV_BF16 = 0, RKV_F32 = 1, RKV_FP8_E4M3 = 2 } rkv_dtype_t;
                                    scored by forming each pair of key tiles once; beta = 1 only).  A cross-check. */
 
 /* stage bits for rkv_compress_stages */
-#define RKV_STAGE_PREP 1u    /* key inverse norms and per-tile sums of normalised keys; on the two-pass tensor-core route, which reads
-                              * the keys here anyway, Eq. 2-3 pooled logits as well */
-#define RKV_STAGE_SCORES 2u  /* Eq. 2-3 pooled logits (other routes); Eq. 5 matrix + retention rule + Eq. 6 column means */
+#define RKV_STAGE_PREP 1u    /* key inverse norms and per-tile sums of normalised keys */
+#define RKV_STAGE_SCORES 2u  /* Eq. 2-3 pooled logits; Eq. 5 matrix + retention rule + Eq. 6 column means */
 #define RKV_STAGE_SELECT 4u  /* Eq. 3 softmax, Eq. 4, Eq. 6 softmax, Eq. 7, top-k, index list */
 #define RKV_STAGE_GATHER 8u  /* in-place compaction of K and V, seq_lens update */
 #define RKV_STAGE_ALL 15u
@@ -209,7 +208,10 @@ RKV_API int rkv_compress_ex(const rkv_desc_t *desc, void *k_cache, void *v_cache
                     int32_t *out_idx, void *stream);
 
 /* The same, running only the stages in stage_mask (RKV_STAGE_*); stages hand their results on through the
- * workspace, so running them one by one in order equals one full call.  For per-stage timing and tests. */
+ * workspace, so running them one by one in order equals one full call.  For per-stage timing and tests.
+ * Each stage reads its inputs when it runs: q_window counts as it stands when RKV_STAGE_SCORES runs, seq_lens and (for 8-bit caches,
+ * which are scored on a copy then) the keys as they stand when RKV_STAGE_PREP runs.  A call that has PREP and SCORES in its mask forms
+ * the logits while prep reads the keys; SCORES in a call of its own reads the keys once more for them. */
 RKV_API int rkv_compress_stages(const rkv_desc_t *desc, void *k_cache, void *v_cache, const void *q_window,
                         int32_t *seq_lens, int32_t budget, int32_t buffer, int32_t alpha, float lambda,
                         int32_t *out_idx, void *stream, uint32_t stage_mask);

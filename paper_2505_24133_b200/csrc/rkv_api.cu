@@ -215,7 +215,11 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
     // What the gather moves is the caller's caches as they are stored; where a copy is scored every stage before it reads the
     // bf16 copy of the keys (contiguous: the block table, if any, is followed once, by the widening kernel).
     Params stored = p;
-    p.codes = direct_codes(d) ? 1 : 0;
+    // The queries that count, and of 8-bit caches the keys, are those of the stages that always read them: the queries at the
+    // scores, 8-bit keys at prep.  Both at once only where one call has both stages.
+    const bool at_once = (stages & RKV_STAGE_PREP) && (stages & RKV_STAGE_SCORES);
+    p.form_logits = p.tri && at_once ? 1 : 0;
+    p.codes = direct_codes(d) && at_once ? 1 : 0;
     const bool copies = needs_copy(d) && !p.codes;
     if (copies) {
         p.k_cache = ws + lay.k_wide;
@@ -238,6 +242,7 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
     }
     if ((e = mark(1)) != cudaSuccess) return cuda_fail(e, "cudaEventRecord");
     if (stages & RKV_STAGE_SCORES) {
+        if (p.tri && !at_once && (e = launch_logits_sm100(p, s)) != cudaSuccess) return cuda_fail(e, "logits launch");
         e = use_simt(d) ? launch_scores_simt(p, s)
                         : (p.tri ? launch_scores_tri_sm100(p, s) : launch_scores_sm100(p, s));
         if (e != cudaSuccess) return cuda_fail(e, "scores launch");
@@ -620,6 +625,8 @@ int rkv_launch_count(const rkv_desc_t *desc, uint32_t stage_mask)
     // the kernel that writes the scoring copy, or the one that records the lengths
     if (desc && (stage_mask & RKV_STAGE_PREP) && (needs_copy(desc) || lengths_ahead(desc))) c += 1;
     if (desc && (stage_mask & RKV_STAGE_SELECT) && (desc->flags & RKV_FLAG_HEAD_MEAN)) c += 1;   // per-sequence selection
+    // the two-pass route's logits, where they are not formed by a prep kernel of the same call
+    if (desc && (stage_mask & RKV_STAGE_SCORES) && !(stage_mask & RKV_STAGE_PREP) && use_tri(desc)) c += 2;
     // the two-pass scoring path is the first pass plus up to two rounds of (listing, second pass) while the
     // retention rule is on
     if (desc && (stage_mask & RKV_STAGE_SCORES) && use_tri(desc) && desc->beta > 0 && desc->sim_threshold < 1.0f) {

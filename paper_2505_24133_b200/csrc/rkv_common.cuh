@@ -36,7 +36,8 @@ struct Params {
     int dtype;                      // of the keys the scoring stages read (bf16 where a widened copy of 8-bit caches is scored)
     int store_row_bytes;            // bytes of a row of the caches as stored (what the gather moves)
     float logit_scale;              // Eq. 2's 1 / sqrt(d) with the caches' own head dimension (d above may be a padded one)
-    int lengths_done;               // 1: a kernel of its own records the lengths and clears the counters ahead of prep
+    int lengths_done;               // 1: the lengths are recorded and the counters cleared when the prep kernel starts
+    int form_logits;                // 1: the prep kernel forms Eq. 2-3's logits
     int codes;                      // 1: the keys are scored as they are stored, E4M3 codes of 128 dimensions
     int fused_codes;                // 1: prep writes the scoring copy itself (k_cache above) from stored rows of 128 E4M3 codes
     const void *fuse_src;           // the stored keys
@@ -295,6 +296,7 @@ size_t compression_bytes(const rkv_desc_t *d, int budget, int buffer, int alpha)
 
 // launchers (one per stage); each returns cudaGetLastError() of its launch
 cudaError_t launch_prep(const Params &p, cudaStream_t s);
+cudaError_t launch_logits_sm100(Params p, cudaStream_t s);      // two-pass route, the scores without the stage before: Eq. 2-3's logits
 cudaError_t launch_widen_keys(const Params &stored, __nv_bfloat16 *wide, int wide_d, const void *q_src, void *q_dst,
                               bool keys, cudaStream_t s);
 cudaError_t launch_scores_simt(const Params &p, cudaStream_t s);

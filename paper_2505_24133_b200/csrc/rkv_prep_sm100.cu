@@ -126,7 +126,7 @@ __device__ __forceinline__ PrepUnit prep_unit_at(const Params &p, int idx, bool 
     return w;
 }
 
-// bf16 caches of 64 dimensions: the lengths are recorded and the counters cleared ahead of the prep kernel.
+// Where the lengths are recorded and the counters cleared ahead of the prep kernel (Params::lengths_done).
 constexpr int kLengthThreads = 256;
 __global__ void __launch_bounds__(kLengthThreads) lengths_kernel(Params p)
 {
@@ -629,8 +629,8 @@ cudaError_t launch_for(const Params &p, cudaStream_t s)
     int dev = 0, sms = 0;
     cudaError_t e = device_sms(&dev, &sms);
     if (e != cudaSuccess || (e = allow_smem_once(done, dev, prep_sm100_kernel<D, kCodes>, kSmemLimit)) != cudaSuccess) return e;
-    // the logits are left to the other scoring kernels where those form them
-    const int q_rows_pad = p.tri ? (p.group * p.alpha + 15) / 16 * 16 : 0;
+    // the logits are left to the other scoring kernels where those form them, and to a later call that scores
+    const int q_rows_pad = p.form_logits ? (p.group * p.alpha + 15) / 16 * 16 : 0;
     const int copy = kCodes ? p.fused_codes : 0;
     const int32_t *table = copy ? p.fuse_table : p.block_table;
     const uint64_t rows = table ? (uint64_t)p.pool_pages * kTile : (uint64_t)p.batch * p.hkv * p.cap;
@@ -640,9 +640,6 @@ cudaError_t launch_for(const Params &p, cudaStream_t s)
                     (!copy || make_map(&map_wide, p.k_cache, (uint64_t)p.batch * p.hkv * p.cap + kTile, kTile));
     if (!ok) return cudaErrorInvalidValue;
     if (!copy) map_wide = map_k;
-    if (p.lengths_done &&
-        (e = launch_early(lengths_kernel, (unsigned)((p.batch + kLengthThreads - 1) / kLengthThreads), kLengthThreads, 0, s, 1, p)) != cudaSuccess)
-        return e;
     const int total = (p.tiles + F::kSub - 1) / F::kSub * p.batch * p.hkv;
     int groups = std::min(kMaxGroups, (int)kTmemCols / (16 + F::kSub * q_rows_pad));
     while (groups > 1 && make_plan<D, kCodes>(q_rows_pad, groups).stages < groups) --groups;
@@ -654,7 +651,22 @@ cudaError_t launch_for(const Params &p, cudaStream_t s)
 
 cudaError_t launch_prep_sm100(const Params &p, cudaStream_t s)
 {
-    const cudaError_t e = p.fused_codes || p.codes ? launch_for<128, true>(p, s) : p.d == 64 ? launch_for<64, false>(p, s) : launch_for<128, false>(p, s);
+    cudaError_t e = cudaSuccess;
+    if (p.lengths_done)
+        e = launch_early(lengths_kernel, (unsigned)((p.batch + kLengthThreads - 1) / kLengthThreads), kLengthThreads, 0, s, 1, p);
+    if (e != cudaSuccess) return e;
+    e = p.fused_codes || p.codes ? launch_for<128, true>(p, s) : p.d == 64 ? launch_for<64, false>(p, s) : launch_for<128, false>(p, s);
+    return e == cudaSuccess ? launch_head_sum(p, s) : e;
+}
+
+// The queries belong to the stage that scores: where that is called by itself, the prep kernel goes over the keys once more with the
+// lengths recorded before, and leaves the logits beside what it left then.  (The head sums' kernel is what sees that a block gave up.)
+cudaError_t launch_logits_sm100(Params p, cudaStream_t s)
+{
+    p.lengths_done = p.form_logits = 1;
+    p.seq_lens = p.meta;
+    p.budgets = p.meta + p.batch;
+    const cudaError_t e = p.d == 64 ? launch_for<64, false>(p, s) : launch_for<128, false>(p, s);
     return e == cudaSuccess ? launch_head_sum(p, s) : e;
 }
 

@@ -123,6 +123,11 @@ def test_rkv_compress_needs_a_current_descriptor(rkv):
     assert rkv.rkv_launch_count_for(_desc(rkv), 64, 32, 8, rkv.RKV_STAGE_ALL) == 5          # one key tile: no second pass
     assert rkv.rkv_launch_count_for(_desc(rkv), 8, 128, 8, rkv.RKV_STAGE_ALL) == 0           # invalid sizes
     assert rkv.rkv_launch_count_for(_desc(rkv, flags=rkv.RKV_FLAG_HEAD_MEAN), 1024, 128, 8, rkv.RKV_STAGE_ALL) == 8
+    # the scores by themselves: the two-pass route's logits take two launches of their own
+    for flags, more in ((0, 2), (rkv.RKV_FLAG_ROWBLOCK_SCORES, 0), (rkv.RKV_FLAG_SIMT_SCORES, 0)):
+        d = _desc(rkv, flags=flags)
+        apart = sum(rkv.rkv_launch_count_for(d, 1024, 128, 8, bit) for bit in (1, 2, 4, 8))
+        assert apart == rkv.rkv_launch_count_for(d, 1024, 128, 8, rkv.RKV_STAGE_ALL) + more
 
 
 def test_product_package_does_not_touch_the_oracle():

@@ -3,7 +3,8 @@ import pytest
 import torch
 
 import rkv_inputs as ri
-from test_gpu_parity import rkv, run_and_check, small_spec  # noqa: F401  (rkv: the fixture)
+from parity_util import check_batch
+from test_gpu_parity import DEFAULTS, rkv, run_and_check, small_spec  # noqa: F401  (rkv: the fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -131,3 +132,36 @@ def test_decode_attention_in_two_chunks(rkv, dtype, head_dim, hq, heads, cap):  
     got = out[rows].cpu().numpy().astype(np.float64)
     scale = np.maximum(np.abs(ref).max(axis=-1, keepdims=True), 1e-30)
     assert (np.abs(got - ref) <= 1e-3 * scale + 1e-7).all(), float((np.abs(got - ref) / scale).max())
+
+
+@pytest.mark.parametrize("head_dim,dtype,budget,buffer", [(64, "bf16", 300, 100), (128, "bf16", 300, 100), (128, "bf16", 90, 30),
+                                                          (128, "fp8", 300, 84), (128, "fp8", 300, 100), (64, "fp8", 300, 84)])
+@pytest.mark.parametrize("beta,T", [(1, 0.5), (1, 1.0)])
+def test_stages_read_their_inputs_when_they_run(rkv, head_dim, dtype, budget, buffer, beta, T):  # noqa: F811
+    """The queries that count are those at the scores; lengths, and 8-bit keys, those at prep: what changes afterwards plays no part."""
+    cap = budget + buffer
+    lens = [cap, cap - 1, budget + 1, budget]
+    spec = small_spec("when", batch=4, hkv=2, hq=8, budget=budget, buffer=buffer, head_dim=head_dim, dtype=dtype, span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=591 + budget, seq_lens=torch.tensor(lens))
+    k0, v0, q0, s0 = wl.k_cache.clone(), wl.v_cache.clone(), wl.q_window.clone(), wl.seq_lens.clone()
+    comp = rkv.Compressor(4, 2, 8, budget, buffer, spec.alpha, 0.1, dtype=spec.torch_dtype, head_dim=head_dim, beta=beta, sim_threshold=T,
+                          dump_scores=True)
+    args = wl.k_cache, wl.v_cache, wl.q_window, wl.seq_lens
+    wl.q_window.normal_(generator=torch.Generator(device="cuda").manual_seed(3)).mul_(4)
+    comp.compress(*args, stages=rkv.RKV_STAGE_PREP)
+    wl.q_window.copy_(q0)
+    wl.seq_lens.copy_(s0.flip(0))
+    if dtype == "fp8":
+        wl.k_cache.view(torch.uint8).fill_(0x38)
+    comp.compress(*args, stages=rkv.RKV_STAGE_SCORES)
+    wl.q_window.zero_()
+    wl.k_cache.copy_(k0)
+    comp.compress(*args, stages=rkv.RKV_STAGE_SELECT)
+    wl.seq_lens.copy_(s0)
+    idx = comp.compress(*args, stages=rkv.RKV_STAGE_GATHER)
+    torch.cuda.synchronize()
+    comp.check_status()
+    rep = check_batch(k0, v0, q0, s0, budget=budget, alpha=spec.alpha, lam=0.1, gpu_idx=idx, gpu_k=wl.k_cache, gpu_v=wl.v_cache,
+                      gpu_seq=wl.seq_lens, gpu_scores=comp.scores, **{**DEFAULTS, "beta": beta, "T": T})
+    assert rep.ok(), rep.errors
+    assert rep.compressed_heads == 2 * sum(L > budget for L in lens)
