@@ -132,11 +132,18 @@ __device__ __forceinline__ uint32_t small_off(int g, int k)
 }
 
 // With kFp8, kBarFull / kBarEmpty [0 .. kConvBufs) stand for the widened tiles (filled by the softmax threads, 128 arrivals).
-// kTwo: blocks of more tiles than one chunk takes (an instance of its own: small calls are latency, 6.3 us without this code, 6.5 with it).
+// kForm: instances of their own, since a block's time is a chain of latencies that code for the others' sake lengthens.
+//   kPlain  the length first, then what it says there is
+//   kEarly  small grids, which nothing but latencies bound: the queries and the first key tile are under way together with the length (the
+//           tile is part of the cache whatever that is), and the merge asks for all that the other blocks hold before it uses any of it
+//           (8 heads of one tile 6.5 us, 5.6; 8 of 9 tiles 6.8, 6.5).  In larger ones the tiles of idle splits are bytes taken from the others
+//           (1024 heads of 9 tiles, three quarters of the sequences empty: 25.4 us, and 32.2 with the early tiles).
+//   kTwo    blocks of more tiles than one chunk takes
 // kSrc: 0 = bf16 caches of 128 dimensions (tiles go to the tensor cores as they land), 1 = E4M3 codes of 128 dimensions,
 // 2 = bf16 caches of 64 dimensions (both: rows of 128 bytes, widened / padded with zeros into bf16 operand tiles of
 // 128 dimensions; the queries of the 64-dimension case fill the first half of their operand, the rest stays zero).
-template <int G, int kSrc, bool kTwo>
+enum { kPlain, kEarly, kTwo };
+template <int G, int kSrc, int kForm>
 __global__ void __launch_bounds__(kTcThreads, 2)
 attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                  const __grid_constant__ CUtensorMap map_q)
@@ -180,7 +187,7 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
                      ::"r"(smem_u32(tmem_holder)), "r"(kTcTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (warp == 4 && lane == 0)
+    if (kForm == kEarly && warp == 4 && lane == 0)
         for (const CUtensorMap *m : {&map_q, &map_k, &map_v}) prefetch_map(m);
     // the P buffers start as zeros: rows of queries the group does not have are never written (and so does the query
     // operand: with 64 dimensions only its first half is loaded)
@@ -199,29 +206,29 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     auto tile_y = [&](int t) -> int {
         return p.block_table ? p.block_table[(size_t)head * (p.cap / kTile) + t] * kTile : head * p.cap + t * kTile;
     };
-    // source tile i of the block (the K tiles, then the V tiles) into its place in the ring
-    auto fetch_tile = [&](const CUtensorMap *map, int i, int t) {
+    // tile i of the block's source tiles (the K tiles, then the V tiles), from row y on, into its place in the ring
+    auto fetch_tile = [&](const CUtensorMap *map, int i, int y) {
         if (kFp8) {
             const int s = i % kRawStages;
             mbar_expect_tx(bar(kBarRawFull + s), kRawBytes);
-            tma_load_2d(sbase + kOffRaw + s * kRawBytes, map, 0, tile_y(t), bar(kBarRawFull + s));
+            tma_load_2d(sbase + kOffRaw + s * kRawBytes, map, 0, y, bar(kBarRawFull + s));
         } else {
-            const int s = i % kTcStages, y = tile_y(t);
+            const int s = i % kTcStages;
             const uint32_t dst = sbase + kOffRing + s * kTcTileBytes;
             mbar_expect_tx(bar(kBarFull + s), kTcTileBytes);
             tma_load_2d(dst, map, 0, y, bar(kBarFull + s));
             tma_load_2d(dst + kTcHalf, map, 64, y, bar(kBarFull + s));
         }
     };
-    // The queries and the first key tile are under way together with the length (the tile is part of the cache whatever that is): a
-    // small call is a chain of latencies.  With the maps and the merge's loads early too, 8 heads of one tile 6.5 -> 5.6 us, 128 of one
-    // 6.0 -> 5.4, 8 of 9 tiles 6.9 -> 6.3, 600 of 9 as before.
-    if (warp == 4 && lane == 0) {
+    auto fetch_queries = [&]() {
         mbar_expect_tx(bar(kBarQ), kSrc == 2 ? kTcSmall / 2 : kTcSmall);
         const int qy = b * p.hq + h * G;                 // the group's G query rows (the rows after them are not used)
         tma_load_2d(sbase + kOffQ, &map_q, 0, qy, bar(kBarQ));
         if (kSrc != 2) tma_load_2d(sbase + kOffQ + kTcSmall / 2, &map_q, 64, qy, bar(kBarQ));
-        fetch_tile(&map_k, 0, t0);
+    };
+    if (kForm == kEarly && warp == 4 && lane == 0) {
+        fetch_queries();
+        fetch_tile(&map_k, 0, tile_y(t0));
     }
     int L = p.seq_lens[b];
     if (L < 0 || L > p.cap) {               // reported, and treated as an empty cache
@@ -230,10 +237,10 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     }
     const int T = min(p.tiles_per_split, (L + kTile - 1) / kTile - t0);      // its tiles (<= 0: none)
     // more than a block's columns hold the scores of: two chunks, one after the other, each with its own maximum and output columns
-    const int chunks = kTwo && T > kTcMaxTiles ? 2 : 1, T0 = chunks == 2 ? (T + 1) / 2 : T;        // T0: tiles of the first chunk
+    const int chunks = kForm == kTwo && T > kTcMaxTiles ? 2 : 1, T0 = chunks == 2 ? (T + 1) / 2 : T;        // T0: tiles of the first chunk
     // in the order of the ring -- the first chunk's K tiles, its V tiles, the second's -- tile i is this one of the block, of K or of V
     auto source = [&](int i, bool *value) -> int {
-        const int c = kTwo && i >= 2 * T0, j = c ? i - 2 * T0 : i, n = c ? T - T0 : T0;
+        const int c = kForm == kTwo && i >= 2 * T0, j = c ? i - 2 * T0 : i, n = c ? T - T0 : T0;
         *value = j >= n;
         return (c ? T0 : 0) + (j >= n ? j - n : j);
     };
@@ -244,11 +251,13 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     float *out = p.out + ((size_t)b * p.hq + (size_t)h * G) * kDim;
 
     if (T <= 0) {       // no cached row falls into this split (uniform for the block)
-        if (warp == 4 && lane == 0) {                    // what is under way lands before the block's memory is given up
-            mbar_wait(bar(kBarQ), 0, abort_flag, sink);
-            mbar_wait(bar(kFp8 ? kBarRawFull : kBarFull), 0, abort_flag, sink);
+        if (kForm == kEarly) {                           // what is under way lands before the block's memory is given up
+            if (warp == 4 && lane == 0) {
+                mbar_wait(bar(kBarQ), 0, abort_flag, sink);
+                mbar_wait(bar(kFp8 ? kBarRawFull : kBarFull), 0, abort_flag, sink);
+            }
+            __syncwarp();
         }
-        __syncwarp();
         if (p.splits == 1) {
             for (int x = threadIdx.x; x < G * kDim; x += kTcThreads) out[x] = 0.f;
         } else {
@@ -265,11 +274,12 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
             constexpr int kRing = kFp8 ? kRawStages : kTcStages, kEmpty = kFp8 ? kBarRawEmpty : kBarEmpty;
-            for (int i = 1; i < 2 * T; ++i) {                // the other K tiles, then the V tiles
-                if (!mbar_wait(bar(kEmpty + i % kRing), ((i / kRing) & 1) ^ 1, abort_flag, sink)) break;
+            if (kForm != kEarly) fetch_queries();
+            for (int i = kForm == kEarly ? 1 : 0; i < 2 * T; ++i) {
                 bool value;
-                const int t = source(i, &value);
-                fetch_tile(value ? &map_v : &map_k, i, t0 + t);
+                const int y = tile_y(t0 + source(i, &value));
+                if (!mbar_wait(bar(kEmpty + i % kRing), ((i / kRing) & 1) ^ 1, abort_flag, sink)) break;
+                fetch_tile(value ? &map_v : &map_k, i, y);
             }
         }
         __syncwarp();
@@ -282,7 +292,7 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
             // f32 accumulate, bf16 x bf16, A MN-major (bit 15), B K-major, M = 128, N = 16
             const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
             int i = 0;                                       // tiles of the ring so far
-            for (int c = 0; c < (kTwo ? chunks : 1) && ok; ++c) {
+            for (int c = 0; c < (kForm == kTwo ? chunks : 1) && ok; ++c) {
                 const int n = c ? T - T0 : T0, done = c ? T0 : 0;
                 // (the second chunk's scores take the columns of the first's: the last of its weights have been waited for)
                 for (int t = 0; t < n && ok; ++t, ++i) {     // scores of key tile t into its own 16 columns
@@ -358,7 +368,7 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
         float m[G], l[G], m0[G], l0[G];              // of the present chunk, and of the first
 #pragma unroll
         for (int g = 0; g < G; ++g) m0[g] = -INFINITY, l0[g] = 0.f;
-        for (int c = 0; c < (kTwo ? chunks : 1); ++c) {
+        for (int c = 0; c < (kForm == kTwo ? chunks : 1); ++c) {
             const int n = c ? T - T0 : T0, done = c ? T0 : 0;
             if (kFp8)
                 for (int t = 0; t < n && ok; ++t) ok = widen_tile(2 * done + t);
@@ -399,7 +409,7 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
                 uint32_t acc[16];
                 tmem_ld16(lane_base + 16 * (chunks + t), acc);
                 tmem_wait16(acc);
-                tc_fence_before();                       // (the second chunk's scores are written behind this thread's arrival below)
+                if (kForm == kTwo) tc_fence_before();    // (the second chunk's scores are written behind this thread's arrival below)
                 const bool valid = (t0 + done + t) * kTile + r < L;
                 uint8_t *pt_smem = smem + kOffP + pb * kTcSmall;
 #pragma unroll
@@ -488,16 +498,16 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
         for (int x = split * kTcThreads + threadIdx.x; x < G * kDim; x += p.splits * kTcThreads) {
             const int g = x / kDim, c = x % kDim;
             const uint32_t row = base + (uint32_t)(g * kStride) * 4u;
-            // everything that the other blocks hold is asked for before any of it is used
             float ms[kTcMaxSplits], ns[kTcMaxSplits], ls[kTcMaxSplits], m = -INFINITY, num = 0.f, den = 0.f;
 #pragma unroll
             for (int s = 0; s < kTcMaxSplits; ++s) {
                 ms[s] = -INFINITY;
-                ns[s] = ls[s] = 0.f;
                 if (s < p.splits) {
                     ms[s] = ld_cluster(row + kHeadDim * 4u, s);
-                    ns[s] = ld_cluster(row + (uint32_t)c * 4u, s);
-                    ls[s] = ld_cluster(row + (kHeadDim + 1) * 4u, s);
+                    if (kForm == kEarly) {
+                        ns[s] = ld_cluster(row + (uint32_t)c * 4u, s);
+                        ls[s] = ld_cluster(row + (kHeadDim + 1) * 4u, s);
+                    }
                 }
             }
 #pragma unroll
@@ -506,8 +516,8 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
             for (int s = 0; s < kTcMaxSplits; ++s) {                   // fixed order; a split without rows has m = -inf
                 if (ms[s] == -INFINITY) continue;
                 const float w = exp2f(ms[s] - m);
-                num = fmaf(w, ns[s], num);
-                den = fmaf(w, ls[s], den);
+                num = fmaf(w, kForm == kEarly ? ns[s] : ld_cluster(row + (uint32_t)c * 4u, s), num);
+                den = fmaf(w, kForm == kEarly ? ls[s] : ld_cluster(row + (kHeadDim + 1) * 4u, s), den);
             }
             out[x] = den > 0.f ? num / den : 0.f;
         }
@@ -524,25 +534,36 @@ attend_tc_kernel(AttendTcParams p, const __grid_constant__ CUtensorMap map_k, co
     }
 }
 
-template <int G, int kSrc, bool kTwo>
+template <int G, int kSrc, int kForm>
 cudaError_t launch_tc_one(const AttendTcParams &p, int heads, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
-                          cudaStream_t s)
+                          int dev, cudaStream_t s)
 {
     static PerDevice done;
-    int dev = 0, sms = 0;
-    cudaError_t e = device_sms(&dev, &sms);
-    if (e != cudaSuccess || (e = allow_smem_once(done, dev, attend_tc_kernel<G, kSrc, kTwo>, kTcSmem, true)) != cudaSuccess) return e;
-    return launch_early(attend_tc_kernel<G, kSrc, kTwo>, (unsigned)(heads * p.splits), kTcThreads, kTcSmem, s,
+    const cudaError_t e = allow_smem_once(done, dev, attend_tc_kernel<G, kSrc, kForm>, kTcSmem, true);
+    if (e != cudaSuccess) return e;
+    return launch_early(attend_tc_kernel<G, kSrc, kForm>, (unsigned)(heads * p.splits), kTcThreads, kTcSmem, s,
                         p.separate ? 1u : (unsigned)p.splits, p, mk, mv, mq);
+}
+template <int G, int kSrc>
+cudaError_t launch_tc_form(const AttendTcParams &p, int heads, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq, cudaStream_t s)
+{
+    int dev = 0, sms = 0;
+    const cudaError_t e = device_sms(&dev, &sms);
+    if (e != cudaSuccess) return e;
+    if (p.tiles_per_split > kTcMaxTiles) return launch_tc_one<G, kSrc, kTwo>(p, heads, mk, mv, mq, dev, s);
+    // A block per SM, or two of few tiles: beside a second block of many an idle one's tile costs more than an early start gives (32 heads of 9
+    // tiles, 288 blocks of one: 13.0 us, 12.1 early; 256 blocks of nine, 256 heads of which half are empty: 12.6, 13.2; 128 heads of 17 tiles, 1000
+    // tokens: 15.6, 16.0).
+    const long long blocks = (long long)heads * p.splits;
+    return blocks <= sms || (blocks <= 2ll * sms && p.tiles_per_split <= 4) ? launch_tc_one<G, kSrc, kEarly>(p, heads, mk, mv, mq, dev, s)
+                                                                            : launch_tc_one<G, kSrc, kPlain>(p, heads, mk, mv, mq, dev, s);
 }
 template <int G>
 cudaError_t launch_tc_for(const AttendTcParams &p, int heads, int src, const CUtensorMap &mk, const CUtensorMap &mv, const CUtensorMap &mq,
                           cudaStream_t s)
 {
-    const bool two = p.tiles_per_split > kTcMaxTiles;
-    if (src == 1) return two ? launch_tc_one<G, 1, true>(p, heads, mk, mv, mq, s) : launch_tc_one<G, 1, false>(p, heads, mk, mv, mq, s);
-    if (src == 2) return two ? launch_tc_one<G, 2, true>(p, heads, mk, mv, mq, s) : launch_tc_one<G, 2, false>(p, heads, mk, mv, mq, s);
-    return two ? launch_tc_one<G, 0, true>(p, heads, mk, mv, mq, s) : launch_tc_one<G, 0, false>(p, heads, mk, mv, mq, s);
+    return src == 1 ? launch_tc_form<G, 1>(p, heads, mk, mv, mq, s) : src == 2 ? launch_tc_form<G, 2>(p, heads, mk, mv, mq, s)
+                                                                           : launch_tc_form<G, 0>(p, heads, mk, mv, mq, s);
 }
 
 }  // namespace

@@ -165,3 +165,43 @@ def test_stages_read_their_inputs_when_they_run(rkv, head_dim, dtype, budget, bu
                       gpu_seq=wl.seq_lens, gpu_scores=comp.scores, **{**DEFAULTS, "beta": beta, "T": T})
     assert rep.ok(), rep.errors
     assert rep.compressed_heads == 2 * sum(L > budget for L in lens)
+
+
+@pytest.mark.parametrize("dtype,head_dim,hq", [("bf16", 128, 4), ("fp8", 128, 3), ("bf16", 64, 8)])
+@pytest.mark.parametrize("heads,cap", [(8, 1152), (32, 1152), (128, 2176), (296, 2176), (148, 4224), (600, 384)])
+@pytest.mark.parametrize("paged", [False, True])
+def test_decode_attention_forms(rkv, dtype, head_dim, hq, heads, cap, paged):  # noqa: F811
+    """Small grids that fetch before they know the length, large ones, blocks of two chunks: empty sequences, splits without a row, pages
+    that a short sequence does not have (-1 in its table).  Weights are carried to 2^-17 each, sums in fp32: that much of the largest output, against 64 bits."""
+    import numpy as np
+    import oracle
+    from parity_util import random_block_table, to_paged
+    spec = ri.CacheSpec("forms", 1, heads // 2, 2, 2 * hq, head_dim, cap - 64, 64, 8, 0.1, dtype, 16, 0.3, 0.05, 4, 8.0)
+    some = [cap, 0, 1, cap - 1, 128, 129, 0, cap // 2, 300, cap // 2 + 1]
+    lens = [min(some[b % len(some)], cap) for b in range(heads // 2)]
+    wl = ri.make_workload(spec, device="cuda", seed=621, seq_lens=torch.tensor(lens))
+    raw, nan = (torch.int16, 0x7FC0) if dtype == "bf16" else (torch.uint8, 0x7F)
+    for b, L in enumerate(lens):
+        for t in (wl.k_cache, wl.v_cache):
+            t.view(raw)[b, :, L:] = nan
+    k, v, more = wl.k_cache, wl.v_cache, {}
+    if paged:
+        pages = cap // 128
+        table = random_block_table(heads // 2, 2, pages, heads * pages + 7, seed=9)
+        k, v = (to_paged(t.view(raw), heads * pages + 7, table, fill=nan).view(t.dtype) for t in (k, v))
+        for b, L in enumerate(lens):
+            table[b, :, -(-L // 128):] = -1
+        more = dict(block_table=table, pool_pages=heads * pages + 7)
+    q_new = torch.randn(heads // 2, 2 * hq, head_dim, generator=torch.Generator(device="cuda").manual_seed(7), device="cuda").to(torch.bfloat16)
+    comp = rkv.Compressor(heads // 2, 2, 2 * hq, spec.budget, spec.buffer, spec.alpha, 0.1, dtype=spec.torch_dtype, head_dim=head_dim, **more)
+    out = torch.full((heads // 2, 2 * hq, head_dim), 7.0, device="cuda")
+    assert rkv.rkv_decode_attention(comp.desc, k, v, q_new, wl.seq_lens, out, spec.budget, spec.buffer) == 0
+    torch.cuda.synchronize()
+    comp.check_status()
+    rows = list(range(min(10, heads // 2))) + list(range(10, heads // 2, 17))
+    K, V = (torch.nan_to_num(t[rows].float(), nan=0.0).cpu().numpy() for t in (wl.k_cache, wl.v_cache))
+    ref = oracle.oracle_decode_attention(K, V, q_new[rows].float().cpu().numpy(), np.array([lens[r] for r in rows], dtype=np.int32))
+    got = out[rows].cpu().numpy().astype(np.float64)
+    err = np.abs(got - ref).max() / np.abs(ref).max()
+    assert np.isfinite(got).all() and err <= 2.0 ** -17, err
+    assert all(np.all(got[i] == 0.0) for i, r in enumerate(rows) if lens[r] == 0)
