@@ -60,9 +60,9 @@ struct Form {
 enum {
     kBarFull = 0,                            // [kMaxStages] unit landed
     kBarEmpty = kBarFull + kMaxStages,       // [kMaxStages] ... and no longer read (both products; codes: the 4 warps that widened it)
-    kBarQFull = kBarEmpty + kMaxStages,      // [2] a head's queries landed
-    kBarQEmpty = kBarQFull + 2,              // [2] ... no longer read
-    kBarReady = kBarQEmpty + 2,              // [kMaxGroups] r_i (codes: and the operand tile) written by the group's 4 warps
+    kBarQFull = kBarEmpty + kMaxStages,      // [kMaxStages] a head's queries landed
+    kBarQEmpty = kBarQFull + kMaxStages,     // [kMaxStages] ... no longer read
+    kBarReady = kBarQEmpty + kMaxStages,              // [kMaxGroups] r_i (codes: and the operand tile) written by the group's 4 warps
     kBarLogits = kBarReady + kMaxGroups,     // [kMaxGroups] logits in TMEM
     kBarSums = kBarLogits + kMaxGroups,      // [kMaxGroups] key sums in TMEM
     kBarTaken = kBarSums + kMaxGroups,       // [kMaxGroups] both taken out (4 warps)
@@ -71,29 +71,49 @@ enum {
     kNumBars
 };
 
+// How a block's shared memory is cut up.
 struct Plan {
     int stages, q_bytes, off_own, off_q, off_sum, off_bar, off_units, off_misc, total;
 };
-// groups: as many as there are stages at most.  A group waits for unit k by the parity of its stage's phase, which is exact once the unit
-// before in that stage, k - stages, has landed; what a group knows to have landed is everything up to its own unit before, k - groups
-// (its key sums were issued in order).
 template <int D, bool kCodes>
-__host__ __device__ inline Plan make_plan(int q_rows_pad, int groups)
+__host__ __device__ inline Plan make_plan(int q_rows_pad, int groups, int q_bufs)
 {
     Plan pl;
     pl.q_bytes = q_rows_pad * D * 2;
     const int own = kCodes ? groups * kOperandBytes : 0;
-    const int fixed = own + 2 * pl.q_bytes + groups * kSumB + kNumBars * 8 + 16 + (kMaxStages + kMaxGroups) * 16 + 32 + 1024;      // + alignment slack
+    const int fixed = own + q_bufs * pl.q_bytes + groups * kSumB + kNumBars * 8 + 16 + (kMaxStages + kMaxGroups) * 16 + 32 + 1024;      // + alignment slack
     const int stages = (kSmemLimit - fixed) / Form<D, kCodes>::kStageBytes;
     pl.stages = stages > kMaxStages ? kMaxStages : stages;
     pl.off_own = pl.stages * Form<D, kCodes>::kStageBytes;
     pl.off_q = pl.off_own + own;
-    pl.off_sum = pl.off_q + 2 * pl.q_bytes;
+    pl.off_sum = pl.off_q + q_bufs * pl.q_bytes;
     pl.off_bar = pl.off_sum + groups * kSumB;
     pl.off_units = pl.off_bar + (kNumBars * 8 + 15) / 16 * 16;
     pl.off_misc = pl.off_units + (kMaxStages + kMaxGroups) * 16;
     pl.total = pl.off_misc + 32 + 1024;
     return pl;
+}
+// The groups: as many as have room for their accumulators (64 dimensions: three from 64 query rows on, two from 80), and no more than there
+// are stages.  A group waits for unit k by the parity of its stage's phase, which is exact once the unit before in that stage, k -
+// stages, has landed; what a group knows to have landed is everything up to its own unit before, k - groups (its key sums were
+// issued in order).
+//
+// The rings: q_bufs heads' queries and so many units as fit beside them.  A unit can be asked for once its head's queries can, that is
+// when the head q_bufs before it is done with: of heads of u units (q_bufs - 1) u + 1 units can be under way, and no more than there are
+// stages.  The plan is the one with the most units under way, the fewest query blocks among those.
+template <int D, bool kCodes>
+void choose_plan(int q_rows_pad, int units_per_head, int *groups, int *q_bufs)
+{
+    int best = 0;
+    *groups = 1 + std::min(kMaxGroups, (int)kTmemCols / (16 + Form<D, kCodes>::kSub * q_rows_pad));
+    while (best == 0) {
+        --*groups;
+        for (int n = 2; n <= kMaxStages; ++n) {
+            const int stages = make_plan<D, kCodes>(q_rows_pad, *groups, n).stages;
+            const int under_way = std::min(stages, q_rows_pad ? (n - 1) * units_per_head + 1 : stages);
+            if ((stages >= *groups || *groups == 1) && under_way > best) best = under_way, *q_bufs = n;
+        }
+    }
 }
 
 // One unit of the work list: which head-problem, which tiles, how many candidate rows from its first tile on.
@@ -291,13 +311,12 @@ __device__ __forceinline__ void pool_logits(const Params &p, uint32_t qbase, boo
     else pool_any_window(qbase, row_ok, logits, G, p.alpha, p.cap_pad, p.gqa_mean_pool != 0, scale);
 }
 
-// map_k: the stored keys.  map_wide, copy: see above.  q_rows_pad: 0 where another kernel forms the logits.  table: the block table of
-// the stored keys.  groups: as many as have room for their accumulators (64 dimensions: three from 64 query rows on, two from 80), and for
-// no fewer ring stages (codes: three from 48 query rows on).
+// map_k: the stored keys.  map_wide, copy: see above.  table: the block table of the stored keys.  q_rows_pad: 0 where another kernel forms the
+// logits.  groups, q_bufs: see choose_plan.
 template <int D, bool kCodes>
 __global__ void __launch_bounds__(kThreads, 1)
 prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_q,
-                  const __grid_constant__ CUtensorMap map_wide, const int32_t *table, int copy, int total, int q_rows_pad, int groups)
+                  const __grid_constant__ CUtensorMap map_wide, const int32_t *table, int copy, int total, int q_rows_pad, int groups, int q_bufs)
 {
     using F = Form<D, kCodes>;
     constexpr int kSub = F::kSub;
@@ -305,7 +324,7 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
     extern __shared__ uint8_t prep_raw[];
     uint8_t *smem = align_smem(prep_raw);
     const uint32_t sbase = smem_u32(smem);
-    const Plan pl = make_plan<D, kCodes>(q_rows_pad, groups);
+    const Plan pl = make_plan<D, kCodes>(q_rows_pad, groups, q_bufs);
     const uint32_t stages = (uint32_t)pl.stages;
     int *misc = reinterpret_cast<int *>(smem + pl.off_misc);           // TMEM base, abort flag, units and query blocks asked for
     volatile int *abort_flag = misc + 1;
@@ -321,8 +340,6 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
         for (int s = 0; s < kMaxStages; ++s) {
             mbar_init(bar(kBarFull + s), 1);
             mbar_init(bar(kBarEmpty + s), kCodes ? 4 : 2);
-        }
-        for (int s = 0; s < 2; ++s) {
             mbar_init(bar(kBarQFull + s), 1);
             mbar_init(bar(kBarQEmpty + s), 1);
         }
@@ -350,6 +367,8 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(misc);
+    // (The next kernel is let in by this one's end: a head's sums waiting beside the last units cost 256 heads of 9 tiles 123.0 us a call, 121.4
+    // without; 1024 of 2 tiles 124.0, 122.6.)
     pdl_wait();                             // the set-up above touches no global memory
     if (!p.lengths_done) clear_counters(p);
 
@@ -359,7 +378,7 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
             auto row0 = [&](int head, int tile) -> int {
                 return table ? table[(size_t)head * (p.cap / kTile) + tile] * kTile : head * p.cap + tile * kTile;
             };
-            int q_head = -1, qn = 0, k = 0, seq = -1;
+            int q_head = -1, qn = 0, qb = 0, q_phase = 1, k = 0, seq = -1;
             PrepUnit w = prep_unit_at<kSub>(p, first, false);
             for (; k < units; ++k) {
                 const uint32_t s = (uint32_t)k % stages, full = bar(kBarFull + s);
@@ -381,16 +400,6 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
                     mbar_arrive(full);
                     continue;
                 }
-                if (q_rows_pad && w.head != q_head) {
-                    if (!mbar_wait(bar(kBarQEmpty + (qn & 1)), ((qn >> 1) & 1) ^ 1, abort_flag, sink)) break;
-                    const uint32_t q_full = bar(kBarQFull + (qn & 1)), dst = sbase + pl.off_q + (qn & 1) * pl.q_bytes;
-                    const int q_row = (w.head / p.hkv * p.hq + w.head % p.hkv * p.group) * p.alpha;
-                    mbar_expect_tx(q_full, (uint32_t)pl.q_bytes);
-#pragma unroll
-                    for (int x = 0; x < D / 64; ++x) tma_load_2d(dst + x * q_rows_pad * 128, &map_q, x * 64, q_row, q_full);
-                    q_head = w.head;
-                    ++qn;
-                }
                 const bool both = kSub == 1 || w.rows_here > kTile;
                 const uint32_t dst = sbase + s * F::kStageBytes;
                 const int y = row0(w.head, w.tile);
@@ -398,18 +407,31 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
                 tma_load_2d(dst, &map_k, 0, y, full);
                 if (D == 128 && !kCodes) tma_load_2d(dst + kBoxBytes, &map_k, 64, y, full);
                 if (kSub == 2 && both) tma_load_2d(dst + kBoxBytes, &map_k, 0, row0(w.head, w.tile + 1), full);
+                if (q_rows_pad && w.head != q_head) {         // (the keys first: they do not wait for a query block to come free)
+                    if (!mbar_wait(bar(kBarQEmpty + qb), (uint32_t)q_phase, abort_flag, sink)) {
+                        ++k;                                  // the unit's keys are under way
+                        break;
+                    }
+                    const uint32_t q_full = bar(kBarQFull + qb), q_dst = sbase + pl.off_q + qb * pl.q_bytes;
+                    const int q_row = (w.head / p.hkv * p.hq + w.head % p.hkv * p.group) * p.alpha;
+                    mbar_expect_tx(q_full, (uint32_t)pl.q_bytes);
+#pragma unroll
+                    for (int x = 0; x < D / 64; ++x) tma_load_2d(q_dst + x * q_rows_pad * 128, &map_q, x * 64, q_row, q_full);
+                    q_head = w.head;
+                    ++qn;
+                    if (++qb == q_bufs) qb = 0, q_phase ^= 1;
+                }
             }
             misc[2] = k;
             misc[3] = qn;
-            pdl_trigger();                  // nothing is left to ask for: the next kernel may be let in
         }
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------------ products for the logits
         if (lane == 0) {
             const uint32_t idesc_q = instr_desc(kTile, q_rows_pad);
-            int q_head = -1, qn = 0, g = 0;
-            uint32_t turn = 0, s = 0, round = 0;
+            int q_head = -1, q_next = 0, q_phase = 0, g = 0;
+            uint32_t turn = 0, s = 0, round = 0, q_bar = 0, q = 0;
             for (int k = 0; k < units; ++k) {
                 if (!(kCodes ? mbar_wait(bar(kBarReady + g), turn & 1u, abort_flag, sink) : mbar_wait(bar(kBarFull + s), round & 1u, abort_flag, sink))) break;
                 const int4 w = kCodes ? group_unit[g] : unit_at[s];
@@ -419,14 +441,15 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
                     if (!kCodes) mbar_arrive(bar(kBarEmpty + s));
                 } else {
                     if (w.x != q_head) {
-                        if (qn > 0) umma_commit(bar(kBarQEmpty + ((qn - 1) & 1)));       // the head before is through
-                        if (!mbar_wait(bar(kBarQFull + (qn & 1)), (qn >> 1) & 1, abort_flag, sink)) break;
+                        if (!mbar_wait(bar(kBarQFull + q_next), (uint32_t)q_phase, abort_flag, sink)) break;
                         q_head = w.x;
-                        ++qn;
+                        q_bar = bar(kBarQEmpty + q_next);
+                        q = sbase + pl.off_q + q_next * pl.q_bytes;
+                        if (++q_next == q_bufs) q_next = 0, q_phase ^= 1;
                     }
                     tc_fence_after();
                     const uint32_t tile = kCodes ? sbase + pl.off_own + g * kOperandBytes : sbase + s * F::kStageBytes;
-                    const uint32_t q = sbase + pl.off_q + ((qn - 1) & 1) * pl.q_bytes, d_tmem = tmem + g * group_cols + 16u;
+                    const uint32_t d_tmem = tmem + g * group_cols + 16u;
                     if (D == 64) {
                         umma_tile_k64(d_tmem, tile, q, idesc_q);
                         if (w.w > kTile) umma_tile_k64(d_tmem + (uint32_t)q_rows_pad, tile + kBoxBytes, q, idesc_q);
@@ -435,6 +458,7 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
                     }
                     umma_commit(bar(kBarLogits + g));
                     if (!kCodes) umma_commit(bar(kBarEmpty + s));
+                    if ((w.y + kSub) * kTile >= w.z) umma_commit(q_bar);         // the head's last candidates
                 }
                 if (++g == groups) g = 0, ++turn;
                 if (++s == stages) s = 0, ++round;
@@ -607,7 +631,7 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
         }
         if (threadIdx.x == 0) {
             for (int k = max(misc[2] - (int)stages, 0); k < misc[2]; ++k) drain(bar(kBarFull + (uint32_t)k % stages), ((uint32_t)k / stages) & 1u);
-            for (int q = max(misc[3] - 2, 0); q < misc[3]; ++q) drain(bar(kBarQFull + (q & 1)), (q >> 1) & 1);
+            for (int q = max(misc[3] - q_bufs, 0); q < misc[3]; ++q) drain(bar(kBarQFull + q % q_bufs), (uint32_t)(q / q_bufs) & 1u);
             for (int k = 0; k < units; ++k) {
                 const PrepUnit w = prep_unit_at<kSub>(p, first + k, !p.lengths_done);
                 for (int u = 0; u < kSub && w.tile + u < p.tiles; ++u) p.inv_norm[(size_t)w.head * p.cap_pad + (w.tile + u) * kTile] = kGaveUp;
@@ -641,10 +665,10 @@ cudaError_t launch_for(const Params &p, cudaStream_t s)
     if (!ok) return cudaErrorInvalidValue;
     if (!copy) map_wide = map_k;
     const int total = (p.tiles + F::kSub - 1) / F::kSub * p.batch * p.hkv;
-    int groups = std::min(kMaxGroups, (int)kTmemCols / (16 + F::kSub * q_rows_pad));
-    while (groups > 1 && make_plan<D, kCodes>(q_rows_pad, groups).stages < groups) --groups;
-    return launch_early(prep_sm100_kernel<D, kCodes>, (unsigned)std::min(total, sms), kThreads, (size_t)make_plan<D, kCodes>(q_rows_pad, groups).total, s, 1, p,
-                        map_k, map_q, map_wide, table, copy, total, q_rows_pad, groups);
+    int groups = 1, q_bufs = 2;
+    choose_plan<D, kCodes>(q_rows_pad, (p.tiles + F::kSub - 1) / F::kSub, &groups, &q_bufs);
+    return launch_early(prep_sm100_kernel<D, kCodes>, (unsigned)std::min(total, sms), kThreads, (size_t)make_plan<D, kCodes>(q_rows_pad, groups, q_bufs).total, s,
+                        1, p, map_k, map_q, map_wide, table, copy, total, q_rows_pad, groups, q_bufs);
 }
 
 }  // namespace

@@ -38,6 +38,22 @@ def test_logits_where_blocks_take_many_units(rkv, head_dim, dtype, hq):  # noqa:
     comp.check_status()
 
 
+@pytest.mark.parametrize("hq", [8, 32, 112])
+@pytest.mark.parametrize("head_dim,dtype", [(64, "bf16"), (128, "bf16"), (128, "fp8")])
+@pytest.mark.parametrize("budget,buffer", [(60, 36), (200, 184), (420, 92)])
+def test_logits_of_short_heads(rkv, head_dim, dtype, hq, budget, buffer):  # noqa: F811
+    """2400 heads of one, three and four tiles (64 dimensions: one or two units): as many heads' queries are under way as the ring of units
+    reaches over; sequences that are not compressed, whose queries nobody asks for, lie between the others."""
+    cap = budget + buffer
+    some = [cap, budget + 1, budget, cap - 1, 3, cap, 0, budget + buffer // 2]
+    lens = [some[b % 7 if b < 280 else 2] for b in range(300)]
+    spec = small_spec("short", batch=300, hkv=8, hq=hq, budget=budget, buffer=buffer, head_dim=head_dim, dtype=dtype, span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=555 + budget, seq_lens=torch.tensor(lens))
+    rep, comp = run_and_check(rkv, wl, check_rows=[0, 1, 2, 3, 5, 100, 101, 150, 199, 278, 279, 299])
+    assert rep.ok(), rep.errors
+    comp.check_status()
+
+
 @pytest.mark.parametrize("beta,T", [(1, 0.5), (1, 0.95), (3, 0.5), (1, 1.0)])
 @pytest.mark.parametrize("budget,buffer,lens", [(100, 28, [128, 127, 101]), (100, 36, [136, 135, 101]), (1500, 164, [1664, 1545, 1501])])
 def test_codes_scored_as_they_are_stored(rkv, beta, T, budget, buffer, lens):  # noqa: F811
