@@ -136,7 +136,6 @@ scores_dense_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 mbar_arrive(bar(L::kBarQFull + qs));
                 ++k_item;
             }
-            pdl_trigger();                  // no item is left: the next kernel may be let in
             if (!*abort_flag) {             // terminator (skipped when the block is aborting)
                 const uint32_t qs = k_item % kItemSlotsD;
                 if (mbar_wait(bar(L::kBarQEmpty + qs), ((k_item / kItemSlotsD) & 1) ^ 1, abort_flag, sink)) {

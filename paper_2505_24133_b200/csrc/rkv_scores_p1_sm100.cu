@@ -192,7 +192,6 @@ scores_stream_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, 
                 }
                 ++k_item;
             }
-            pdl_trigger();                  // no item is left: the next kernel may be let in
             // terminator: tells the other roles that no item follows (skipped when the block is aborting)
             if (!*abort_flag) {
                 const uint32_t slot = k_item & 1;

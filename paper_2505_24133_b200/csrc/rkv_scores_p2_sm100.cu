@@ -233,7 +233,6 @@ scores_pass2_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, c
                 for (int it = 0; k_item < 2 && (desc.z >> 16) >= 4 && it < 4; ++it) prefetch_tile(desc.x, desc.w - it);
                 ++k_item;
             }
-            pdl_trigger();                  // no item is left: the next kernel may be let in
             // terminator: tells the other roles that no item follows (skipped when the block is aborting)
             if (!*abort_flag) {
                 const uint32_t qs = k_item % kItemSlots;
