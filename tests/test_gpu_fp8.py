@@ -266,9 +266,9 @@ def test_fp8_every_code_through_the_attention_and_the_widening_kernels(rkv):
 
 @pytest.mark.parametrize("dtype,head_dim", [("fp8", 128), ("bf16", 64)])
 def test_scoring_copy_with_budgets_and_pages(rkv, dtype, head_dim):
-    """The prep kernel that writes the scoring copy itself (8-bit codes of 128 dimensions, bf16 keys of 64; capacity a
-    whole number of tiles), together with per-sequence budgets and a block table: the stored tiles are fetched through
-    the table, the copy is contiguous, the compaction moves the stored rows page by page."""
+    """Keys scored as they are stored (8-bit codes of 128 dimensions, bf16 keys of 64; capacity a whole number of tiles), together
+    with per-sequence budgets and a block table: the stored tiles are fetched through the table, the compaction moves the
+    stored rows page by page."""
     budget, buffer = 896, 128
     lens = [1024, 1000, 600, 1024]
     budgets = [896, 700, 896, 512]

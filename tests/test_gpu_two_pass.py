@@ -3,7 +3,7 @@ import pytest
 import torch
 
 import rkv_inputs as ri
-from parity_util import check_batch
+from parity_util import check_batch, pick
 from test_gpu_parity import DEFAULTS, rkv, run_and_check, small_spec  # noqa: F401  (rkv: the fixture)
 
 pytestmark = pytest.mark.gpu
@@ -85,6 +85,39 @@ def test_codes_by_either_route(rkv, budget, buffer):  # noqa: F811
         comp.check_status()
         got.append(idx.clone())
     assert torch.equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("route", ["ROWBLOCK_SCORES", "SIMT_SCORES", "stages"])
+@pytest.mark.parametrize("paged", [False, True])
+def test_copy_where_blocks_take_many_units(rkv, route, paged):  # noqa: F811
+    """The widened copy of 1600 heads of two whole tiles, which the prep kernel writes (also where prep and scores are calls of their own):
+    every group of warps takes several units, so operand tiles are written again behind their own stores; lengths inside
+    a tile, sequences that are not compressed, pages of other owners full of NaN."""
+    from parity_util import from_paged, random_block_table, to_paged
+    budget, buffer, B = 180, 76, 200
+    lens = [(256, 255, 181, 180, 129)[b % 5] for b in range(B)]
+    spec = small_spec("copies", batch=B, hkv=8, hq=8, budget=budget, buffer=buffer, dtype="fp8", span=8)
+    wl = ri.make_workload(spec, device="cuda", seed=577, seq_lens=torch.tensor(lens))
+    k0, v0, q0, s0 = wl.k_cache.clone(), wl.v_cache.clone(), wl.q_window.clone(), wl.seq_lens.clone()
+    k, v, more = wl.k_cache, wl.v_cache, {}
+    if paged:
+        pool_pages = B * 8 * 2 + 11
+        table = random_block_table(B, 8, 2, pool_pages, seed=15)
+        k, v = (to_paged(t.view(torch.uint8), pool_pages, table, fill=0x7F).view(t.dtype) for t in (k, v))
+        more = dict(block_table=table, pool_pages=pool_pages)
+    comp = rkv.Compressor(B, 8, 8, budget, buffer, spec.alpha, spec.lam, dtype=spec.torch_dtype, dump_scores=True,
+                          flags=0 if route == "stages" else getattr(rkv, "RKV_FLAG_" + route), **more)
+    for st in (rkv.RKV_STAGE_PREP, rkv.RKV_STAGE_ALL & ~rkv.RKV_STAGE_PREP) if route == "stages" else (rkv.RKV_STAGE_ALL,):
+        idx = comp.compress(k, v, wl.q_window, wl.seq_lens, stages=st)
+    torch.cuda.synchronize()
+    comp.check_status()
+    if paged:
+        k, v = (from_paged(t.view(torch.uint8), table).view(t.dtype) for t in (k, v))
+    sel = torch.tensor([0, 1, 2, 3, 4, 70, 71, 72, 140, 141, 197, 198, 199], device="cuda")
+    rep = check_batch(*(pick(t, sel) for t in (k0, v0)), q0[sel], s0[sel], budget=budget, alpha=spec.alpha, lam=spec.lam, gpu_idx=idx[sel],
+                      gpu_k=pick(k, sel), gpu_v=pick(v, sel), gpu_seq=wl.seq_lens[sel], gpu_scores=comp.scores[:, sel], **DEFAULTS)
+    assert rep.ok(), rep.errors
+    assert rep.compressed_heads == 8 * sum(lens[i] > budget for i in sel.tolist())
 
 
 @pytest.mark.parametrize("size", [0.0, 1e-3, 1.0, 400.0])
