@@ -223,7 +223,7 @@ __device__ __forceinline__ void widen16(const uint4 &codes, uint4 *lo, uint4 *hi
 // path (__ldg) asks for data that nothing writes from the kernel's first block to its last.  The second pass, the symmetric
 // scan and its finish may use it for keys and norms: they are launched after a listing kernel, which is launched when the
 // first pass is through, and the first pass waited for all that was written before it.
-// The persistent kernels (prep, both passes, the symmetric scan) let nothing in before they end.  Blocks that wait beside them take from
+// The persistent scoring kernels (both passes, the symmetric scan) let nothing in before they end.  Blocks that wait beside them take from
 // them (the symmetric scan of 2048 heads of 4216 tokens, T = 0.9: 5105 us beside waiting blocks, 4764 without), and where there are few
 // heads a pass runs on for long when the first blocks are out of items: a call with 32 heads of 4216 tokens 166 us when the passes let
 // the next kernel in at that point, 147 so; 16 of 1700 98, 89; 32 of 4216 in 8 bits 162, 136; 256 of 1144 128.3, 126.7.

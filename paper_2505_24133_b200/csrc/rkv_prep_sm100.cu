@@ -50,6 +50,10 @@ constexpr int kSumB = 8 * 16 * 32;                         // B operand of the k
 constexpr int kMaxStages = 8;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kSmemLimit = 227 * 1024;
+// From more units a block on the next kernel is let in when nothing is left to ask for, below by this one's end: the head sums waiting
+// beside the last units cost 256 heads of 9 tiles (16 units a block) 123.0 us a call, 121.4 without; 1024 of 2 tiles (14) 124.0, 122.6;
+// of 4096 heads of 33 tiles in 8 bits (913) the stage takes 764 us when they come after it, 747 beside it.
+constexpr int kManyUnits = 32;
 
 template <int D, bool kCodes>
 struct Form {
@@ -60,9 +64,9 @@ struct Form {
 enum {
     kBarFull = 0,                            // [kMaxStages] unit landed
     kBarEmpty = kBarFull + kMaxStages,       // [kMaxStages] ... and no longer read (both products; codes: the 4 warps that widened it)
-    kBarQFull = kBarEmpty + kMaxStages,      // [kMaxStages] a head's queries landed
+    kBarQFull = kBarEmpty + kMaxStages,      // [kMaxStages] a head's queries landed (choose_plan says how many of them are used)
     kBarQEmpty = kBarQFull + kMaxStages,     // [kMaxStages] ... no longer read
-    kBarReady = kBarQEmpty + kMaxStages,              // [kMaxGroups] r_i (codes: and the operand tile) written by the group's 4 warps
+    kBarReady = kBarQEmpty + kMaxStages,     // [kMaxGroups] r_i (codes: and the operand tile) written by the group's 4 warps
     kBarLogits = kBarReady + kMaxGroups,     // [kMaxGroups] logits in TMEM
     kBarSums = kBarLogits + kMaxGroups,      // [kMaxGroups] key sums in TMEM
     kBarTaken = kBarSums + kMaxGroups,       // [kMaxGroups] both taken out (4 warps)
@@ -367,8 +371,6 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(misc);
-    // (The next kernel is let in by this one's end: a head's sums waiting beside the last units cost 256 heads of 9 tiles 123.0 us a call, 121.4
-    // without; 1024 of 2 tiles 124.0, 122.6.)
     pdl_wait();                             // the set-up above touches no global memory
     if (!p.lengths_done) clear_counters(p);
 
@@ -424,6 +426,7 @@ prep_sm100_kernel(Params p, const __grid_constant__ CUtensorMap map_k, const __g
             }
             misc[2] = k;
             misc[3] = qn;
+            if (units > kManyUnits) pdl_trigger();
         }
         __syncwarp();
     } else if (warp == 1) {
