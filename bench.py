@@ -360,8 +360,19 @@ def kernel_table(rkv, timed: Timed, kw, KB, peaks):
     n = spec.cap - spec.alpha
     esz = wl.k_cache.element_size()
     row = spec.head_dim * esz
-    wide_row = spec.head_dim * 2                       # a row of the bf16 scoring copy (8-bit caches)
     P = spec.head_problems
+    # prep: K once, r_i and Kbar_i.Kbar_i out; on the two-pass route the 16-byte slices and the pooled logits as well; a scoring copy,
+    # where one is made, written (by prep itself for whole tiles of 128-dimension codes, else by a pass of its own, and read back)
+    simt, rowblock = (comp_ev.desc.flags & f for f in (rkv.RKV_FLAG_SIMT_SCORES, rkv.RKV_FLAG_ROWBLOCK_SCORES))
+    two_pass = esz < 4 and spec.head_dim != 256 and not simt and not rowblock
+    padded = spec.head_dim == 64 and esz < 4 and rowblock and not simt
+    wide_row = 256 if padded else spec.head_dim * 2
+    if padded or (esz == 1 and not (two_pass and spec.head_dim == 128)):
+        in_prep = esz == 1 and spec.head_dim == 128 and spec.cap % 128 == 0
+        prep_bytes = n * (row + wide_row) if in_prep else spec.cap * (row + wide_row) + n * wide_row
+    else:
+        prep_bytes = n * row
+    prep_bytes += spec.cap * 24 + n * 4 * spec.alpha if two_pass else spec.cap * 8
     T = (n + 127) // 128
     # one tile product = 128 x 128 outputs over K = 128 + 16: the head dimension plus the one extra K = 16 step that
     # folds the threshold test into the accumulator (both scoring passes issue it for every key tile)
@@ -373,10 +384,7 @@ def kernel_table(rkv, timed: Timed, kw, KB, peaks):
     pass2_useful = pairs2 * 2.0 * 128 * (spec.head_dim + 16)     # listed tokens x keys of the streamed tiles x 2 (d + 16)
     # algorithmic work per launch: bytes a kernel has to move / flops it has to execute, nothing it merely could
     work = {
-        # K once; r_i, Kbar_i.Kbar_i, the 16-byte slice and the pooled logits out.  8-bit caches of other than 128 dimensions: their bf16
-        # copy by a pass of its own, which is read back
-        "prep": ("hbm", P * (n * row + spec.cap * (24 + 4 * spec.alpha)) if esz > 1 or spec.head_dim == 128 else
-                 P * (spec.cap * row + spec.cap * wide_row + n * wide_row + spec.cap * (24 + 4 * spec.alpha))),
+        "prep": ("hbm", P * prep_bytes),
         "scores_pass1": ("tensor", pass1_flops),
         "scores_list": ("hbm", P * n / 8),                 # a bit per token (and what it lists)
         "scores_pass2": ("tensor", pass2_flops),

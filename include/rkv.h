@@ -298,8 +298,8 @@ RKV_API int rkv_push_query(const rkv_desc_t *desc, void *q_window, const void *q
  * two bf16 parts, i.e. to fp32 accuracy), softmax in fp32; fp32 caches: fp32 arithmetic throughout.  head_dim 128 (any
  * cache type) or 64 (bf16 caches: tiles padded to 128 on their way to the tensor cores), and G = n_q_heads /
  * n_kv_heads up to 8 (RKV_ERR_UNSUPPORTED otherwise).  The rows of a head are cut into splits (with
- * few head-problems, to fill the GPU; for bf16 and 8-bit caches also whenever budget + buffer exceeds 1920 rows, what one block
- * holds scores for).  Their partial results may go through desc->workspace (always with fp32 caches; with 8-bit caches and
+ * few head-problems, to fill the GPU; for bf16 and 8-bit caches also whenever budget + buffer exceeds 3584 rows, what one block
+ * takes in two chunks).  Their partial results may go through desc->workspace (always with fp32 caches; with 8-bit caches and
  * head_dim 64 where there are many blocks; otherwise they stay in shared memory): rkv_decode_workspace_bytes() says how
  * much a call asks for (0 when the head-problems fill the GPU by themselves and a block holds a head's scores; never more than
  * rkv_workspace_bytes() of the same shape, so one workspace serves both).  Enqueues one or two kernels on `stream`; return codes as for rkv_compress_ex.

@@ -50,8 +50,8 @@ bool needs_copy(const rkv_desc_t *d) { return d->dtype == RKV_FP8_E4M3 || pads_d
 int scoring_dim(const rkv_desc_t *d) { return pads_dim(d) ? kHeadDim : d->head_dim; }
 // bf16 caches of 64 dimensions on the two-pass route: a kernel ahead of prep records the lengths.
 bool lengths_ahead(const rkv_desc_t *d) { return d->head_dim == 64 && use_tri(d) && !needs_copy(d); }
-// Tensor-core scoring of 64 dimensions, by either route.  Its workspace has room for the padded copy, used or not: callers
-// have relied on the size.
+// Tensor-core scoring of 64 dimensions, by either route.  Its workspace has room for the padded copy, used or not: one workspace
+// serves every route, and the stages one by one, at the size that rkv_workspace_bytes() has always told.
 bool tensor64(const rkv_desc_t *d) { return d->head_dim == 64 && !use_simt(d); }
 // Rows of 128 E4M3 codes are scored as they are stored on the two-pass route.  For the other routes the prep kernel writes the widened
 // copy itself (instead of a widening pass in front of it) where the capacity is a whole number of 128-row tiles.
@@ -231,7 +231,8 @@ int run(const rkv_desc_t *d, void *k_cache, void *v_cache, const void *q_window,
         p.fuse_src = stored.k_cache;
         p.fuse_table = stored.block_table;
     }
-    // (launches that callers count on: a kernel of its own records the lengths where the capacity is not a whole number of tiles)
+    // (8-bit codes whose capacity is no whole number of tiles: prep could record the lengths itself; the kernel stands in for the
+    // widening pass of before, so that the number of launches that rkv_launch_count_for() tells stays what it was)
     p.lengths_done = lengths_ahead(d) || (p.codes && lay.cap % kTile != 0) ? 1 : 0;
     if (stages & RKV_STAGE_PREP) {
         if (copies &&

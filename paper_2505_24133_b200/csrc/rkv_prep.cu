@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kPrepThreads, D <= 128 ? 5 : 2) prep_kernel(Pa
 // the streaming kernel), also as three bf16 rows whose sum is s to fp32 accuracy (rows 3..15 of the 16-row block are
 // zero): behind the rows of the last key tile they let the first scoring pass form Kbar_i . s in its own product.
 // kCodes: as E4M3 codes, for keys that are.  A part holds what the parts before it left, 16 times as large: four more bits of the
-// sum each, so that seven hold all that fp32 does, down to components 2^-24 of the largest.
+// sum each, so that seven hold all that fp32 does of components down to 2^-17 of the largest; of smaller ones they leave 2^-42 of the largest.
 template <int D, bool kCodes = false>        // (D >= 64, the most tiles that a head can have)
 __global__ void __launch_bounds__(D) head_sum_kernel(Params p)
 {

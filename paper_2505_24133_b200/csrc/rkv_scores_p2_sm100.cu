@@ -1,4 +1,4 @@
-// Stage "scores", second pass, for bf16 caches: the tokens that the first pass (rkv_scores_p1_sm100.cu) left short
+// Stage "scores", second pass, for bf16 caches of 64 and 128 dimensions and E4M3 codes of 128: the tokens that the first pass (rkv_scores_p1_sm100.cu) left short
 // of partners against the key tiles BELOW the last one, last to first.  tcgen05.mma with TMEM accumulators, fed by
 // TMA, one persistent block per SM.
 //
